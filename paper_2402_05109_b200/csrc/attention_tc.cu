@@ -181,9 +181,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   uint32_t tmem_base;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
 
-  const int nr = min(max((rs.n_rows ? rs.n_rows[b] : rs.tc) - a.row_off, 0), QROWS);
-  const int p_call = rs.pos0[b];                         // first cache slot written by this forward call
-  const int p0 = p_call + a.row_off;                     // first slot of this launch's rows
+  int nr, p_call, p0, seq, q_row0;                       // p_call: first cache slot written by this forward call; p0: first slot of this CTA's rows
+  if (rs.blocks) {
+    const AttBlock blk = rs.blocks[b];
+    seq = blk.seq; q_row0 = blk.row0; nr = min(blk.n, QROWS); p0 = blk.pos0; p_call = blk.call0;
+  } else {
+    seq = b; q_row0 = b * rs.tc + a.row_off;
+    nr = min(max((rs.n_rows ? rs.n_rows[b] : rs.tc) - a.row_off, 0), QROWS);
+    p_call = rs.pos0[b]; p0 = p_call + a.row_off;
+  }
   const int total = p0 + nr;
   const int nt = (total + TILE - 1) / TILE;
   const int tile0 = chunk_first_tile(c, nt, nchunks), tile1 = chunk_first_tile(c + 1, nt, nchunks);
@@ -197,7 +203,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   if (warp == 2) {
     if (lane == 0 && has_work) {
       const uint64_t pol = policy_evict_first(), pol_q = policy_evict_last();
-      const int row0 = (b * H + h) * a.max_seq;
+      const int row0 = (seq * H + h) * a.max_seq;
       auto request_k = [&](int i) {
         const int s = i % NSK;
         const uint32_t k_dst = ring_s + s * C::K_BYTES;
@@ -233,7 +239,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       for (int pl = 0; pl < NP; ++pl)
 #pragma unroll
         for (int hf = 0; hf < C::NHALF; ++hf)
-          tma_load_2d(q_s + pl * C::QP_BYTES + hf * QROWS * 128, &tmQ, h * HD + hf * 64, pl * a.q_plane_rows + b * rs.tc + a.row_off, q_full, pol_q);
+          tma_load_2d(q_s + pl * C::QP_BYTES + hf * QROWS * 128, &tmQ, h * HD + hf * 64, pl * a.q_plane_rows + q_row0, q_full, pol_q);
       // K stage i % NSK was last read by the scores of tile i - NSK (completion i / NSK - 1 of its empty barrier), V stage
       // i % NSV by the P V product of tile i - NSV; whichever ring has room is served first, K ahead of V
       uint32_t idle = 0;
@@ -502,7 +508,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     constexpr int V4 = HD / 4;
     const uint32_t xo_s = ring_s, xml_s = ring_s + QROWS * HD * 4;
     const int d = H * HD;
-    const int rows_cap = min(rs.tc - a.row_off, QROWS);
+    const int rows_cap = rs.blocks ? nr : min(rs.tc - a.row_off, QROWS);
     const int my_rows = rows_cap > c ? (rows_cap - c + nchunks - 1) / nchunks : 0;
     // chunk weights of my rows, normalised: w_c = 2^(m_c - M) / sum_c l_c 2^(m_c - M)  (one thread per row, all (m, l) loads in flight together)
     for (int t = tid; t < my_rows; t += C::NTHREADS) {
@@ -549,7 +555,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         for (int cc = 0; cc < MAX_CHUNKS; ++cc) {
           acc.x += v[ib][cc].x * w[ib][cc]; acc.y += v[ib][cc].y * w[ib][cc]; acc.z += v[ib][cc].z * w[ib][cc]; acc.w += v[ib][cc].w * w[ib][cc];
         }
-        bf16* dst = a.out + ((size_t)b * rs.tc + a.row_off + i) * d + h * HD + k4 * 4;      // rows past nr get zeros
+        bf16* dst = a.out + (size_t)(q_row0 + i) * d + h * HD + k4 * 4;      // rows past nr get zeros
         const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
         *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
         if (a.out_ps) {
@@ -604,9 +610,10 @@ hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc
   AttArgs a{};
   a.rs = rs; a.out = out; a.out_ps = out_ps; a.H = H; a.max_seq = max_seq; a.status = status; a.wait_limit = WAIT_LIMIT;
   a.q_plane_rows = q_rows; a.kv_plane_rows = (int)cache_rows; a.early = stable_lengths ? 1 : 0; a.row_off = row_off;
-  a.nchunks = pick_chunks(H * rs.batch, len_upper, sm_count());
+  const int groups = rs.blocks ? rs.n_blocks : rs.batch;
+  a.nchunks = pick_chunks(H * groups, len_upper, sm_count());
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(H, rs.batch, a.nchunks); cfg.blockDim = dim3(C::NTHREADS); cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
+  cfg.gridDim = dim3(H, groups, a.nchunks); cfg.blockDim = dim3(C::NTHREADS); cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)a.nchunks;
@@ -621,7 +628,7 @@ hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc
 template <int NP>
 hydra_status dispatch(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, RowSet rs, bf16* out, size_t out_ps,
                       int H, int hd, int max_seq, int len_upper, int* status, bool stable_lengths, cudaStream_t st) {
-  const bool wide = rs.tc > 64;
+  const bool wide = rs.blocks ? attention_block_rows(hd, NP) > 64 : rs.tc > 64;
   if (hd == 128 && wide && NP == 2) {
     // Q, P and the rings of two planes for 128 query rows exceed the shared memory of an SM: 64 rows per launch; the rows of
     // an earlier launch are cache rows to a later one (the preceding kernel has appended the K and V rows of the whole chunk)
@@ -640,10 +647,13 @@ hydra_status dispatch(const __half* q, int q_rows, const __half* kc, const __hal
 
 }  // namespace
 
+// Query rows of a packed attention block: two planes of Q, P and the rings for 128 rows exceed an SM's shared memory at head_dim 128.
+int attention_block_rows(int head_dim, int planes) { return head_dim == 128 && planes == 2 ? 64 : 128; }
+
 hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, int planes, RowSet rs,
                                bf16* out, size_t out_ps, int H, int hd, int max_seq, int len_upper, int* status, bool stable_lengths,
                                cudaStream_t st) {
-  if (rs.tc > 128 || (rs.mask && rs.tc > 64) || (planes != 1 && planes != 2)) return HYDRA_ERR_UNSUPPORTED;
+  if ((!rs.blocks && (rs.tc > 128 || (rs.mask && rs.tc > 64))) || (planes != 1 && planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (!tensor_map_encoder_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
   if (((uintptr_t)q | (uintptr_t)kc | (uintptr_t)vc) & 15) return HYDRA_ERR_INVALID;
   return planes == 2 ? dispatch<2>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, hd, max_seq, len_upper, status, stable_lengths, st)

@@ -131,15 +131,29 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+// A run of consecutive prompt rows of one sequence that an attention CTA takes as its query tile (packed row sets).
+struct AttBlock {
+  int seq, row0;           // sequence; the run's first row in the row set
+  int pos0, n;             // cache slot of the first row; rows
+  int call0;               // first cache slot that the forward call writes for this sequence
+  int pad[3];
+};
+
 // Rows of one forward call: `batch` sequences with `tc` row slots each; sequence b uses its first
 // n_rows[b] slots (all tc when n_rows is null).  Row i of b has KV slot pos0[b]+i, rotary position
 // pos0[b]+depth[i] and may attend to cache slots < pos0[b] and to slot pos0[b]+j iff bit j of mask[i].
+// With row_at the set is packed instead: n_packed causal rows back to back, row r = (sequence, cache slot = rotary position),
+// cut into n_blocks attention blocks; the fields above are unused.
 struct RowSet {
   int batch, tc;
   const int* n_rows;      // device [batch] or null
   const int* pos0;        // device [batch]
   const int* depth;       // device [tc]
   const uint64_t* mask;   // device [tc]; null: a causal chunk (row i sees new slots 0..i), bfloat16 model path only
+  const int2* row_at = nullptr;          // device [n_packed]
+  const AttBlock* blocks = nullptr;      // device [n_blocks]
+  int n_packed = 0, n_blocks = 0;
+  __host__ __device__ int rows() const { return row_at ? n_packed : batch * tc; }
 };
 
 }  // namespace hydra

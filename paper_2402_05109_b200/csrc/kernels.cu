@@ -257,8 +257,9 @@ hydra_status residual_rmsnorm(const float* res, const float* part, SplitDesc sd,
 __global__ void rope_table_kernel(RowSet rs, float2* __restrict__ table, int half, float theta) {
   pdl_wait();
   pdl_trigger();
-  int r = blockIdx.x, b = r / rs.tc, i = r % rs.tc;
-  int pos = rs.pos0[b] + rs.depth[i];
+  int r = blockIdx.x, pos;
+  if (rs.row_at) pos = rs.row_at[r].y;
+  else pos = rs.pos0[r / rs.tc] + rs.depth[r % rs.tc];
   for (int j = threadIdx.x; j < half; j += blockDim.x) {
     double inv = exp2(-((double)j / (double)half) * log2((double)theta));
     double s, c;
@@ -267,7 +268,7 @@ __global__ void rope_table_kernel(RowSet rs, float2* __restrict__ table, int hal
   }
 }
 hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cudaStream_t st) {
-  launch_pdl(rope_table_kernel, dim3(rs.batch * rs.tc), dim3(64), 0, st, rs, table, head_dim / 2, theta);
+  launch_pdl(rope_table_kernel, dim3(rs.rows()), dim3(64), 0, st, rs, table, head_dim / 2, theta);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -283,11 +284,18 @@ __global__ void __launch_bounds__(256) qkv_rope_store_kernel(const float* __rest
                                                              int* status) {
   pdl_trigger();
   pdl_wait();
-  const int r = blockIdx.x, b = r / rs.tc, i = r % rs.tc;
-  const int nr = rs.n_rows ? rs.n_rows[b] : rs.tc;
-  if (i >= nr) return;
+  const int r = blockIdx.x;
+  int b, slot;
+  if (rs.row_at) {
+    const int2 at = rs.row_at[r];
+    b = at.x; slot = at.y;
+  } else {
+    const int i = r % rs.tc;
+    b = r / rs.tc;
+    if (i >= (rs.n_rows ? rs.n_rows[b] : rs.tc)) return;
+    slot = rs.pos0[b] + i;
+  }
   const int d = H * hd, half = hd >> 1;
-  const int slot = rs.pos0[b] + i;
   if (slot < 0 || slot >= max_seq) { if (threadIdx.x == 0 && blockIdx.y == 0) atomicOr(status, ST_BOUNDS); return; }
   const int tph = half >> 2;                                       // threads per head
   const int h = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
@@ -329,7 +337,7 @@ hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table
   // 128 threads per CTA: with 64 rows twice as many SMs pull the partial sums as with 256
   const int threads = 128 % (hd / 8) == 0 ? 128 : 256;
   const int heads_per_block = threads / (hd / 8);
-  dim3 grid(rs.batch * rs.tc, (H + heads_per_block - 1) / heads_per_block);
+  dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block);
   if (dtype == 0)
     launch_pdl(qkv_rope_store_kernel<float>, grid, dim3(threads), 0, st, part, sd, table, (float*)q, q_ps, (float*)kcache, (float*)vcache,
                kv_ps, rs, H, hd, max_seq, status);
@@ -999,6 +1007,40 @@ __global__ void capture_last_kernel(const float* h, const int* prompt_len, int c
 hydra_status capture_last(const float* h, const int* prompt_len, int chunk, int tc, float* h_new, int kp1, int* n_new,
                           int* len, int batch, int d, cudaStream_t st) {
   launch_pdl(capture_last_kernel, dim3(batch), dim3(256), 0, st, h, prompt_len, chunk, tc, h_new, kp1, n_new, len, d);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
+}
+
+// Packed prompts: token g of the concatenated prompts (base = offsets[0]) is a slot of the sequence b whose range holds it.
+__global__ void pack_rows_kernel(const int* offsets, int batch, int2* row_at, int base, int total) {
+  pdl_trigger();
+  pdl_wait();
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= total) return;
+  int b = 0;
+  while (b + 1 < batch && offsets[b + 1] - base <= g) ++b;
+  row_at[g] = make_int2(b, g - (offsets[b] - base));
+}
+hydra_status pack_rows(const int* offsets, int batch, int2* row_at, int base, int total, cudaStream_t st) {
+  launch_pdl(pack_rows_kernel, dim3((total + 255) / 256), dim3(256), 0, st, offsets, batch, row_at, base, total);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
+}
+
+// h holds the hidden rows of tokens g0 .. g0+rows-1 of the concatenated prompts
+__global__ void capture_last_packed_kernel(const float* h, const int* offsets, int g0, int rows, float* h_new, int kp1, int* n_new,
+                                           int* len, int d) {
+  pdl_trigger();
+  pdl_wait();
+  const int b = blockIdx.x, i = offsets[b + 1] - 1 - g0;
+  if (i < 0 || i >= rows) return;
+  for (int c = threadIdx.x * 4; c < d; c += blockDim.x * 4)                                  // d % 4 == 0
+    *reinterpret_cast<float4*>(h_new + (size_t)b * kp1 * d + c) = *reinterpret_cast<const float4*>(h + (size_t)i * d + c);
+  if (threadIdx.x == 0) { n_new[b] = 1; len[b] = offsets[b + 1] - offsets[b]; }
+}
+hydra_status capture_last_packed(const float* h, const int* offsets, int g0, int rows, float* h_new, int kp1, int* n_new, int* len,
+                                 int batch, int d, cudaStream_t st) {
+  launch_pdl(capture_last_packed_kernel, dim3(batch), dim3(256), 0, st, h, offsets, g0, rows, h_new, kp1, n_new, len, d);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

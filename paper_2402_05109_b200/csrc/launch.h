@@ -44,6 +44,7 @@ hydra_status tree_attention_f32(const float* q, const float* kcache, const float
 // [planes][cache_batch][H][max_seq][hd] are float16 in 1 or 2 planes (hi = f16(v), lo = f16(v - hi)); out is bfloat16
 // [rows][H*hd] in two planes out_ps elements apart (0: hi only).  rs.mask == null selects a causal chunk (row i sees
 // the committed slots and new slots 0..i) of up to 128 rows (one plane, or head_dim 64); with a mask, up to 64 rows.
+// A packed row set runs one CTA column per attention block of at most attention_block_rows(...) rows.
 // stable_lengths: rs.pos0 / rs.n_rows and every cache row below pos0 were written by kernels that had COMPLETED before the
 // kernel preceding this one in the stream started (true inside a forward call of the library, whose first kernel holds
 // its successors back until everything earlier has completed); the kernel then requests committed cache tiles before it
@@ -51,6 +52,7 @@ hydra_status tree_attention_f32(const float* q, const float* kcache, const float
 hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, int planes, RowSet rs,
                                bf16* out, size_t out_ps, int n_heads, int head_dim, int max_seq, int len_upper, int* status,
                                bool stable_lengths, cudaStream_t st);
+int attention_block_rows(int head_dim, int planes);
 hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, int dtype,
                       cudaStream_t st);
 // amax[r] = argmax_v of the summed partial logits (lowest id among equal maxima); the sums go to logits_out if given
@@ -108,6 +110,11 @@ hydra_status gather_chunk_tokens(const int* tokens, const int* offsets, int chun
 // for sequences whose last prompt row lies in this chunk: h_new[b][0] = h[b*tc + i], n_new = 1, len = prompt_len
 hydra_status capture_last(const float* h, const int* prompt_len, int chunk, int tc, float* h_new, int kp1, int* n_new,
                           int* len, int batch, int d, cudaStream_t st);
+// packed prompts (bfloat16 path): row_at[g] = (sequence, slot) of token g of the concatenated prompts
+hydra_status pack_rows(const int* offsets, int batch, int2* row_at, int base, int total, cudaStream_t st);
+// capture_last for a packed pass over tokens g0 .. g0+rows-1
+hydra_status capture_last_packed(const float* h, const int* offsets, int g0, int rows, float* h_new, int kp1, int* n_new, int* len,
+                                 int batch, int d, cudaStream_t st);
 // pos0[b] = len[b] - n_new[b]; n_rows[b] = n_new[b]
 hydra_status prefix_rowset(const int* len, const int* n_new, int* pos0, int* n_rows, int batch, cudaStream_t st);
 // hprime[b] = x[b*tc + n_rows[b]-1]

@@ -2,6 +2,7 @@
 // not the tensor-core GEMM).  float or bfloat16 storage, float arithmetic.
 #include "launch.h"
 #include <math.h>
+#include <vector>
 
 namespace hydra {
 
@@ -948,15 +949,41 @@ hydra_status softmax_row_stats(const float* logits, float4* row_stats, int rows,
   return HYDRA_OK;
 }
 
-hydra_status accept_compact(const AcceptArgs& a, cudaStream_t st) {
+static dim3 accept_grid(const AcceptArgs& a) {
   long long units = (long long)a.n_layers * 2 * a.kv_planes * a.n_heads * (a.head_dim * a.esize / 16);
   int G = (int)((units + 255) / 256);
   int cap = (sm_count() * 4 + a.batch - 1) / a.batch;
   if (G > cap) G = cap;
   if (G < 1) G = 1;
-  launch_pdl(accept_compact_kernel, dim3(dim3(G, a.batch)), dim3(256), 0, st, a);
+  return dim3(G, a.batch);
+}
+hydra_status accept_compact(const AcceptArgs& a, cudaStream_t st) {
+  launch_pdl(accept_compact_kernel, accept_grid(a), dim3(256), 0, st, a);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
+}
+cudaError_t accept_graph_node(cudaGraph_t graph, cudaGraphNode_t* node) {
+  size_t n = 0;
+  cudaError_t e = cudaGraphGetNodes(graph, nullptr, &n);
+  if (e != cudaSuccess) return e;
+  std::vector<cudaGraphNode_t> nodes(n);
+  if ((e = cudaGraphGetNodes(graph, nodes.data(), &n)) != cudaSuccess) return e;
+  for (size_t i = n; i-- > 0;) {                           // the last launch of a step
+    cudaGraphNodeType t;
+    cudaKernelNodeParams p{};
+    if ((e = cudaGraphNodeGetType(nodes[i], &t)) != cudaSuccess) return e;
+    if (t != cudaGraphNodeTypeKernel) continue;
+    if ((e = cudaGraphKernelNodeGetParams(nodes[i], &p)) != cudaSuccess) return e;
+    if (p.func == (void*)accept_compact_kernel) { *node = nodes[i]; return cudaSuccess; }
+  }
+  return cudaErrorInvalidValue;
+}
+cudaError_t accept_graph_update(cudaGraphExec_t exec, cudaGraphNode_t node, const AcceptArgs& a) {
+  AcceptArgs copy = a;
+  void* args[] = {&copy};
+  cudaKernelNodeParams p{};
+  p.func = (void*)accept_compact_kernel; p.gridDim = accept_grid(a); p.blockDim = dim3(256); p.sharedMemBytes = 0; p.kernelParams = args;
+  return cudaGraphExecKernelNodeSetParams(exec, node, &p);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -102,6 +102,9 @@ struct AcceptArgs {
 // row_stats[r] for every logits row (typical acceptance)
 hydra_status softmax_row_stats(const float* logits, float4* row_stats, int rows, int vocab, float tau, cudaStream_t st);
 hydra_status accept_compact(const AcceptArgs& a, cudaStream_t st);
+// the acceptance node of a captured step, and new arguments for it in an instantiated graph
+cudaError_t accept_graph_node(cudaGraph_t graph, cudaGraphNode_t* node);
+cudaError_t accept_graph_update(cudaGraphExec_t exec, cudaGraphNode_t node, const AcceptArgs& a);
 
 // ---- small state kernels
 hydra_status set_chunk(const int* prompt_len, int chunk, int tc, int* pos0, int* n_rows, int batch, cudaStream_t st);

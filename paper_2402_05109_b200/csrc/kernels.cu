@@ -350,27 +350,31 @@ hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table
 }
 
 // ------------------------------------------------------------------------------------------------
-// Tree attention, split over the KV length.  One CTA per (head, sequence, KV chunk); the chunk's K,V
-// rows are read once; every query row keeps an online softmax (running max, sum, weighted V) per warp.
+// Tree attention of the float path, split over the KV length and the query rows.  One CTA per (head, sequence, KV chunk, row
+// group of 8 RPW rows); a warp keeps an online softmax (running max, sum, weighted V) for RPW rows.  The small decoders this
+// path serves have a handful of (head, sequence) pairs and one chunk, so the time is the serial chain inside a warp: few rows
+// per warp spread it over the SMs (each row group reads the chunk's K,V again, out of L2), and with a single chunk the kernel
+// writes the result itself instead of leaving it to the combine kernel.  Measured at 16 rows x 4 heads x 48..80 slots: 28 us with
+// eight consecutive rows per warp and the combine kernel, 10 us now.
 // ------------------------------------------------------------------------------------------------
 constexpr int ATT_CHUNK = ATT_CHUNK_ROWS;
 constexpr int ATT_TILE = 32;      // KV rows staged per iteration
 constexpr int ATT_WARPS = 8;
 
-template <typename T, int HD>
+template <typename T, int HD, int RPW>
 __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc,
                                                                    const T* __restrict__ vc, RowSet rs,
                                                                    float* __restrict__ part_o, float* __restrict__ part_ml,
-                                                                   int H, int max_seq, int nchunks) {
+                                                                   T* __restrict__ out, int H, int max_seq, int nchunks) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ float smem[];
-  constexpr int RPW = 8;                                  // query rows per warp (tc <= 64)
   constexpr int KPL = HD / 32;                            // output dims per lane
-  float* qs = smem;                                       // [64][HD]
-  float* ks = qs + 64 * HD;                               // [ATT_TILE][HD+1]
+  constexpr int ROWS = ATT_WARPS * RPW;                   // query rows of this CTA
+  float* qs = smem;                                       // [ROWS][HD]
+  float* ks = qs + ROWS * HD;                             // [ATT_TILE][HD+1]
   float* vs = ks + ATT_TILE * (HD + 1);                   // [ATT_TILE][HD]
-  const int h = blockIdx.x, b = blockIdx.y, c = blockIdx.z;
+  const int h = blockIdx.x, b = blockIdx.y, c = blockIdx.z % nchunks, r0 = blockIdx.z / nchunks * ROWS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nr = rs.n_rows ? rs.n_rows[b] : rs.tc;
   const int p0 = rs.pos0[b];
@@ -380,16 +384,16 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
   const int d = H * HD;
   const float scale = rsqrtf((float)HD);
 
-  for (int e = threadIdx.x; e < nr * HD; e += blockDim.x) {
-    int i = e / HD, k = e % HD;
-    qs[i * HD + k] = to_f<T>(q[((size_t)(b * rs.tc + i)) * d + h * HD + k]) * scale;
+  for (int e = threadIdx.x * 4; e < min(ROWS, nr - r0) * HD; e += blockDim.x * 4) {
+    const float4 v = load4<T>(q + ((size_t)(b * rs.tc + r0 + e / HD)) * d + h * HD + e % HD);
+    *reinterpret_cast<float4*>(qs + e) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
   }
   float m[RPW], l[RPW], o[RPW][KPL];
   uint64_t msk[RPW];
 #pragma unroll
-  for (int j = 0; j < RPW; ++j) {
+  for (int j = 0; j < RPW; ++j) {                         // row j of this warp: r0 + 8 j + warp
     m[j] = -INFINITY; l[j] = 0.f;
-    int r = warp * RPW + j;
+    const int r = r0 + j * ATT_WARPS + warp;
     msk[j] = r < nr ? rs.mask[r] : 0ull;
 #pragma unroll
     for (int kk = 0; kk < KPL; ++kk) o[j][kk] = 0.f;
@@ -397,25 +401,26 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
   const T* kbase = kc + ((size_t)b * H + h) * max_seq * HD;
   const T* vbase = vc + ((size_t)b * H + h) * max_seq * HD;
 
-  for (int t0 = s0; t0 < s1; t0 += ATT_TILE) {
+  for (int t0 = s0; t0 < s1 && r0 < nr; t0 += ATT_TILE) {
     __syncthreads();
-    for (int e = threadIdx.x; e < ATT_TILE * HD; e += blockDim.x) {
-      int j = e / HD, k = e % HD;
-      int slot = t0 + j;
-      float kv = 0.f, vv = 0.f;
-      if (slot < s1) { kv = to_f<T>(kbase[(size_t)slot * HD + k]); vv = to_f<T>(vbase[(size_t)slot * HD + k]); }
-      ks[j * (HD + 1) + k] = kv;
-      vs[j * HD + k] = vv;
+#pragma unroll
+    for (int e = threadIdx.x * 4; e < ATT_TILE * HD; e += ATT_WARPS * 32 * 4) {
+      const int j = e / HD, k = e % HD, slot = t0 + j;
+      float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
+      if (slot < s1) { kv = load4<T>(kbase + (size_t)slot * HD + k); vv = load4<T>(vbase + (size_t)slot * HD + k); }
+      float* kd = ks + j * (HD + 1) + k;
+      kd[0] = kv.x; kd[1] = kv.y; kd[2] = kv.z; kd[3] = kv.w;
+      *reinterpret_cast<float4*>(vs + e) = vv;
     }
     __syncthreads();
     const int slot = t0 + lane;
 #pragma unroll
     for (int j = 0; j < RPW; ++j) {
-      const int r = warp * RPW + j;
+      const int r = r0 + j * ATT_WARPS + warp;
       if (r >= nr) continue;
       bool valid = slot < s1 && (slot < p0 || ((msk[j] >> (slot - p0)) & 1ull));
       float sc = 0.f;
-      const float* qr = qs + r * HD;
+      const float* qr = qs + (r - r0) * HD;
       const float* kr = ks + lane * (HD + 1);
 #pragma unroll 8
       for (int k = 0; k < HD; ++k) sc += qr[k] * kr[k];
@@ -428,6 +433,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
       float acc[KPL];
 #pragma unroll
       for (int kk = 0; kk < KPL; ++kk) acc[kk] = o[j][kk] * alpha;
+#pragma unroll 8
       for (int jj = 0; jj < ATT_TILE; ++jj) {
         float pj = __shfl_sync(0xffffffffu, p, jj);
 #pragma unroll
@@ -440,7 +446,14 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
   }
 #pragma unroll
   for (int j = 0; j < RPW; ++j) {
-    const int r = warp * RPW + j;
+    const int r = r0 + j * ATT_WARPS + warp;
+    if (r >= rs.tc) continue;
+    if (out) {                                            // the only chunk: normalise; rows past nr come out as zeros
+      T* dst = out + (size_t)(b * rs.tc + r) * d + h * HD;
+#pragma unroll
+      for (int kk = 0; kk < KPL; ++kk) dst[lane + 32 * kk] = from_f<T>(r < nr ? o[j][kk] / l[j] : 0.f);
+      continue;
+    }
     if (r >= nr) continue;
     size_t idx = ((size_t)(b * rs.tc + r) * H + h) * nchunks + c;
 #pragma unroll
@@ -479,6 +492,22 @@ size_t attention_scratch_bytes(int batch, int tc, int n_heads, int head_dim, int
   return (size_t)batch * tc * n_heads * nchunks * (head_dim + 2) * sizeof(float);
 }
 
+template <typename T, int HD, int RPW>
+static hydra_status launch_tree_attn(const T* q, const T* kc, const T* vc, RowSet rs, float* part_o, float* part_ml, T* out, int H, int max_seq,
+                                     int nchunks, cudaStream_t st) {
+  const size_t smem = (size_t)(ATT_WARPS * RPW * HD + ATT_TILE * (HD + 1) + ATT_TILE * HD) * sizeof(float);
+  static PerDeviceFlag attr_done;
+  if (!attr_done.get()) {
+    HYDRA_CUDA(cudaFuncSetAttribute(tree_attn_kernel<T, HD, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    attr_done.set();
+  }
+  const int groups = (rs.tc + ATT_WARPS * RPW - 1) / (ATT_WARPS * RPW);
+  launch_pdl(tree_attn_kernel<T, HD, RPW>, dim3(H, rs.batch, nchunks * groups), dim3(ATT_WARPS * 32), smem, st, q, kc, vc, rs, part_o, part_ml,
+             nchunks == 1 ? out : (T*)nullptr, H, max_seq, nchunks);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
+}
+
 template <typename T, int HD>
 static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSet rs, T* out, float* scratch, int H,
                                      int max_seq, int len_upper, cudaStream_t st) {
@@ -489,15 +518,12 @@ static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSe
   size_t rows = (size_t)rs.batch * rs.tc;
   float* part_o = scratch;
   float* part_ml = scratch + rows * H * nchunks_max * HD;
-  size_t smem = (size_t)(64 * HD + ATT_TILE * (HD + 1) + ATT_TILE * HD) * sizeof(float);
-  static PerDeviceFlag attr_done;
-  if (!attr_done.get()) {
-    HYDRA_CUDA(cudaFuncSetAttribute(tree_attn_kernel<T, HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr_done.set();
-  }
-  launch_pdl(tree_attn_kernel<T, HD>, dim3(dim3(H, rs.batch, nchunks)), dim3(ATT_WARPS * 32), smem, st, q, kc, vc, rs, part_o, part_ml, H,
-                                                                                   max_seq, nchunks);
-  HYDRA_LAUNCH_CHECK();
+  // one row per warp while that leaves at most two CTAs per SM; more rows per warp share the staged K,V tile instead
+  const long ctas1 = (long)H * rs.batch * nchunks * ((rs.tc + ATT_WARPS - 1) / ATT_WARPS), cap = 2L * sm_count();
+  if (ctas1 <= cap) HYDRA_TRY((launch_tree_attn<T, HD, 1>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  else if (ctas1 <= 2 * cap) HYDRA_TRY((launch_tree_attn<T, HD, 2>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  else HYDRA_TRY((launch_tree_attn<T, HD, 8>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  if (nchunks == 1) return HYDRA_OK;
   launch_pdl(tree_attn_combine_kernel<T, HD>, dim3(dim3((unsigned)rows, H)), dim3(HD), 0, st, part_o, part_ml, rs, out, H, nchunks);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;

@@ -243,7 +243,8 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  * library image (every GPU that loads the library holds it until the process exits).
  *   - x [m][k], w [n][k] bfloat16, out [m][n] float, status_dev as in hydra_gemm: all caller-owned device
  *     memory; n % 128 == 0, k % 64 == 0.
- *   - hydra_gemm_partial_floats(m, n, k, 1, 0) * 4 bytes must fit in the 8 MiB array, otherwise HYDRA_ERR_CAPACITY (text in
+ *   - m * n * 4 bytes must fit in the 8 MiB array (the work is shared out among as many CTAs as the partial sums in it
+ *     allow), otherwise HYDRA_ERR_CAPACITY (text in
  *     hydra_last_error) and nothing is launched.
  *   - The call allocates nothing on the device.  The first call on each device looks up the array's device
  *     address (cudaGetSymbolAddress, with that device current); make that first call outside any stream

@@ -3,20 +3,18 @@
 //   part[slot][m][n] = sum over one K range of x[m][k] * w[n][k]        (float accumulate, float out)
 //
 // The weight matrix is the large operand (read once from HBM); the activation slab is small (tree rows x
-// batch) and L2 resident.  So the roles are swapped with respect to the usual GEMM: a 128-row weight tile
-// [128 n][64 k] is the MMA "A" operand (M = 128 TMEM lanes), the activation tile [MT rows][64 k] is the "B"
-// operand (N = MT columns).  Both are K-major and land in shared memory through TMA with the 128-byte
-// swizzle; accumulators live in tensor memory.
+// batch) and L2 resident.  So the roles are swapped with respect to the usual GEMM: weight rows [n][64 k] are the MMA "A"
+// operand (M: TMEM lanes), activation rows [64 k] the "B" operand (N: TMEM columns).  Both are K-major and land in shared
+// memory through TMA with the 128-byte swizzle; accumulators live in tensor memory.
 //
 // Work decomposition (stream-K): the (tile, k-block) pairs of the whole GEMM are laid out in one line,
-// tile-major, and cut into equal contiguous ranges, one per CTA (at most one CTA per SM), so that every SM
+// tile-major, and cut into equal contiguous ranges, one per CTA, so that every SM
 // streams the same number of weight bytes without interruption.  A CTA's range covers the tail of one tile,
 // possibly whole tiles, and the head of another; each such run is a "segment" whose partial sum goes to
-// slot (cta - first cta of the tile) of the partial buffer.  The consumer kernel adds the slots of a tile in
+// slot (CTA - first CTA of the tile) of the partial buffer.  The consumer kernel adds the slots of a tile in
 // fixed order (SplitDesc), so results are deterministic.
 //
-// A unit carries NH = 1 or 2 such weight tiles (256 weight rows in one TMA box) that share the unit's activation
-// tile and accumulate side by side in tensor memory: wide outputs use 2.
+// A unit is 64 k of NH = 1 or 2 weight tiles of 128 rows (one TMA box, one accumulator each) that share the activation tile.
 //
 // Warp roles (192 threads): warp 0 = TMA producer (one lane), warp 1 = TMEM allocation + MMA issue (one
 // lane), warps 2..5 = epilogue (TMEM -> registers -> global, coalesced along n).  Two accumulator sets in
@@ -25,7 +23,7 @@
 // before griddepcontrol.wait, activations and all global writes after it.
 // Precision: weights are bfloat16 (exact: the reference model's weights are the same bfloat16 values).  The
 // activation operand comes as TWO bfloat16 planes, hi = bf16(v) and lo = bf16(v - hi), i.e. about 16 mantissa
-// bits; each weight tile is multiplied with both planes into the same accumulator.  This doubles the MMA work
+// bits; each weight tile is multiplied with both planes.  This doubles the MMA work
 // (irrelevant while the kernel is HBM-bound) and the L2-resident activation traffic, not the HBM traffic, and
 // keeps the hidden states within 1e-2 of a float reference over 32+ layers (plain bfloat16 operands drift to
 // 4e-2).  x_lo_rows = 0 selects a single plane.
@@ -93,118 +91,120 @@ constexpr int A_BYTES = BLOCK_N * BLOCK_K * 2;
 // Instruction descriptor: D = f32, A = B = bf16, both K-major, M = 128, N = MT.
 __host__ __device__ constexpr uint32_t instr_desc(int mt) { return instr_desc_f16(1, BLOCK_N, mt, 0); }
 
-// One accumulator buffer (MT columns, plus MT more holding W*lo when `cat`) of this thread's lane -> partial-sum rows
-// m0.. of column dst; 64 columns per batch of tensor-memory loads when the tile has that many.
-template <int MT>
-__device__ __forceinline__ void store_accumulator(uint32_t taddr, bool cat, float* dst, int m0, int m, int n) {
-  if constexpr (MT >= 64) {
+// Accumulator columns of this thread's lane -> rows (distance n) of the partial buffer; with `cat` the W*lo columns, mt further
+// on, are added.  Batches of 32 in a rolled loop: code unrolled for every shape does not
+// stay in the instruction cache, and fetching it is what the epilogue then waits for (64 rows: 5.5 us with 64-column batches
+// and a 16-column remainder unrolled, 1.5 us rolled).  Reads whole batches, so accumulators are spaced accordingly.
+__device__ __forceinline__ void store_accumulator(uint32_t taddr, bool cat, int mt, float* dst, int rows, int n) {
 #pragma unroll 1
-    for (int c = 0; c < MT; c += 64) {
-      if (m0 + c >= m) break;
-      uint32_t r[64];
-      if (cat) {
-        uint32_t r2[64];
-        tmem_ld64x2(taddr + (uint32_t)c, taddr + (uint32_t)(MT + c), r, r2);
+  for (; rows > 0; rows -= 32, taddr += 32u, dst += (size_t)32 * n) {
+    uint32_t r[32];
+    if (cat) {
+      uint32_t r2[32];
+      tmem_ld32x2(taddr, taddr + (uint32_t)mt, r, r2);
 #pragma unroll
-        for (int j = 0; j < 64; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
-      } else {
-        tmem_ld64(taddr + (uint32_t)c, r);
-      }
-#pragma unroll
-      for (int j = 0; j < 64; ++j)
-        if (m0 + c + j < m) __stcg(dst + (size_t)(m0 + c + j) * n, __uint_as_float(r[j]));
+      for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
+    } else {
+      tmem_ld32(taddr, r);
     }
-  } else {
+    float* p = dst;
+#pragma unroll
+    for (int j = 0; j < 32; ++j, p += n)
+      if (j < rows) __stcg(p, __uint_as_float(r[j]));
+  }
+}
+// Up to 16 rows (decoding without a tree, draft levels); one row: all tiles and planes in one tensor-memory round trip.
+template <int NH>
+__device__ __forceinline__ void store_few(uint32_t taddr, int acc_cols, bool cat, int mt, float* dst, int rows, int n, int tiles_in) {
+  const uint32_t lo = cat ? (uint32_t)mt : 0u, t1 = taddr + (uint32_t)(NH == 2 ? acc_cols : 0);
+  if (rows == 1) {
+    uint32_t h0, l0, h1, l1;
+    tmem_ld1x4(taddr, taddr + lo, t1, t1 + lo, h0, l0, h1, l1);
+    __stcg(dst, cat ? __uint_as_float(h0) + __uint_as_float(l0) : __uint_as_float(h0));
+    if (NH == 2 && tiles_in == 2) __stcg(dst + BLOCK_N, cat ? __uint_as_float(h1) + __uint_as_float(l1) : __uint_as_float(h1));
+    return;
+  }
 #pragma unroll 1
-    for (int c = 0; c < MT; c += 16) {
-      if (m0 + c >= m) break;
-      uint32_t r[16];
-      tmem_ld16(taddr + (uint32_t)c, r);
-      if (cat) {                                         // add the W*lo columns
-        uint32_t r2[16];
-        tmem_ld16(taddr + (uint32_t)(MT + c), r2);
+  for (int hh = 0; hh < tiles_in; ++hh, taddr += acc_cols, dst += BLOCK_N) {
+    uint32_t r[16], q[16];
+    tmem_ld16x2(taddr, taddr + lo, r, q);
+    if (!cat) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(r2[j]));
-      }
-#pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (m0 + c + j < m) __stcg(dst + (size_t)(m0 + c + j) * n, __uint_as_float(r[j]));
+      for (int j = 0; j < 16; ++j) q[j] = 0u;
     }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (j < rows) __stcg(dst + (size_t)j * n, __uint_as_float(r[j]) + __uint_as_float(q[j]));
   }
 }
 
-template <int MT, int BUDGET_KB, int NH = 1> struct TileCfg {        // NH: 128-row weight tiles per unit (they share the activation tile)
-  static constexpr int SMEM_BUDGET = BUDGET_KB * 1024;
-  static constexpr int B_PLANE = MT * BLOCK_K * 2;               // one activation plane of a stage
-  static constexpr int B_BYTES = 2 * B_PLANE;                    // hi + lo
-  static constexpr int W_BYTES = NH * A_BYTES;                   // weight rows of a unit: NH * 128
-  static constexpr int STAGE_BYTES = W_BYTES + B_BYTES;
-  static constexpr int STAGES = (SMEM_BUDGET / STAGE_BYTES) > 10 ? 10 : ((SMEM_BUDGET / STAGE_BYTES) < 2 ? 2 : (SMEM_BUDGET / STAGE_BYTES));
-  // Two planes, MT <= 128: the hi and lo activation tiles sit back to back in shared memory and form ONE MMA B
-  // operand of 2*MT rows, so each weight tile is read from shared memory once; accumulator columns [0, MT) hold
-  // W*hi, [MT, 2MT) hold W*lo and the epilogue adds them.  MT = 256: two accumulating passes over the weight tile.
-  static constexpr bool CAT = MT <= 128;
-  static constexpr int ACC_COLS = CAT ? (2 * MT < 32 ? 32 : 2 * MT) : MT;   // columns of one accumulator buffer
-  static constexpr int NBUF = 2 * NH * ACC_COLS <= 512 ? 2 : 1;   // accumulator sets: two when tensor memory allows
-  static constexpr int TMEM_COLS = NBUF * NH * ACC_COLS;          // power of two, <= 512
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
-};
-
 struct GemmArgs {
   float* part; size_t slot_stride;
-  int m, n, kb, n_tiles, total_units, q;
+  int m, n, kb, m_tiles, total_units, q;
   int x_lo_rows;                 // row offset of the lo plane inside the activation tensor map (0: single plane)
+  // activation rows per tile, boxes (planes) of a stage, MMA passes over a weight tile and columns of one, ring stages,
+  // accumulator columns and buffers, tensor-memory columns
+  int mt, x_boxes, passes, mma_n, stages, acc_cols, acc_bufs, tmem_cols;
+  int cat;                       // hi and lo planes are the halves of one MMA operand: columns [mt, 2 mt) hold W*lo
   int* status;
   int* diag;                     // optional int[8]: where the first bounded wait gave up (site, cta, unit, units, grid, m, n, kb)
   uint32_t wait_limit;           // polls before a barrier wait gives up
   int skip_unit;                 // >= 0: CTA 0 leaves out the weight-tile request of this unit (a test of the bounded waits), else -1
 };
 
-// Records the first wait that ran out (site: 1 producer/empty, 2 mma/acc-empty, 3 mma/full-w, 4 mma/full-x, 5 epilogue/acc-full).
+// Records the first wait that ran out (site: 1 producer/empty, 2 mma/acc-empty, 3 mma/full, 5 epilogue/acc-full).
 #define GIVE_UP(site, unit) do { atomicOr(a.status, ST_TIMEOUT); \
     if (a.diag && atomicCAS(a.diag, 0, (site)) == 0) { a.diag[1] = blockIdx.x; a.diag[2] = (unit); a.diag[3] = n_units; \
       a.diag[4] = gridDim.x; a.diag[5] = a.m; a.diag[6] = a.n; a.diag[7] = a.kb; } } while (0)
 
-template <int MT, int BUDGET_KB, int NH>
-__global__ void __launch_bounds__(192, 1)
+constexpr int MAX_STAGES = 10;
+constexpr int EPI_WARPS = 4;                             // one per quadrant of tensor memory (two measured no faster: the L2 takes the stores no sooner)
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int RING_BYTES = 200 * 1024;
+constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
+
+// Shapes are run-time arguments (one copy of the code for all row counts); NH: 128-row weight tiles per CTA and unit.
+template <int NH>
+__global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const GemmArgs a) {
-  using C = TileCfg<MT, BUDGET_KB, NH>;
-  constexpr int BN = NH * BLOCK_N;                       // weight rows of a unit
+  constexpr int W_BYTES = NH * A_BYTES, BN = NH * BLOCK_N;        // weight rows of a unit
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t bars = tiles + C::STAGES * C::STAGE_BYTES;
-  auto fullw_bar = [&](int s) { return bars + 8u * s; };
-  auto fullx_bar = [&](int s) { return bars + 8u * (C::STAGES + s); };
-  auto empty_bar = [&](int s) { return bars + 8u * (2 * C::STAGES + s); };
-  auto accfull_bar = [&](int i) { return bars + 8u * (3 * C::STAGES + i); };
-  auto accempty_bar = [&](int i) { return bars + 8u * (3 * C::STAGES + 2 + i); };
-  const uint32_t tmem_slot = bars + 8u * (3 * C::STAGES + 4);
+  const int stages = a.stages;
+  const uint32_t x_box_bytes = (uint32_t)a.mt * (BLOCK_K * 2), x_bytes = a.x_boxes * x_box_bytes, stage_bytes = W_BYTES + x_bytes;
+  const uint32_t bars = tiles + RING_BYTES;
+  auto full_bar = [&](int s) { return bars + 8u * s; };
+  auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
+  auto accfull_bar = [&](int i) { return bars + 8u * (2 * MAX_STAGES + i); };
+  auto accempty_bar = [&](int i) { return bars + 8u * (2 * MAX_STAGES + 2 + i); };
+  const uint32_t tmem_slot = bars + 8u * (2 * MAX_STAGES + 4);
   __shared__ int s_abort;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u_begin = blockIdx.x * a.q;
   const int u_end = min(u_begin + a.q, a.total_units);
-  const int n_units = u_end - u_begin;
+  const int n_units = u_end - u_begin, pre = n_units < stages ? n_units : stages;
 
   if (threadIdx.x == 0) {
     s_abort = 0;
-    for (int s = 0; s < C::STAGES; ++s) { mbar_init(fullw_bar(s), 1); mbar_init(fullx_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(accfull_bar(i), 1); mbar_init(accempty_bar(i), 4); }
+    for (int s = 0; s < stages; ++s) { mbar_init(full_bar(s), 2); mbar_init(empty_bar(s), 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(accfull_bar(i), 1); mbar_init(accempty_bar(i), EPI_WARPS); }
     mbar_init_fence();
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmX);
     // weights do not depend on the preceding kernel: request the first ring of weight tiles right away, before the
     // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait
-    const uint64_t pol_w0 = policy_evict_first();
-    const int pre0 = n_units < C::STAGES ? n_units : C::STAGES;
-    for (int i = 0; i < pre0; ++i) {
-      const int u = u_begin + i, tile = u / a.kb;
-      if (u == a.skip_unit) continue;
-      mbar_arrive_expect_tx(fullw_bar(i), C::W_BYTES);
-      tma_load_2d(tiles + i * C::STAGE_BYTES, &tmW, (u - tile * a.kb) * BLOCK_K, (tile % a.n_tiles) * BN, fullw_bar(i), pol_w0);
+    const uint64_t pol = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal();
+    int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_tiles * BN;
+    for (int i = 0; i < pre; ++i) {
+      if (u_begin + i != a.skip_unit) {
+        mbar_arrive_expect_tx(full_bar(i), W_BYTES);
+        tma_load_2d(tiles + i * stage_bytes, &tmW, kb * BLOCK_K, nrow, full_bar(i), pol);
+      }
+      if (++kb == a.kb) { kb = 0; nrow = ++tile / a.m_tiles * BN; }
     }
   }
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
+  if (warp == 1) tmem_alloc(tmem_slot, a.tmem_cols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -214,102 +214,96 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
-      const int pre = n_units < C::STAGES ? n_units : C::STAGES;      // weight tiles already requested in the prologue
-      // (k column, weight row, activation row) of the unit being issued, advanced without divisions
-      int kcol = 0, nrow = 0, mrow = 0;
+      const uint64_t pol_w = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
+      int kcol = 0, nrow = 0, mrow = 0;                  // (k column, weight row, activation row) of the unit being issued, advanced without divisions
       if (n_units > 0) {
         const int tile = u_begin / a.kb;
-        kcol = (u_begin - tile * a.kb) * BLOCK_K; nrow = (tile % a.n_tiles) * BN; mrow = (tile / a.n_tiles) * MT;
+        kcol = (u_begin - tile * a.kb) * BLOCK_K; nrow = tile / a.m_tiles * BN; mrow = tile % a.m_tiles * a.mt;
       }
-      const int kend = a.kb * BLOCK_K, nend = a.n_tiles * BN, lo_rows = a.x_lo_rows;
-      const uint32_t x_bytes = lo_rows ? C::B_BYTES : C::B_PLANE;
+      const int kend = a.kb * BLOCK_K, mend = a.m_tiles * a.mt;
       int s = 0; uint32_t eph = 1;                       // ring stage, parity of its empty barrier
-      grid_dep_wait();                     // activations are the preceding kernel's output
+      grid_dep_wait();                                   // activations are the preceding kernel's output
       for (int i = 0; i < n_units; ++i) {
-        const uint32_t a_dst = tiles + s * C::STAGE_BYTES;
+        const uint32_t dst = tiles + s * stage_bytes;
         if (i >= pre) {
           if (!mbar_wait(empty_bar(s), eph, a.wait_limit)) { GIVE_UP(1, i); s_abort = 1; break; }
           if (u_begin + i != a.skip_unit) {
-            mbar_arrive_expect_tx(fullw_bar(s), C::W_BYTES);
-            tma_load_2d(a_dst, &tmW, kcol, nrow, fullw_bar(s), pol_w);
+            mbar_arrive_expect_tx(full_bar(s), W_BYTES);
+            tma_load_2d(dst, &tmW, kcol, nrow, full_bar(s), pol_w);
           }
         }
-        mbar_arrive_expect_tx(fullx_bar(s), x_bytes);
-        tma_load_2d(a_dst + C::W_BYTES, &tmX, kcol, mrow, fullx_bar(s), pol_x);
-        if (lo_rows) tma_load_2d(a_dst + C::W_BYTES + C::B_PLANE, &tmX, kcol, lo_rows + mrow, fullx_bar(s), pol_x);
-        if (++s == C::STAGES) { s = 0; eph ^= 1u; }
-        if ((kcol += BLOCK_K) == kend) { kcol = 0; if ((nrow += BN) == nend) { nrow = 0; mrow += MT; } }
+        mbar_arrive_expect_tx(full_bar(s), x_bytes);
+        tma_load_2d(dst + W_BYTES, &tmX, kcol, mrow, full_bar(s), pol_x);
+        if (a.x_boxes == 2) tma_load_2d(dst + W_BYTES + x_box_bytes, &tmX, kcol, mrow + a.x_lo_rows, full_bar(s), pol_x);
+        if (++s == stages) { s = 0; eph ^= 1u; }
+        if ((kcol += BLOCK_K) == kend) { kcol = 0; if ((mrow += a.mt) == mend) { mrow = 0; nrow += BN; } }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      const bool cat = C::CAT && a.x_lo_rows != 0;
-      const uint32_t idesc = cat ? instr_desc(2 * MT) : instr_desc(MT);
-      int seg = 0, s = 0;
-      uint32_t ph = 0;                                   // ring stage, parity of its full barriers
+      const uint32_t idesc = instr_desc_f16(1, BLOCK_N, a.mma_n, 0);
+      const uint64_t ring_desc = smem_desc_sw128(tiles);                       // + offset / 16 inside the ring
+      int s = 0, acc = 0;
+      uint32_t ph = 0, acc_ph = 0;                       // parities of the stage's full barrier and of the accumulator's barriers
       bool ok = true;
-      const bool two_pass = a.x_lo_rows && !cat;
       int seg_len = n_units > 0 ? min((u_begin / a.kb + 1) * a.kb, u_end) - u_begin : 0;      // first segment: the tail of a tile
       for (int i = 0; i < n_units && ok;) {
-        const int acc = seg % C::NBUF;
-        const uint32_t acc_ph = (seg / C::NBUF) & 1;
         if (!mbar_wait(accempty_bar(acc), acc_ph ^ 1u, a.wait_limit)) { GIVE_UP(2, i); ok = false; break; }      // epilogue has drained this buffer
         tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * NH * C::ACC_COLS);
+        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * NH * a.acc_cols);
         for (int j = 0; j < seg_len; ++j, ++i) {
-          if (!mbar_wait(fullw_bar(s), ph, a.wait_limit)) { GIVE_UP(3, i); ok = false; break; }
-          if (!mbar_wait(fullx_bar(s), ph, a.wait_limit)) { GIVE_UP(4, i); ok = false; break; }
+          if (!mbar_wait(full_bar(s), ph, a.wait_limit)) { GIVE_UP(3, i); ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = tiles + s * C::STAGE_BYTES;
-          const uint64_t bdesc = smem_desc_sw128(a_addr + C::W_BYTES);
+          const uint64_t wdesc = ring_desc + (uint64_t)((s * stage_bytes) >> 4), xdesc = wdesc + (uint64_t)(W_BYTES >> 4);
 #pragma unroll
-          for (int hh = 0; hh < NH; ++hh) {              // the unit's weight tiles, one accumulator each, same activation tile
-            const uint64_t adesc = smem_desc_sw128(a_addr + hh * A_BYTES);
-            const uint32_t d_h = tmem_d + (uint32_t)(hh * C::ACC_COLS);
+          for (int hh = 0; hh < NH; ++hh)                // the unit's weight tiles, one accumulator each, same activation tile
 #pragma unroll
             for (int k = 0; k < BLOCK_K / 16; ++k)       // 16 bf16 = 32 bytes per MMA: +2 in 16-byte units
-              umma_f16(d_h, adesc + 2u * k, bdesc + 2u * k, idesc, (uint32_t)((j | k) != 0));
-            if (two_pass) {                              // the low-order plane of the activations, same weights
-              const uint64_t ldesc = smem_desc_sw128(a_addr + C::W_BYTES + C::B_PLANE);
+              umma_f16(tmem_d + (uint32_t)(hh * a.acc_cols), wdesc + (uint64_t)(hh * (A_BYTES >> 4) + 2 * k), xdesc + 2u * k, idesc, (uint32_t)((j | k) != 0));
+          if (a.passes == 2) {                           // the low-order plane of the activations, same weights
+            const uint64_t ldesc = xdesc + (uint64_t)(x_box_bytes >> 4);
 #pragma unroll
-              for (int k = 0; k < BLOCK_K / 16; ++k) umma_f16(d_h, adesc + 2u * k, ldesc + 2u * k, idesc, 1u);
-            }
+            for (int hh = 0; hh < NH; ++hh)
+#pragma unroll
+              for (int k = 0; k < BLOCK_K / 16; ++k)
+                umma_f16(tmem_d + (uint32_t)(hh * a.acc_cols), wdesc + (uint64_t)(hh * (A_BYTES >> 4) + 2 * k), ldesc + 2u * k, idesc, 1u);
           }
-          umma_commit(empty_bar(s));                     // frees the stage once these MMAs have read it
-          if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+          umma_commit(empty_bar(s));                       // frees the stage once these MMAs have read it
+          if (++s == stages) { s = 0; ph ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(accfull_bar(acc));                   // segment complete: hand the accumulator to the epilogue
-        ++seg;
+        umma_commit(accfull_bar(acc));                   // segment complete: hand the accumulators to the epilogue
+        if (++acc == a.acc_bufs) { acc = 0; acc_ph ^= 1u; }
         seg_len = min(a.kb, n_units - i);                // every later segment starts a tile
       }
       if (!ok) { atomicOr(a.status, ST_TIMEOUT); s_abort = 1; }
     }
   } else {
     const int quarter = warp & 3;                        // TMEM lanes this warp may read
-    const int epi_tid = quarter * 32 + lane;             // column of the tile this thread owns
     grid_dep_wait();                                     // the partial buffer may still be read by the preceding kernel
-    int seg = 0;
-    for (int i = 0; i < n_units;) {
-      const int u = u_begin + i;
-      const int tile = u / a.kb;
-      const int seg_len = min((tile + 1) * a.kb, u_end) - u;
-      const int acc = seg % C::NBUF;
-      const uint32_t acc_ph = (seg / C::NBUF) & 1;
-      if (!mbar_wait(accfull_bar(acc), acc_ph, a.wait_limit)) { if (lane == 0) GIVE_UP(5, i); break; }
+    int acc = 0;
+    uint32_t acc_ph = 0;
+    for (int i = 0, tile = u_begin / a.kb; i < n_units; ++tile) {
+      // where the segment goes, worked out while its accumulator fills
+      const int seg_len = min((tile + 1) * a.kb, u_end) - (u_begin + i), slot = (int)blockIdx.x - tile * a.kb / a.q;
+      const int n_tile = tile / a.m_tiles, n0 = n_tile * BN, m0 = (tile - n_tile * a.m_tiles) * a.mt, rows = min(a.mt, a.m - m0);
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * NH * a.acc_cols);
+      float* dst = a.part + (size_t)slot * a.slot_stride + (size_t)m0 * a.n + n0 + quarter * 32 + lane;
+      const int tiles_in = NH == 2 && n0 + BLOCK_N < a.n ? 2 : 1;      // an output that is no multiple of the unit's width ends inside its last unit
+      const bool ok = mbar_wait(accfull_bar(acc), acc_ph, a.wait_limit);
+      if (!__all_sync(0xffffffffu, ok)) { if (lane == 0) GIVE_UP(5, i); s_abort = 1; break; }
       tc_fence_after();
-      const int slot = blockIdx.x - (int)(((long long)tile * a.kb) / a.q);
-      const int n0 = (tile % a.n_tiles) * BN, m0 = (tile / a.n_tiles) * MT;
-      float* dst = a.part + (size_t)slot * a.slot_stride + n0 + epi_tid;
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * NH * C::ACC_COLS);
-#pragma unroll
-      for (int hh = 0; hh < NH; ++hh)
-        store_accumulator<MT>(taddr + (uint32_t)(hh * C::ACC_COLS), C::CAT && a.x_lo_rows != 0, dst + hh * BLOCK_N, m0, a.m, a.n);
+      if (rows <= 16) {
+        store_few<NH>(taddr, a.acc_cols, a.cat, a.mt, dst, rows, a.n, tiles_in);
+      } else {
+#pragma unroll 1
+        for (int hh = 0; hh < tiles_in; ++hh) store_accumulator(taddr + (uint32_t)(hh * a.acc_cols), a.cat, a.mt, dst + hh * BLOCK_N, rows, a.n);
+      }
       tc_fence_before();
-      if (lane == 0) mbar_arrive(accempty_bar(acc));     // the MMA warp may reuse this accumulator
+      __syncwarp();
+      if (lane == 0) mbar_arrive(accempty_bar(acc));     // the MMA lane may reuse this accumulator
       i += seg_len;
-      ++seg;
+      if (++acc == a.acc_bufs) { acc = 0; acc_ph ^= 1u; }
     }
   }
   __syncwarp();                                          // the one-lane roles rejoin their warps before the block-wide barrier
@@ -318,109 +312,110 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   if (s_abort) {                                         // let copies in flight land before the CTA retires
     for (int i = 0; i < 2000; ++i) __nanosleep(100);
   }
-  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, C::TMEM_COLS); }
+  if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, a.tmem_cols); }
 }
 
-template <int MT, int BUDGET_KB, int NH>
-hydra_status launch_b(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, cudaStream_t st) {
-  using C = TileCfg<MT, BUDGET_KB, NH>;
+template <int NH>
+hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, cudaStream_t st) {
   static PerDeviceFlag attr_done;
   if (!attr_done.get()) {
-    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<MT, BUDGET_KB, NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     attr_done.set();
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  HYDRA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<MT, BUDGET_KB, NH>, tw, tx, a));
+  HYDRA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<NH>, tw, tx, a));
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
-}
-
-// Shared memory per CTA: a deep ring, one CTA per SM (a 100 KB ring that lets the CTAs of two consecutive,
-// programmatically overlapped GEMMs share an SM measured no faster).
-template <int MT, int NH>
-hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, cudaStream_t st) {
-  return launch_b<MT, 200, NH>(tw, tx, a, grid, st);
 }
 
 }  // namespace
 
 bool gemm_tc_available() { return tensor_map_encoder_available(); }
 
-int gemm_tile_rows(int m) { return m <= 16 ? 16 : m <= 32 ? 32 : m <= 64 ? 64 : m <= 128 ? 128 : 256; }
-
-// Stream-K plan: equal contiguous unit ranges, one per CTA, at most one CTA per SM and at least 4 k-blocks each.
-// 128-row weight tiles per unit: outputs of 4096 columns and more take two (half the activation-tile traffic and half
-// the issue work per weight byte, a third more weight bytes in flight: -5 % step time at the 7B shape).  Above 64
-// activation rows tensor memory holds one set of two accumulators only (the epilogue no longer overlaps the next
-// segment), still a small gain.
-int gemm_tile_halves(int m, int n) {
-  return n % (2 * BLOCK_N) == 0 && n >= 4096 ? 2 : 1;
+// Tile shape.  128 or 256 weight rows per unit, measured with the reduction of the partial sums (us; n x k):
+//  * units of 256 rows take enough of them for ~4 per SM: 2048 x 2048, 1 row: 4.8 (128) against 5.6 (256); 3072 x 3072: 8.4 / 7.6
+//  * up to 64 activation rows 256 (fewer activation bytes per weight byte, more weight bytes in flight): 22016 x 4096, 1 row: 32.1 /
+//    30.2, 64 rows: 42.2 / 42.4; 4096 x 11008, 1 row: 19.0 / 17.5, 64 rows: 20.9 / 20.3
+//  * above, 128 (tensor memory then holds two accumulators, and fewer partial sums are left): 12288 x 4096, 96 rows: 29.4 / 30.9;
+//    4096 x 4096, 128 rows: 16.0 / 19.0; 22016 x 4096, 192 rows: 77 / 82; except for
+//  * tall row tiles with 16 and more units per SM, where the activation tile is most of what an SM takes in: 22016 x 4096, 256
+//    rows: 111 / 103, 512 rows: 222 / 192; 4096 x 11008, 512 rows: 96 / 91; but 4096 x 4096, 512 rows: 49 / 54
+struct GemmShape { int nh, mt, m_tiles; };
+static GemmShape gemm_shape(int m, int n, int k) {
+  // equal row tiles of a multiple of 16 rows, so that the MMA work and the activation traffic follow m
+  const int row_tiles = (m + 255) / 256, mt = ((m + row_tiles - 1) / row_tiles + 15) / 16 * 16;
+  const long long units = (long long)row_tiles * (n / 256) * (k / BLOCK_K), sms = sm_count();
+  const bool wide = m <= 64 ? 4 * units >= 15 * sms : (mt > 192 || row_tiles > 1) && units >= 16 * sms;
+  return GemmShape{wide ? 2 : 1, mt, (m + mt - 1) / mt};
 }
 
-SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, int force_nh) {
+// Stream-K plan: equal contiguous unit ranges, one per CTA, at most one CTA per SM and at least 4 k-blocks each.
+SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap) {
   SplitDesc sd{};
-  const int mt = gemm_tile_rows(m);
-  const int nh = force_nh ? force_nh : gemm_tile_halves(m, n);
-  sd.mt = mt; sd.n_tiles = n / (nh * BLOCK_N); sd.bn_shift = nh == 2 ? 8 : 7; sd.kb = k / BLOCK_K; sd.stride = (size_t)m * n;
-  const int tiles = sd.n_tiles * ((m + mt - 1) / mt);
+  const GemmShape sh = gemm_shape(m, n, k);
+  sd.mt = sh.mt; sd.m_tiles = sh.m_tiles; sd.kb = k / BLOCK_K; sd.stride = (size_t)m * n;
+  sd.bn_shift = sh.nh == 2 ? 8 : 7;
+  const int tiles = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles;
   const long long total = (long long)tiles * sd.kb;
   long long g = sm_count();
   if (g > total / 4) g = total / 4 > 0 ? total / 4 : 1;
   sd.q = (int)((total + g - 1) / g);
-  if (grid) *grid = (int)((total + sd.q - 1) / sd.q);
-  if (max_slots) {
-    int mx = 1;
-    for (int t = 0; t < tiles; ++t) {
-      long long u0 = (long long)t * sd.kb;
-      int ns = (int)((u0 + sd.kb - 1) / sd.q - u0 / sd.q) + 1;
-      mx = ns > mx ? ns : mx;
-    }
-    *max_slots = mx;
+  if (max_slots || part_cap) {
+    auto slots = [&]() {
+      int mx = 1;
+      for (int t = 0; t < tiles; ++t) {
+        long long u0 = (long long)t * sd.kb;
+        int ns = (int)((u0 + sd.kb - 1) / sd.q - u0 / sd.q) + 1;
+        mx = ns > mx ? ns : mx;
+      }
+      return mx;
+    };
+    int mx = slots();
+    // whole tiles per CTA need one slot
+    while (part_cap && mx > 1 && (size_t)mx * sd.stride > part_cap) { sd.q = sd.q < sd.kb ? sd.q + 1 : (sd.q + sd.kb) / sd.kb * sd.kb; mx = slots(); }
+    if (max_slots) *max_slots = mx;
   }
+  if (grid) *grid = (int)((total + sd.q - 1) / sd.q);
   return sd;
 }
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
-                     SplitDesc* sd_out, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st) {
+                     SplitDesc* sd_out, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
   int grid = 1;
-  SplitDesc sd = gemm_tc_plan(m, n, k, &grid, nullptr, 0);
+  const SplitDesc sd = gemm_tc_plan(m, n, k, &grid, nullptr, part_cap);
+  const GemmShape sh = gemm_shape(m, n, k);
   if (x_rows_alloc < m) x_rows_alloc = m;
+  GemmArgs a{};
+  a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.m_tiles = sd.m_tiles; a.mt = sd.mt;
+  a.total_units = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles * sd.kb; a.q = sd.q; a.status = status;
+  a.x_lo_rows = x_planes == 2 ? x_rows_alloc : 0; a.diag = diag;
+  a.wait_limit = dbg && dbg->wait_limit ? dbg->wait_limit : WAIT_LIMIT; a.skip_unit = dbg ? dbg->skip_unit : -1;
+  // Two planes, up to 128 rows: the hi and lo activation tiles sit back to back and form ONE MMA operand of 2 mt rows, so each
+  // weight tile is read from shared memory once; taller tiles take a pass per plane.
+  a.cat = x_planes == 2 && sd.mt <= 128;
+  a.passes = x_planes == 2 && !a.cat ? 2 : 1;
+  a.x_boxes = x_planes; a.mma_n = a.cat ? 2 * sd.mt : sd.mt;
+  const int read_cols = (sd.mt + 31) / 32 * 32;          // the epilogue reads whole batches of 32 columns
+  a.acc_cols = a.cat ? sd.mt + read_cols : read_cols;
+  a.acc_bufs = 2 * sh.nh * a.acc_cols <= 512 ? 2 : 1;
+  for (a.tmem_cols = 32; a.tmem_cols < a.acc_bufs * sh.nh * a.acc_cols;) a.tmem_cols *= 2;
+  const int stage_bytes = sh.nh * A_BYTES + a.x_boxes * sd.mt * BLOCK_K * 2;
+  a.stages = RING_BYTES / stage_bytes < MAX_STAGES ? RING_BYTES / stage_bytes : MAX_STAGES;
   CUtensorMap tw, tx;
-  const int nh = sd.bn_shift == 8 ? 2 : 1;
-  if (!get_tensor_map(w, (uint64_t)n, (uint64_t)k, (uint32_t)(nh * BLOCK_N), false, &tw) ||
+  if (!get_tensor_map(w, (uint64_t)n, (uint64_t)k, (uint32_t)(sh.nh * BLOCK_N), false, &tw) ||
       !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes, (uint64_t)k, (uint32_t)sd.mt, false, &tx)) {
     set_last_error("cuTensorMapEncodeTiled", cudaErrorUnknown);
     return HYDRA_ERR_CUDA;
   }
-  GemmArgs a{};
-  a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.n_tiles = sd.n_tiles;
-  a.total_units = sd.n_tiles * ((m + sd.mt - 1) / sd.mt) * sd.kb; a.q = sd.q; a.status = status;
-  a.x_lo_rows = x_planes == 2 ? x_rows_alloc : 0; a.diag = diag;
-  a.wait_limit = dbg && dbg->wait_limit ? dbg->wait_limit : WAIT_LIMIT; a.skip_unit = dbg ? dbg->skip_unit : -1;
   if (sd_out) *sd_out = sd;
-  if (nh == 2) {
-    switch (sd.mt) {
-      case 16: return launch<16, 2>(tw, tx, a, grid, st);
-      case 32: return launch<32, 2>(tw, tx, a, grid, st);
-      case 64: return launch<64, 2>(tw, tx, a, grid, st);
-      case 128: return launch<128, 2>(tw, tx, a, grid, st);
-      default: return launch<256, 2>(tw, tx, a, grid, st);
-    }
-  }
-  switch (sd.mt) {
-    case 16: return launch<16, 1>(tw, tx, a, grid, st);
-    case 32: return launch<32, 1>(tw, tx, a, grid, st);
-    case 64: return launch<64, 1>(tw, tx, a, grid, st);
-    case 128: return launch<128, 1>(tw, tx, a, grid, st);
-    default: return launch<256, 1>(tw, tx, a, grid, st);
-  }
+  return sh.nh == 2 ? launch<2>(tw, tx, a, grid, st) : launch<1>(tw, tx, a, grid, st);
 }
 
 }  // namespace hydra

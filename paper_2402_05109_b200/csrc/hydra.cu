@@ -48,7 +48,7 @@ struct Bump {                      // 256-byte aligned bump allocator; base == n
   }
 };
 
-int pad_rows(int m) { int t = gemm_tile_rows(m); return (m + t - 1) / t * t; }
+int pad_rows(int m) { return (m + 15) / 16 * 16; }
 
 enum State { ST_CREATED = 0, ST_READY = 1, ST_DRAFTED = 2, ST_VERIFIED = 3 };
 

@@ -11,9 +11,10 @@ namespace hydra {
 // dbg (tests of the bounded waits only): a shorter poll limit and one weight-tile request that CTA 0 leaves out.
 struct GemmDebug { uint32_t wait_limit; int skip_unit; };
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
-                     SplitDesc* sd_out, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st);
-SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, int force_nh = 0);   // force_nh: 128-row weight tiles per unit (0: the kernel's own choice)
-int gemm_tile_rows(int m);                // activation rows per MMA tile for an m-row GEMM: 16, 32, 64, 128 or 256
+                     SplitDesc* sd_out, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
+                     size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/);
+// grid: CTAs.  part_cap (floats, 0: no limit): fewer CTAs, hence fewer slots, where the partial sums would not fit otherwise.
+SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap = 0);
 bool gemm_tc_available();                 // driver entry point for tensor-map encoding found
 // SIMT path (float or bfloat16 operands), single slot.
 hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, cudaStream_t st);

@@ -26,7 +26,8 @@ extern "C" hydra_status hydra_gemm_noalloc(const void* x, const void* w, float* 
   if (!x || !w || !out || !status || m < 1 || n < 1 || k < 1) return HYDRA_ERR_INVALID;
   if (n % 128 || k % 64) return HYDRA_ERR_UNSUPPORTED;
   int slots = 1;
-  gemm_tc_plan(m, n, k, nullptr, &slots);
+  constexpr size_t CAP = NOALLOC_SCRATCH_BYTES / sizeof(float);
+  gemm_tc_plan(m, n, k, nullptr, &slots, CAP);
   if ((size_t)slots * (size_t)m * (size_t)n * sizeof(float) > NOALLOC_SCRATCH_BYTES) {
     set_last_error("hydra_gemm_noalloc: the partial sums exceed the 8 MiB built-in scratch", cudaErrorInvalidValue);
     return HYDRA_ERR_CAPACITY;
@@ -47,6 +48,6 @@ extern "C" hydra_status hydra_gemm_noalloc(const void* x, const void* w, float* 
   float* part = reinterpret_cast<float*>(addr);
   // every partial element the reduction reads is written by the GEMM first, so nothing has to be cleared
   SplitDesc sd;
-  HYDRA_TRY(gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, &sd, status, nullptr, nullptr, st));
+  HYDRA_TRY(gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, &sd, status, nullptr, nullptr, st, CAP));
   return reduce_splits(part, sd, out, m, n, st);
 }

@@ -1,0 +1,22 @@
+"""Tensor-core GEMM at the edges of its tile choice: row tiles of any multiple of 16 rows, 16 / 17 rows (epilogue paths), 64 / 65, 128 / 129
+(one pass, a pass per plane), two row tiles; 128 and 256 weight rows per unit, an output that ends inside its last unit."""
+import pytest
+import torch
+
+from synth import normal_
+from tests.parity import split_hi_lo
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m", [1, 2, 15, 16, 17, 47, 64, 65, 80, 112, 128, 129, 176, 256, 257, 308, 513])
+@pytest.mark.parametrize("n,k", [(128, 64), (384, 704), (4096 + 128, 1024), (4096, 4096)])
+def test_gemm_tile_edges(m, n, k):
+    from paper_2402_05109_b200 import gemm
+    x = normal_(torch.empty(m, k, device="cuda"), 61, m + k, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 62, n, 0.02)
+    # planes hold 16 bits, products are exact, only the order of the float sums differs: k terms of size ~0.02, a few ulp of the largest sum
+    for planes in (split_hi_lo(x), x.to(torch.bfloat16)):
+        ref = (planes.double().sum(0) if planes.dim() == 3 else planes.double()) @ w.double().T
+        out = gemm(planes, w, mode=0).double()
+        assert float((out - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5

@@ -162,53 +162,62 @@ template <> __device__ __forceinline__ void put4<bf16>(bf16* p, size_t ps, float
   if (ps) store4<bf16>(p + ps, make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w));
 }
 
+template <typename T> struct alignas(4 * sizeof(T)) Raw4 { T v[4]; };      // four elements as stored
 constexpr int NORM_THREADS = 1024;
 // x_out = res + sum of the partial-sum slots; with `gain`, also xn = rmsnorm(x_out) * gain (operand planes) and hn (float).
-// A row is shared by the CS CTAs of a thread-block cluster (CTA `part` owns d / CS consecutive columns), so that few rows
-// still pull their partial sums through many SMs; the CTAs push their sums of squares into each other's shared memory and
-// add them in rank order after one cluster barrier.
+// A row is shared by the CS CTAs of a thread-block cluster (CTA `rank` owns d / CS consecutive columns), so that few rows
+// still pull their partial sums through many SMs.  The kernel is a chain of latencies (a few hundred KB in all), so what does
+// not depend on the preceding kernel - the slot counts with their integer divisions, the gain - comes before the wait for it,
+// and every warp leaves its sum of squares in the shared memory of all CTAs of the row, so that one barrier is the only one.
 template <typename T, int CS>
 __global__ void __launch_bounds__(NORM_THREADS) residual_rmsnorm_kernel(const float* res, const float* __restrict__ part,
                                                                         SplitDesc sd, float* x_out,
                                                                         const T* __restrict__ gain, T* __restrict__ xn, size_t xn_ps,
                                                                         float* __restrict__ hn, int d, float eps) {
   pdl_trigger();
-  pdl_wait();
-  __shared__ float sh[32];
-  __shared__ float s_ss[CS];
+  __shared__ float s_ss[CS * 32];
   const int row = blockIdx.x / CS, rank = blockIdx.x % CS;
-  const int dc = d / CS, c0 = rank * dc;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int dc = d / CS, c0 = rank * dc, i0 = c0 + threadIdx.x * 4;
   const size_t base = (size_t)row * d;
+  int ns0 = part && i0 < c0 + dc ? split_count(sd, row, i0) : 0;
+  Raw4<T> g0{};
+  if (gain && i0 < c0 + dc) g0 = *reinterpret_cast<const Raw4<T>*>(gain + i0);
+  pdl_wait();
   float ss = 0.f;
   float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f);                          // this thread's first piece stays in registers
-  for (int i = c0 + threadIdx.x * 4, it = 0; i < c0 + dc; i += blockDim.x * 4, ++it) {   // one 16-byte piece per thread and round, all its slot loads in flight together
+  for (int i = i0; i < c0 + dc; i += blockDim.x * 4) {                  // one 16-byte piece per thread and round, all its slot loads in flight together
     size_t off[1] = {base + i};
-    int ns[1] = {part ? split_count(sd, row, i) : 0};
+    int ns[1] = {i == i0 ? ns0 : part ? split_count(sd, row, i) : 0};
     float4 acc[1];
     float4 v = res ? *reinterpret_cast<const float4*>(res + base + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     sum_slots_multi<1, 12>(part, sd.stride, off, ns, acc);             // narrow outputs are cut into up to ~11 slots per tile
     v.x += acc[0].x; v.y += acc[0].y; v.z += acc[0].z; v.w += acc[0].w;
     *reinterpret_cast<float4*>(x_out + base + i) = v;
     ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-    if (it == 0) v0 = v;
+    if (i == i0) v0 = v;
   }
   if (!gain) return;
-  float tot = block_sum(ss, sh);
+  ss = warp_sum(ss);
   if constexpr (CS > 1) {
-    if (threadIdx.x < CS) {                                              // thread r leaves this CTA's sum in CTA r's slot `rank`
-      uint32_t local = (uint32_t)__cvta_generic_to_shared(&s_ss[rank]), remote;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((uint32_t)threadIdx.x));
-      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(tot) : "memory");
+    if (lane < CS) {                                                     // lane r leaves the warp's sum in CTA r's table
+      uint32_t local = (uint32_t)__cvta_generic_to_shared(&s_ss[rank * 32 + warp]), remote;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"((uint32_t)lane));
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(ss) : "memory");
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    tot = 0.f;
-#pragma unroll
-    for (int r = 0; r < CS; ++r) tot += s_ss[r];
+  } else {
+    if (lane == 0) s_ss[warp] = ss;
+    __syncthreads();
   }
+  float tot = 0.f;
+#pragma unroll
+  for (int c = 0; c < CS; ++c) tot += lane < nw ? s_ss[c * 32 + lane] : 0.f;
+  tot = warp_sum(tot);
   const float inv = rsqrtf(tot / (float)d + eps);
-  for (int i = c0 + threadIdx.x * 4, it = 0; i < c0 + dc; i += blockDim.x * 4, ++it) {
-    float4 v = it == 0 ? v0 : *reinterpret_cast<const float4*>(x_out + base + i);
-    float4 gn = load4<T>(gain + i);
+  for (int i = i0; i < c0 + dc; i += blockDim.x * 4) {
+    float4 v = i == i0 ? v0 : *reinterpret_cast<const float4*>(x_out + base + i);
+    const float4 gn = i == i0 ? load4<T>(reinterpret_cast<const T*>(&g0)) : load4<T>(gain + i);
     v.x *= inv * gn.x; v.y *= inv * gn.y; v.z *= inv * gn.z; v.w *= inv * gn.w;
     if (xn) put4<T>(xn + base + i, xn_ps, v);
     if (hn) *reinterpret_cast<float4*>(hn + base + i) = v;
@@ -284,8 +293,17 @@ __global__ void __launch_bounds__(256) qkv_rope_store_kernel(const float* __rest
                                                              RowSet rs, int H, int hd, int max_seq,
                                                              int* status) {
   pdl_trigger();
-  pdl_wait();
   const int r = blockIdx.x;
+  const int d = H * hd, half = hd >> 1;
+  const int tph = half >> 2;                                       // threads per head
+  const int h = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
+  const int j = (threadIdx.x % tph) * 4;
+  const int c0 = h * hd + j, c1 = c0 + half;
+  const int cols[6] = {c0, c1, d + c0, d + c1, 2 * d + c0, 2 * d + c1};
+  size_t off[6]; int ns[6];                                        // before the wait: the slot counts take two integer divisions each
+#pragma unroll
+  for (int e = 0; e < 6; ++e) { off[e] = (size_t)r * 3 * d + cols[e]; ns[e] = split_count(sd, r, cols[e]); }
+  pdl_wait();
   int b, slot;
   if (rs.row_at) {
     const int2 at = rs.row_at[r];
@@ -296,21 +314,10 @@ __global__ void __launch_bounds__(256) qkv_rope_store_kernel(const float* __rest
     if (i >= (rs.n_rows ? rs.n_rows[b] : rs.tc)) return;
     slot = rs.pos0[b] + i;
   }
-  const int d = H * hd, half = hd >> 1;
   if (slot < 0 || slot >= max_seq) { if (threadIdx.x == 0 && blockIdx.y == 0) atomicOr(status, ST_BOUNDS); return; }
-  const int tph = half >> 2;                                       // threads per head
-  const int h = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
   if (h >= H) return;
-  const int j = (threadIdx.x % tph) * 4;
-  const int c0 = h * hd + j, c1 = c0 + half;
-  const int cols[6] = {c0, c1, d + c0, d + c1, 2 * d + c0, 2 * d + c1};
   float4 v6[6];
-  {
-    size_t off[6]; int ns[6];
-#pragma unroll
-    for (int e = 0; e < 6; ++e) { off[e] = (size_t)r * 3 * d + cols[e]; ns[e] = split_count(sd, r, cols[e]); }
-    sum_slots_multi<6>(part, sd.stride, off, ns, v6);
-  }
+  sum_slots_multi<6>(part, sd.stride, off, ns, v6);
   const float4 t01 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j);        // (cos, sin) of j, j+1
   const float4 t23 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j + 2);    // (cos, sin) of j+2, j+3
   const float cs[4] = {t01.x, t01.z, t23.x, t23.z}, sn[4] = {t01.y, t01.w, t23.y, t23.w};
@@ -543,12 +550,13 @@ hydra_status tree_attention_f32(const float* q, const float* kc, const float* vc
 template <typename T>
 __global__ void silu_mul_kernel(const float* __restrict__ part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int rows, int f) {
   pdl_trigger();
-  pdl_wait();
-  size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= (size_t)rows * f) return;
-  const int r = (int)(i / f), c = (int)(i % f);
+  const int f4 = f / 4, p = blockIdx.x * blockDim.x + threadIdx.x;            // rows * f / 4 stays below 2^31
+  const int r = p / f4, c = (p - r * f4) * 4;
+  if (r >= rows) return;
+  const size_t i = (size_t)r * f + c;
   size_t off[2] = {(size_t)r * 2 * f + c, (size_t)r * 2 * f + f + c};
   int ns[2] = {split_count(sd, r, c), split_count(sd, r, f + c)};
+  pdl_wait();
   float4 gu[2];
   sum_slots_multi<2>(part, sd.stride, off, ns, gu);
   const float4 g = gu[0], u = gu[1];
@@ -579,10 +587,6 @@ __device__ __forceinline__ void warp_best(float& v, int& i) {
   }
 }
 
-__device__ __forceinline__ float summed(const float* part, const SplitDesc& sd, int row, int col, int n) {
-  return sum_slots_scalar<4>(part, sd.stride, (size_t)row * n + col, split_count(sd, row, col));
-}
-
 // Top-c of every logits row in two stages.  Stage 1: grid (rows, blocks of TOPK_SPAN columns); each block sums the
 // partial slots of its columns (optionally storing the sums as the row's logits); every warp then picks the c best of
 // its register-resident values in c rounds of a warp-wide reduction (no block barrier inside the rounds), and one warp
@@ -596,23 +600,36 @@ __global__ void __launch_bounds__(256) topk_stage1_kernel(const float* __restric
                                                           float* __restrict__ logits_out, float* __restrict__ cand_v,
                                                           int* __restrict__ cand_i, int vocab, int c) {
   pdl_trigger();
-  pdl_wait();
   __shared__ float wv[8][TOPK_MAX];
   __shared__ int wi[8][TOPK_MAX];
   const int row = blockIdx.x, blk = blockIdx.y, nblk = gridDim.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float v[8]; int idx[8];
+  float v[8]; int idx[8], ns[8], ns_max = 0;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int col = blk * TOPK_SPAN + j * 256 + threadIdx.x;
-    idx[j] = col;
-    v[j] = -INFINITY;
-    if (col < vocab) {
-      v[j] = summed(part, sd, row, col, vocab);
-      if (logits_out) logits_out[(size_t)row * vocab + col] = v[j];
-    } else {
-      idx[j] = 0x7fffffff;
-    }
+    ns[j] = col < vocab ? split_count(sd, row, col) : 0;
+    idx[j] = col < vocab ? col : 0x7fffffff;
+    v[j] = col < vocab ? 0.f : -INFINITY;
+    ns_max = max(ns_max, ns[j]);
+  }
+  const float* src = part + (size_t)row * vocab + blk * TOPK_SPAN + threadIdx.x;
+  pdl_wait();
+  for (int s = 0; s < ns_max; s += 4) {                    // four slots of the eight columns in flight together
+    float u[4][8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) u[q][j] = s + q < ns[j] ? __ldcg(src + (s + q) * sd.stride + j * 256) : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] += u[q][j];
+  }
+  if (logits_out) {
+    float* dst = logits_out + (size_t)row * vocab + blk * TOPK_SPAN + threadIdx.x;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) if (ns[j]) dst[j * 256] = v[j];
   }
   for (int t = 0; t < c; ++t) {                            // this warp's c best, in order
     float bv = -INFINITY; int bi = 0x7fffffff;
@@ -758,31 +775,36 @@ hydra_status head_gather(const float* hprime, const void* embed, const int* root
   return HYDRA_OK;
 }
 
+// Four columns per thread in small CTAs (a level has 1 to a few dozen rows); the bias and the slot counts before the wait.
+constexpr int HEAD_ACT_THREADS = 64;
 template <typename T>
-__global__ void head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* __restrict__ part,
+__global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* __restrict__ part,
                                 SplitDesc sd, const T* __restrict__ bias, float* y_out, T* __restrict__ yb, size_t yb_ps,
                                 int rows, int d) {
   pdl_trigger();
+  const int d4 = d / 4, p = blockIdx.x * blockDim.x + threadIdx.x, r = p / d4, c = (p - r * d4) * 4;
+  if (r >= rows) return;
+  const size_t off[1] = {(size_t)r * d + c};
+  const int ns[1] = {split_count(sd, r, c)};
+  float4 v = bias ? load4<T>(bias + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const size_t at = res_is_hprime ? (size_t)(r / rows_per_b) * d + c : off[0];
   pdl_wait();
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)rows * d) return;
-  int r = (int)(i / d), c = (int)(i % d);
-  float v = bias ? to_f<T>(bias[c]) : 0.f;
-  v += sum_slots_scalar<12>(part, sd.stride, i, split_count(sd, r, c));
-  float base = res_is_hprime ? res[(size_t)(r / rows_per_b) * d + c] : res[i];
-  float y = base + silu_f(v);
-  y_out[i] = y;
-  put<T>(yb + i, yb_ps, y);
+  const float4 base = *reinterpret_cast<const float4*>(res + at);
+  float4 acc[1];
+  sum_slots_multi<1, 12>(part, sd.stride, off, ns, acc);
+  const float4 y = make_float4(base.x + silu_f(v.x + acc[0].x), base.y + silu_f(v.y + acc[0].y), base.z + silu_f(v.z + acc[0].z), base.w + silu_f(v.w + acc[0].w));
+  *reinterpret_cast<float4*>(y_out + off[0]) = y;
+  put4<T>(yb + off[0], yb_ps, y);
 }
 hydra_status head_act(const float* res, int res_is_hprime, int rows_per_b, const float* part, SplitDesc sd,
                       const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, int dtype, cudaStream_t st) {
-  size_t n = (size_t)rows * d;
-  unsigned grid = (unsigned)((n + 255) / 256);
+  if (d & 3) return HYDRA_ERR_UNSUPPORTED;
+  const unsigned grid = (unsigned)(((size_t)rows * d / 4 + HEAD_ACT_THREADS - 1) / HEAD_ACT_THREADS);
   if (dtype == 0)
-    launch_pdl(head_act_kernel<float>, dim3(grid), dim3(256), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const float*)bias,
+    launch_pdl(head_act_kernel<float>, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const float*)bias,
                                                  y_out, (float*)yb, yb_ps, rows, d);
   else
-    launch_pdl(head_act_kernel<bf16>, dim3(grid), dim3(256), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const bf16*)bias,
+    launch_pdl(head_act_kernel<bf16>, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const bf16*)bias,
                                                 y_out, (bf16*)yb, yb_ps, rows, d);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;

@@ -78,10 +78,20 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + __expf(-x)
 // 128 or 256 rows; the row tiles that read the same weights are neighbours) owns units [t*kb, (t+1)*kb), so its
 // partial sums sit in slots 0 .. split_count-1 (slot s at part + s*stride + m*N + n), one per CTA that
 // touched the tile, in CTA order.  A single-slot output is described by q = kb = 1.
-struct SplitDesc { int q, kb, m_tiles, mt, bn_shift; size_t stride; };
-__host__ __device__ __forceinline__ int split_count(const SplitDesc& sd, int m, int n) {
-  const int u0 = ((n >> sd.bn_shift) * sd.m_tiles + m / sd.mt) * sd.kb;   // tiles * kb stays far below 2^31
-  return (u0 + sd.kb - 1) / sd.q - u0 / sd.q + 1;
+struct SplitDesc {
+  int q, kb, m_tiles, mt, bn_shift;
+  unsigned long long q_inv, mt_inv;      // ceil(2^40 / q), ceil(2^32 / mt)
+  size_t stride;
+  // u * q_inv >> 40 is u / q while u q < 2^40 (u: units, far below 2^24; q: units / CTAs); m * mt_inv >> 32 is m / mt while m mt < 2^32
+  void set_inverses() {
+    q_inv = ((1ull << 40) + (unsigned)q - 1) / (unsigned)q;
+    mt_inv = ((1ull << 32) + (unsigned)mt - 1) / (unsigned)mt;
+  }
+};
+__device__ __forceinline__ int split_count(const SplitDesc& sd, int m, int n) {
+  const int mi = sd.m_tiles == 1 ? 0 : (int)(((unsigned)m * sd.mt_inv) >> 32);
+  const unsigned u0 = (unsigned)(((n >> sd.bn_shift) * sd.m_tiles + mi) * sd.kb);   // tiles * kb stays far below 2^31
+  return (int)((((u0 + sd.kb - 1) * sd.q_inv) >> 40) - ((u0 * sd.q_inv) >> 40)) + 1;
 }
 // acc[u] = sum over the ns[u] slots of the four floats at element offset off[u] of a slot (all loads of a round in flight together)
 template <int U, int PMAX = 6>
@@ -117,7 +127,11 @@ __device__ __forceinline__ float sum_slots_scalar(const float* part, size_t stri
   for (int p = PMAX; p < ns; ++p) acc += __ldcg(part + p * stride + idx);
   return acc;
 }
-inline SplitDesc single_slot(size_t stride) { return SplitDesc{1 << 30, 1, 1, 1 << 30, 30, stride}; }
+inline SplitDesc single_slot(size_t stride) {
+  SplitDesc sd{1 << 30, 1, 1, 1 << 30, 30, 0, 0, stride};
+  sd.set_inverses();
+  return sd;
+}
 
 // Launch with programmatic stream serialisation allowed (see pdl_wait).
 template <typename... KArgs, typename... Args>

@@ -381,6 +381,7 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
     if (max_slots) *max_slots = mx;
   }
   if (grid) *grid = (int)((total + sd.q - 1) / sd.q);
+  sd.set_inverses();
   return sd;
 }
 

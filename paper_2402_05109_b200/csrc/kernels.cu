@@ -223,6 +223,63 @@ __global__ void __launch_bounds__(NORM_THREADS) residual_rmsnorm_kernel(const fl
     if (hn) *reinterpret_cast<float4*>(hn + base + i) = v;
   }
 }
+// Many rows: one CTA of at most 512 threads per row, P pieces per thread in registers, two CTAs per SM.  (With the kernel above,
+// 1024 threads at 64 registers, one CTA fills an SM and 512 rows run as four latencies one after the other: 20 us at 512 x 4096.)
+constexpr int NORM_ROW_THREADS = 512;
+template <typename T, int P>
+__global__ void __launch_bounds__(NORM_ROW_THREADS, 2) residual_rmsnorm_rows_kernel(const float* res, const float* __restrict__ part, SplitDesc sd,
+                                                                                 float* x_out, const T* __restrict__ gain, T* __restrict__ xn, size_t xn_ps,
+                                                                                 float* __restrict__ hn, int d, float eps) {
+  pdl_trigger();
+  __shared__ float s_ss[NORM_ROW_THREADS / 32];
+  const int row = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5, i0 = threadIdx.x * 4, di = blockDim.x * 4;
+  const size_t base = (size_t)row * d;
+  int ns[P], mx = 0;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    ns[p] = part && i0 + p * di < d ? split_count(sd, row, i0 + p * di) : 0;
+    mx = max(mx, ns[p]);
+  }
+  pdl_wait();
+  float4 v[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p)
+    v[p] = res && i0 + p * di < d ? *reinterpret_cast<const float4*>(res + base + i0 + p * di) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* src = part + base + i0;
+  float4 acc[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+  for (int s = 0; s < mx; ++s) {
+    float4 u[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) u[p] = s < ns[p] ? __ldcg(reinterpret_cast<const float4*>(src + s * sd.stride + p * di)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int p = 0; p < P; ++p) { acc[p].x += u[p].x; acc[p].y += u[p].y; acc[p].z += u[p].z; acc[p].w += u[p].w; }
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    if (i0 + p * di >= d) continue;
+    v[p].x += acc[p].x; v[p].y += acc[p].y; v[p].z += acc[p].z; v[p].w += acc[p].w;
+    *reinterpret_cast<float4*>(x_out + base + i0 + p * di) = v[p];
+    ss += v[p].x * v[p].x + v[p].y * v[p].y + v[p].z * v[p].z + v[p].w * v[p].w;
+  }
+  if (!gain) return;
+  ss = warp_sum(ss);
+  if (lane == 0) s_ss[warp] = ss;
+  __syncthreads();
+  const float inv = rsqrtf(warp_sum(lane < nw ? s_ss[lane] : 0.f) / (float)d + eps);
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const int i = i0 + p * di;
+    if (i >= d) continue;
+    const float4 gn = load4<T>(gain + i);
+    const float4 y = make_float4(v[p].x * (inv * gn.x), v[p].y * (inv * gn.y), v[p].z * (inv * gn.z), v[p].w * (inv * gn.w));
+    if (xn) put4<T>(xn + base + i, xn_ps, y);
+    if (hn) *reinterpret_cast<float4*>(hn + base + i) = y;
+  }
+}
 template <typename T, int CS>
 static cudaError_t launch_norm(int rows, int d, cudaStream_t st, const float* res, const float* part, SplitDesc sd, float* x_out,
                                const void* gain, void* xn, size_t xn_ps, float* hn, float eps) {
@@ -238,21 +295,29 @@ static cudaError_t launch_norm(int rows, int d, cudaStream_t st, const float* re
   cfg.attrs = attr; cfg.numAttrs = CS > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, residual_rmsnorm_kernel<T, CS>, res, part, sd, x_out, (const T*)gain, (T*)xn, xn_ps, hn, d, eps);
 }
+template <typename T>
+static void norm_dispatch(const float* res, const float* part, SplitDesc sd, float* x_out, const void* gain, void* xn, size_t xn_ps, float* hn, int rows,
+                          int d, float eps, cudaStream_t st) {
+  // few rows: 8, 4 or 2 CTAs per row (the columns must split into whole 16-byte pieces); many: one CTA with everything in registers
+  if (rows <= 16 && d % 32 == 0) { launch_norm<T, 8>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps); return; }
+  if (rows <= 40 && d % 16 == 0) { launch_norm<T, 4>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps); return; }
+  if (rows <= 96 && d % 8 == 0) { launch_norm<T, 2>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps); return; }
+  const int pieces = (d / 4 + NORM_ROW_THREADS - 1) / NORM_ROW_THREADS, threads = ((d / 4 + pieces - 1) / pieces + 31) / 32 * 32;
+  auto go = [&](auto kernel) {
+    launch_pdl(kernel, dim3(rows), dim3(threads), 0, st, res, part, sd, x_out, (const T*)gain, (T*)xn, xn_ps, hn, d, eps);
+  };
+  if (pieces == 1) go(residual_rmsnorm_rows_kernel<T, 1>);
+  else if (pieces == 2) go(residual_rmsnorm_rows_kernel<T, 2>);
+  else if (pieces == 3) go(residual_rmsnorm_rows_kernel<T, 3>);
+  else if (pieces == 4) go(residual_rmsnorm_rows_kernel<T, 4>);
+  else launch_norm<T, 1>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
+}
 hydra_status residual_rmsnorm(const float* res, const float* part, SplitDesc sd, float* x_out,
                               const void* gain, void* xn, size_t xn_ps, float* hn, int rows, int d, float eps, int dtype,
                               cudaStream_t st) {
   if (d & 3) return HYDRA_ERR_UNSUPPORTED;
-  // few rows: 4 or 2 CTAs per row (the columns must split into whole 16-byte pieces)
-  const int cs = (rows <= 40 && d % 16 == 0) ? 4 : (rows <= 96 && d % 8 == 0) ? 2 : 1;
-  if (dtype == 0) {
-    if (cs == 4) launch_norm<float, 4>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-    else if (cs == 2) launch_norm<float, 2>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-    else launch_norm<float, 1>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-  } else {
-    if (cs == 4) launch_norm<bf16, 4>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-    else if (cs == 2) launch_norm<bf16, 2>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-    else launch_norm<bf16, 1>(rows, d, st, res, part, sd, x_out, gain, xn, xn_ps, hn, eps);
-  }
+  if (dtype == 0) norm_dispatch<float>(res, part, sd, x_out, gain, xn, xn_ps, hn, rows, d, eps, st);
+  else norm_dispatch<bf16>(res, part, sd, x_out, gain, xn, xn_ps, hn, rows, d, eps, st);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -283,74 +348,69 @@ hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cud
   return HYDRA_OK;
 }
 
-// One thread rotates four consecutive pairs (j..j+3, j+half..j+half+3) of one head of q and k and copies the
-// matching v elements; all loads and stores are 16 bytes wide.
+// One thread takes four consecutive pairs (j..j+3, j+half..j+half+3) of one head of q, k or v (blockIdx.z): q and k are rotated,
+// k and v appended to the cache; all loads and stores are 16 bytes wide.  Three short threads instead of one long one: the sums
+// of two pieces leave registers for twice the warps (512 rows: 23 us with one thread for q, k and v), and 64 rows spread over
+// more SMs.  What the call's earlier kernels cannot change - slot counts, lengths, row table - is read before the wait (the
+// lengths are stable within a forward call, see rope_table_kernel).
 // T: float (float model path) or float16 (bfloat16 model path: q and the caches are float16 in one or two planes).
 template <typename T>
-__global__ void __launch_bounds__(256) qkv_rope_store_kernel(const float* __restrict__ part, SplitDesc sd,
+__global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* __restrict__ part, SplitDesc sd,
                                                              const float2* __restrict__ table, T* __restrict__ q, size_t q_ps,
                                                              T* __restrict__ kc, T* __restrict__ vc, size_t kv_ps,
                                                              RowSet rs, int H, int hd, int max_seq,
                                                              int* status) {
   pdl_trigger();
-  const int r = blockIdx.x;
+  const int r = blockIdx.x, which = blockIdx.z;
   const int d = H * hd, half = hd >> 1;
   const int tph = half >> 2;                                       // threads per head
   const int h = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
   const int j = (threadIdx.x % tph) * 4;
-  const int c0 = h * hd + j, c1 = c0 + half;
-  const int cols[6] = {c0, c1, d + c0, d + c1, 2 * d + c0, 2 * d + c1};
-  size_t off[6]; int ns[6];                                        // before the wait: the slot counts take two integer divisions each
-#pragma unroll
-  for (int e = 0; e < 6; ++e) { off[e] = (size_t)r * 3 * d + cols[e]; ns[e] = split_count(sd, r, cols[e]); }
-  pdl_wait();
+  const int c0 = which * d + h * hd + j;
+  const size_t off[2] = {(size_t)r * 3 * d + c0, (size_t)r * 3 * d + c0 + half};
+  const int ns[2] = {split_count(sd, r, c0), split_count(sd, r, c0 + half)};
   int b, slot;
+  bool live = h < H;
   if (rs.row_at) {
     const int2 at = rs.row_at[r];
     b = at.x; slot = at.y;
   } else {
     const int i = r % rs.tc;
     b = r / rs.tc;
-    if (i >= (rs.n_rows ? rs.n_rows[b] : rs.tc)) return;
+    live = live && i < (rs.n_rows ? rs.n_rows[b] : rs.tc);
     slot = rs.pos0[b] + i;
   }
-  if (slot < 0 || slot >= max_seq) { if (threadIdx.x == 0 && blockIdx.y == 0) atomicOr(status, ST_BOUNDS); return; }
-  if (h >= H) return;
-  float4 v6[6];
-  sum_slots_multi<6>(part, sd.stride, off, ns, v6);
+  const bool in_range = slot >= 0 && slot < max_seq;
+  pdl_wait();
+  if (!live) return;
+  if (!in_range) { if (threadIdx.x == 0 && blockIdx.y == 0 && which == 0) atomicOr(status, ST_BOUNDS); return; }
   const float4 t01 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j);        // (cos, sin) of j, j+1
   const float4 t23 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j + 2);    // (cos, sin) of j+2, j+3
-  const float cs[4] = {t01.x, t01.z, t23.x, t23.z}, sn[4] = {t01.y, t01.w, t23.y, t23.w};
-  auto rot = [&](const float4& a, const float4& bq, float4& lo, float4& hi) {
-    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {bq.x, bq.y, bq.z, bq.w};
+  float4 v2[2];
+  sum_slots_multi<2>(part, sd.stride, off, ns, v2);
+  if (which < 2) {
+    const float cs[4] = {t01.x, t01.z, t23.x, t23.z}, sn[4] = {t01.y, t01.w, t23.y, t23.w};
+    const float av[4] = {v2[0].x, v2[0].y, v2[0].z, v2[0].w}, bv[4] = {v2[1].x, v2[1].y, v2[1].z, v2[1].w};
     float l[4], hh[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) { l[e] = av[e] * cs[e] - bv[e] * sn[e]; hh[e] = bv[e] * cs[e] + av[e] * sn[e]; }
-    lo = make_float4(l[0], l[1], l[2], l[3]); hi = make_float4(hh[0], hh[1], hh[2], hh[3]);
-  };
-  float4 qlo, qhi, klo, khi;
-  rot(v6[0], v6[1], qlo, qhi);
-  rot(v6[2], v6[3], klo, khi);
-  put4h<T>(q + (size_t)r * d + c0, q_ps, qlo);
-  put4h<T>(q + (size_t)r * d + c1, q_ps, qhi);
-  const size_t o = (((size_t)b * H + h) * max_seq + slot) * hd;
-  put4h<T>(kc + o + j, kv_ps, klo);
-  put4h<T>(kc + o + j + half, kv_ps, khi);
-  put4h<T>(vc + o + j, kv_ps, v6[4]);
-  put4h<T>(vc + o + j + half, kv_ps, v6[5]);
+    v2[0] = make_float4(l[0], l[1], l[2], l[3]); v2[1] = make_float4(hh[0], hh[1], hh[2], hh[3]);
+  }
+  T* dst = which == 0 ? q + (size_t)r * d + h * hd : (which == 1 ? kc : vc) + (((size_t)b * H + h) * max_seq + slot) * hd;
+  const size_t ps = which == 0 ? q_ps : kv_ps;
+  put4h<T>(dst + j, ps, v2[0]);
+  put4h<T>(dst + j + half, ps, v2[1]);
 }
 hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table, void* q, size_t q_ps, void* kcache, void* vcache,
                             size_t kv_ps, RowSet rs, int H, int hd, int max_seq, int dtype, int* status, cudaStream_t st) {
-  if (hd % 8) return HYDRA_ERR_UNSUPPORTED;
-  // 128 threads per CTA: with 64 rows twice as many SMs pull the partial sums as with 256
-  const int threads = 128 % (hd / 8) == 0 ? 128 : 256;
-  const int heads_per_block = threads / (hd / 8);
-  dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block);
+  if (hd % 8 || 128 % (hd / 8)) return HYDRA_ERR_UNSUPPORTED;
+  const int heads_per_block = 128 / (hd / 8);
+  dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block, 3);
   if (dtype == 0)
-    launch_pdl(qkv_rope_store_kernel<float>, grid, dim3(threads), 0, st, part, sd, table, (float*)q, q_ps, (float*)kcache, (float*)vcache,
+    launch_pdl(qkv_rope_store_kernel<float>, grid, dim3(128), 0, st, part, sd, table, (float*)q, q_ps, (float*)kcache, (float*)vcache,
                kv_ps, rs, H, hd, max_seq, status);
   else
-    launch_pdl(qkv_rope_store_kernel<__half>, grid, dim3(threads), 0, st, part, sd, table, (__half*)q, q_ps, (__half*)kcache, (__half*)vcache,
+    launch_pdl(qkv_rope_store_kernel<__half>, grid, dim3(128), 0, st, part, sd, table, (__half*)q, q_ps, (__half*)kcache, (__half*)vcache,
                kv_ps, rs, H, hd, max_seq, status);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
@@ -548,26 +608,23 @@ hydra_status tree_attention_f32(const float* q, const float* kc, const float* vc
 // SiLU(gate) * up from the gate/up partial sums
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void silu_mul_kernel(const float* __restrict__ part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int rows, int f) {
+__global__ void __launch_bounds__(256) silu_mul_kernel(const float* __restrict__ part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int f) {
   pdl_trigger();
-  const int f4 = f / 4, p = blockIdx.x * blockDim.x + threadIdx.x;            // rows * f / 4 stays below 2^31
-  const int r = p / f4, c = (p - r * f4) * 4;
-  if (r >= rows) return;
-  const size_t i = (size_t)r * f + c;
-  size_t off[2] = {(size_t)r * 2 * f + c, (size_t)r * 2 * f + f + c};
-  int ns[2] = {split_count(sd, r, c), split_count(sd, r, f + c)};
+  const int r = blockIdx.y, c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const size_t off[2] = {(size_t)r * 2 * f + c, (size_t)r * 2 * f + f + c};
+  const int ns[2] = {split_count(sd, r, c), split_count(sd, r, f + c)};
   pdl_wait();
+  if (c >= f) return;
   float4 gu[2];
-  sum_slots_multi<2>(part, sd.stride, off, ns, gu);
+  sum_slots_multi<2, 4>(part, sd.stride, off, ns, gu);     // the widest output: few CTAs, hence few slots, per tile
   const float4 g = gu[0], u = gu[1];
-  put4<T>(act + i, act_ps, make_float4(silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w));
+  put4<T>(act + (size_t)r * f + c, act_ps, make_float4(silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w));
 }
 hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, int dtype, cudaStream_t st) {
   if (f & 3) return HYDRA_ERR_UNSUPPORTED;
-  size_t n = (size_t)rows * f / 4;
-  unsigned grid = (unsigned)((n + 255) / 256);
-  if (dtype == 0) launch_pdl(silu_mul_kernel<float>, dim3(grid), dim3(256), 0, st, part, sd, (float*)act, act_ps, rows, f);
-  else launch_pdl(silu_mul_kernel<bf16>, dim3(grid), dim3(256), 0, st, part, sd, (bf16*)act, act_ps, rows, f);
+  const dim3 grid((f / 4 + 255) / 256, rows);
+  if (dtype == 0) launch_pdl(silu_mul_kernel<float>, grid, dim3(256), 0, st, part, sd, (float*)act, act_ps, f);
+  else launch_pdl(silu_mul_kernel<bf16>, grid, dim3(256), 0, st, part, sd, (bf16*)act, act_ps, f);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -783,12 +840,12 @@ __global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float*
                                 int rows, int d) {
   pdl_trigger();
   const int d4 = d / 4, p = blockIdx.x * blockDim.x + threadIdx.x, r = p / d4, c = (p - r * d4) * 4;
-  if (r >= rows) return;
   const size_t off[1] = {(size_t)r * d + c};
   const int ns[1] = {split_count(sd, r, c)};
   float4 v = bias ? load4<T>(bias + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   const size_t at = res_is_hprime ? (size_t)(r / rows_per_b) * d + c : off[0];
   pdl_wait();
+  if (r >= rows) return;
   const float4 base = *reinterpret_cast<const float4*>(res + at);
   float4 acc[1];
   sum_slots_multi<1, 12>(part, sd.stride, off, ns, acc);

@@ -21,43 +21,109 @@ template <> struct Vec4<bf16> {
     v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b); }
 };
 
-template <typename T, int MR>
+// Sum of v[r] over the warp, for R values at once: lanes first trade halves of the values (R-1 shuffles for R values), then the
+// remaining lane bits are folded.  Value warp_sum_owner(lane) ends up in lanes 0..R-1.
+template <int R>
+__device__ __forceinline__ float warp_sum_multi(float (&v)[R], int lane) {
+#pragma unroll
+  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int r = 0; r < n; ++r) {
+      const float give = up ? v[r] : v[r + n], keep = up ? v[r + n] : v[r];
+      v[r] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
+  }
+  float s = v[0];
+#pragma unroll
+  for (int bit = R; bit < 32; bit *= 2) s += __shfl_xor_sync(0xffffffffu, s, bit);
+  return s;
+}
+// which of the R values: the lowest lane bit chose the upper half, the next bit the upper quarter, ...
+template <int R>
+__device__ __forceinline__ int warp_sum_owner(int lane) {
+  int r = 0;
+#pragma unroll
+  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) r += (lane & bit) ? n : 0;
+  return r;
+}
+
+// MR activation rows; KS warps share an output column (each every KS-th 512-byte piece of its weight row), 8 / KS columns per
+// block.  The small models of the float path spend their time in the chain launch -> loads -> reduction: the first WPRE weight
+// pieces of a lane are loaded before the wait for the preceding kernel, the MR sums share one transposing reduction, and the
+// split keeps the activation loads of a lane to one or two rounds and fills the SMs (16 x 256 x 688: 10.5 us with one warp per
+// column, 32 blocks).
+template <typename T, int MR, int KS>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w,
                                                         float* __restrict__ out, int m, int n, int k) {
+  constexpr int WPRE = 2;
   pdl_trigger();
-  pdl_wait();
+  __shared__ float s_part[8][MR];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int col = blockIdx.x * 8 + warp;
+  const int col = blockIdx.x * (8 / KS) + warp / KS, k0 = (warp % KS) * 128 + lane * 4;
   const int m0 = blockIdx.y * MR;
-  if (col >= n) return;
+  const T* wr = w + (size_t)min(col, n - 1) * k;
+  float wv[WPRE][4];
+#pragma unroll
+  for (int i = 0; i < WPRE; ++i)
+    if (k0 + i * KS * 128 < k) Vec4<T>::load(wr + k0 + i * KS * 128, wv[i]);
+  pdl_wait();
   float acc[MR];
 #pragma unroll
   for (int r = 0; r < MR; ++r) acc[r] = 0.f;
-  const T* wr = w + (size_t)col * k;
-  for (int kk = lane * 4; kk < k; kk += 128) {
-    float wv[4];
-    Vec4<T>::load(wr + kk, wv);
+  auto step = [&](int kk, const float (&wk)[4]) {
 #pragma unroll
     for (int r = 0; r < MR; ++r) {
-      int row = m0 + r < m ? m0 + r : m - 1;
+      const int row = m0 + r < m ? m0 + r : m - 1;
       float xv[4];
       Vec4<T>::load(x + (size_t)row * k + kk, xv);
-      acc[r] += wv[0] * xv[0] + wv[1] * xv[1] + wv[2] * xv[2] + wv[3] * xv[3];
+      acc[r] += wk[0] * xv[0] + wk[1] * xv[1] + wk[2] * xv[2] + wk[3] * xv[3];
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < WPRE; ++i)
+    if (k0 + i * KS * 128 < k) step(k0 + i * KS * 128, wv[i]);
+  for (int kk = k0 + WPRE * KS * 128; kk < k; kk += KS * 128) {
+    float wk[4];
+    Vec4<T>::load(wr + kk, wk);
+    step(kk, wk);
+  }
+  float s = warp_sum_multi<MR>(acc, lane);
+  const int r = warp_sum_owner<MR>(lane);
+  if constexpr (KS > 1) {
+    if (lane < MR) s_part[warp][r] = s;
+    __syncthreads();
+    if (warp % KS) return;
+    if (lane < MR) {
+#pragma unroll
+      for (int q = 1; q < KS; ++q) s += s_part[warp + q][r];
     }
   }
-#pragma unroll
-  for (int r = 0; r < MR; ++r) {
-    float s = warp_sum(acc[r]);
-    if (lane == 0 && m0 + r < m) out[(size_t)(m0 + r) * n + col] = s;
-  }
+  if (lane < MR && m0 + r < m && col < n) out[(size_t)(m0 + r) * n + col] = s;
 }
 
+template <typename T, int MR>
+static void launch_gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, cudaStream_t st) {
+  const int groups = (m + MR - 1) / MR;
+  auto go = [&](auto kernel, int ks) {
+    launch_pdl(kernel, dim3((n * ks + 7) / 8, groups), dim3(256), 0, st, (const T*)x, (const T*)w, out, m, n, k);
+  };
+  // warps per column: until there are two blocks per SM or a lane has one piece
+  const int pieces = (k + 127) / 128, want = 2 * sm_count();
+  if (pieces >= 4 && (long)n * groups / 4 <= want) go(gemm_simt_kernel<T, MR, 4>, 4);
+  else if (pieces >= 2 && (long)n * groups / 8 <= want) go(gemm_simt_kernel<T, MR, 2>, 2);
+  else go(gemm_simt_kernel<T, MR, 1>, 1);
+}
 hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0 || (k & 3)) return HYDRA_ERR_UNSUPPORTED;
-  constexpr int MR = 16;
-  dim3 grid((n + 7) / 8, (m + MR - 1) / MR);
-  if (dtype == 0) launch_pdl(gemm_simt_kernel<float, MR>, dim3(grid), dim3(256), 0, st, (const float*)x, (const float*)w, out, m, n, k);
-  else launch_pdl(gemm_simt_kernel<bf16, MR>, dim3(grid), dim3(256), 0, st, (const bf16*)x, (const bf16*)w, out, m, n, k);
+  auto rows = [&](auto zero) {
+    typedef decltype(zero) T;
+    if (m == 1) launch_gemm_simt<T, 1>(x, w, out, m, n, k, st);
+    else if (m <= 4) launch_gemm_simt<T, 4>(x, w, out, m, n, k, st);
+    else if (m <= 8) launch_gemm_simt<T, 8>(x, w, out, m, n, k, st);
+    else launch_gemm_simt<T, 16>(x, w, out, m, n, k, st);
+  };
+  if (dtype == 0) rows(float{}); else rows(bf16{});
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -422,10 +488,10 @@ hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table
 // path serves have a handful of (head, sequence) pairs and one chunk, so the time is the serial chain inside a warp: few rows
 // per warp spread it over the SMs (each row group reads the chunk's K,V again, out of L2), and with a single chunk the kernel
 // writes the result itself instead of leaving it to the combine kernel.  Measured at 16 rows x 4 heads x 48..80 slots: 28 us with
-// eight consecutive rows per warp and the combine kernel, 10 us now.
+// eight consecutive rows per warp and the combine kernel, 10 us with one row per warp; two keys per lane shorten the chain further.
 // ------------------------------------------------------------------------------------------------
 constexpr int ATT_CHUNK = ATT_CHUNK_ROWS;
-constexpr int ATT_TILE = 32;      // KV rows staged per iteration
+constexpr int ATT_TILE = 64;      // KV rows staged per iteration: two keys per lane
 constexpr int ATT_WARPS = 8;
 
 template <typename T, int HD, int RPW>
@@ -480,34 +546,41 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
       *reinterpret_cast<float4*>(vs + e) = vv;
     }
     __syncthreads();
-    const int slot = t0 + lane;
+    const int sl0 = t0 + lane, sl1 = sl0 + 32;
 #pragma unroll
     for (int j = 0; j < RPW; ++j) {
       const int r = r0 + j * ATT_WARPS + warp;
       if (r >= nr) continue;
-      bool valid = slot < s1 && (slot < p0 || ((msk[j] >> (slot - p0)) & 1ull));
-      float sc = 0.f;
+      const bool ok0 = sl0 < s1 && (sl0 < p0 || ((msk[j] >> (sl0 - p0)) & 1ull)), ok1 = sl1 < s1 && (sl1 < p0 || ((msk[j] >> (sl1 - p0)) & 1ull));
       const float* qr = qs + (r - r0) * HD;
-      const float* kr = ks + lane * (HD + 1);
+      const float *kr0 = ks + lane * (HD + 1), *kr1 = kr0 + 32 * (HD + 1);
+      float a0[2] = {0.f, 0.f}, a1[2] = {0.f, 0.f};       // two chains per key
 #pragma unroll 8
-      for (int k = 0; k < HD; ++k) sc += qr[k] * kr[k];
-      sc = valid ? sc : -INFINITY;
-      float mn = fmaxf(m[j], warp_max(sc));
+      for (int k = 0; k < HD; k += 2) {
+        const float2 qv = *reinterpret_cast<const float2*>(qr + k);
+        a0[0] += qv.x * kr0[k]; a0[1] += qv.y * kr0[k + 1];
+        a1[0] += qv.x * kr1[k]; a1[1] += qv.y * kr1[k + 1];
+      }
+      const float sc0 = ok0 ? a0[0] + a0[1] : -INFINITY, sc1 = ok1 ? a1[0] + a1[1] : -INFINITY;
+      const float mn = fmaxf(m[j], warp_max(fmaxf(sc0, sc1)));
       if (mn == -INFINITY) continue;
-      float alpha = expf(m[j] - mn);
-      float p = valid ? expf(sc - mn) : 0.f;
-      l[j] = l[j] * alpha + warp_sum(p);
-      float acc[KPL];
+      const float alpha = expf(m[j] - mn);
+      const float w0 = ok0 ? expf(sc0 - mn) : 0.f, w1 = ok1 ? expf(sc1 - mn) : 0.f;
+      l[j] = l[j] * alpha + warp_sum(w0 + w1);
+      float acc0[KPL], acc1[KPL];
 #pragma unroll
-      for (int kk = 0; kk < KPL; ++kk) acc[kk] = o[j][kk] * alpha;
+      for (int kk = 0; kk < KPL; ++kk) { acc0[kk] = o[j][kk] * alpha; acc1[kk] = 0.f; }
 #pragma unroll 8
-      for (int jj = 0; jj < ATT_TILE; ++jj) {
-        float pj = __shfl_sync(0xffffffffu, p, jj);
+      for (int jj = 0; jj < 32; ++jj) {
+        const float p0j = __shfl_sync(0xffffffffu, w0, jj), p1j = __shfl_sync(0xffffffffu, w1, jj);
 #pragma unroll
-        for (int kk = 0; kk < KPL; ++kk) acc[kk] += pj * vs[jj * HD + lane + 32 * kk];
+        for (int kk = 0; kk < KPL; ++kk) {
+          acc0[kk] += p0j * vs[jj * HD + lane + 32 * kk];
+          acc1[kk] += p1j * vs[(jj + 32) * HD + lane + 32 * kk];
+        }
       }
 #pragma unroll
-      for (int kk = 0; kk < KPL; ++kk) o[j][kk] = acc[kk];
+      for (int kk = 0; kk < KPL; ++kk) o[j][kk] = acc0[kk] + acc1[kk];
       m[j] = mn;
     }
   }

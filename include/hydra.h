@@ -240,7 +240,7 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  * Serving loops that must stay clear of the allocator's locks and implicit synchronisation, plugins living
  * inside a host's fixed memory budget, and processes whose free memory already belongs to a pool cannot
  * supply hydra_gemm's partial_dev buffer; here the partial sums live in an 8 MiB array that is part of the
- * library image (every GPU that loads the library holds it until the process exits).
+ * library image (every GPU that loads the library holds it, and a 64 KiB table of counters, until the process exits).
  *   - x [m][k], w [n][k] bfloat16, out [m][n] float, status_dev as in hydra_gemm: all caller-owned device
  *     memory; n % 128 == 0, k % 64 == 0.
  *   - m * n * 4 bytes must fit in the 8 MiB array (the work is shared out among as many CTAs as the partial sums in it
@@ -250,7 +250,7 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  *     address (cudaGetSymbolAddress, with that device current); make that first call outside any stream
  *     capture.
  *   - All calls on a GPU share the one array and it keeps the previous call's partial sums; the GEMM
- *     overwrites every element it later reads, so no clearing is needed, but two calls whose kernels overlap
+ *     overwrites every element it later reads and leaves the counters at zero, so no clearing is needed, but two calls whose kernels overlap
  *     on the GPU (different streams, different threads) race on it: serialise them. */
 hydra_status hydra_gemm_noalloc(const void* x_dev, const void* w_dev, float* out_dev, int m, int n, int k,
                                 int32_t* status_dev, void* stream);

@@ -87,7 +87,7 @@ def _check(code: int, what: str):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())      # torch.cuda.current_stream().cuda_stream without the wrapper object
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -244,8 +244,8 @@ def _need(cond: bool, what: str):
 
 
 def _dense_cuda(t: torch.Tensor, dtype, name: str):
-    _need(isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype == dtype,
-          "%s must be a contiguous CUDA tensor of %s" % (name, dtype))
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype == dtype):
+        raise HydraError("bad argument: %s must be a contiguous CUDA tensor of %s" % (name, dtype))
 
 
 def gemm(x: torch.Tensor, w: torch.Tensor, mode: int = 0) -> torch.Tensor:

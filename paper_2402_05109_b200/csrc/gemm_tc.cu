@@ -138,8 +138,24 @@ __device__ __forceinline__ void store_few(uint32_t taddr, int acc_cols, bool cat
   }
 }
 
+// The slots of one tile (128 columns) added in slot order into the output by the 128 epilogue threads: a warp per row, 16 bytes
+// per lane, two rows with all their slots in flight.
+__device__ __forceinline__ void sum_tile(const float* part, size_t stride, int slots, float* out, int rows, int n, int e) {
+  const int c = (e & 31) * 4;
+#pragma unroll 1
+  for (int r = e >> 5; r < rows; r += 8) {
+    const size_t off[2] = {(size_t)r * n + c, (size_t)(r + 4) * n + c};
+    const int ns[2] = {slots, r + 4 < rows ? slots : 0};
+    float4 v[2];
+    sum_slots_multi<2, 12>(part, stride, off, ns, v);
+    *reinterpret_cast<float4*>(out + off[0]) = v[0];
+    if (ns[1]) *reinterpret_cast<float4*>(out + off[1]) = v[1];
+  }
+}
+
 struct GemmArgs {
   float* part; size_t slot_stride;
+  float* out; unsigned int* arrived;       // REDUCE only: the output, and per tile how many of its CTAs have stored (zero between calls)
   int m, n, kb, m_tiles, total_units, q;
   int x_lo_rows;                 // row offset of the lo plane inside the activation tensor map (0: single plane)
   // activation rows per tile, boxes (planes) of a stage, MMA passes over a weight tile and columns of one, ring stages,
@@ -157,6 +173,20 @@ struct GemmArgs {
     if (a.diag && atomicCAS(a.diag, 0, (site)) == 0) { a.diag[1] = blockIdx.x; a.diag[2] = (unit); a.diag[3] = n_units; \
       a.diag[4] = gridDim.x; a.diag[5] = a.m; a.diag[6] = a.n; a.diag[7] = a.kb; } } while (0)
 
+__device__ __forceinline__ void epilogue_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ bool epilogue_all(bool v) {       // v of all 128 epilogue threads
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, 128, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
+
 constexpr int MAX_STAGES = 10;
 constexpr int EPI_WARPS = 4;                             // one per quadrant of tensor memory (two measured no faster: the L2 takes the stores no sooner)
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
@@ -164,7 +194,9 @@ constexpr int RING_BYTES = 200 * 1024;
 constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
 
 // Shapes are run-time arguments (one copy of the code for all row counts); NH: 128-row weight tiles per CTA and unit.
-template <int NH>
+// REDUCE (stand-alone calls): the last CTA to store a tile's partial sums adds them, so the call is one launch.  (Inside a
+// forward call the consumer kernels add them: there the extra round trip through the counters is on the critical path.)
+template <int NH, bool REDUCE>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const GemmArgs a) {
   constexpr int W_BYTES = NH * A_BYTES, BN = NH * BLOCK_N;        // weight rows of a unit
@@ -178,7 +210,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   auto accfull_bar = [&](int i) { return bars + 8u * (2 * MAX_STAGES + i); };
   auto accempty_bar = [&](int i) { return bars + 8u * (2 * MAX_STAGES + 2 + i); };
   const uint32_t tmem_slot = bars + 8u * (2 * MAX_STAGES + 4);
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_last;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u_begin = blockIdx.x * a.q;
@@ -290,7 +322,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * NH * a.acc_cols);
       float* dst = a.part + (size_t)slot * a.slot_stride + (size_t)m0 * a.n + n0 + quarter * 32 + lane;
       const int tiles_in = NH == 2 && n0 + BLOCK_N < a.n ? 2 : 1;      // an output that is no multiple of the unit's width ends inside its last unit
-      const bool ok = mbar_wait(accfull_bar(acc), acc_ph, a.wait_limit);
+      bool ok = mbar_wait(accfull_bar(acc), acc_ph, a.wait_limit);
+      if constexpr (REDUCE) ok = epilogue_all(ok);       // the four warps meet at barriers below: they give up together
       if (!__all_sync(0xffffffffu, ok)) { if (lane == 0) GIVE_UP(5, i); s_abort = 1; break; }
       tc_fence_after();
       if (rows <= 16) {
@@ -302,6 +335,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(accempty_bar(acc));     // the MMA lane may reuse this accumulator
+      if constexpr (REDUCE) {
+        const int slots = ((tile + 1) * a.kb - 1) / a.q - tile * a.kb / a.q + 1;
+        epilogue_barrier();
+        if (threadIdx.x == 64) {                         // one fence covers what the barrier has ordered before it
+          __threadfence();
+          s_last = atomicAdd(a.arrived + tile, 1u) == (unsigned)(slots - 1);
+          __threadfence();
+        }
+        epilogue_barrier();
+        if (s_last) {
+          if (threadIdx.x == 64) a.arrived[tile] = 0u;   // for the next call
+          const size_t at = (size_t)m0 * a.n + n0;
+#pragma unroll 1
+          for (int hh = 0; hh < tiles_in; ++hh) sum_tile(a.part + at + hh * BLOCK_N, a.slot_stride, slots, a.out + at + hh * BLOCK_N, rows, a.n, (int)threadIdx.x - 64);
+        }
+      }
       i += seg_len;
       if (++acc == a.acc_bufs) { acc = 0; acc_ph ^= 1u; }
     }
@@ -315,11 +364,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, a.tmem_cols); }
 }
 
-template <int NH>
+template <int NH, bool REDUCE>
 hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, cudaStream_t st) {
   static PerDeviceFlag attr_done;
   if (!attr_done.get()) {
-    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<NH, REDUCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
     attr_done.set();
   }
   cudaLaunchConfig_t cfg = {};
@@ -328,7 +377,7 @@ hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  HYDRA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<NH>, tw, tx, a));
+  HYDRA_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<NH, REDUCE>, tw, tx, a));
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -386,7 +435,8 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
 }
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
-                     SplitDesc* sd_out, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap) {
+                     SplitDesc* sd_out, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap, float* out,
+                     unsigned int* arrived) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
   int grid = 1;
@@ -416,7 +466,15 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
     return HYDRA_ERR_CUDA;
   }
   if (sd_out) *sd_out = sd;
-  return sh.nh == 2 ? launch<2>(tw, tx, a, grid, st) : launch<1>(tw, tx, a, grid, st);
+  // One launch where issuing a second one is what takes the time: up to 16 rows and a weight matrix that passes in a few microseconds
+  // (back to back, one launch / two: 11 x 2048 x 2048 6.3 / 8.3 us, 4 x 3456 x 640 6.4 / 8.3, 8 x 640 x 5632 8.0 / 8.2; but
+  // 11 x 4096 x 2048 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x 1024 10.2 / 8.3: the sums of a tile are one CTA's work)
+  if (out && m <= 16 && (long long)n * k <= 6 * 1000 * 1000) {
+    a.out = out; a.arrived = arrived;
+    return sh.nh == 2 ? launch<2, true>(tw, tx, a, grid, st) : launch<1, true>(tw, tx, a, grid, st);
+  }
+  const hydra_status s = sh.nh == 2 ? launch<2, false>(tw, tx, a, grid, st) : launch<1, false>(tw, tx, a, grid, st);
+  return s == HYDRA_OK && out ? reduce_splits(part, sd, out, m, n, st) : s;
 }
 
 }  // namespace hydra

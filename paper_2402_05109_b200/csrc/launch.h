@@ -12,7 +12,9 @@ namespace hydra {
 struct GemmDebug { uint32_t wait_limit; int skip_unit; };
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
                      SplitDesc* sd_out, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
-                     size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/);
+                     size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/,
+                     float* out = nullptr /*[m][n]: the sums themselves*/, unsigned int* arrived = nullptr /*with out: a zeroed counter per tile, left zeroed*/);
+constexpr size_t GEMM_TILE_COLS = 128;    // an output has at most n / GEMM_TILE_COLS * ceil(m / 16) tiles
 // grid: CTAs.  part_cap (floats, 0: no limit): fewer CTAs, hence fewer slots, where the partial sums would not fit otherwise.
 SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap = 0);
 bool gemm_tc_available();                 // driver entry point for tensor-map encoding found

@@ -12,7 +12,10 @@ namespace {
 // Partial sums of the stream-K GEMM: hydra_gemm_partial_floats(m, n, k, 1, 0) floats.  8 MiB per GPU that loads the library, held until
 // the process exits.  Shared by every call (and every thread) on that GPU.
 constexpr size_t NOALLOC_SCRATCH_BYTES = 8u << 20;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
+// behind them a counter per output tile (how many CTAs have stored it; zero between calls): m n floats fit in the scratch, a tile has
+// 128 columns, and row tiles multiply only where there are hundreds of rows, so 2^21 / 128 counters cover every call
+constexpr size_t NOALLOC_TILES = NOALLOC_SCRATCH_BYTES / sizeof(float) / hydra::GEMM_TILE_COLS;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_TILES * sizeof(unsigned int)];
 
 // device address of the array, per device; 0 until the first call on that device has looked it up (any thread may
 // make that call: the slot is an atomic, and two threads racing on it store the same address)
@@ -25,10 +28,7 @@ extern "C" hydra_status hydra_gemm_noalloc(const void* x, const void* w, float* 
   using namespace hydra;
   if (!x || !w || !out || !status || m < 1 || n < 1 || k < 1) return HYDRA_ERR_INVALID;
   if (n % 128 || k % 64) return HYDRA_ERR_UNSUPPORTED;
-  int slots = 1;
-  constexpr size_t CAP = NOALLOC_SCRATCH_BYTES / sizeof(float);
-  gemm_tc_plan(m, n, k, nullptr, &slots, CAP);
-  if ((size_t)slots * (size_t)m * (size_t)n * sizeof(float) > NOALLOC_SCRATCH_BYTES) {
+  if ((size_t)m * (size_t)n * sizeof(float) > NOALLOC_SCRATCH_BYTES) {
     set_last_error("hydra_gemm_noalloc: the partial sums exceed the 8 MiB built-in scratch", cudaErrorInvalidValue);
     return HYDRA_ERR_CAPACITY;
   }
@@ -44,10 +44,8 @@ extern "C" hydra_status hydra_gemm_noalloc(const void* x, const void* w, float* 
     g_scratch_ptr[dev].store(addr, std::memory_order_release);
   }
   if (!gemm_tc_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
-  cudaStream_t st = (cudaStream_t)stream;
   float* part = reinterpret_cast<float*>(addr);
-  // every partial element the reduction reads is written by the GEMM first, so nothing has to be cleared
-  SplitDesc sd;
-  HYDRA_TRY(gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, &sd, status, nullptr, nullptr, st, CAP));
-  return reduce_splits(part, sd, out, m, n, st);
+  // every partial element that is added is written first, and the counters are left at zero, so nothing has to be cleared
+  return gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, nullptr, status, nullptr, nullptr, (cudaStream_t)stream,
+                 NOALLOC_SCRATCH_BYTES / sizeof(float), out, reinterpret_cast<unsigned int*>(addr + NOALLOC_SCRATCH_BYTES));
 }

@@ -20,3 +20,19 @@ def test_gemm_tile_edges(m, n, k):
         ref = (planes.double().sum(0) if planes.dim() == 3 else planes.double()) @ w.double().T
         out = gemm(planes, w, mode=0).double()
         assert float((out - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 64), (1, 256, 256), (11, 2048, 2048), (16, 640, 5632), (16, 1408, 4288), (17, 1408, 4288), (3, 4096, 4096)])
+def test_gemm_noalloc_one_and_two_launches(m, n, k):
+    """Both sides of the choice between adding the partial sums in the GEMM's own launch and in a second one; several calls in a
+    row, because the counters of one call have to be left clean for the next."""
+    from paper_2402_05109_b200 import gemm_noalloc
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 63, n, 0.02)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for i in range(4):
+        x = normal_(torch.empty(m, k, dtype=torch.bfloat16, device="cuda"), 64 + i, m + k, 1.0)
+        out = torch.full((m, n), float("nan"), device="cuda")
+        gemm_noalloc(x, w, out, status)
+        ref = x.double() @ w.double().T
+        assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+    assert int(status.item()) == 0

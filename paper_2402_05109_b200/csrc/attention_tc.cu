@@ -83,8 +83,6 @@ struct AttArgs {
   int H, max_seq, nchunks;
   int* status;
   uint32_t wait_limit;
-  int row_off;                         // first row (of each sequence's rs.tc row slots) this launch computes: a wide causal chunk
-                                       // runs as several launches of QROWS rows, each seeing the earlier ones as cache rows
   int early;                           // the lengths (rs.pos0, rs.n_rows) and the committed cache rows were written by kernels that
                                        // completed before the preceding kernel started (see tree_attention_tc)
 };
@@ -100,7 +98,11 @@ template <int HD, int QROWS, int NP> struct AttCfg {
   static constexpr int V_BYTES = NP * NHALF * TILE * 128;     // a V tile: [plane][half][key][128 bytes] (N blocks of 64 output columns)
   // K and V tiles travel through rings of their own: a K stage is free again as soon as the scores of its tile are done,
   // long before the tile's P V product frees the V stage, so K runs further ahead inside the same shared memory.
-  static constexpr int NSK = K_BYTES >= 32768 ? 3 : 4;            // K ring stages
+  // Two planes of 128 query rows at head_dim 128 take 64 KB of Q and 32 KB per P tile: one P buffer (written when the previous
+  // tile's P V product is done) and two stages each just fit.  A tile of 128 rows costs the tensor pipe what one of 64 does.
+  static constexpr bool TIGHT = Q_BYTES > 32768;
+  static constexpr int NPB = TIGHT ? 1 : 2;                       // P buffers
+  static constexpr int NSK = TIGHT ? 2 : K_BYTES >= 32768 ? 3 : 4;      // K ring stages
   static constexpr int NSV = V_BYTES >= 32768 ? 2 : 4;            // V ring stages
   // MMA M is 128 whatever QROWS is: with 64 query rows the upper 64 accumulator lanes are unused (M = 64 instructions
   // measured slower per instruction), and the operand reads of a 64-row Q or P tile run 8 KB past the tile, into the next
@@ -114,9 +116,9 @@ template <int HD, int QROWS, int NP> struct AttCfg {
   // their row maxima through XM_BYTES of shared memory.  128 rows: one warp per quadrant, thread = row, all keys.
   static constexpr bool SPLIT = QROWS == 64;
   static constexpr int KPT = SPLIT ? TILE / 2 : TILE;                // keys per softmax thread and tile
-  static constexpr int XM_BYTES = 2 * 2 * 64 * 4;                    // [tile parity][key half][row]
+  static constexpr int XM_BYTES = SPLIT ? 2 * 2 * 64 * 4 : 0;        // [tile parity][key half][row]
   static constexpr int NBAR = 1 + 2 * NSK + 2 * NSV + 8 + 4;
-  static constexpr int SMEM_BYTES = 1024 + Q_BYTES + 2 * P_BYTES + (RING_BYTES > MERGE_BYTES ? RING_BYTES : MERGE_BYTES) + XM_BYTES + NBAR * 8 + 16;
+  static constexpr int SMEM_BYTES = 1024 + Q_BYTES + NPB * P_BYTES + (RING_BYTES > MERGE_BYTES ? RING_BYTES : MERGE_BYTES) + XM_BYTES + NBAR * 8 + 16;
   static constexpr int NTHREADS = 256;
   static constexpr int S_COLS = NP * TILE;                    // one score buffer: [Q_hi K_hi + Q_lo K_hi | Q_hi K_lo]
   static constexpr int O_COLS = NP * HD;                      // the output accumulator: [P_hi V_hi + P_lo V_hi | P_hi V_lo]
@@ -136,7 +138,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   constexpr int NSK = C::NSK, NSV = C::NSV;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t q_s = base, p_s = q_s + C::Q_BYTES, ring_s = p_s + 2 * C::P_BYTES, vring_s = ring_s + C::KRING_BYTES;
+  const uint32_t q_s = base, p_s = q_s + C::Q_BYTES, ring_s = p_s + C::NPB * C::P_BYTES, vring_s = ring_s + C::KRING_BYTES;
   const uint32_t xm_s = ring_s + (C::RING_BYTES > C::MERGE_BYTES ? C::RING_BYTES : C::MERGE_BYTES);
   const uint32_t bars = xm_s + C::XM_BYTES;
   const uint32_t q_full = bars;
@@ -186,9 +188,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     const AttBlock blk = rs.blocks[b];
     seq = blk.seq; q_row0 = blk.row0; nr = min(blk.n, QROWS); p0 = blk.pos0; p_call = blk.call0;
   } else {
-    seq = b; q_row0 = b * rs.tc + a.row_off;
-    nr = min(max((rs.n_rows ? rs.n_rows[b] : rs.tc) - a.row_off, 0), QROWS);
-    p_call = rs.pos0[b]; p0 = p_call + a.row_off;
+    seq = b; q_row0 = b * rs.tc;
+    nr = min(rs.n_rows ? rs.n_rows[b] : rs.tc, QROWS);
+    p0 = p_call = rs.pos0[b];
   }
   const int total = p0 + nr;
   const int nt = (total + TILE - 1) / TILE;
@@ -290,7 +292,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         if (!mbar_wait(p_full(i & 1), (uint32_t)((i >> 1) & 1), limit)) { ok = false; break; }
         if (!mbar_wait(v_full(s), (uint32_t)((i / NSV) & 1), limit)) { ok = false; break; }
         tc_fence_after();
-        const uint64_t vd = v_desc + (uint64_t)((s * C::V_BYTES) >> 4), pd = p_desc + (uint64_t)(((i & 1) * C::P_BYTES) >> 4);
+        const uint64_t vd = v_desc + (uint64_t)((s * C::V_BYTES) >> 4), pd = p_desc + (uint64_t)(((i % C::NPB) * C::P_BYTES) >> 4);
         const uint32_t d_o = tmem_base + (uint32_t)C::O_COL0;
 #pragma unroll
         for (int kk = 0; kk < TILE / 16; ++kk)
@@ -398,8 +400,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           }
         }
         l = l * alpha + sum;
-        // P buffer i & 1 was last read by P V of tile i - 2; the row's accumulator by P V of tile i - 1
-        if (i >= 2 && !mbar_wait(pv_done(i & 1), (uint32_t)(((i >> 1) - 1) & 1), limit)) { ok = false; break; }
+        // P buffer i % NPB was last read by P V of tile i - NPB; the row's accumulator by P V of tile i - 1
+        if (i >= C::NPB && !mbar_wait(pv_done((i - C::NPB) & 1), (uint32_t)(((i - C::NPB) >> 1) & 1), limit)) { ok = false; break; }
         if (__any_sync(0xffffffffu, rescale)) {            // both warps of a quadrant decide alike; each scales its half of the columns
           if (i >= 1 && !mbar_wait(pv_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), limit)) { ok = false; break; }
           tc_fence_after();
@@ -413,7 +415,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             tmem_st32(lane_addr + (uint32_t)(C::O_COL0 + c0), o);
           }
         }
-        const uint32_t prow = p_s + (i & 1) * C::P_BYTES + (uint32_t)row * 128u;
+        const uint32_t prow = p_s + (i % C::NPB) * C::P_BYTES + (uint32_t)row * 128u;
         if (row_valid) {
 #pragma unroll
           for (int ch = 0; ch < KPT / 8; ++ch) {
@@ -434,7 +436,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           }
         }
       } else {
-        if (i >= 2 && !mbar_wait(pv_done(i & 1), (uint32_t)(((i >> 1) - 1) & 1), limit)) { ok = false; break; }
+        if (i >= C::NPB && !mbar_wait(pv_done((i - C::NPB) & 1), (uint32_t)(((i - C::NPB) >> 1) & 1), limit)) { ok = false; break; }
       }
       if (t0 + TILE > total) {
         // rows of the V tile past the end of the sequence hold whatever the cache holds: zero them, so that a
@@ -508,7 +510,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     constexpr int V4 = HD / 4;
     const uint32_t xo_s = ring_s, xml_s = ring_s + QROWS * HD * 4;
     const int d = H * HD;
-    const int rows_cap = rs.blocks ? nr : min(rs.tc - a.row_off, QROWS);
+    const int rows_cap = rs.blocks ? nr : min(rs.tc, QROWS);
     const int my_rows = rows_cap > c ? (rows_cap - c + nchunks - 1) / nchunks : 0;
     // chunk weights of my rows, normalised: w_c = 2^(m_c - M) / sum_c l_c 2^(m_c - M)  (one thread per row, all (m, l) loads in flight together)
     for (int t = tid; t < my_rows; t += C::NTHREADS) {
@@ -592,7 +594,7 @@ int pick_chunks(int pairs, int len_upper, int sms) {
 
 template <int HD, int QROWS, int NP>
 hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, RowSet rs, bf16* out, size_t out_ps,
-                 int H, int max_seq, int len_upper, int* status, bool stable_lengths, int row_off, cudaStream_t st) {
+                 int H, int max_seq, int len_upper, int* status, bool stable_lengths, cudaStream_t st) {
   using C = AttCfg<HD, QROWS, NP>;
   CUtensorMap tq, tk, tv;
   const uint64_t cache_rows = (uint64_t)cache_batch * H * max_seq;
@@ -609,7 +611,7 @@ hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc
   }
   AttArgs a{};
   a.rs = rs; a.out = out; a.out_ps = out_ps; a.H = H; a.max_seq = max_seq; a.status = status; a.wait_limit = WAIT_LIMIT;
-  a.q_plane_rows = q_rows; a.kv_plane_rows = (int)cache_rows; a.early = stable_lengths ? 1 : 0; a.row_off = row_off;
+  a.q_plane_rows = q_rows; a.kv_plane_rows = (int)cache_rows; a.early = stable_lengths ? 1 : 0;
   const int groups = rs.blocks ? rs.n_blocks : rs.batch;
   a.nchunks = pick_chunks(H * groups, len_upper, sm_count());
   cudaLaunchConfig_t cfg = {};
@@ -628,27 +630,16 @@ hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc
 template <int NP>
 hydra_status dispatch(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, RowSet rs, bf16* out, size_t out_ps,
                       int H, int hd, int max_seq, int len_upper, int* status, bool stable_lengths, cudaStream_t st) {
-  const bool wide = rs.blocks ? attention_block_rows(hd, NP) > 64 : rs.tc > 64;
-  if (hd == 128 && wide && NP == 2) {
-    // Q, P and the rings of two planes for 128 query rows exceed the shared memory of an SM: 64 rows per launch; the rows of
-    // an earlier launch are cache rows to a later one (the preceding kernel has appended the K and V rows of the whole chunk)
-    for (int off = 0; off < rs.tc; off += 64) {
-      hydra_status r = run<128, 64, 2>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, off, st);
-      if (r != HYDRA_OK) return r;
-    }
-    return HYDRA_OK;
-  }
-  if (hd == 128) return wide ? run<128, 128, 1>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, 0, st)
-                             : run<128, 64, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, 0, st);
-  if (hd == 64) return wide ? run<64, 128, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, 0, st)
-                            : run<64, 64, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, 0, st);
+  const bool wide = rs.blocks || rs.tc > 64;
+  if (hd == 128) return wide ? run<128, 128, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, st)
+                             : run<128, 64, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, st);
+  if (hd == 64) return wide ? run<64, 128, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, st)
+                            : run<64, 64, NP>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, max_seq, len_upper, status, stable_lengths, st);
   return HYDRA_ERR_UNSUPPORTED;
 }
 
 }  // namespace
 
-// Query rows of a packed attention block: two planes of Q, P and the rings for 128 rows exceed an SM's shared memory at head_dim 128.
-int attention_block_rows(int head_dim, int planes) { return head_dim == 128 && planes == 2 ? 64 : 128; }
 
 hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, int planes, RowSet rs,
                                bf16* out, size_t out_ps, int H, int hd, int max_seq, int len_upper, int* status, bool stable_lengths,

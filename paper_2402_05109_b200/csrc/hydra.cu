@@ -360,7 +360,7 @@ hydra_status run_prefix(hydra_ctx* c, const float* src, const RowSet& rs, int le
 // of consecutive rows of one sequence.  Synchronises the stream once (the block table is a host buffer).
 hydra_status prompt_packed(hydra_ctx* c, const int* tokens, const int* offs, cudaStream_t st) {
   const hydra_model_cfg& m = c->m;
-  const int B = c->batch, base = offs[0], total = offs[B] - base, qrows = attention_block_rows(m.head_dim, c->kv_planes);
+  const int B = c->batch, base = offs[0], total = offs[B] - base, qrows = ATT_BLOCK_ROWS;
   const int passes = (total + PROMPT_ROWS - 1) / PROMPT_ROWS;
   const int step = ((total + passes - 1) / passes + CHUNK - 1) / CHUNK * CHUNK;
   struct Pass { int g0, rows, block0, n_blocks, len_upper; };
@@ -376,6 +376,8 @@ hydra_status prompt_packed(hydra_ctx* c, const int* tokens, const int* offs, cud
       p.len_upper = std::max(p.len_upper, end - (offs[s] - base));
     }
     p.n_blocks = (int)blocks.size() - p.block0;
+    // the longest first: with more CTAs than SMs the short ones fill the end
+    std::stable_sort(blocks.begin() + p.block0, blocks.end(), [](const AttBlock& a, const AttBlock& b) { return a.pos0 + a.n > b.pos0 + b.n; });
     plan.push_back(p);
   }
   if (blocks.size() > prompt_blocks_cap(m)) return HYDRA_ERR_CAPACITY;

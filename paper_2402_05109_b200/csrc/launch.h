@@ -46,8 +46,8 @@ hydra_status tree_attention_f32(const float* q, const float* kcache, const float
 // bfloat16 model path: tensor-core kernel (attention_tc.cu).  q [planes][q_rows][H*hd] and the caches
 // [planes][cache_batch][H][max_seq][hd] are float16 in 1 or 2 planes (hi = f16(v), lo = f16(v - hi)); out is bfloat16
 // [rows][H*hd] in two planes out_ps elements apart (0: hi only).  rs.mask == null selects a causal chunk (row i sees
-// the committed slots and new slots 0..i) of up to 128 rows (one plane, or head_dim 64); with a mask, up to 64 rows.
-// A packed row set runs one CTA column per attention block of at most attention_block_rows(...) rows.
+// the committed slots and new slots 0..i) of up to 128 rows; with a mask, up to 64 rows.
+// A packed row set runs one CTA column per attention block of at most ATT_BLOCK_ROWS rows.
 // stable_lengths: rs.pos0 / rs.n_rows and every cache row below pos0 were written by kernels that had COMPLETED before the
 // kernel preceding this one in the stream started (true inside a forward call of the library, whose first kernel holds
 // its successors back until everything earlier has completed); the kernel then requests committed cache tiles before it
@@ -55,7 +55,7 @@ hydra_status tree_attention_f32(const float* q, const float* kcache, const float
 hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, int planes, RowSet rs,
                                bf16* out, size_t out_ps, int n_heads, int head_dim, int max_seq, int len_upper, int* status,
                                bool stable_lengths, cudaStream_t st);
-int attention_block_rows(int head_dim, int planes);
+constexpr int ATT_BLOCK_ROWS = 128;
 hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, int dtype,
                       cudaStream_t st);
 // amax[r] = argmax_v of the summed partial logits (lowest id among equal maxima); the sums go to logits_out if given

@@ -112,7 +112,7 @@ hydra_status hydra_destroy(hydra_ctx*);
  * "Prefix Attention"); leaves, per sequence, the committed length, the root token (argmax after the last
  * prompt token) and the last hidden state.  tokens_dev holds the prompts back to back; seq_offsets_host
  * has batch+1 entries (read before the call returns).  The prompts are processed in passes, every pass
- * streaming the weights once: of up to 512 tokens of the prompts packed back to back (dtype 1), or of 64 rows per sequence
+ * streaming the weights once: of up to 768 tokens of the prompts packed back to back (dtype 1), or of 64 rows per sequence
  * (dtype 0).  Synchronises the stream once (see Conventions).
  * Errors: INVALID (null pointer, batch outside 1..max_batch, empty prompt), CAPACITY (prompt + tree rows
  * exceed max_seq). */

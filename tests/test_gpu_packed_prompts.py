@@ -1,4 +1,4 @@
-"""The packed prompt pass of the bfloat16 path (prompts back to back, at most 512 tokens a pass) against the oracle, in lock-step."""
+"""The packed prompt pass of the bfloat16 path (prompts back to back, at most 768 tokens a pass) against the oracle, in lock-step."""
 import pytest
 
 from synth import load_tree
@@ -9,7 +9,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("head_dim,kv_planes,lens", [
-    (128, 2, [512]), (128, 2, [513]), (128, 2, [1100]),                  # one full pass; one row more; several passes of one sequence
+    (128, 2, [512]), (128, 2, [513]), (128, 2, [768]), (128, 2, [769]), (128, 2, [1600]),      # up to one full pass; one row more; several passes
+    (128, 2, [700, 67, 1]), (128, 2, [700, 67, 1, 1]), (128, 1, [500, 300, 12, 800]),
     (128, 2, [300, 211, 1, 1, 130, 64]), (128, 1, [500, 12, 1]),         # passes that end inside, at the end of and just after a sequence
     (64, 2, [129, 383, 127]), (64, 1, [1, 511, 2])])
 def test_packed_prompt_passes(head_dim, kv_planes, lens):

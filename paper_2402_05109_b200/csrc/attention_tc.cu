@@ -3,43 +3,53 @@
 //
 // Operand format: q, the K cache (post-RoPE), the V cache and the softmax weights are float16 (the values are O(1),
 // far inside the float16 range) in NP planes.  NP = 2: hi = f16(v), lo = f16(v - hi), about 22 significant bits;
-// a product x y is taken as x_hi y_hi + x_hi y_lo + x_lo y_hi.  Stacking the planes of the B operand along its N
+// a product x y is taken as x_hi y_hi + x_hi y_lo + x_lo y_hi.  For the scores, stacking the planes of K along the N
 // dimension gives the first two terms in ONE instruction sequence (accumulator columns [0, n) and [n, 2n), added
-// when the accumulator is read); the third is a second sequence into columns [0, n).  NP = 1: hi only, 11 bits
+// when the accumulator is read); the third is a second sequence into columns [0, n).  For P V, all three go into the
+// same head_dim columns.  NP = 1: hi only, 11 bits
 // (half the cache bytes; hidden states then drift to a few 1e-3 of a float reference over 32 layers).
 // Scores, running maxima, sums and the output accumulate in float.  The result leaves as two bfloat16 planes
 // (hi = bf16(v), lo = bf16(v - hi)), the operand format of the GEMM that consumes it.
 //
 // One CTA per (head, sequence, KV chunk).  A sequence's KV rows are cut into 64-row tiles and the tiles are dealt
 // to the launch's chunks in equal contiguous runs, computed on the device from the real length (a captured graph
-// keeps balanced chunks as the sequence grows).  256 threads:
-//   warp 2 (one lane)  TMA producer: Q once, then K tiles and V tiles through rings of their own (a K stage is free
+// keeps balanced chunks as the sequence grows).  Roles (256 threads for 64 query rows, 320 for 128):
+//   one producer lane  TMA: Q once, then K tiles and V tiles through rings of their own (a K stage is free
 //                      as soon as the scores of its tile are done, a V stage after the tile's P V product), each stage
 //                      with its own "full" barrier, so the scores of a tile start before its V has landed;
-//   warp 3 (one lane)  MMA issue: S_i = Q K_i^T (M = 128 query lanes, N = 64 keys) into one of two score buffers in
-//                      tensor memory, issued one tile ahead; O += P_i V_i (N = head_dim, V read as an MN-major operand
-//                      straight from its [key][dim] tile) into one accumulator that lives across the chunk;
-//   four softmax warps thread = query row (a tensor-memory lane).  With 64 query rows two warps share a quadrant of
-//                      tensor memory (warps 0 and 4: rows 0..31, warps 1 and 5: rows 32..63) and each takes half of a
-//                      tile's keys; the two swap their row maxima through shared memory, keep the same reference
-//                      maximum and each its own part of the row sum.  With 128 rows warps 4..7 take a quadrant each
-//                      and all keys.  A thread reads its scores from tensor memory, applies the scale and
+//   one MMA lane       S_i = Q K_i^T (M = 128 query lanes, N = 64 keys) into one of two score buffers in
+//                      tensor memory; O += P_i V_i (N = head_dim, V read as an MN-major operand
+//                      straight from its [key][dim] tile) into one accumulator that lives across the chunk; whichever of
+//                      the next S and the next P V has its operands is issued;
+//   softmax warps      thread = query row (a tensor-memory lane), all 64 keys of a tile.  Two groups of warps take the tiles in
+//                      turn, even and odd, so that one group's exponentials run while the other waits for scores, loads
+//                      them or stores its P.  A thread reads its scores from tensor memory, applies
 //                      the mask (committed slots are visible to every row; tree slot j to row i iff bit j of the
-//                      row's ancestor bitmask, or j <= i for a causal chunk), keeps the row's running reference
-//                      maximum and sum in the exp2 domain, writes P_i as float16 into a swizzled shared-memory
-//                      tile for the MMA.  The reference maximum only moves when a tile's maximum exceeds it by
+//                      row's ancestor bitmask, or j <= i for a causal chunk), takes the row's running reference
+//                      maximum (exp2 domain) over from the other group, hands it on, and writes P_i as float16 into tensor
+//                      memory, the A operand of the P V product.  The reference maximum only moves when a tile's maximum exceeds it by
 //                      more than 8 (a factor 256, harmless in float16 and float); only then is the row's output
 //                      accumulator rescaled in tensor memory (load, scale, store), so the common tile needs no
-//                      round trip through registers for O.
+//                      round trip through registers for O.  Each group keeps its own row sum.
+// What bounds a tile of the loop (two planes, head_dim 128): 64 KB from memory (1.1 us with 120 CTAs at 7 TB/s), about 1800
+// cycles of shared memory and 1540 of the tensor pipe (see S_COLS), 512 of exponentials per 32 rows; a softmax step is a chain of
+// about 1600 cycles, of which two run at a time.  With one group of softmax warps (a tile of 64 rows shared by two warps), P in
+// shared memory and the rows of one chunk merged like those of several, a layer took, against now: 64 rows x 8 sequences of 250 to
+// 1100 tokens x 32 heads 49.7 -> 42.7 us, 40 heads x 2000 tokens 30.5 -> 26.8 us, 32 heads x 600 tokens 12.0 -> 10.9 us; 768 prompt
+// rows of two sequences 41.6 -> 27 us, of one sequence at 2000 tokens (40 heads) 85 -> 68 us, of four (52 heads) 84 -> 62 us.
 // Query rows beyond the row count of the call ride along as unused lanes of the M = 128 tile.
-// The chunks of a (head, sequence) pair (at most 8) form a thread-block cluster: every CTA leaves its partial rows
+// One chunk: the softmax warps normalise their rows out of tensor memory and write them, through a warp's own piece of the
+// idle ring for whole 128-byte stores; no cluster, no merge.
+// Several chunks of a (head, sequence) pair (at most 8) form a thread-block cluster: every CTA leaves its partial rows
 // (un-normalised output, reference maximum, sum) in its own shared memory, and each CTA merges a share of the rows
 // out of its peers' shared memory, in chunk order (deterministic; no scratch traffic, no atomics).
+// (Sending the rows to the CTA that merges them, instead of reading them from there, took longer: 1.5 us for 64 rows of a chunk.)
 // Every barrier wait is bounded; when one runs out the CTA raises the time-out bit of the status word, skips its
 // stores, still takes part in the cluster barriers, frees its tensor memory and returns.
 #include "tc.cuh"
 #include <cuda_fp16.h>
 #include <math.h>
+#include <algorithm>
 
 namespace hydra {
 
@@ -66,6 +76,11 @@ __device__ __forceinline__ float4 ld_peer4(uint32_t addr) {
   asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
   return v;
 }
+__device__ __forceinline__ float4 ld_smem4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -74,6 +89,33 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   __half2 v = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+// two floats in one register pair: one instruction for both
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1,%2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0,%1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 v;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+  return v;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 v;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+  return v;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float v;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(v) : "f"(a), "f"(b), "f"(c));
+  return v;
 }
 
 struct AttArgs {
@@ -91,55 +133,53 @@ template <int HD, int QROWS, int NP> struct AttCfg {
   static constexpr int NHALF = HD / 64;                       // 64-column (128-byte) halves of a head row
   static constexpr int QP_BYTES = NHALF * QROWS * 128;        // one plane of Q: [half][query row][128 bytes]
   static constexpr int Q_BYTES = NP * QP_BYTES;
-  static constexpr int PP_BYTES = QROWS * 128;                // one plane of a P tile: [query row][64 keys] float16
-  static constexpr int P_BYTES = NP * PP_BYTES;
   static constexpr int KH_BYTES = NP * TILE * 128;            // one half of a K tile: [plane][key][128 bytes] (the planes stacked along N)
   static constexpr int K_BYTES = NHALF * KH_BYTES;
   static constexpr int V_BYTES = NP * NHALF * TILE * 128;     // a V tile: [plane][half][key][128 bytes] (N blocks of 64 output columns)
   // K and V tiles travel through rings of their own: a K stage is free again as soon as the scores of its tile are done,
   // long before the tile's P V product frees the V stage, so K runs further ahead inside the same shared memory.
-  // Two planes of 128 query rows at head_dim 128 take 64 KB of Q and 32 KB per P tile: one P buffer (written when the previous
-  // tile's P V product is done) and two stages each just fit.  A tile of 128 rows costs the tensor pipe what one of 64 does.
-  static constexpr bool TIGHT = Q_BYTES > 32768;
-  static constexpr int NPB = TIGHT ? 1 : 2;                       // P buffers
-  static constexpr int NSK = TIGHT ? 2 : K_BYTES >= 32768 ? 3 : 4;      // K ring stages
-  static constexpr int NSV = V_BYTES >= 32768 ? 2 : 4;            // V ring stages
+  // Two planes at head_dim 128: 64 KB a tile, 32 KB (64 query rows) or 64 KB (128) of Q.
+  static constexpr int NSK = K_BYTES >= 32768 ? 3 : 4;           // K ring stages
+  static constexpr int NSV = V_BYTES >= 32768 ? (Q_BYTES > 32768 ? 2 : 3) : 4;      // V ring stages
   // MMA M is 128 whatever QROWS is: with 64 query rows the upper 64 accumulator lanes are unused (M = 64 instructions
-  // measured slower per instruction), and the operand reads of a 64-row Q or P tile run 8 KB past the tile, into the next
-  // piece of Q, of P or of the ring (never read back), so the order Q, P0, P1, ring keeps them inside the allocation.
+  // measured slower per instruction), and the operand reads of a 64-row Q tile run 8 KB past the tile, into the next
+  // piece of Q or the ring (never read back).
   static constexpr int MROWS = 128;
-  static constexpr int RPW = MROWS / 4;                       // accumulator rows (tensor-memory lanes) per softmax warp
   static constexpr int KRING_BYTES = NSK * K_BYTES;
   static constexpr int RING_BYTES = KRING_BYTES + NSV * V_BYTES;
-  static constexpr int MERGE_BYTES = QROWS * HD * 4 + QROWS * 16;    // a chunk's partial rows + (max, sum, max, sum of the other key half); aliases the ring
-  // 64 query rows: two softmax warps per tensor-memory quadrant, each with half of a tile's keys (SPLIT); they exchange
-  // their row maxima through XM_BYTES of shared memory.  128 rows: one warp per quadrant, thread = row, all keys.
-  static constexpr bool SPLIT = QROWS == 64;
-  static constexpr int KPT = SPLIT ? TILE / 2 : TILE;                // keys per softmax thread and tile
-  static constexpr int XM_BYTES = SPLIT ? 2 * 2 * 64 * 4 : 0;        // [tile parity][key half][row]
-  static constexpr int NBAR = 1 + 2 * NSK + 2 * NSV + 8 + 4;
-  static constexpr int SMEM_BYTES = 1024 + Q_BYTES + NPB * P_BYTES + (RING_BYTES > MERGE_BYTES ? RING_BYTES : MERGE_BYTES) + XM_BYTES + NBAR * 8 + 16;
-  static constexpr int NTHREADS = 256;
-  static constexpr int S_COLS = NP * TILE;                    // one score buffer: [Q_hi K_hi + Q_lo K_hi | Q_hi K_lo]
-  static constexpr int O_COLS = NP * HD;                      // the output accumulator: [P_hi V_hi + P_lo V_hi | P_hi V_lo]
-  static constexpr int O_COL0 = 2 * S_COLS;
-  static constexpr int TMEM_COLS = O_COL0 + O_COLS <= 256 ? 256 : 512;
-  static_assert(RING_BYTES >= MERGE_BYTES + 128 * MAX_CHUNKS * 4, "merge area and chunk weights must fit in the ring");
-  static_assert(MERGE_BYTES % 16 == 0, "alignment of the chunk weights");
-  static_assert(O_COL0 + O_COLS <= 512, "tensor memory");
+  static constexpr int MERGE_BYTES = QROWS * HD * 4 + QROWS * 16;    // a chunk's partial rows + (max, sum) of either group; aliases the ring
+  // softmax warps: group g (even / odd tiles), quadrant q of tensor memory -> warp 4 g + q; 64 query rows only fill quadrants
+  // 0 and 1, which leaves warps 2 and 3 for the producer and the MMA lane
+  static constexpr int NQUAD = QROWS / 32;
+  static constexpr int NTHREADS = QROWS == 64 ? 256 : 320;
+  static constexpr int W_PRODUCER = QROWS == 64 ? 2 : 8, W_MMA = W_PRODUCER + 1;
+  static constexpr int XM_BYTES = 2 * QROWS * 4;                     // [group][row] reference maximum
+  static constexpr int BUF_BYTES = NHALF * NQUAD * 2 * 32 * 128;     // one-chunk result on its way out: 32 rows x 64 columns x 2 planes per warp; aliases the ring
+  static constexpr int NBAR = 1 + 2 * NSK + 2 * NSV + 9 + 2 * NQUAD;
+  static constexpr int SMEM_BYTES = 1024 + Q_BYTES + RING_BYTES + XM_BYTES + NBAR * 8 + 16;
+  // tensor memory: two score buffers [Q_hi K_hi + Q_lo K_hi | Q_hi K_lo], the output accumulator, two P buffers (32 columns a
+  // plane, two keys a column): P is the A operand of P V, so neither its stores nor its reads pass through shared memory,
+  // whose 128 bytes a cycle bound a tile (64 KB in from memory, 112 KB of operands for the scores, 48 KB of V: 1800 cycles; with P
+  // in shared memory 2300)
+  static constexpr int S_COLS = NP * TILE;
+  static constexpr int O_COL0 = 2 * S_COLS, O_COLS = HD;
+  static constexpr int P_COL0 = O_COL0 + O_COLS, P_COLS = NP * TILE / 2;
+  static constexpr int TMEM_COLS = P_COL0 + 2 * P_COLS <= 256 ? 256 : 512;
+  static_assert(RING_BYTES >= MERGE_BYTES && RING_BYTES >= BUF_BYTES + QROWS * 16, "what follows the last tile must fit in the ring");
+  static_assert(P_COL0 + 2 * P_COLS <= 512, "tensor memory");
   static_assert(SMEM_BYTES <= 232448, "shared memory of one SM");
 };
 
 template <int HD, int QROWS, int NP>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(AttCfg<HD, QROWS, NP>::NTHREADS, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const AttArgs a) {
   using C = AttCfg<HD, QROWS, NP>;
   constexpr int NSK = C::NSK, NSV = C::NSV;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  const uint32_t q_s = base, p_s = q_s + C::Q_BYTES, ring_s = p_s + C::NPB * C::P_BYTES, vring_s = ring_s + C::KRING_BYTES;
-  const uint32_t xm_s = ring_s + (C::RING_BYTES > C::MERGE_BYTES ? C::RING_BYTES : C::MERGE_BYTES);
+  const uint32_t q_s = base, ring_s = q_s + C::Q_BYTES, vring_s = ring_s + C::KRING_BYTES;
+  const uint32_t xm_s = ring_s + C::RING_BYTES;
   const uint32_t bars = xm_s + C::XM_BYTES;
   const uint32_t q_full = bars;
   auto k_full = [&](int s) { return bars + 8u * (1 + s); };
@@ -151,11 +191,10 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   auto s_empty = [&](int i) { return bars + 8u * (B0 + 2 + i); };
   auto p_full = [&](int i) { return bars + 8u * (B0 + 4 + i); };
   auto pv_done = [&](int i) { return bars + 8u * (B0 + 6 + i); };
-  auto xm_bar = [&](int par, int quad) { return bars + 8u * (B0 + 8 + 2 * par + quad); };   // both key halves of a quadrant have left their maxima
+  const uint32_t o_done = bars + 8u * (B0 + 8);          // every P V product of the chunk
+  auto xm_bar = [&](int g, int quad) { return bars + 8u * (B0 + 9 + C::NQUAD * g + quad); };   // group g has left the quadrant's reference maxima
   const uint32_t tmem_slot = bars + 8u * C::NBAR;
   __shared__ int s_abort;
-  // normalised chunk weights of the rows this CTA merges: in the idle ring, behind the merge area its peers read
-  float* const s_w = reinterpret_cast<float*>(smem_raw + (ring_s - smem_u32(smem_raw)) + C::MERGE_BYTES);
 
   const RowSet& rs = a.rs;
   const int h = blockIdx.x, b = blockIdx.y, c = blockIdx.z;
@@ -164,15 +203,15 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 
   if (tid == 0) {
     s_abort = 0;
-    mbar_init(q_full, 1);
+    mbar_init(q_full, 1); mbar_init(o_done, 1);
     for (int s = 0; s < NSK; ++s) { mbar_init(k_full(s), 1); mbar_init(k_empty(s), 1); }
     for (int s = 0; s < NSV; ++s) { mbar_init(v_full(s), 1); mbar_init(v_empty(s), 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(s_full(i), 1); mbar_init(s_empty(i), 4); mbar_init(p_full(i), 4); mbar_init(pv_done(i), 1); }
-    for (int i = 0; i < 4; ++i) mbar_init(xm_bar(i >> 1, i & 1), 2);
+    for (int i = 0; i < 2; ++i) { mbar_init(s_full(i), 1); mbar_init(s_empty(i), C::NQUAD); mbar_init(p_full(i), C::NQUAD); mbar_init(pv_done(i), 1); }
+    for (int i = 0; i < 2 * C::NQUAD; ++i) mbar_init(xm_bar(0, i), 1);
     mbar_init_fence();
     prefetch_tensormap(&tmQ); prefetch_tensormap(&tmK); prefetch_tensormap(&tmV);
   }
-  if (warp == 3) tmem_alloc(tmem_slot, C::TMEM_COLS);
+  if (warp == C::W_MMA) tmem_alloc(tmem_slot, C::TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -198,11 +237,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const bool has_work = tile0 < tile1 && nr > 0 && p0 >= 0 && total <= a.max_seq;
   const int ntiles = has_work ? tile1 - tile0 : 0;
   const uint32_t limit = a.wait_limit;
+  const int rows_cap = rs.blocks ? nr : min(rs.tc, QROWS);     // output rows of this pair; those past nr get zeros
 
-  // warp 2: TMA producer (one lane); warp 3: MMA issue (one lane); softmax: warps 0, 1, 4, 5 (quadrants 0, 1, 0, 1; key halves
-  // 0, 0, 1, 1) for 64 query rows, warps 4..7 (quadrants 0..3) for 128
-  const bool softmax_warp = C::SPLIT ? (warp & 2) == 0 : warp >= 4;
-  if (warp == 2) {
+  if (warp == C::W_PRODUCER) {
     if (lane == 0 && has_work) {
       const uint64_t pol = policy_evict_first(), pol_q = policy_evict_last();
       const int row0 = (seq * H + h) * a.max_seq;
@@ -253,20 +290,17 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         else if (++idle > limit) { atomicOr(a.status, ST_TIMEOUT); s_abort = 1; break; }
       }
     }
-  } else if (warp == 3) {
+  } else if (warp == C::W_MMA) {
     if (lane == 0 && has_work) {
       constexpr uint32_t idesc_s = instr_desc_f16(0, C::MROWS, NP * TILE, 0);      // Q_hi x [K_hi ; K_lo]
       constexpr uint32_t idesc_s2 = instr_desc_f16(0, C::MROWS, TILE, 0);          // Q_lo x K_hi
-      constexpr uint32_t idesc_pv = instr_desc_f16(0, C::MROWS, NP * HD, 1);       // P_hi x [V_hi | V_lo]
-      constexpr uint32_t idesc_pv2 = instr_desc_f16(0, C::MROWS, HD, 1);           // P_lo x V_hi
+      constexpr uint32_t idesc_pv = instr_desc_f16(0, C::MROWS, HD, 1);            // P x V
       // operand descriptors: built once; a byte offset inside shared memory adds offset / 16 to the start-address field
-      const uint64_t q_desc = smem_desc_sw128(q_s), p_desc = smem_desc_sw128(p_s), k_desc = smem_desc_sw128(ring_s),
+      const uint64_t q_desc = smem_desc_sw128(q_s), k_desc = smem_desc_sw128(ring_s),
                      v_desc = smem_desc_sw128_mn(vring_s, TILE * 128);
       bool ok = mbar_wait(q_full, 0, limit);
       auto issue_s = [&](int i) {                        // S_i = Q K_i^T into score buffer i & 1
         const int s = i % NSK;
-        if (!mbar_wait(k_full(s), (uint32_t)((i / NSK) & 1), limit)) return false;
-        if (i >= 2 && !mbar_wait(s_empty(i & 1), (uint32_t)(((i >> 1) - 1) & 1), limit)) return false;
         tc_fence_after();
         const uint64_t kd = k_desc + (uint64_t)((s * C::K_BYTES) >> 4);
         const uint32_t d_s = tmem_base + (uint32_t)((i & 1) * C::S_COLS);
@@ -282,132 +316,151 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         }
         umma_commit(k_empty(s));                        // frees the K stage once these MMAs have read it
         umma_commit(s_full(i & 1));
-        return true;
       };
-      if (ok) ok = issue_s(0);
-      for (int i = 0; i < ntiles && ok; ++i) {
-        if (i + 1 < ntiles) ok = issue_s(i + 1);
-        if (!ok) break;
+      auto issue_pv = [&](int i) {
         const int s = i % NSV;
-        if (!mbar_wait(p_full(i & 1), (uint32_t)((i >> 1) & 1), limit)) { ok = false; break; }
-        if (!mbar_wait(v_full(s), (uint32_t)((i / NSV) & 1), limit)) { ok = false; break; }
         tc_fence_after();
-        const uint64_t vd = v_desc + (uint64_t)((s * C::V_BYTES) >> 4), pd = p_desc + (uint64_t)(((i % C::NPB) * C::P_BYTES) >> 4);
-        const uint32_t d_o = tmem_base + (uint32_t)C::O_COL0;
+        const uint64_t vd = v_desc + (uint64_t)((s * C::V_BYTES) >> 4);
+        const uint32_t d_o = tmem_base + (uint32_t)C::O_COL0, p_t = tmem_base + (uint32_t)(C::P_COL0 + (i & 1) * C::P_COLS);
 #pragma unroll
-        for (int kk = 0; kk < TILE / 16; ++kk)
-          umma_f16(d_o, pd + (uint64_t)((kk * 32) >> 4), vd + (uint64_t)((kk * 2048) >> 4), idesc_pv, (uint32_t)((i | kk) != 0));
+        for (int kk = 0; kk < TILE / 16; ++kk)             // P_hi V_hi
+          umma_f16_ts(d_o, p_t + (uint32_t)(kk * 8), vd + (uint64_t)((kk * 2048) >> 4), idesc_pv, (uint32_t)((i | kk) != 0));
         if (NP == 2) {
 #pragma unroll
-          for (int kk = 0; kk < TILE / 16; ++kk)
-            umma_f16(d_o, pd + (uint64_t)((C::PP_BYTES + kk * 32) >> 4), vd + (uint64_t)((kk * 2048) >> 4), idesc_pv2, 1u);
+          for (int kk = 0; kk < TILE / 16; ++kk) {         // + P_hi V_lo + P_lo V_hi
+            umma_f16_ts(d_o, p_t + (uint32_t)(kk * 8), vd + (uint64_t)((C::V_BYTES / 2 + kk * 2048) >> 4), idesc_pv, 1u);
+            umma_f16_ts(d_o, p_t + (uint32_t)(TILE / 2 + kk * 8), vd + (uint64_t)((kk * 2048) >> 4), idesc_pv, 1u);
+          }
         }
         umma_commit(v_empty(s));
         umma_commit(pv_done(i & 1));
+      };
+      // S_i waits for its K tile and for the softmax group to have read S_(i-2); P_i V_i for P_i and its V tile
+      int is = 0, ip = 0;
+      uint32_t idle = 0;
+      while (ok && ip < ntiles) {
+        bool did = false;
+        if (is < ntiles && (is < 2 || mbar_test(s_empty(is & 1), (uint32_t)(((is >> 1) - 1) & 1))) && mbar_test(k_full(is % NSK), (uint32_t)((is / NSK) & 1))) {
+          issue_s(is++); did = true;
+        }
+        if (ip < is && mbar_test(p_full(ip & 1), (uint32_t)((ip >> 1) & 1)) && mbar_test(v_full(ip % NSV), (uint32_t)((ip / NSV) & 1))) {
+          issue_pv(ip++); did = true;
+        }
+        if (did) idle = 0;
+        else if (++idle > limit) ok = false;
       }
+      if (ok) umma_commit(o_done);
       if (!ok) { atomicOr(a.status, ST_TIMEOUT); s_abort = 1; }
     }
-  } else if (softmax_warp) {
-    // ---- softmax warps: thread = accumulator row = a tensor-memory lane of the warp's quadrant; KPT of the tile's keys
-    constexpr int KPT = C::KPT;
-    const int quad = warp & 3, half = C::SPLIT ? warp >> 2 : 0, row = quad * C::RPW + lane;
-    const int kb0 = half * KPT;                           // first key of the tile this thread looks at
-    const bool row_valid = row < QROWS;
-    const bool warp_rows = quad * C::RPW < nr;            // any row of this warp in use
-    const bool row_live = row_valid && row < nr;
+  } else if ((warp & 3) < C::NQUAD) {
+    // ---- softmax warps: thread = accumulator row = a tensor-memory lane of the warp's quadrant
+    const int quad = warp & 3, grp = warp >> 2, row = quad * 32 + lane;
+    const bool warp_rows = quad * 32 < nr;            // any row of this warp in use
+    const bool row_live = row < nr;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(quad * 32) << 16);
     const uint64_t mask = (row_live && rs.mask) ? rs.mask[row] : 0ull;
     const bool causal = rs.mask == nullptr;
     const float sc = rsqrtf((float)HD) * 1.4426950408889634f;   // 1/sqrt(hd) * log2(e)
-    float m_ref = -INFINITY, l = 0.f;                     // l: the sum over this thread's keys only
+    float m_ref = -INFINITY, l = 0.f;                     // after this group's last tile; l: the sum over its tiles
     bool ok = true;
-    const int st = (C::SPLIT ? half * 2 + quad : warp - 4) * 32 + lane;      // 0..127 among the softmax threads
-    for (int i = 0; i < ntiles; ++i) {
+    const int gt = quad * 32 + lane;                      // thread of the group
+    for (int i = grp; i < ntiles; i += 2) {
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }     // a wait that ran out in one lane ends the walk for the whole warp
       const int t0 = (tile0 + i) * TILE;
-      if (!mbar_wait(s_full(i & 1), (uint32_t)((i >> 1) & 1), limit)) { ok = false; break; }
+      if (!mbar_wait(s_full(grp), (uint32_t)((i >> 1) & 1), limit)) { ok = false; break; }
       tc_fence_after();
-      uint32_t r[KPT];
+      f32x2 s2[TILE / 2];                                  // raw scores, two keys each
       if (warp_rows) {
-        const uint32_t s_addr = lane_addr + (uint32_t)((i & 1) * C::S_COLS + kb0);
-        if constexpr (NP == 1) {
-          if constexpr (KPT == 64) tmem_ld64(s_addr, r); else tmem_ld32(s_addr, r);
-        } else {                                           // the two column halves of the score buffer in one round trip, added
-          uint32_t y[KPT];
-          if constexpr (KPT == 64) tmem_ld64x2(s_addr, s_addr + (uint32_t)TILE, r, y); else tmem_ld32x2(s_addr, s_addr + (uint32_t)TILE, r, y);
+        const uint32_t s_addr = lane_addr + (uint32_t)(grp * C::S_COLS);
 #pragma unroll
-          for (int j = 0; j < KPT; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(y[j]));
+        for (int c0 = 0; c0 < TILE; c0 += 32) {            // NP = 2: the two column halves of the score buffer, added
+          uint32_t x[32], y[32];
+          if constexpr (NP == 1) tmem_ld32(s_addr + (uint32_t)c0, x); else tmem_ld32x2(s_addr + (uint32_t)c0, s_addr + (uint32_t)(TILE + c0), x, y);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const f32x2 v = pack2(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+            if constexpr (NP == 1) s2[c0 / 2 + j] = v;
+            else s2[c0 / 2 + j] = add2(v, pack2(__uint_as_float(y[2 * j]), __uint_as_float(y[2 * j + 1])));
+          }
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(s_empty(i & 1));
-      float alpha = 1.f;
+      if (lane == 0) mbar_arrive(s_empty(grp));
       if (warp_rows) {
-        // visibility word of this row for the tile's 64 keys (bit j: key t0 + j), built once per tile
-        uint64_t vis = row_live ? ~0ull : 0ull;
-        if (t0 + TILE > p0 && row_live) {                  // the tile reaches into the new rows (or past the end)
-          const int shift = t0 - p0;                       // new-slot index of the tile's first key; negative: it is a committed row
-          if (causal) {                                    // new slots 0..row: keys j <= row - shift
-            const int n = row - shift + 1;
-            vis = n >= 64 ? ~0ull : (n <= 0 ? 0ull : ((1ull << n) - 1ull));
-          } else if (shift >= 0) {
-            vis = shift < 64 ? mask >> shift : 0ull;
-          } else {
-            vis = (mask << (-shift)) | ((1ull << (-shift)) - 1ull);
+        if (t0 + TILE > p0) {                              // the tile reaches into the new rows (or past the end): hide keys
+          // visibility word of this row for the tile's 64 keys (bit j: key t0 + j)
+          uint64_t vis = 0ull;
+          if (row_live) {
+            const int shift = t0 - p0;                     // new-slot index of the tile's first key; negative: it is a committed row
+            if (causal) {                                  // new slots 0..row: keys j <= row - shift
+              const int n = row - shift + 1;
+              vis = n >= 64 ? ~0ull : (n <= 0 ? 0ull : ((1ull << n) - 1ull));
+            } else if (shift >= 0) {
+              vis = shift < 64 ? mask >> shift : 0ull;
+            } else {
+              vis = (mask << (-shift)) | ((1ull << (-shift)) - 1ull);
+            }
+            const int nv = total - t0;                     // keys of the tile that exist
+            if (nv < 64) vis &= (1ull << nv) - 1ull;
           }
-          const int nv = total - t0;                       // keys of the tile that exist
-          if (nv < 64) vis &= (1ull << nv) - 1ull;
-        }
-        if constexpr (C::SPLIT) vis >>= kb0;
-        float mx = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < KPT; ++j) {
-          const float v = ((vis >> j) & 1ull) ? __uint_as_float(r[j]) * sc : -INFINITY;
-          r[j] = __float_as_uint(v);
-          mx = fmaxf(mx, v);
+          for (int j = 0; j < TILE / 2; ++j) {
+            const float2 v = unpack2(s2[j]);
+            s2[j] = pack2((vis >> (2 * j)) & 1ull ? v.x : -INFINITY, (vis >> (2 * j + 1)) & 1ull ? v.y : -INFINITY);
+          }
         }
-        if constexpr (C::SPLIT) {
-          // the row's maximum over all 64 keys: the two warps of the quadrant swap theirs (buffer and barrier of the tile's
-          // parity; a buffer is rewritten two tiles later, after the P V product that followed this read has been issued)
-          const uint32_t xm = xm_s + (uint32_t)(((i & 1) * 2) * 64 * 4);
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(xm + (uint32_t)((half * 64 + row) * 4)), "f"(mx) : "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(xm_bar(i & 1, quad));
-          if (!mbar_wait(xm_bar(i & 1, quad), (uint32_t)((i >> 1) & 1), limit)) { ok = false; break; }
-          float other;
-          asm volatile("ld.shared.f32 %0, [%1];" : "=f"(other) : "r"(xm + (uint32_t)(((half ^ 1) * 64 + row) * 4)) : "memory");
-          mx = fmaxf(mx, other);
+        float mx = -INFINITY, mx1 = -INFINITY;             // scores of dead rows are whatever Q holds there; nothing of theirs is used
+#pragma unroll
+        for (int j = 0; j < TILE / 2; j += 2) {
+          const float2 v = unpack2(s2[j]), v1 = unpack2(s2[j + 1]);
+          mx = max3(mx, v.x, v.y); mx1 = max3(mx1, v1.x, v1.y);
         }
-        float m_new = m_ref;
-        if (mx > m_ref + RESCALE_STEP) m_new = mx;          // also the first finite maximum (m_ref = -inf)
-        const bool rescale = m_ref != -INFINITY && m_new != m_ref;
-        if (rescale) alpha = ex2(m_ref - m_new);
+        mx = fmaxf(mx, mx1) * sc;
+        // the reference maximum after tile i - 1 from the other group's warp of the quadrant, the one after this tile back to it
+        float m_in = -INFINITY;
+        const uint32_t xm = xm_s + (uint32_t)(row * 4);
+        if (i > 0) {
+          if (!mbar_wait(xm_bar(grp ^ 1, quad), (uint32_t)(((i - 1) >> 1) & 1), limit)) { ok = false; break; }
+          asm volatile("ld.shared.f32 %0, [%1];" : "=f"(m_in) : "r"(xm + (uint32_t)((grp ^ 1) * QROWS * 4)) : "memory");
+        }
+        const float m_new = mx > m_in + RESCALE_STEP ? mx : m_in;      // also the first finite maximum (m_in = -inf)
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(xm + (uint32_t)(grp * QROWS * 4)), "f"(m_new) : "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(xm_bar(grp, quad));
+        const bool rescale = row_live && m_in != -INFINITY && m_new != m_in;
+        if (m_ref != m_new) l *= ex2(m_ref - m_new);
         m_ref = m_new;
-        const float bse = m_new == -INFINITY ? 0.f : m_new;
-        float sum = 0.f;
-        uint32_t pk[KPT / 2];
+        const float bse = m_new == -INFINITY ? 0.f : -m_new;
+        const f32x2 sc2 = pack2(sc, sc), bse2 = pack2(bse, bse);
+        f32x2 sum2 = 0ull;
+        uint32_t ph[TILE / 2], pl[NP == 2 ? TILE / 2 : 1];
 #pragma unroll
-        for (int j = 0; j < KPT / 2; ++j) {
-          const float p0v = ex2(__uint_as_float(r[2 * j]) - bse), p1v = ex2(__uint_as_float(r[2 * j + 1]) - bse);
-          pk[j] = pack_half2(p0v, p1v);
-          if (NP == 1) {
-            const __half2 hv = *reinterpret_cast<const __half2*>(&pk[j]);
-            sum += __low2float(hv) + __high2float(hv);     // the sum of what the MMA will really weigh V with
+        for (int j = 0; j < TILE / 2; ++j) {
+          const float2 e = unpack2(fma2(s2[j], sc2, bse2));
+          const f32x2 p = pack2(ex2(e.x), ex2(e.y));
+          const float2 pv = unpack2(p);
+          ph[j] = pack_half2(pv.x, pv.y);
+          const __half2 hv = *reinterpret_cast<const __half2*>(&ph[j]);
+          const f32x2 hi = pack2(__low2float(hv), __high2float(hv));
+          if constexpr (NP == 1) {
+            sum2 = add2(sum2, hi);                         // the sum of what the MMA will really weigh V with
           } else {
-            sum += p0v + p1v;
-            r[2 * j] = __float_as_uint(p0v); r[2 * j + 1] = __float_as_uint(p1v);     // kept for the lo plane
+            sum2 = add2(sum2, p);
+            const float2 lo = unpack2(fma2(hi, pack2(-1.f, -1.f), p));       // lo = f16(p - f16(p))
+            pl[j] = pack_half2(lo.x, lo.y);
           }
         }
-        l = l * alpha + sum;
-        // P buffer i % NPB was last read by P V of tile i - NPB; the row's accumulator by P V of tile i - 1
-        if (i >= C::NPB && !mbar_wait(pv_done((i - C::NPB) & 1), (uint32_t)(((i - C::NPB) >> 1) & 1), limit)) { ok = false; break; }
-        if (__any_sync(0xffffffffu, rescale)) {            // both warps of a quadrant decide alike; each scales its half of the columns
+        const float2 sum = unpack2(sum2);
+        l += sum.x + sum.y;
+        if (i >= 2 && !mbar_wait(pv_done(grp), (uint32_t)(((i - 2) >> 1) & 1), limit)) { ok = false; break; }      // the P buffer is free
+        if (__any_sync(0xffffffffu, rescale)) {
+          const float alpha = rescale ? ex2(m_in - m_new) : 1.f;
+          // P V of tile i - 2 is done, so the other buffer's barrier is at tile i - 1; it cannot pass it before this tile's P
           if (i >= 1 && !mbar_wait(pv_done((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), limit)) { ok = false; break; }
           tc_fence_after();
-          constexpr int OC = C::SPLIT ? C::O_COLS / 2 : C::O_COLS;
 #pragma unroll 1
-          for (int c0 = half * OC; c0 < (half + 1) * OC; c0 += 32) {
+          for (int c0 = 0; c0 < C::O_COLS; c0 += 32) {
             uint32_t o[32];
             tmem_ld32(lane_addr + (uint32_t)(C::O_COL0 + c0), o);
 #pragma unroll
@@ -415,28 +468,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             tmem_st32(lane_addr + (uint32_t)(C::O_COL0 + c0), o);
           }
         }
-        const uint32_t prow = p_s + (i % C::NPB) * C::P_BYTES + (uint32_t)row * 128u;
-        if (row_valid) {
-#pragma unroll
-          for (int ch = 0; ch < KPT / 8; ++ch) {
-            const uint32_t dst = prow + (uint32_t)(((kb0 / 8 + ch) ^ (row & 7)) * 16);
-            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(pk[4 * ch]), "r"(pk[4 * ch + 1]), "r"(pk[4 * ch + 2]), "r"(pk[4 * ch + 3]) : "memory");
-          }
-          if (NP == 2) {
-#pragma unroll
-            for (int j = 0; j < KPT / 2; ++j) {            // lo = f16(p - f16(p))
-              const __half2 hv = *reinterpret_cast<const __half2*>(&pk[j]);
-              pk[j] = pack_half2(__uint_as_float(r[2 * j]) - __low2float(hv), __uint_as_float(r[2 * j + 1]) - __high2float(hv));
-            }
-#pragma unroll
-            for (int ch = 0; ch < KPT / 8; ++ch) {
-              const uint32_t dst = prow + (uint32_t)(C::PP_BYTES + ((kb0 / 8 + ch) ^ (row & 7)) * 16);
-              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(pk[4 * ch]), "r"(pk[4 * ch + 1]), "r"(pk[4 * ch + 2]), "r"(pk[4 * ch + 3]) : "memory");
-            }
-          }
-        }
+        const uint32_t p_addr = lane_addr + (uint32_t)(C::P_COL0 + grp * C::P_COLS);
+        tmem_st32(p_addr, ph);
+        if constexpr (NP == 2) tmem_st32(p_addr + (uint32_t)(TILE / 2), pl);
       } else {
-        if (i >= C::NPB && !mbar_wait(pv_done((i - C::NPB) & 1), (uint32_t)(((i - C::NPB) >> 1) & 1), limit)) { ok = false; break; }
+        if (i >= 2 && !mbar_wait(pv_done(grp), (uint32_t)(((i - 2) >> 1) & 1), limit)) { ok = false; break; }
       }
       if (t0 + TILE > total) {
         // rows of the V tile past the end of the sequence hold whatever the cache holds: zero them, so that a
@@ -446,147 +482,166 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         const uint32_t v_src = vring_s + s * C::V_BYTES;
         const int first = total - t0;                       // first row to clear (>= 1)
         constexpr int BLK = NP * C::NHALF;                  // 64-column blocks of a V tile
-        for (int e = st; e < (TILE - first) * BLK * 8; e += 128) {
+        for (int e = gt; e < (TILE - first) * BLK * 8; e += QROWS) {
           const int rr = first + e / (BLK * 8), rem = e % (BLK * 8);
           const uint32_t dst = v_src + (uint32_t)((rem >> 3) * TILE * 128 + rr * 128 + (rem & 7) * 16);
           asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst), "r"(0u) : "memory");
         }
+        fence_proxy_async();                               // the cleared rows become visible to the tensor core
       }
-      fence_proxy_async();                                 // P (and the cleared V rows) become visible to the tensor core
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full(i & 1));
+      if (lane == 0) mbar_arrive(p_full(grp));
     }
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) { atomicOr(a.status, ST_TIMEOUT); s_abort = 1; }
-    // ---- this chunk's partial rows -> shared memory (the ring is idle once the last P V has completed)
-    if (ok && ntiles > 0 && !mbar_wait(pv_done((ntiles - 1) & 1), (uint32_t)(((ntiles - 1) >> 1) & 1), limit)) {
+    // (not pv_done of the last tile: a group does not follow the other's phases, and a parity only tells neighbouring ones apart)
+    if (ok && ntiles > 0 && !mbar_wait(o_done, 0, limit)) {
       ok = false; atomicOr(a.status, ST_TIMEOUT); s_abort = 1;
     }
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
-    {
-      const uint32_t xo = ring_s + (uint32_t)row * (HD * 4), xml = ring_s + QROWS * HD * 4 + (uint32_t)row * 16 + (uint32_t)half * 8;
-      const bool have = ok && ntiles > 0 && row_live && m_ref != -INFINITY;
-      if (ok && ntiles > 0 && warp_rows) {
-        // 64 output columns (both planes' halves) per tensor-memory round trip; with two warps per quadrant each takes
-        // every other block of 64
+    // 32 output columns of this thread's row in one tensor-memory round trip
+    auto read_o = [&](int c0, uint32_t (&o)[32]) { tmem_ld32(lane_addr + (uint32_t)(C::O_COL0 + c0), o); };
+    if (nchunks == 1) {
+      // the other group's maximum and sum; the output is relative to the larger maximum (the one after the last tile)
+      const uint32_t xl = ring_s + (uint32_t)(C::BUF_BYTES + row * 16);
+      asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(xl + (uint32_t)grp * 8u), "f"(m_ref), "f"(l) : "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(2 * QROWS) : "memory");       // the softmax warps
+      const float4 ml = ld_smem4(xl);
+      const float M = fmaxf(ml.x, ml.z);
+      const bool have = ok && row_live && M != -INFINITY;
+      const float L = have ? ml.y * ex2(ml.x - M) + ml.w * ex2(ml.z - M) : 0.f;
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+      if (a.early) pdl_wait();                             // (the producer lane has waited already) before the first global store
+      const int w_rows = min(32, rows_cap - quad * 32);    // rows of this warp that exist
+      const uint32_t buf = ring_s + (uint32_t)(grp * C::NQUAD + quad) * (2 * 32 * 128);
+      if (ok && w_rows > 0) {
 #pragma unroll 1
-        for (int c0 = half * 64; c0 < HD; c0 += C::SPLIT ? 128 : 64) {
-          uint32_t o[64];
-          if (NP == 2) {
-            uint32_t o2[64];
-            tmem_ld64x2(lane_addr + (uint32_t)(C::O_COL0 + c0), lane_addr + (uint32_t)(C::O_COL0 + HD + c0), o, o2);
+        for (int c0 = grp * 64; c0 < HD; c0 += 128) {        // the two warps of a quadrant take every other block of 64 columns
+#pragma unroll 1
+          for (int c1 = 0; c1 < 64; c1 += 32) {
+            uint32_t o[32];
+            if (ntiles > 0) read_o(c0 + c1, o);
 #pragma unroll
-            for (int j = 0; j < 64; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) + __uint_as_float(o2[j]));
-          } else {
-            tmem_ld64(lane_addr + (uint32_t)(C::O_COL0 + c0), o);
-          }
-          if (row_valid) {
+            for (int j = 0; j < 4; ++j) {                  // 8 columns: 16 bytes of either plane; piece p of row `lane` sits at position p ^ (lane & 7)
+              uint32_t hi[4], lo[4];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {                 // float4 piece k4 of row i sits at position k4 ^ (i & (HD/4 - 1))
-              const int k4 = c0 / 4 + j;
-              const uint32_t dst = xo + (uint32_t)((k4 ^ (row & (HD / 4 - 1))) * 16);
-              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(o[4 * j]), "r"(o[4 * j + 1]), "r"(o[4 * j + 2]), "r"(o[4 * j + 3]) : "memory");
+              for (int k = 0; k < 4; ++k) {
+                const float x = have ? __uint_as_float(o[8 * j + 2 * k]) * inv : 0.f, y = have ? __uint_as_float(o[8 * j + 2 * k + 1]) * inv : 0.f;
+                const __nv_bfloat162 hv = __floats2bfloat162_rn(x, y);
+                const __nv_bfloat162 lv = __floats2bfloat162_rn(x - __low2float(hv), y - __high2float(hv));
+                hi[k] = *reinterpret_cast<const uint32_t*>(&hv); lo[k] = *reinterpret_cast<const uint32_t*>(&lv);
+              }
+              const uint32_t dst = buf + (uint32_t)(lane * 128 + (((c1 / 8 + j) ^ (lane & 7)) * 16));
+              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(hi[0]), "r"(hi[1]), "r"(hi[2]), "r"(hi[3]) : "memory");
+              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + 32u * 128u), "r"(lo[0]), "r"(lo[1]), "r"(lo[2]), "r"(lo[3]) : "memory");
             }
           }
+          __syncwarp();
+          const int piece = lane & 7;
+#pragma unroll 4
+          for (int it = 0; it < 8; ++it) {
+            const int i = it * 4 + (lane >> 3);
+            if (i < w_rows) {
+              const uint32_t src = buf + (uint32_t)(i * 128 + ((piece ^ (i & 7)) * 16));
+              bf16* dst = a.out + (size_t)(q_row0 + quad * 32 + i) * (H * HD) + h * HD + c0 + piece * 8;
+              *reinterpret_cast<float4*>(dst) = ld_smem4(src);
+              if (a.out_ps) *reinterpret_cast<float4*>(dst + a.out_ps) = ld_smem4(src + 32u * 128u);
+            }
+          }
+          __syncwarp();
         }
       }
-      if (row_valid) {                                     // (max, this thread's part of the sum); without a second key half its slot reads (max, 0)
-        const float2 ml = have ? make_float2(m_ref, l) : make_float2(-INFINITY, 0.f);
-        asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(xml), "f"(ml.x), "f"(ml.y) : "memory");
-        if constexpr (!C::SPLIT) asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(xml + 8u), "f"(ml.x), "f"(0.f) : "memory");
+    } else {
+      if (ok && ntiles > 0 && warp_rows) {
+        const uint32_t xo = ring_s + (uint32_t)row * (HD * 4);
+#pragma unroll 1
+        for (int c0 = grp * (HD / 2); c0 < (grp + 1) * (HD / 2); c0 += 32) {       // the two warps of a quadrant take half of the columns each
+          uint32_t o[32];
+          read_o(c0, o);
+#pragma unroll
+          for (int j = 0; j < 8; ++j)                      // float4 piece k4 of row i sits at position k4 ^ (i & (HD/4 - 1))
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(xo + (uint32_t)(((c0 / 4 + j) ^ (row & (HD / 4 - 1))) * 16)),
+                         "r"(o[4 * j]), "r"(o[4 * j + 1]), "r"(o[4 * j + 2]), "r"(o[4 * j + 3]) : "memory");
+        }
       }
+      const bool have = ok && row_live;
+      asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(ring_s + (uint32_t)(QROWS * HD * 4 + row * 16 + grp * 8)),
+                   "f"(have ? m_ref : -INFINITY), "f"(have ? l : 0.f) : "memory");
     }
   }
   __syncwarp();                                           // the one-lane roles rejoin their warps before the block-wide barrier
   tc_fence_before();
-  __syncthreads();
-  // ---- merge the chunks of this (head, sequence): out[r][h][:] = sum_c o_c 2^(m_c - M) / sum_c l_c 2^(m_c - M),
-  // chunks in order; this CTA takes rows c, c + nchunks, ...
-  cluster_sync_all();                                     // every chunk's rows are in its shared memory
-  if (a.early) pdl_wait();                                // (the producer lane has waited already) before the first global store
-  {
-    constexpr int V4 = HD / 4;
-    const uint32_t xo_s = ring_s, xml_s = ring_s + QROWS * HD * 4;
-    const int d = H * HD;
-    const int rows_cap = rs.blocks ? nr : min(rs.tc, QROWS);
-    const int my_rows = rows_cap > c ? (rows_cap - c + nchunks - 1) / nchunks : 0;
-    // chunk weights of my rows, normalised: w_c = 2^(m_c - M) / sum_c l_c 2^(m_c - M)  (one thread per row, all (m, l) loads in flight together)
-    for (int t = tid; t < my_rows; t += C::NTHREADS) {
-      const int i = c + t * nchunks;
-      float mc[MAX_CHUNKS], lc[MAX_CHUNKS];
-      float M = -INFINITY, L = 0.f;
-#pragma unroll
-      for (int cc = 0; cc < MAX_CHUNKS; ++cc) {
-        mc[cc] = -INFINITY; lc[cc] = 0.f;
-        if (cc < nchunks && i < nr) { const float4 ml = ld_peer4(peer_smem(xml_s + (uint32_t)i * 16u, (uint32_t)cc)); mc[cc] = ml.x; lc[cc] = ml.y + ml.w; }
-      }
-#pragma unroll
-      for (int cc = 0; cc < MAX_CHUNKS; ++cc) M = fmaxf(M, mc[cc]);
-#pragma unroll
-      for (int cc = 0; cc < MAX_CHUNKS; ++cc) { mc[cc] = mc[cc] == -INFINITY ? 0.f : exp2f(mc[cc] - M); L += lc[cc] * mc[cc]; }
-      const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-      for (int cc = 0; cc < MAX_CHUNKS; ++cc) s_w[t * MAX_CHUNKS + cc] = mc[cc] * inv;
-    }
+  if (nchunks == 1) {
     __syncthreads();
-    // two output pieces per thread and round, all their peer loads in flight together (a load that waits for the
-    // previous one's use costs a shared-memory round trip across the cluster each)
-    for (int e0 = tid; e0 < my_rows * V4; e0 += 2 * C::NTHREADS) {
-      float4 v[2][MAX_CHUNKS];
-      float w[2][MAX_CHUNKS];
+  } else {
+    cluster_sync_all();                                   // every chunk's rows are in its shared memory
+    if (a.early) pdl_wait();                              // (the producer lane has waited already) before the first global store
+    // out[r][h][:] = sum_c o_c 2^(m_c - M) / sum_c l_c 2^(m_c - M), chunks in order, M the maximum so far; this CTA takes
+    // rows c, c + nchunks, ...; the loads of up to four chunks are in flight together
+    constexpr int V4 = HD / 4;
+    const int d = H * HD;
+    const int my_rows = rows_cap > c ? (rows_cap - c + nchunks - 1) / nchunks : 0;
+#pragma unroll 1
+    for (int e = tid; e < my_rows * V4 && !s_abort; e += C::NTHREADS) {
+      const int k4 = e % V4, i = c + (e / V4) * nchunks;
+      const uint32_t xo = ring_s + (uint32_t)(i * (HD * 4) + ((k4 ^ (i & (V4 - 1))) * 16)), xml = ring_s + (uint32_t)(QROWS * HD * 4 + i * 16);
+      float M = -INFINITY, L = 0.f;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (int c0 = 0; c0 < nchunks; c0 += 4) {
+        float4 ml[4], v[4];
 #pragma unroll
-      for (int ib = 0; ib < 2; ++ib) {
-        const int e = e0 + ib * C::NTHREADS, t = e / V4, i = c + t * nchunks, k4 = e % V4;
-        const bool live = e < my_rows * V4;
+        for (int u = 0; u < 4; ++u) {
+          ml[u] = make_float4(-INFINITY, 0.f, -INFINITY, 0.f); v[u] = acc;
+          if (c0 + u < nchunks) { ml[u] = ld_peer4(peer_smem(xml, (uint32_t)(c0 + u))); v[u] = ld_peer4(peer_smem(xo, (uint32_t)(c0 + u))); }
+        }
 #pragma unroll
-        for (int cc = 0; cc < MAX_CHUNKS; ++cc) {
-          w[ib][cc] = live && cc < nchunks ? s_w[t * MAX_CHUNKS + cc] : 0.f;
-          v[ib][cc] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (w[ib][cc] != 0.f)                              // a chunk of weight zero may hold nothing at all
-            v[ib][cc] = ld_peer4(peer_smem(xo_s + (uint32_t)(i * HD * 4 + ((k4 ^ (i & (V4 - 1))) * 16)), (uint32_t)cc));
+        for (int u = 0; u < 4; ++u) {
+          const float mu = fmaxf(ml[u].x, ml[u].z);        // the output is relative to the larger maximum of the two groups
+          if (mu != -INFINITY) {                           // a chunk that saw no key of this row holds anything at all in its place
+            const float m1 = fmaxf(M, mu), f = ex2(M - m1), w = ex2(mu - m1);
+            M = m1;
+            L = L * f + ml[u].y * ex2(ml[u].x - m1) + ml[u].w * ex2(ml[u].z - m1);
+            acc.x = acc.x * f + v[u].x * w; acc.y = acc.y * f + v[u].y * w; acc.z = acc.z * f + v[u].z * w; acc.w = acc.w * f + v[u].w * w;
+          }
         }
       }
-#pragma unroll
-      for (int ib = 0; ib < 2; ++ib) {
-        const int e = e0 + ib * C::NTHREADS, t = e / V4, i = c + t * nchunks, k4 = e % V4;
-        if (e >= my_rows * V4 || s_abort) continue;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int cc = 0; cc < MAX_CHUNKS; ++cc) {
-          acc.x += v[ib][cc].x * w[ib][cc]; acc.y += v[ib][cc].y * w[ib][cc]; acc.z += v[ib][cc].z * w[ib][cc]; acc.w += v[ib][cc].w * w[ib][cc];
-        }
-        bf16* dst = a.out + (size_t)(q_row0 + i) * d + h * HD + k4 * 4;      // rows past nr get zeros
-        const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
-        *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-        if (a.out_ps) {
-          const __nv_bfloat162 l0 = __floats2bfloat162_rn(acc.x - __low2float(h0), acc.y - __high2float(h0));
-          const __nv_bfloat162 l1 = __floats2bfloat162_rn(acc.z - __low2float(h1), acc.w - __high2float(h1));
-          *reinterpret_cast<uint2*>(dst + a.out_ps) = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
-        }
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+      acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+      bf16* dst = a.out + (size_t)(q_row0 + i) * d + h * HD + k4 * 4;      // rows past nr get zeros
+      const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
+      *reinterpret_cast<uint2*>(dst) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+      if (a.out_ps) {
+        const __nv_bfloat162 l0 = __floats2bfloat162_rn(acc.x - __low2float(h0), acc.y - __high2float(h0));
+        const __nv_bfloat162 l1 = __floats2bfloat162_rn(acc.z - __low2float(h1), acc.w - __high2float(h1));
+        *reinterpret_cast<uint2*>(dst + a.out_ps) = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
       }
     }
+    cluster_sync_all();                                   // peers may still be reading this CTA's rows
   }
-  cluster_sync_all();                                     // peers may still be reading this CTA's rows
   if (s_abort) {                                          // let copies in flight land before the CTA retires
     for (int i = 0; i < 2000; ++i) __nanosleep(100);
   }
-  if (warp == 3) { tc_fence_after(); tmem_dealloc(tmem_base, C::TMEM_COLS); }
+  if (warp == C::W_MMA) { tc_fence_after(); tmem_dealloc(tmem_base, C::TMEM_COLS); }
 }
 
-// Number of KV chunks per (head, sequence) for lengths up to len_upper: the count (at most 8) that minimises the
-// largest number of tiles any SM walks, with about three tiles' worth of set-up and merging per CTA; ties go to
-// fewer chunks.  One CTA per SM (the rings take nearly all of its shared memory).
-int pick_chunks(int pairs, int len_upper, int sms) {
-  const int nt = (len_upper + TILE - 1) / TILE;
+// Number of KV chunks per (head, sequence) or (head, block): the count (at most 8) with the least estimated time, in tiles; ties go
+// to fewer chunks.  One CTA per SM (the rings take nearly all of its shared memory), nt tiles in the longest pair, `tiles` in
+// all of a head's.  Besides its tiles a CTA pays about 3 tiles' time for set-up and its result, with a merge 4 and one more per 32
+// rows (measured: 3.9 us, 7.3 with 64 rows, 10.5 with 128 at 1.35 us a tile).  Packed prompt blocks come longest first, so the SMs
+// even out: the longest CTA or the mean load counts.  Otherwise all pairs may have nt tiles: whole waves count.
+// 32 pairs of 10 tiles, 64 rows: 1, 2, 3, 4, 5 chunks take 18.1, 15.1, 13.6, 12.0, 21.8 us; 256 pairs of up to 18: 46.7 and 74 us.
+// Blocks of prompts (192 of up to 10 tiles): 1, 2, 3 chunks take 27.7, 41.5, 55.6 us.
+int pick_chunks(int pairs, int nt, long tiles, bool packed, int rows, int sms) {
   int hi = nt < MAX_CHUNKS ? nt : MAX_CHUNKS;
   if (hi < 1) hi = 1;
-  auto cost = [&](int n) {
-    const long per_sm = ((long)pairs * n + sms - 1) / sms, tiles = (nt + n - 1) / n;
-    return per_sm * (tiles + 3);
+  auto cost = [&](int n) -> double {
+    const double own = n == 1 ? 3 : 4 + rows / 32, longest = (double)nt / n + own;
+    return packed ? std::max(longest, (tiles + pairs * n * own) / sms) : (pairs * n + sms - 1) / sms * longest;
   };
-  int best = 1; long best_cost = cost(1);
+  int best = 1; double best_cost = cost(1);
   for (int n = 2; n <= hi; ++n)
     if (cost(n) < best_cost) { best = n; best_cost = cost(n); }
   return best;
@@ -613,7 +668,8 @@ hydra_status run(const __half* q, int q_rows, const __half* kc, const __half* vc
   a.rs = rs; a.out = out; a.out_ps = out_ps; a.H = H; a.max_seq = max_seq; a.status = status; a.wait_limit = WAIT_LIMIT;
   a.q_plane_rows = q_rows; a.kv_plane_rows = (int)cache_rows; a.early = stable_lengths ? 1 : 0;
   const int groups = rs.blocks ? rs.n_blocks : rs.batch;
-  a.nchunks = pick_chunks(H * groups, len_upper, sm_count());
+  a.nchunks = pick_chunks(H * groups, (len_upper + TILE - 1) / TILE, (long)H * rs.n_tiles, rs.blocks != nullptr, rs.blocks ? QROWS : rs.tc, sm_count());
+  if (a.nchunks == 1 && ((uintptr_t)out & 15)) a.nchunks = 2;      // one chunk writes 16 bytes at a time, the merge 8
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(H, groups, a.nchunks); cfg.blockDim = dim3(C::NTHREADS); cfg.dynamicSmemBytes = C::SMEM_BYTES; cfg.stream = st;
   cudaLaunchAttribute attr[2];

@@ -115,18 +115,6 @@ __device__ __forceinline__ void sum_slots_multi(const float* part, size_t stride
         acc[u].x += v.x; acc[u].y += v.y; acc[u].z += v.z; acc[u].w += v.w;
       }
 }
-// one float: the slots of element `idx` summed in slot order, the first PMAX loads in flight together
-template <int PMAX = 12>
-__device__ __forceinline__ float sum_slots_scalar(const float* part, size_t stride, size_t idx, int ns) {
-  float v[PMAX];
-#pragma unroll
-  for (int p = 0; p < PMAX; ++p) v[p] = p < ns ? __ldcg(part + p * stride + idx) : 0.f;
-  float acc = 0.f;
-#pragma unroll
-  for (int p = 0; p < PMAX; ++p) acc += v[p];
-  for (int p = PMAX; p < ns; ++p) acc += __ldcg(part + p * stride + idx);
-  return acc;
-}
 inline SplitDesc single_slot(size_t stride) {
   SplitDesc sd{1 << 30, 1, 1, 1 << 30, 30, 0, 0, stride};
   sd.set_inverses();
@@ -167,6 +155,7 @@ struct RowSet {
   const int2* row_at = nullptr;          // device [n_packed]
   const AttBlock* blocks = nullptr;      // device [n_blocks]
   int n_packed = 0, n_blocks = 0;
+  int n_tiles = 0;                       // 64-key tiles that the blocks of one head walk, all together
   __host__ __device__ int rows() const { return row_at ? n_packed : batch * tc; }
 };
 

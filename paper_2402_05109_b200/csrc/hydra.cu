@@ -366,11 +366,11 @@ hydra_status prompt_packed(hydra_ctx* c, const int* tokens, const int* offs, cud
   const int B = c->batch, base = offs[0], total = offs[B] - base, qrows = ATT_BLOCK_ROWS;
   const int passes = (total + PROMPT_ROWS - 1) / PROMPT_ROWS;
   const int step = ((total + passes - 1) / passes + 255) / 256 * 256;
-  struct Pass { int g0, rows, block0, n_blocks, len_upper; };
+  struct Pass { int g0, rows, block0, n_blocks, len_upper, n_tiles; };
   std::vector<Pass> plan;
   std::vector<AttBlock> blocks;
   for (int g0 = 0, b = 0; g0 < total; g0 += step) {
-    Pass p{g0, std::min(step, total - g0), (int)blocks.size(), 0, 0};
+    Pass p{g0, std::min(step, total - g0), (int)blocks.size(), 0, 0, 0};
     while (base + g0 >= offs[b + 1]) ++b;
     for (int g = g0, s = b; g < g0 + p.rows; ++s) {
       const int end = std::min(g0 + p.rows, offs[s + 1] - base), call0 = g - (offs[s] - base);
@@ -379,6 +379,7 @@ hydra_status prompt_packed(hydra_ctx* c, const int* tokens, const int* offs, cud
       p.len_upper = std::max(p.len_upper, end - (offs[s] - base));
     }
     p.n_blocks = (int)blocks.size() - p.block0;
+    for (int i = p.block0; i < p.block0 + p.n_blocks; ++i) p.n_tiles += (blocks[i].pos0 + blocks[i].n + 63) / 64;
     // the longest first: with more CTAs than SMs the short ones fill the end
     std::stable_sort(blocks.begin() + p.block0, blocks.end(), [](const AttBlock& a, const AttBlock& b) { return a.pos0 + a.n > b.pos0 + b.n; });
     plan.push_back(p);
@@ -389,7 +390,7 @@ hydra_status prompt_packed(hydra_ctx* c, const int* tokens, const int* offs, cud
   HYDRA_TRY(pack_rows(c->d_offsets, B, c->d_row_at, base, total, st));
   for (const Pass& p : plan) {
     RowSet rs{B, 0, nullptr, nullptr, nullptr, nullptr};
-    rs.row_at = c->d_row_at + p.g0; rs.n_packed = p.rows; rs.blocks = c->d_blocks + p.block0; rs.n_blocks = p.n_blocks;
+    rs.row_at = c->d_row_at + p.g0; rs.n_packed = p.rows; rs.blocks = c->d_blocks + p.block0; rs.n_blocks = p.n_blocks; rs.n_tiles = p.n_tiles;
     HYDRA_TRY(run_base(c, tokens + base + p.g0, rs, p.len_upper, nullptr, 0, nullptr, true, st));
     HYDRA_TRY(capture_last_packed(c->h_tree, c->d_offsets, base + p.g0, p.rows, c->h_new, c->h.n_heads + 1, c->d_n_new, c->d_len, B, m.d_model, st));
     if (c->h.prefix_attn) HYDRA_TRY(run_prefix(c, c->h_tree, rs, p.len_upper, st));

@@ -468,6 +468,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             tmem_st32(lane_addr + (uint32_t)(C::O_COL0 + c0), o);
           }
         }
+        tc_fence_after();                                  // the product that read this buffer is over
         const uint32_t p_addr = lane_addr + (uint32_t)(C::P_COL0 + grp * C::P_COLS);
         tmem_st32(p_addr, ph);
         if constexpr (NP == 2) tmem_st32(p_addr + (uint32_t)(TILE / 2), pl);

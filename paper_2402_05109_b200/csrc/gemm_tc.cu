@@ -30,6 +30,7 @@
 // Every mbarrier wait is bounded: when one runs out the CTA raises ST_TIMEOUT in the status word, stops
 // storing, lets its copies settle, frees its tensor memory and returns.
 #include "tc.cuh"
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -415,14 +416,11 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
   if (g > total / 4) g = total / 4 > 0 ? total / 4 : 1;
   sd.q = (int)((total + g - 1) / g);
   if (max_slots || part_cap) {
-    auto slots = [&]() {
-      int mx = 1;
-      for (int t = 0; t < tiles; ++t) {
-        long long u0 = (long long)t * sd.kb;
-        int ns = (int)((u0 + sd.kb - 1) / sd.q - u0 / sd.q) + 1;
-        mx = ns > mx ? ns : mx;
-      }
-      return mx;
+    auto slots = [&]() {                                   // CTAs that touch a tile, at most: tile t begins rem units into a CTA's range
+      const unsigned q = (unsigned)sd.q, kb = (unsigned)sd.kb, top = (q + kb - 2) / q + 1;
+      unsigned mx = 1, rem = 0;
+      for (int t = 0; t < tiles && mx < top; ++t, rem = (rem + kb) % q) mx = std::max(mx, (rem + kb - 1) / q + 1);
+      return (int)mx;
     };
     int mx = slots();
     // whole tiles per CTA need one slot

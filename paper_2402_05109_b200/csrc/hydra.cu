@@ -198,12 +198,14 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
     const int shapes[][2] = {{3 * d, d}, {d, d}, {2 * f, d}, {d, f}, {V, d}};
     const int per_seq[] = {T, K + 1, 1, m.dtype == 1 ? 1 : CHUNK};
     for (auto& sh : shapes) {
-      for (int rows : per_seq)
-        for (int bb = 1; bb <= m.max_batch; ++bb) need(rows * bb, sh[0], sh[1]);
-      // packed prompt passes of any row count: the plan depends on the count rounded up to 16 rows
+      // packed prompt passes have any row count; the plan depends on the count rounded up to 16 rows
       if (m.dtype == 1) for (int rows = 16; rows <= PROMPT_ROWS; rows += 16) need(rows, sh[0], sh[1]);
+      for (int rows : per_seq)
+        for (int bb = 1; bb <= m.max_batch; ++bb)
+          if (m.dtype != 1 || rows * bb > PROMPT_ROWS) need(rows * bb, sh[0], sh[1]);
     }
-    for (int mm = 1; mm <= m.max_batch * t.maxP; ++mm) {
+    const int g = m.dtype == 1 ? 16 : 1;
+    for (int mm = g; mm < m.max_batch * t.maxP + g; mm += g) {
       for (int i = 1; i <= K; ++i) need(mm, d, (i + 1) * d);
       need(mm, d, d);
       need(mm, V, d);
@@ -531,8 +533,6 @@ hydra_status hydra_create(hydra_ctx** out, const hydra_model_cfg* m, const hydra
   if (th.K > 0 && h->n_mlp_layers > 1 && (!w->head_wr || (h->has_bias && !w->head_br))) return HYDRA_ERR_INVALID;
   if (h->prefix_attn && (!w->pfx_attn_norm || !w->pfx_wqkv || !w->pfx_wo || !w->pfx_ffn_norm || !w->pfx_w_gate_up || !w->pfx_w_down))
     return HYDRA_ERR_INVALID;
-  size_t need = carve(nullptr, *m, *h, th, nullptr);
-  if (ws_bytes < need) return HYDRA_ERR_CAPACITY;
   if (m->dtype == 1 && !gemm_tc_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
   hydra_ctx* c = new (std::nothrow) hydra_ctx();
   if (!c) return HYDRA_ERR_INVALID;
@@ -553,7 +553,8 @@ hydra_status hydra_create(hydra_ctx** out, const hydra_model_cfg* m, const hydra
     if (!c->head_w1[i] || (h->n_mlp_layers > 1 && !c->head_wr[i])) { delete c; return HYDRA_ERR_INVALID; }
   }
   c->embed = w->embed; c->lm_head = w->lm_head; c->final_norm = w->final_norm;
-  carve(c, *m, *h, th, (char*)ws);
+  const size_t need = carve(c, *m, *h, th, (char*)ws);
+  if (ws_bytes < need) { delete c; return HYDRA_ERR_CAPACITY; }
   c->batch = 0; c->state = ST_CREATED; c->gemm_mode = 0; c->plant = nullptr; c->launches = 0; c->timing = 0; c->steps_done = 0;
   c->use_graph = 1;
   c->acc_mode = 0; c->acc_tau = 1.f; c->acc_eps = 0.f; c->acc_alpha = 0.f; c->acc_u = nullptr; c->last_logits = nullptr;

@@ -241,7 +241,7 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  * supply hydra_gemm's partial_dev buffer; here the partial sums live in an 8 MiB array that is part of the
  * library image (every GPU that loads the library holds it, and a 64 KiB table of counters, until the process exits).
  *   - x [m][k], w [n][k] bfloat16, out [m][n] float, status_dev as in hydra_gemm: all caller-owned device
- *     memory; n % 128 == 0, k % 64 == 0.
+ *     memory; n % 128 == 0, k % 64 == 0; x and w on 16-byte boundaries (INVALID otherwise), out on a float's.
  *   - m * n * 4 bytes must fit in the 8 MiB array (the work is shared out among as many CTAs as the partial sums in it
  *     allow), otherwise HYDRA_ERR_CAPACITY (text in
  *     hydra_last_error) and nothing is launched.

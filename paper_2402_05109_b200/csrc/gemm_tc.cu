@@ -466,8 +466,9 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   if (sd_out) *sd_out = sd;
   // One launch where issuing a second one is what takes the time: up to 16 rows and a weight matrix that passes in a few microseconds
   // (back to back, one launch / two: 11 x 2048 x 2048 6.3 / 8.3 us, 4 x 3456 x 640 6.4 / 8.3, 8 x 640 x 5632 8.0 / 8.2; but
-  // 11 x 4096 x 2048 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x 1024 10.2 / 8.3: the sums of a tile are one CTA's work)
-  if (out && m <= 16 && (long long)n * k <= 6 * 1000 * 1000) {
+  // 11 x 4096 x 2048 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x 1024 10.2 / 8.3: the sums of a tile are one CTA's work).
+  // sum_tile stores 16 bytes at a time; a result buffer off that boundary takes the second launch, which stores single floats
+  if (out && m <= 16 && (long long)n * k <= 6 * 1000 * 1000 && !((uintptr_t)out & 15)) {
     a.out = out; a.arrived = arrived;
     return sh.nh == 2 ? launch<2, true>(tw, tx, a, grid, st) : launch<1, true>(tw, tx, a, grid, st);
   }

@@ -36,3 +36,19 @@ def test_gemm_noalloc_one_and_two_launches(m, n, k):
         ref = x.double() @ w.double().T
         assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 64), (11, 2048, 2048), (3, 4096, 4096)])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_gemm_noalloc_result_off_a_16_byte_boundary(m, n, k, offset):
+    """The result may be any float tensor, a view into a larger buffer included, at sizes on both sides of the one-launch choice."""
+    from paper_2402_05109_b200 import gemm_noalloc
+    x = normal_(torch.empty(m, k, dtype=torch.bfloat16, device="cuda"), 65, m + k, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 66, n, 0.02)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    buf = torch.full((m * n + 8,), 7.0, device="cuda")
+    out = buf[offset:offset + m * n].view(m, n)
+    gemm_noalloc(x, w, out, status)
+    ref = x.double() @ w.double().T
+    assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+    assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + m * n:] == 7.0).all()) and int(status.item()) == 0

@@ -152,6 +152,12 @@ template <> __device__ __forceinline__ float4 load4<float>(const float* p) { ret
 template <> __device__ __forceinline__ float4 load4<bf16>(const bf16* p) {
   float v[4]; Vec4<bf16>::load(p, v); return make_float4(v[0], v[1], v[2], v[3]);
 }
+// Four elements at an element boundary (VEC: at a boundary of four).
+template <typename T> inline bool on_vec4(const T* p) { return ((uintptr_t)p & (4 * sizeof(T) - 1)) == 0; }
+template <bool VEC, typename T> __device__ __forceinline__ float4 load4_at(const T* p) {
+  if constexpr (VEC) return load4<T>(p);
+  else return make_float4(to_f<T>(p[0]), to_f<T>(p[1]), to_f<T>(p[2]), to_f<T>(p[3]));
+}
 
 template <typename T>
 __global__ void embed_rows_kernel(const T* __restrict__ embed, const int* __restrict__ tok, float* __restrict__ x, int d,
@@ -494,7 +500,7 @@ constexpr int ATT_CHUNK = ATT_CHUNK_ROWS;
 constexpr int ATT_TILE = 64;      // KV rows staged per iteration: two keys per lane
 constexpr int ATT_WARPS = 8;
 
-template <typename T, int HD, int RPW>
+template <typename T, int HD, int RPW, bool VEC>
 __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc,
                                                                    const T* __restrict__ vc, RowSet rs,
                                                                    float* __restrict__ part_o, float* __restrict__ part_ml,
@@ -518,7 +524,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
   const float scale = rsqrtf((float)HD);
 
   for (int e = threadIdx.x * 4; e < min(ROWS, nr - r0) * HD; e += blockDim.x * 4) {
-    const float4 v = load4<T>(q + ((size_t)(b * rs.tc + r0 + e / HD)) * d + h * HD + e % HD);
+    const float4 v = load4_at<VEC>(q + ((size_t)(b * rs.tc + r0 + e / HD)) * d + h * HD + e % HD);
     *reinterpret_cast<float4*>(qs + e) = make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale);
   }
   float m[RPW], l[RPW], o[RPW][KPL];
@@ -540,7 +546,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
     for (int e = threadIdx.x * 4; e < ATT_TILE * HD; e += ATT_WARPS * 32 * 4) {
       const int j = e / HD, k = e % HD, slot = t0 + j;
       float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
-      if (slot < s1) { kv = load4<T>(kbase + (size_t)slot * HD + k); vv = load4<T>(vbase + (size_t)slot * HD + k); }
+      if (slot < s1) { kv = load4_at<VEC>(kbase + (size_t)slot * HD + k); vv = load4_at<VEC>(vbase + (size_t)slot * HD + k); }
       float* kd = ks + j * (HD + 1) + k;
       kd[0] = kv.x; kd[1] = kv.y; kd[2] = kv.z; kd[3] = kv.w;
       *reinterpret_cast<float4*>(vs + e) = vv;
@@ -632,17 +638,17 @@ size_t attention_scratch_bytes(int batch, int tc, int n_heads, int head_dim, int
   return (size_t)batch * tc * n_heads * nchunks * (head_dim + 2) * sizeof(float);
 }
 
-template <typename T, int HD, int RPW>
+template <typename T, int HD, int RPW, bool VEC = true>
 static hydra_status launch_tree_attn(const T* q, const T* kc, const T* vc, RowSet rs, float* part_o, float* part_ml, T* out, int H, int max_seq,
                                      int nchunks, cudaStream_t st) {
   const size_t smem = (size_t)(ATT_WARPS * RPW * HD + ATT_TILE * (HD + 1) + ATT_TILE * HD) * sizeof(float);
   static PerDeviceFlag attr_done;
   if (!attr_done.get()) {
-    HYDRA_CUDA(cudaFuncSetAttribute(tree_attn_kernel<T, HD, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    HYDRA_CUDA(cudaFuncSetAttribute(tree_attn_kernel<T, HD, RPW, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     attr_done.set();
   }
   const int groups = (rs.tc + ATT_WARPS * RPW - 1) / (ATT_WARPS * RPW);
-  launch_pdl(tree_attn_kernel<T, HD, RPW>, dim3(H, rs.batch, nchunks * groups), dim3(ATT_WARPS * 32), smem, st, q, kc, vc, rs, part_o, part_ml,
+  launch_pdl(tree_attn_kernel<T, HD, RPW, VEC>, dim3(H, rs.batch, nchunks * groups), dim3(ATT_WARPS * 32), smem, st, q, kc, vc, rs, part_o, part_ml,
              nchunks == 1 ? out : (T*)nullptr, H, max_seq, nchunks);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
@@ -660,7 +666,9 @@ static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSe
   float* part_ml = scratch + rows * H * nchunks_max * HD;
   // one row per warp while that leaves at most two CTAs per SM; more rows per warp share the staged K,V tile instead
   const long ctas1 = (long)H * rs.batch * nchunks * ((rs.tc + ATT_WARPS - 1) / ATT_WARPS), cap = 2L * sm_count();
-  if (ctas1 <= cap) HYDRA_TRY((launch_tree_attn<T, HD, 1>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  // the stand-alone call takes operands on any element boundary: loads of one element then (the rows of a warp do not change a result)
+  if (!on_vec4(q) || !on_vec4(kc) || !on_vec4(vc)) HYDRA_TRY((launch_tree_attn<T, HD, 8, false>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  else if (ctas1 <= cap) HYDRA_TRY((launch_tree_attn<T, HD, 1>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else if (ctas1 <= 2 * cap) HYDRA_TRY((launch_tree_attn<T, HD, 2>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else HYDRA_TRY((launch_tree_attn<T, HD, 8>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   if (nchunks == 1) return HYDRA_OK;

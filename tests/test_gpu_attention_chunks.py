@@ -51,3 +51,22 @@ def test_result_buffer_off_a_16_byte_boundary():
     # both round the same float result to bfloat16, summed in a different order: at most one bfloat16 step (2^-8) apart
     assert float((got - want.float()).abs().max()) <= float(want.float().abs().max()) * 2.0 ** -8
     assert int(status) == 0 and float(buf[:4].abs().max()) == 0.0 and float(buf[-4:].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("hd,S,tc", [(64, 96, 16), (128, 96, 64), (64, 400, 64), (128, 300, 5)])      # one chunk of keys and several
+@pytest.mark.parametrize("which", ["q", "k", "v"])
+def test_float_operands_off_a_16_byte_boundary(hd, S, tc, which):
+    """Float q, K and V may be any float tensors, views into larger buffers included: bit for bit the result of aligned ones."""
+    from paper_2402_05109_b200 import tree_attention
+    B, H = 2, 3
+    ops = {n: rnd(s, 37, i, torch.float32).cuda() for i, (n, s) in enumerate({"q": (B * tc, H, hd), "k": (B, H, S, hd), "v": (B, H, S, hd)}.items())}
+    pos0, n_rows = (torch.tensor(x, dtype=torch.int32).cuda() for x in ([S - tc, 7], [tc, tc - 1]))
+    mask = torch.tensor([(1 << (i + 1)) - 1 if i < 63 else -1 for i in range(tc)], dtype=torch.int64).cuda()
+    want = tree_attention(ops["q"], ops["k"], ops["v"], pos0, n_rows, mask, tc)
+    for off in (1, 2, 3):
+        t = ops[which]
+        buf = torch.empty(t.numel() + 4, device="cuda")
+        view = buf[off:off + t.numel()].view(t.shape)
+        view.copy_(t)
+        moved = dict(ops, **{which: view})
+        assert torch.equal(tree_attention(moved["q"], moved["k"], moved["v"], pos0, n_rows, mask, tc), want)

@@ -915,8 +915,9 @@ hydra_status head_gather(const float* hprime, const void* embed, const int* root
 }
 
 // Four columns per thread in small CTAs (a level has 1 to a few dozen rows); the bias and the slot counts before the wait.
+// VEC: the bias, a caller's vector, lies on a boundary of four elements.
 constexpr int HEAD_ACT_THREADS = 64;
-template <typename T>
+template <typename T, bool VEC>
 __global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* __restrict__ part,
                                 SplitDesc sd, const T* __restrict__ bias, float* y_out, T* __restrict__ yb, size_t yb_ps,
                                 int rows, int d) {
@@ -924,7 +925,7 @@ __global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float*
   const int d4 = d / 4, p = blockIdx.x * blockDim.x + threadIdx.x, r = p / d4, c = (p - r * d4) * 4;
   const size_t off[1] = {(size_t)r * d + c};
   const int ns[1] = {split_count(sd, r, c)};
-  float4 v = bias ? load4<T>(bias + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v = bias ? load4_at<VEC>(bias + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   const size_t at = res_is_hprime ? (size_t)(r / rows_per_b) * d + c : off[0];
   pdl_wait();
   if (r >= rows) return;
@@ -939,12 +940,12 @@ hydra_status head_act(const float* res, int res_is_hprime, int rows_per_b, const
                       const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, int dtype, cudaStream_t st) {
   if (d & 3) return HYDRA_ERR_UNSUPPORTED;
   const unsigned grid = (unsigned)(((size_t)rows * d / 4 + HEAD_ACT_THREADS - 1) / HEAD_ACT_THREADS);
-  if (dtype == 0)
-    launch_pdl(head_act_kernel<float>, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const float*)bias,
-                                                 y_out, (float*)yb, yb_ps, rows, d);
-  else
-    launch_pdl(head_act_kernel<bf16>, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const bf16*)bias,
-                                                y_out, (bf16*)yb, yb_ps, rows, d);
+  auto go = [&](auto zero, auto kernel) {
+    typedef decltype(zero) T;
+    launch_pdl(kernel, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const T*)bias, y_out, (T*)yb, yb_ps, rows, d);
+  };
+  if (dtype == 0) on_vec4((const float*)bias) ? go(float{}, head_act_kernel<float, true>) : go(float{}, head_act_kernel<float, false>);
+  else on_vec4((const bf16*)bias) ? go(bf16{}, head_act_kernel<bf16, true>) : go(bf16{}, head_act_kernel<bf16, false>);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

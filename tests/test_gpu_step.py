@@ -56,6 +56,32 @@ def test_prompt_lengths_around_the_prefill_chunk(head_dim, kv_planes):
     assert st.steps == 2
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_head_biases_off_a_boundary_of_four(dtype, offset):
+    """Bias vectors may be any tensors, views into one flat parameter buffer included: the logits of the last level and the drafted
+    tokens are bit for bit those of aligned biases."""
+    from paper_2402_05109_b200 import Hydra
+    m = ModelCfg(1, 256, 4, 64, 512, 1024, dtype=dtype)
+    h = HeadCfg(3, 3, False)
+    w = {k: v.cuda() for k, v in make_weights(m, h, 41).items()}
+    assert float(w["H1.b1"].float().abs().max()) > 0.0 and float(w["H1.br"].float().abs().max()) > 0.0
+    moved = dict(w)
+    for k, v in w.items():
+        if k.endswith((".b1", ".br")):
+            buf = torch.empty(v.numel() + 4, dtype=v.dtype, device="cuda")
+            moved[k] = buf[offset:offset + v.numel()].view(v.shape).copy_(v)
+    outs = []
+    for weights in (w, moved):
+        g = Hydra(m, h, load_tree("tree15_d3"), weights, 2, 64)
+        g.prefill(make_prompts(41, [9, 14], m.vocab))
+        tok = g.draft()
+        g.poll_status()
+        outs.append((tok.cpu(), g.get_buffer("HEAD_LOGITS").cpu().clone()))
+        g.close()
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
 @pytest.mark.parametrize("dtype,mlp,prefix", [("bf16", 1, False), ("bf16", 3, True), ("fp32", 2, False)])
 def test_medusa_mode_heads(dtype, mlp, prefix):
     """Sequentially independent heads (the Medusa baseline): head i sees the hidden state alone, one logits row per

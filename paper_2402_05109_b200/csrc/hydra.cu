@@ -280,7 +280,7 @@ hydra_status run_gemm(hydra_ctx* c, const void* x, int x_rows_alloc, const void*
     return gemm_tc((const bf16*)x, x_rows_alloc, c->planes, (const bf16*)w, c->part, m, n, k, sd, c->d_status, c->d_status + 8, nullptr, st);
   }
   *sd = single_slot((size_t)m * n);
-  return gemm_simt(x, w, c->part, m, n, k, c->m.dtype, st);      // bfloat16: the hi plane only (debug mode)
+  return gemm_simt(x, w, c->part, m, n, k, c->m.dtype, true, st);      // bfloat16: the hi plane only (debug mode)
 }
 
 // element distance between the hi and lo planes of an operand buffer of `rows_alloc` rows of `cols` (0 for float)
@@ -856,7 +856,7 @@ hydra_status hydra_gemm(const void* x, const void* w, float* out, float* partial
     HYDRA_TRY(gemm_tc((const bf16*)x, m, x_planes, (const bf16*)w, partial, m, n, k, &sd, status, nullptr, nullptr, st));
     return reduce_splits(partial, sd, out, m, n, st);
   }
-  return gemm_simt(x, w, out, m, n, k, dtype, st);
+  return gemm_simt(x, w, out, m, n, k, dtype, false, st);
 }
 
 hydra_status hydra_gemm_bounded_wait_probe(const void* x, const void* w, float* partial, int m, int n, int k, int skip_unit,

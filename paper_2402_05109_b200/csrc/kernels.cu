@@ -50,12 +50,13 @@ __device__ __forceinline__ int warp_sum_owner(int lane) {
 
 // MR activation rows; KS warps share an output column (each every KS-th 512-byte piece of its weight row), 8 / KS columns per
 // block.  The small models of the float path spend their time in the chain launch -> loads -> reduction: the first WPRE weight
-// pieces of a lane are loaded before the wait for the preceding kernel, the MR sums share one transposing reduction, and the
+// pieces of a lane are loaded before the wait for the preceding kernel (w_const: the weights of a context, which no kernel writes; a
+// stand-alone call's w may be the preceding kernel's result), the MR sums share one transposing reduction, and the
 // split keeps the activation loads of a lane to one or two rounds and fills the SMs (16 x 256 x 688: 10.5 us with one warp per
 // column, 32 blocks).
 template <typename T, int MR, int KS>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w,
-                                                        float* __restrict__ out, int m, int n, int k) {
+__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w,      // not __restrict__: such loads may be moved over the wait
+                                                        float* __restrict__ out, int m, int n, int k, int w_const) {
   constexpr int WPRE = 2;
   pdl_trigger();
   __shared__ float s_part[8][MR];
@@ -64,10 +65,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ x,
   const int m0 = blockIdx.y * MR;
   const T* wr = w + (size_t)min(col, n - 1) * k;
   float wv[WPRE][4];
+  if (!w_const) pdl_wait();
 #pragma unroll
   for (int i = 0; i < WPRE; ++i)
     if (k0 + i * KS * 128 < k) Vec4<T>::load(wr + k0 + i * KS * 128, wv[i]);
-  pdl_wait();
+  if (w_const) pdl_wait();
   float acc[MR];
 #pragma unroll
   for (int r = 0; r < MR; ++r) acc[r] = 0.f;
@@ -103,10 +105,10 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ x,
 }
 
 template <typename T, int MR>
-static void launch_gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, cudaStream_t st) {
+static void launch_gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, bool w_const, cudaStream_t st) {
   const int groups = (m + MR - 1) / MR;
   auto go = [&](auto kernel, int ks) {
-    launch_pdl(kernel, dim3((n * ks + 7) / 8, groups), dim3(256), 0, st, (const T*)x, (const T*)w, out, m, n, k);
+    launch_pdl(kernel, dim3((n * ks + 7) / 8, groups), dim3(256), 0, st, (const T*)x, (const T*)w, out, m, n, k, (int)w_const);
   };
   // warps per column: until there are two blocks per SM or a lane has one piece
   const int pieces = (k + 127) / 128, want = 2 * sm_count();
@@ -114,14 +116,14 @@ static void launch_gemm_simt(const void* x, const void* w, float* out, int m, in
   else if (pieces >= 2 && (long)n * groups / 8 <= want) go(gemm_simt_kernel<T, MR, 2>, 2);
   else go(gemm_simt_kernel<T, MR, 1>, 1);
 }
-hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, cudaStream_t st) {
+hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, bool w_const, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0 || (k & 3)) return HYDRA_ERR_UNSUPPORTED;
   auto rows = [&](auto zero) {
     typedef decltype(zero) T;
-    if (m == 1) launch_gemm_simt<T, 1>(x, w, out, m, n, k, st);
-    else if (m <= 4) launch_gemm_simt<T, 4>(x, w, out, m, n, k, st);
-    else if (m <= 8) launch_gemm_simt<T, 8>(x, w, out, m, n, k, st);
-    else launch_gemm_simt<T, 16>(x, w, out, m, n, k, st);
+    if (m == 1) launch_gemm_simt<T, 1>(x, w, out, m, n, k, w_const, st);
+    else if (m <= 4) launch_gemm_simt<T, 4>(x, w, out, m, n, k, w_const, st);
+    else if (m <= 8) launch_gemm_simt<T, 8>(x, w, out, m, n, k, w_const, st);
+    else launch_gemm_simt<T, 16>(x, w, out, m, n, k, w_const, st);
   };
   if (dtype == 0) rows(float{}); else rows(bf16{});
   HYDRA_LAUNCH_CHECK();

@@ -18,8 +18,9 @@ constexpr size_t GEMM_TILE_COLS = 128;    // an output has at most n / GEMM_TILE
 // grid: CTAs.  part_cap (floats, 0: no limit): fewer CTAs, hence fewer slots, where the partial sums would not fit otherwise.
 SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap = 0);
 bool gemm_tc_available();                 // driver entry point for tensor-map encoding found
-// SIMT path (float or bfloat16 operands), single slot.
-hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, cudaStream_t st);
+// SIMT path (float or bfloat16 operands), single slot.  w_const: no kernel in flight writes w (the weights of a context), so it is
+// read ahead of the preceding kernel's completion.
+hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, bool w_const, cudaStream_t st);
 // out[m][n] = sum of the slots of part
 hydra_status reduce_splits(const float* part, SplitDesc sd, float* out, int m, int n, cudaStream_t st);
 

@@ -19,8 +19,9 @@
 // Warp roles (192 threads): warp 0 = TMA producer (one lane), warp 1 = TMEM allocation + MMA issue (one
 // lane), warps 2..5 = epilogue (TMEM -> registers -> global, coalesced along n).  Two accumulator sets in
 // TMEM (where 512 columns allow) let the epilogue of one segment overlap the main loop of the next.  The kernel is launched with
-// programmatic stream serialisation: weight tiles (which never depend on the preceding kernel) are requested
-// before griddepcontrol.wait, activations and all global writes after it.
+// programmatic stream serialisation: the weight tiles of a context's call (no kernel writes those) are requested
+// before griddepcontrol.wait, activations and all global writes after it.  A stand-alone call takes any matrix as w, the preceding
+// kernel's result included, so it only fetches the first tiles into the L2 (which changes nothing that is read) and requests them after the wait.
 // Precision: weights are bfloat16 (exact: the reference model's weights are the same bfloat16 values).  The
 // activation operand comes as TWO bfloat16 planes, hi = bf16(v) and lo = bf16(v - hi), i.e. about 16 mantissa
 // bits; each weight tile is multiplied with both planes.  This doubles the MMA work
@@ -166,6 +167,7 @@ struct GemmArgs {
   int* status;
   int* diag;                     // optional int[8]: where the first bounded wait gave up (site, cta, unit, units, grid, m, n, kb)
   uint32_t wait_limit;           // polls before a barrier wait gives up
+  int w_const;                   // no kernel in flight writes w
   int skip_unit;                 // >= 0: CTA 0 leaves out the weight-tile request of this unit (a test of the bounded waits), else -1
 };
 
@@ -216,7 +218,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u_begin = blockIdx.x * a.q;
   const int u_end = min(u_begin + a.q, a.total_units);
-  const int n_units = u_end - u_begin, pre = n_units < stages ? n_units : stages;
+  const int n_units = u_end - u_begin, ring = n_units < stages ? n_units : stages, pre = a.w_const ? ring : 0;     // pre: weight tiles requested up front
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -226,11 +228,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmX);
     // weights do not depend on the preceding kernel: request the first ring of weight tiles right away, before the
-    // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait
+    // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait; where they may, bring them nearer
     const uint64_t pol = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal();
     int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_tiles * BN;
-    for (int i = 0; i < pre; ++i) {
-      if (u_begin + i != a.skip_unit) {
+    for (int i = 0; i < ring; ++i) {
+      if (!a.w_const) {
+        tma_prefetch_2d(&tmW, kb * BLOCK_K, nrow);
+      } else if (u_begin + i != a.skip_unit) {
         mbar_arrive_expect_tx(full_bar(i), W_BYTES);
         tma_load_2d(tiles + i * stage_bytes, &tmW, kb * BLOCK_K, nrow, full_bar(i), pol);
       }
@@ -259,7 +263,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       for (int i = 0; i < n_units; ++i) {
         const uint32_t dst = tiles + s * stage_bytes;
         if (i >= pre) {
-          if (!mbar_wait(empty_bar(s), eph, a.wait_limit)) { GIVE_UP(1, i); s_abort = 1; break; }
+          if (!mbar_wait(empty_bar(s), eph, a.wait_limit)) { GIVE_UP(1, i); s_abort = 1; break; }      // (passes at once the first time round)
           if (u_begin + i != a.skip_unit) {
             mbar_arrive_expect_tx(full_bar(s), W_BYTES);
             tma_load_2d(dst, &tmW, kcol, nrow, full_bar(s), pol_w);
@@ -433,7 +437,7 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
 }
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
-                     SplitDesc* sd_out, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap, float* out,
+                     SplitDesc* sd_out, bool w_const, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap, float* out,
                      unsigned int* arrived) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
@@ -445,7 +449,7 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.m_tiles = sd.m_tiles; a.mt = sd.mt;
   a.total_units = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles * sd.kb; a.q = sd.q; a.status = status;
   a.x_lo_rows = x_planes == 2 ? x_rows_alloc : 0; a.diag = diag;
-  a.wait_limit = dbg && dbg->wait_limit ? dbg->wait_limit : WAIT_LIMIT; a.skip_unit = dbg ? dbg->skip_unit : -1;
+  a.wait_limit = dbg && dbg->wait_limit ? dbg->wait_limit : WAIT_LIMIT; a.skip_unit = dbg ? dbg->skip_unit : -1; a.w_const = w_const;
   // Two planes, up to 128 rows: the hi and lo activation tiles sit back to back and form ONE MMA operand of 2 mt rows, so each
   // weight tile is read from shared memory once; taller tiles take a pass per plane.
   a.cat = x_planes == 2 && sd.mt <= 128;

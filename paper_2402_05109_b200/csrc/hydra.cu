@@ -277,7 +277,7 @@ hydra_status run_gemm(hydra_ctx* c, const void* x, int x_rows_alloc, const void*
     int slots = 1;
     gemm_tc_plan(m, n, k, nullptr, &slots);
     if ((size_t)slots * m * n > c->part_floats) return HYDRA_ERR_CAPACITY;
-    return gemm_tc((const bf16*)x, x_rows_alloc, c->planes, (const bf16*)w, c->part, m, n, k, sd, c->d_status, c->d_status + 8, nullptr, st);
+    return gemm_tc((const bf16*)x, x_rows_alloc, c->planes, (const bf16*)w, c->part, m, n, k, sd, true, c->d_status, c->d_status + 8, nullptr, st);
   }
   *sd = single_slot((size_t)m * n);
   return gemm_simt(x, w, c->part, m, n, k, c->m.dtype, true, st);      // bfloat16: the hi plane only (debug mode)
@@ -853,7 +853,7 @@ hydra_status hydra_gemm(const void* x, const void* w, float* out, float* partial
     if (!status) return HYDRA_ERR_INVALID;
     if (!gemm_tc_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
     SplitDesc sd;
-    HYDRA_TRY(gemm_tc((const bf16*)x, m, x_planes, (const bf16*)w, partial, m, n, k, &sd, status, nullptr, nullptr, st));
+    HYDRA_TRY(gemm_tc((const bf16*)x, m, x_planes, (const bf16*)w, partial, m, n, k, &sd, false, status, nullptr, nullptr, st));
     return reduce_splits(partial, sd, out, m, n, st);
   }
   return gemm_simt(x, w, out, m, n, k, dtype, false, st);
@@ -869,7 +869,7 @@ hydra_status hydra_gemm_bounded_wait_probe(const void* x, const void* w, float* 
   CounterScope cs(nullptr);
   GemmDebug dbg{wait_limit, skip_unit};
   SplitDesc sd;
-  return gemm_tc((const bf16*)x, m, 1, (const bf16*)w, partial, m, n, k, &sd, status, diag, &dbg, (cudaStream_t)stream);
+  return gemm_tc((const bf16*)x, m, 1, (const bf16*)w, partial, m, n, k, &sd, false, status, diag, &dbg, (cudaStream_t)stream);
 }
 
 size_t hydra_attention_scratch_bytes(int batch, int tc, int n_heads, int head_dim, int max_seq) {

@@ -8,10 +8,11 @@ namespace hydra {
 // tcgen05 path (bfloat16 operands).  x_rows_alloc = rows the x buffer really holds (>= m); rows of the last
 // tile beyond m are computed and dropped.  part needs gemm_tc_plan(...)'s max_slots * m * n floats.
 // x holds x_planes (1 or 2) planes of x_rows_alloc rows each: plane 0 = bf16(v), plane 1 = bf16(v - plane 0).
+// w_const: no kernel in flight writes w (the weights of a context); its first tiles are then read ahead of the preceding kernel's completion.
 // dbg (tests of the bounded waits only): a shorter poll limit and one weight-tile request that CTA 0 leaves out.
 struct GemmDebug { uint32_t wait_limit; int skip_unit; };
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
-                     SplitDesc* sd_out, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
+                     SplitDesc* sd_out, bool w_const, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
                      size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/,
                      float* out = nullptr /*[m][n]: the sums themselves*/, unsigned int* arrived = nullptr /*with out: a zeroed counter per tile, left zeroed*/);
 constexpr size_t GEMM_TILE_COLS = 128;    // an output has at most n / GEMM_TILE_COLS * ceil(m / 16) tiles

@@ -46,6 +46,6 @@ extern "C" hydra_status hydra_gemm_noalloc(const void* x, const void* w, float* 
   if (!gemm_tc_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
   float* part = reinterpret_cast<float*>(addr);
   // every partial element that is added is written first, and the counters are left at zero, so nothing has to be cleared
-  return gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, nullptr, status, nullptr, nullptr, (cudaStream_t)stream,
+  return gemm_tc((const bf16*)x, m, 1, (const bf16*)w, part, m, n, k, nullptr, false, status, nullptr, nullptr, (cudaStream_t)stream,
                  NOALLOC_SCRATCH_BYTES / sizeof(float), out, reinterpret_cast<unsigned int*>(addr + NOALLOC_SCRATCH_BYTES));
 }

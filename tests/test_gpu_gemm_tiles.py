@@ -52,3 +52,34 @@ def test_gemm_noalloc_result_off_a_16_byte_boundary(m, n, k, offset):
     ref = x.double() @ w.double().T
     assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
     assert bool((buf[:offset] == 7.0).all()) and bool((buf[offset + m * n:] == 7.0).all()) and int(status.item()) == 0
+
+
+@pytest.mark.parametrize("m", [3, 64])
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_weights_written_by_the_preceding_kernel(m, noalloc):
+    """The weights of a stand-alone call may be the result of the kernel before it on the stream (here the library's attention, which
+    lets its successor start early): stream order alone has to be enough."""
+    from paper_2402_05109_b200 import tree_attention
+    from paper_2402_05109_b200.binding import lib, _stream
+    B, tc, H, hd, S = 2, 64, 8, 128, 2048
+    n, k = B * tc, H * hd
+    half = lambda shape, i: normal_(torch.empty(shape, dtype=torch.float16, device="cuda"), 81, i, 1.0)
+    q, kc, vc = half((n, H, hd), 1), half((B, H, S, hd), 2), half((B, H, S, hd), 3)
+    pos0 = torch.tensor([S - tc, S - 2 * tc], dtype=torch.int32, device="cuda")
+    x = normal_(torch.empty(m, k, dtype=torch.bfloat16, device="cuda"), 82, m, 1.0)
+    w = tree_attention(q, kc, vc, pos0, None, None, tc)
+    ref = x.double() @ w.double().T
+    part = torch.empty(lib.hydra_gemm_partial_floats(m, n, k, 1, 0), device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(20):
+        w.fill_(float("nan"))
+        out = torch.empty(m, n, device="cuda")
+        torch.cuda.synchronize()
+        assert lib.hydra_tree_attention(q.data_ptr(), kc.data_ptr(), vc.data_ptr(), pos0.data_ptr(), None, None, w.data_ptr(), None,
+                                        B, tc, H, hd, S, 1, 1, 1, status.data_ptr(), _stream()) == 0
+        if noalloc:
+            assert lib.hydra_gemm_noalloc(x.data_ptr(), w.data_ptr(), out.data_ptr(), m, n, k, status.data_ptr(), _stream()) == 0
+        else:
+            assert lib.hydra_gemm(x.data_ptr(), w.data_ptr(), out.data_ptr(), part.data_ptr(), m, n, k, 1, 0, 1, status.data_ptr(), _stream()) == 0
+        assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+    assert int(status.item()) == 0

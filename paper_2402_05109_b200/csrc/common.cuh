@@ -80,18 +80,23 @@ __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + __expf(-x)
 // touched the tile, in CTA order.  A single-slot output is described by q = kb = 1.
 struct SplitDesc {
   int q, kb, m_tiles, mt, bn_shift;
-  unsigned long long q_inv, mt_inv;      // ceil(2^40 / q), ceil(2^32 / mt)
+  unsigned long long q_inv, mt_inv;      // ceil(2^63 / q), ceil(2^32 / mt)
   size_t stride;
-  // u * q_inv >> 40 is u / q while u q < 2^40 (u: units, far below 2^24; q: units / CTAs); m * mt_inv >> 32 is m / mt while m mt < 2^32
   void set_inverses() {
-    q_inv = ((1ull << 40) + (unsigned)q - 1) / (unsigned)q;
+    q_inv = ((1ull << 63) + (unsigned)q - 1) / (unsigned)q;
     mt_inv = ((1ull << 32) + (unsigned)mt - 1) / (unsigned)mt;
   }
+  // u / q, exact for all u, q < 2^31 (u * q_inv >> 63; the excess of q_inv, below 1, adds less than u / 2^63 < 1 / q); two multiplications
+  __host__ __device__ unsigned div_q(unsigned u) const {
+    return (unsigned)(((unsigned long long)u * (unsigned)(q_inv >> 32) + ((unsigned long long)u * (unsigned)q_inv >> 32)) >> 31);
+  }
+  // m / mt, exact while m mt < 2^32; row tiles of 256 (every m above 4096 has tiles of more than 240, that is 256 rows) are exact for all m
+  __host__ __device__ int div_mt(int m) const { return (int)(((unsigned)m * mt_inv) >> 32); }
 };
-__device__ __forceinline__ int split_count(const SplitDesc& sd, int m, int n) {
-  const int mi = sd.m_tiles == 1 ? 0 : (int)(((unsigned)m * sd.mt_inv) >> 32);
-  const unsigned u0 = (unsigned)(((n >> sd.bn_shift) * sd.m_tiles + mi) * sd.kb);   // tiles * kb stays far below 2^31
-  return (int)((((u0 + sd.kb - 1) * sd.q_inv) >> 40) - ((u0 * sd.q_inv) >> 40)) + 1;
+__host__ __device__ __forceinline__ int split_count(const SplitDesc& sd, int m, int n) {
+  const int mi = sd.m_tiles == 1 ? 0 : sd.div_mt(m);
+  const unsigned u0 = (unsigned)(((n >> sd.bn_shift) * sd.m_tiles + mi) * sd.kb);   // tiles * kb stays below 2^31
+  return (int)(sd.div_q(u0 + sd.kb - 1) - sd.div_q(u0)) + 1;
 }
 // acc[u] = sum over the ns[u] slots of the four floats at element offset off[u] of a slot (all loads of a round in flight together)
 template <int U, int PMAX = 6>

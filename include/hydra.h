@@ -239,7 +239,7 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  * Serving loops that must stay clear of the allocator's locks and implicit synchronisation, plugins living
  * inside a host's fixed memory budget, and processes whose free memory already belongs to a pool cannot
  * supply hydra_gemm's partial_dev buffer; here the partial sums live in an 8 MiB array that is part of the
- * library image (every GPU that loads the library holds it, and a 64 KiB table of counters, until the process exits).
+ * library image (every GPU that loads the library holds it, and 6 KiB of counters, until the process exits).
  *   - x [m][k], w [n][k] bfloat16, out [m][n] float, status_dev as in hydra_gemm: all caller-owned device
  *     memory; n % 128 == 0, k % 64 == 0; x and w on 16-byte boundaries (INVALID otherwise), out on a float's.
  *   - m * n * 4 bytes must fit in the 8 MiB array (the work is shared out among as many CTAs as the partial sums in it
@@ -249,10 +249,15 @@ hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, fl
  *     address (cudaGetSymbolAddress, with that device current); make that first call outside any stream
  *     capture.
  *   - All calls on a GPU share the one array and it keeps the previous call's partial sums; the GEMM
- *     overwrites every element it later reads and leaves the counters at zero, so no clearing is needed, but two calls whose kernels overlap
- *     on the GPU (different streams, different threads) race on it: serialise them. */
+ *     overwrites every element it later reads, so no clearing is needed, but two calls whose kernels overlap
+ *     on the GPU (different streams, different threads) race on it: serialise them.  What a call that timed out or was
+ *     overlapped leaves behind does not reach later calls.
+ *   - May be captured into a graph (then always as two launches; outside a capture, small calls are one). */
 hydra_status hydra_gemm_noalloc(const void* x_dev, const void* w_dev, float* out_dev, int m, int n, int k,
                                 int32_t* status_dev, void* stream);
+/* Introspection for tests: the device address of the current device's array, and the bytes of its partial sums and of the counters
+ * behind them (8-byte words; each an earlier call's number in the upper 48 bits and how many CTAs have stored the tile below). */
+hydra_status hydra_gemm_noalloc_scratch(void** dev_ptr, size_t* partial_bytes, size_t* counter_bytes);
 /* hydra_gemm_bounded_wait_probe: exercises the give-up path of the tensor-core GEMM's bounded waits.  Runs the
  * GEMM of hydra_gemm (dtype 1, mode 0, x_planes 1) on a problem small enough for ONE CTA (else UNSUPPORTED), with
  * barrier waits limited to wait_limit polls (1..65536) and with the weight-tile request of k-block `skip_unit` left

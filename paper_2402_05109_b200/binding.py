@@ -68,6 +68,7 @@ lib.hydra_gemm_partial_floats.restype = _sz
 lib.hydra_gemm_partial_floats.argtypes = [_i] * 5
 lib.hydra_gemm.argtypes = [_vp, _vp, _vp, _vp, _i, _i, _i, _i, _i, _i, _vp, _vp]
 lib.hydra_gemm_noalloc.argtypes = [_vp, _vp, _vp, _i, _i, _i, _vp, _vp]
+lib.hydra_gemm_noalloc_scratch.argtypes = [C.POINTER(_vp), C.POINTER(_sz), C.POINTER(_sz)]
 lib.hydra_gemm_bounded_wait_probe.argtypes = [_vp, _vp, _vp, _i, _i, _i, _i, C.c_uint, _vp, _vp, _vp]
 lib.hydra_attention_scratch_bytes.restype = _sz
 lib.hydra_attention_scratch_bytes.argtypes = [_i] * 5

@@ -157,7 +157,7 @@ __device__ __forceinline__ void sum_tile(const float* part, size_t stride, int s
 
 struct GemmArgs {
   float* part; size_t slot_stride;
-  float* out; unsigned int* arrived;       // REDUCE only: the output, and per tile how many of its CTAs have stored (zero between calls)
+  float* out; GemmArrivals arr;            // REDUCE only: the output, and per tile how many of its CTAs have stored
   int m, n, kb, m_tiles, total_units, q;
   int x_lo_rows;                 // row offset of the lo plane inside the activation tensor map (0: single plane)
   // activation rows per tile, boxes (planes) of a stage, MMA passes over a weight tile and columns of one, ring stages,
@@ -326,6 +326,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const int n_tile = tile / a.m_tiles, n0 = n_tile * BN, m0 = (tile - n_tile * a.m_tiles) * a.mt, rows = min(a.mt, a.m - m0);
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * NH * a.acc_cols);
       float* dst = a.part + (size_t)slot * a.slot_stride + (size_t)m0 * a.n + n0 + quarter * 32 + lane;
+      if (REDUCE && threadIdx.x == 64) atomicMax(a.arr.count + tile, a.arr.ticket << 16);      // an older call's count, if one is left, is gone
       const int tiles_in = NH == 2 && n0 + BLOCK_N < a.n ? 2 : 1;      // an output that is no multiple of the unit's width ends inside its last unit
       bool ok = mbar_wait(accfull_bar(acc), acc_ph, a.wait_limit);
       if constexpr (REDUCE) ok = epilogue_all(ok);       // the four warps meet at barriers below: they give up together
@@ -345,12 +346,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         epilogue_barrier();
         if (threadIdx.x == 64) {                         // one fence covers what the barrier has ordered before it
           __threadfence();
-          s_last = atomicAdd(a.arrived + tile, 1u) == (unsigned)(slots - 1);
+          s_last = (atomicAdd(a.arr.count + tile, 1ull) & 0xffff) == (unsigned)(slots - 1);
           __threadfence();
         }
         epilogue_barrier();
         if (s_last) {
-          if (threadIdx.x == 64) a.arrived[tile] = 0u;   // for the next call
+          if (threadIdx.x == 64) a.arr.count[tile] = 0ull;      // threads may enqueue on one stream in another order than their tickets'
           const size_t at = (size_t)m0 * a.n + n0;
 #pragma unroll 1
           for (int hh = 0; hh < tiles_in; ++hh) sum_tile(a.part + at + hh * BLOCK_N, a.slot_stride, slots, a.out + at + hh * BLOCK_N, rows, a.n, (int)threadIdx.x - 64);
@@ -438,7 +439,7 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
                      SplitDesc* sd_out, bool w_const, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap, float* out,
-                     unsigned int* arrived) {
+                     const GemmArrivals* arrivals) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
   int grid = 1;
@@ -472,8 +473,8 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   // (back to back, one launch / two: 11 x 2048 x 2048 6.3 / 8.3 us, 4 x 3456 x 640 6.4 / 8.3, 8 x 640 x 5632 8.0 / 8.2; but
   // 11 x 4096 x 2048 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x 1024 10.2 / 8.3: the sums of a tile are one CTA's work).
   // sum_tile stores 16 bytes at a time; a result buffer off that boundary takes the second launch, which stores single floats
-  if (out && m <= 16 && (long long)n * k <= 6 * 1000 * 1000 && !((uintptr_t)out & 15)) {
-    a.out = out; a.arrived = arrived;
+  if (out && arrivals && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && !((uintptr_t)out & 15)) {
+    a.out = out; a.arr = *arrivals;
     return sh.nh == 2 ? launch<2, true>(tw, tx, a, grid, st) : launch<1, true>(tw, tx, a, grid, st);
   }
   const hydra_status s = sh.nh == 2 ? launch<2, false>(tw, tx, a, grid, st) : launch<1, false>(tw, tx, a, grid, st);

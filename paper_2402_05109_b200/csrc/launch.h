@@ -11,11 +11,17 @@ namespace hydra {
 // w_const: no kernel in flight writes w (the weights of a context); its first tiles are then read ahead of the preceding kernel's completion.
 // dbg (tests of the bounded waits only): a shorter poll limit and one weight-tile request that CTA 0 leaves out.
 struct GemmDebug { uint32_t wait_limit; int skip_unit; };
+struct GemmArrivals { unsigned long long* count; unsigned long long ticket; };
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
                      SplitDesc* sd_out, bool w_const, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
                      size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/,
-                     float* out = nullptr /*[m][n]: the sums themselves*/, unsigned int* arrived = nullptr /*with out: a zeroed counter per tile, left zeroed*/);
-constexpr size_t GEMM_TILE_COLS = 128;    // an output has at most n / GEMM_TILE_COLS * ceil(m / 16) tiles
+                     float* out = nullptr /*[m][n]: the sums themselves*/, const GemmArrivals* arrivals = nullptr /*with out: for one-launch calls*/);
+// Stand-alone calls of up to GEMM_ONE_LAUNCH_WEIGHTS weights and 16 rows add their partial sums in the GEMM's own launch (gemm_tc.cu has the
+// figures).  A counter per tile (128 columns, at least 64 k) says how many CTAs have stored it: the call's ticket in the upper 48 bits,
+// the count below.  Tickets rise from call to call, so whatever an earlier call left in a counter - one that timed out, or that another call
+// overlapped - counts for nothing in a later one.
+constexpr long long GEMM_ONE_LAUNCH_WEIGHTS = 6 * 1000 * 1000;
+constexpr size_t GEMM_ONE_LAUNCH_TILES = GEMM_ONE_LAUNCH_WEIGHTS / (128 * 64);
 // grid: CTAs.  part_cap (floats, 0: no limit): fewer CTAs, hence fewer slots, where the partial sums would not fit otherwise.
 SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap = 0);
 bool gemm_tc_available();                 // driver entry point for tensor-map encoding found

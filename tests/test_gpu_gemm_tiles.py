@@ -83,3 +83,43 @@ def test_weights_written_by_the_preceding_kernel(m, noalloc):
             assert lib.hydra_gemm(x.data_ptr(), w.data_ptr(), out.data_ptr(), part.data_ptr(), m, n, k, 1, 0, 1, status.data_ptr(), _stream()) == 0
         assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
     assert int(status.item()) == 0
+
+
+def _noalloc_counters():
+    """The counters of hydra_gemm_noalloc's one-launch form as an int64 tensor."""
+    import ctypes as C
+    from paper_2402_05109_b200.binding import lib
+    ptr, part, cnt = C.c_void_p(), C.c_size_t(), C.c_size_t()
+    assert lib.hydra_gemm_noalloc_scratch(C.byref(ptr), C.byref(part), C.byref(cnt)) == 0 and part.value == 8 << 20
+
+    class View:
+        __cuda_array_interface__ = dict(shape=(cnt.value // 8,), typestr="<i8", data=(ptr.value + part.value, False), version=2)
+    return torch.as_tensor(View(), device="cuda")
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 128, 64), (11, 2048, 2048), (16, 640, 5632)])
+def test_gemm_noalloc_after_a_call_that_left_its_counters(m, n, k):
+    """A call that timed out, or that another one overlapped, leaves tiles counted in part.  Later calls, and replays of a
+    captured one, must not see it: every counter set to a small count of the first call before each of them."""
+    from paper_2402_05109_b200 import gemm_noalloc
+    counters = _noalloc_counters()
+    x = normal_(torch.empty(m, k, dtype=torch.bfloat16, device="cuda"), 67, m + k, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 68, n, 0.02)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ref = x.double() @ w.double().T
+    tol = 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+    out = torch.empty(m, n, device="cuda")
+    gemm_noalloc(x, w, out, status)
+    assert n // 128 <= counters.numel() and int(counters[: n // 128].abs().max()) == 0
+    graph, replayed = torch.cuda.CUDAGraph(), torch.empty(m, n, device="cuda")
+    with torch.cuda.graph(graph):
+        gemm_noalloc(x, w, replayed, status)
+    for left in range(1, 9):
+        for again, call in ((out, lambda: gemm_noalloc(x, w, out, status)), (replayed, graph.replay)):
+            counters.fill_((1 << 16) + left)
+            again.fill_(float("nan"))
+            call()
+            torch.cuda.synchronize()
+            assert float((again.double() - ref).abs().max()) <= tol
+    counters.zero_()
+    assert int(status.item()) == 0

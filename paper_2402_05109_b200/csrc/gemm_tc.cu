@@ -202,6 +202,7 @@ constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 512 /*barrier
 template <int NH, bool REDUCE>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const GemmArgs a) {
+  static_assert(!REDUCE || NH == 1, "sum_tile takes one weight tile");
   constexpr int W_BYTES = NH * A_BYTES, BN = NH * BLOCK_N;        // weight rows of a unit
   extern __shared__ uint8_t smem_raw[];
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -353,8 +354,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (s_last) {
           if (threadIdx.x == 64) a.arr.count[tile] = 0ull;      // threads may enqueue on one stream in another order than their tickets'
           const size_t at = (size_t)m0 * a.n + n0;
-#pragma unroll 1
-          for (int hh = 0; hh < tiles_in; ++hh) sum_tile(a.part + at + hh * BLOCK_N, a.slot_stride, slots, a.out + at + hh * BLOCK_N, rows, a.n, (int)threadIdx.x - 64);
+          sum_tile(a.part + at, a.slot_stride, slots, a.out + at, rows, a.n, (int)threadIdx.x - 64);
         }
       }
       i += seg_len;
@@ -470,12 +470,14 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   }
   if (sd_out) *sd_out = sd;
   // One launch where issuing a second one is what takes the time: up to 16 rows and a weight matrix that passes in a few microseconds
-  // (back to back, one launch / two: 11 x 2048 x 2048 6.3 / 8.3 us, 4 x 3456 x 640 6.4 / 8.3, 8 x 640 x 5632 8.0 / 8.2; but
-  // 11 x 4096 x 2048 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x 1024 10.2 / 8.3: the sums of a tile are one CTA's work).
-  // sum_tile stores 16 bytes at a time; a result buffer off that boundary takes the second launch, which stores single floats
-  if (out && arrivals && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && !((uintptr_t)out & 15)) {
+  // (back to back, one launch / two: 11 x 2048 x 2048 7.1 / 9.2 us, 4 x 3456 x 640 6.8 / 9.2, 11 x 4096 x 1024 7.0 / 9.3, 8 x 640 x 5632
+  // 8.6 / 9.1; with weight tiles requested before the dependency wait 11 x 4096 x 2048 took 9.2 / 8.4, 11 x 4096 x 4096 12.4 / 10.2, 64 x 512 x
+  // 1024 10.2 / 8.3: the sums of a tile are one CTA's work).
+  // sum_tile stores 16 bytes at a time; a result buffer off that boundary takes the second launch, which stores single floats.  (Units
+  // of two weight tiles begin at 9 million weights on 148 SMs.)
+  if (out && arrivals && sh.nh == 1 && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && !((uintptr_t)out & 15)) {
     a.out = out; a.arr = *arrivals;
-    return sh.nh == 2 ? launch<2, true>(tw, tx, a, grid, st) : launch<1, true>(tw, tx, a, grid, st);
+    return launch<1, true>(tw, tx, a, grid, st);
   }
   const hydra_status s = sh.nh == 2 ? launch<2, false>(tw, tx, a, grid, st) : launch<1, false>(tw, tx, a, grid, st);
   return s == HYDRA_OK && out ? reduce_splits(part, sd, out, m, n, st) : s;

@@ -17,3 +17,12 @@ def test_packed_prompt_passes(head_dim, kv_planes, lens):
     m = ModelCfg(2, 256, 256 // head_dim, head_dim, 512, 1024, dtype="bf16", kv_planes=kv_planes)
     st, _ = run(m, HeadCfg(3, 1, True), load_tree("tree15_d3"), lens, 2, 33, max(lens) + 40, kv_layers=(0, 1))
     assert st.steps == 2
+
+
+@pytest.mark.parametrize("rows", [16, 17, 40, 41, 96, 97])
+@pytest.mark.parametrize("d_model", [256, 1280])
+def test_row_counts_around_the_norm_clusters(rows, d_model):
+    """A pass of few rows shares each row's norm among 8, 4 or 2 CTAs of a cluster, one of many rows does not: the prompt passes at the edges."""
+    m = ModelCfg(1, d_model, d_model // 128, 128, 512, 1024, dtype="bf16")
+    st, _ = run(m, HeadCfg(1, 1, True), [-1, 0], [rows], 1, 34, rows + 16, kv_layers=(0,))
+    assert st.steps == 1

@@ -1,0 +1,21 @@
+"""Orders inside kernels that no run can show to be right: read from the source."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2402_05109_b200", "csrc")
+
+
+def kernel_bodies(name):
+    """Every kernel's text, from its __global__ to the closing brace in the first column."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    return [text[m.start():text.index("\n}", m.start())] for m in re.finditer(r"^__global__", text, re.M)]
+
+
+def test_a_cluster_has_started_before_its_shared_memory_is_stored_to():
+    """Distributed shared memory may be accessed once every CTA of the cluster is known to run: a cluster barrier completes first."""
+    found = 0
+    for body in kernel_bodies("kernels.cu"):
+        if "st.shared::cluster" in body:
+            found += 1
+            assert -1 < body.find("barrier.cluster.arrive") < body.find("barrier.cluster.wait") < body.find("st.shared::cluster")
+    assert found == 1

@@ -67,7 +67,9 @@ __device__ __forceinline__ float warp_max(float v) {
 }
 // Programmatic dependent launch: every kernel of the library starts with pdl_trigger() (lets the next kernel
 // in the stream get resident early) and pdl_wait() (blocks until the preceding kernel has completed and its
-// writes are visible) before it touches memory, so dependencies stay transitive along the stream.
+// writes are visible) before it touches what other kernels write, so dependencies stay transitive along the stream.  What an earlier
+// kernel of the stream writes is never a `const ... __restrict__` parameter: the compiler may take such data as constant for the
+// kernel's lifetime, which here begins before the writer has ended, and move its loads over the wait.  Weights and tables may be.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -130,7 +130,7 @@ hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, i
   return HYDRA_OK;
 }
 
-__global__ void reduce_splits_kernel(const float* __restrict__ part, SplitDesc sd, float* __restrict__ out, int m, int n) {
+__global__ void reduce_splits_kernel(const float* part, SplitDesc sd, float* __restrict__ out, int m, int n) {
   pdl_trigger();
   pdl_wait();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -162,7 +162,7 @@ template <bool VEC, typename T> __device__ __forceinline__ float4 load4_at(const
 }
 
 template <typename T>
-__global__ void embed_rows_kernel(const T* __restrict__ embed, const int* __restrict__ tok, float* __restrict__ x, int d,
+__global__ void embed_rows_kernel(const T* __restrict__ embed, const int* tok, float* __restrict__ x, int d,
                                   int vocab, int* status) {
   pdl_trigger();
   pdl_wait();
@@ -246,7 +246,7 @@ constexpr int NORM_THREADS = 1024;
 // memory may be stored to once that CTA has started: a barrier, arrived at on entry and waited for behind the sums, says so (0.35 % of
 // a 7B step without a tree; waited for ahead of the sums 0.6 %).
 template <typename T, int CS>
-__global__ void __launch_bounds__(NORM_THREADS) residual_rmsnorm_kernel(const float* res, const float* __restrict__ part,
+__global__ void __launch_bounds__(NORM_THREADS) residual_rmsnorm_kernel(const float* res, const float* part,
                                                                         SplitDesc sd, float* x_out,
                                                                         const T* __restrict__ gain, T* __restrict__ xn, size_t xn_ps,
                                                                         float* __restrict__ hn, int d, float eps) {
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(NORM_THREADS) residual_rmsnorm_kernel(const fl
 // 1024 threads at 64 registers, one CTA fills an SM and 512 rows run as four latencies one after the other: 20 us at 512 x 4096, here 12.)
 constexpr int NORM_ROW_THREADS = 512;
 template <typename T, int P>
-__global__ void __launch_bounds__(NORM_ROW_THREADS, 2) residual_rmsnorm_rows_kernel(const float* res, const float* __restrict__ part, SplitDesc sd,
+__global__ void __launch_bounds__(NORM_ROW_THREADS, 2) residual_rmsnorm_rows_kernel(const float* res, const float* part, SplitDesc sd,
                                                                                  float* x_out, const T* __restrict__ gain, T* __restrict__ xn, size_t xn_ps,
                                                                                  float* __restrict__ hn, int d, float eps) {
   pdl_trigger();
@@ -433,8 +433,8 @@ hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cud
 // lengths are stable within a forward call, see rope_table_kernel).
 // T: float (float model path) or float16 (bfloat16 model path: q and the caches are float16 in one or two planes).
 template <typename T>
-__global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* __restrict__ part, SplitDesc sd,
-                                                             const float2* __restrict__ table, T* __restrict__ q, size_t q_ps,
+__global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, SplitDesc sd,
+                                                             const float2* table, T* __restrict__ q, size_t q_ps,
                                                              T* __restrict__ kc, T* __restrict__ vc, size_t kv_ps,
                                                              RowSet rs, int H, int hd, int max_seq,
                                                              int* status) {
@@ -507,8 +507,8 @@ constexpr int ATT_TILE = 64;      // KV rows staged per iteration: two keys per 
 constexpr int ATT_WARPS = 8;
 
 template <typename T, int HD, int RPW, bool VEC>
-__global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __restrict__ q, const T* __restrict__ kc,
-                                                                   const T* __restrict__ vc, RowSet rs,
+__global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* q, const T* kc,
+                                                                   const T* vc, RowSet rs,
                                                                    float* __restrict__ part_o, float* __restrict__ part_ml,
                                                                    T* __restrict__ out, int H, int max_seq, int nchunks) {
   pdl_trigger();
@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* __re
 }
 
 template <typename T, int HD>
-__global__ void tree_attn_combine_kernel(const float* __restrict__ part_o, const float* __restrict__ part_ml, RowSet rs,
+__global__ void tree_attn_combine_kernel(const float* part_o, const float* part_ml, RowSet rs,
                                          T* __restrict__ out, int H, int nchunks) {
   pdl_trigger();
   pdl_wait();
@@ -696,7 +696,7 @@ hydra_status tree_attention_f32(const float* q, const float* kc, const float* vc
 // worked out and that before the wait (512 x 11008: 28 us with a flat index divided by the row length, 21 so; 64 rows: 6.0 and 3.5)
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) silu_mul_kernel(const float* __restrict__ part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int f) {
+__global__ void __launch_bounds__(256) silu_mul_kernel(const float* part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int f) {
   pdl_trigger();
   const int r = blockIdx.y, c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   const size_t off[2] = {(size_t)r * 2 * f + c, (size_t)r * 2 * f + f + c};
@@ -741,7 +741,7 @@ constexpr int TOPK_SPAN = 2048;           // columns per stage-1 block (8 per th
 constexpr int TOPK_MAX = 64;              // a tree node has at most 63 children
 constexpr int TOPK_LISTS_PER_LANE = 4;    // stage 2: at most 128 column blocks (262144 tokens)
 
-__global__ void __launch_bounds__(256) topk_stage1_kernel(const float* __restrict__ part, SplitDesc sd,
+__global__ void __launch_bounds__(256) topk_stage1_kernel(const float* part, SplitDesc sd,
                                                           float* __restrict__ logits_out, float* __restrict__ cand_v,
                                                           int* __restrict__ cand_i, int vocab, int c) {
   pdl_trigger();
@@ -804,7 +804,7 @@ __global__ void __launch_bounds__(256) topk_stage1_kernel(const float* __restric
 
 // out_of(row) and count_of(row): where the winners go.  lv.parents == null: argmax (one winner per row to amax[row]).
 // One warp per winner list; dynamic shared memory: nblk * c (value, index) pairs.
-__global__ void __launch_bounds__(32) topk_stage2_kernel(const float* __restrict__ cand_v, const int* __restrict__ cand_i,
+__global__ void __launch_bounds__(32) topk_stage2_kernel(const float* cand_v, const int* cand_i,
                                                          int nblk, int c, LevelDesc lv, const int* __restrict__ first_child,
                                                          const int* __restrict__ n_child, int* __restrict__ out, int T, int cand_div) {
   pdl_trigger();
@@ -884,8 +884,8 @@ hydra_status topk_children(const float* part, SplitDesc sd, float* logits, Level
 // Hydra heads: input gather and the residual SiLU layer epilogue
 // ------------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) head_gather_kernel(const float* __restrict__ hprime, const T* __restrict__ embed,
-                                                          const int* __restrict__ root_tok, int* tree_tok,
+__global__ void __launch_bounds__(256) head_gather_kernel(const float* hprime, const T* __restrict__ embed,
+                                                          const int* root_tok, int* tree_tok,
                                                           const int* __restrict__ path_tab, LevelDesc lv, int write_root, T* __restrict__ z,
                                                           size_t z_ps, int T_rows, int kp1, int d_model, int vocab, int* status) {
   pdl_trigger();
@@ -924,7 +924,7 @@ hydra_status head_gather(const float* hprime, const void* embed, const int* root
 // VEC: the bias, a caller's vector, lies on a boundary of four elements.
 constexpr int HEAD_ACT_THREADS = 64;
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* __restrict__ part,
+__global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* part,
                                 SplitDesc sd, const T* __restrict__ bias, float* y_out, T* __restrict__ yb, size_t yb_ps,
                                 int rows, int d) {
   pdl_trigger();
@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(256) accept_compact_kernel(AcceptArgs a) {
   }
 }
 // (max, sum exp((l - max)/tau), sum exp((l - max)/tau) (l - max)/tau) of every logits row; one CTA per row, fixed reduction order
-__global__ void __launch_bounds__(1024) softmax_row_stats_kernel(const float* __restrict__ logits, float4* __restrict__ stats, int vocab, float tau) {
+__global__ void __launch_bounds__(1024) softmax_row_stats_kernel(const float* logits, float4* __restrict__ stats, int vocab, float tau) {
   pdl_trigger();
   pdl_wait();
   __shared__ float sh[32];
@@ -1308,7 +1308,7 @@ hydra_status apply_plant(int* tree_tok, const int* plant, int count, cudaStream_
 }
 
 template <typename T>
-__global__ void cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, size_t dst_ps, size_t count) {
+__global__ void cast_rows_kernel(const float* src, T* __restrict__ dst, size_t dst_ps, size_t count) {
   pdl_trigger();
   pdl_wait();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -19,3 +19,11 @@ def test_a_cluster_has_started_before_its_shared_memory_is_stored_to():
             found += 1
             assert -1 < body.find("barrier.cluster.arrive") < body.find("barrier.cluster.wait") < body.find("st.shared::cluster")
     assert found == 1
+
+
+def test_only_weights_and_tables_are_declared_constant():
+    """`const ... __restrict__` lets the compiler move loads over the dependency wait, which is right for data that no kernel writes."""
+    constant = set()
+    for body in kernel_bodies("kernels.cu"):
+        constant |= set(re.findall(r"const \w+\s*\*\s*__restrict__\s+(\w+)", body[:body.index("{")]))
+    assert constant <= {"embed", "gain", "bias", "first_child", "n_child", "path_tab"}

@@ -146,8 +146,9 @@ hydra_status hydra_accept_compact(hydra_ctx*, const int32_t* tree_tok_dev, const
 
 /* One whole decoding step (the three passages above): draft + (optional planting) + verify + accept_compact
  * on the library's own buffers.  n_acc_dev [batch], out_tok_dev [batch][K+1] as in hydra_accept_compact (either
- * may be NULL).  From the second step after a prefill on, the step is captured into a CUDA graph (re-captured
- * when the batch or the planting buffer changes or an attention grid must grow; n_acc_dev and out_tok_dev may change freely) and replayed with one launch, unless the stream
+ * may be NULL).  From the second step of the context on, the step is captured into a CUDA graph (again
+ * when the batch or the planting buffer changes or an attention grid must grow; up to eight graphs are kept, across prompt passes too, until the
+ * acceptance criterion or the GEMM mode changes; n_acc_dev and out_tok_dev may change freely) and replayed with one launch, unless the stream
  * is a default stream (not capturable) or hydra_set_step_graph switched graphs off.  Errors: STATE, CAPACITY. */
 hydra_status hydra_step(hydra_ctx*, int32_t* n_acc_dev, int32_t* out_tok_dev, void* stream);
 /* on = 0: hydra_step launches kernel by kernel (for profilers that list kernels); on = 1 (default): graph replay. */

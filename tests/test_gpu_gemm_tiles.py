@@ -123,3 +123,18 @@ def test_gemm_noalloc_after_a_call_that_left_its_counters(m, n, k):
             assert float((again.double() - ref).abs().max()) <= tol
     counters.zero_()
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("m,n,k", [(64, 11008, 4096), (128, 8192, 2048), (100, 12800, 1024)])
+def test_gemm_noalloc_takes_fewer_ctas_where_the_sums_would_not_fit(m, n, k):
+    """Results that fit the built-in scratch although the partial sums of the usual plan do not: fewer CTAs share the work."""
+    from paper_2402_05109_b200 import gemm_noalloc
+    from paper_2402_05109_b200.binding import lib
+    assert m * n * 4 <= 8 << 20 < 4 * lib.hydra_gemm_partial_floats(m, n, k, 1, 0)
+    x = normal_(torch.empty(m, k, dtype=torch.bfloat16, device="cuda"), 69, m + k, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 70, n, 0.02)
+    status, out = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.full((m, n), float("nan"), device="cuda")
+    gemm_noalloc(x, w, out, status)
+    ref = x.double() @ w.double().T
+    assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+    assert int(status.item()) == 0

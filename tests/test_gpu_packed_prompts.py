@@ -1,7 +1,8 @@
 """The packed prompt pass of the bfloat16 path (prompts back to back, at most 768 tokens a pass) against the oracle, in lock-step."""
 import pytest
+import torch
 
-from synth import load_tree
+from synth import load_tree, make_prompts, make_weights
 from synth.configs import ModelCfg, HeadCfg
 from tests.test_gpu_step import run
 
@@ -26,3 +27,29 @@ def test_row_counts_around_the_norm_clusters(rows, d_model):
     m = ModelCfg(1, d_model, d_model // 128, 128, 512, 1024, dtype="bf16")
     st, _ = run(m, HeadCfg(1, 1, True), [-1, 0], [rows], 1, 34, rows + 16, kv_layers=(0,))
     assert st.steps == 1
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_offsets_may_begin_anywhere_in_the_token_buffer(dtype):
+    """The first offset need not be 0 (prompts inside a larger token buffer): the same root, lengths, hidden rows and caches."""
+    import ctypes as C
+    from paper_2402_05109_b200 import Hydra
+    from paper_2402_05109_b200.binding import lib, _stream
+    m = ModelCfg(2, 256, 2, 128, 512, 1024, dtype=dtype)
+    w = {k: v.cuda() for k, v in make_weights(m, HeadCfg(2, 1, True), 35).items()}
+    prompts = make_prompts(35, [70, 1, 900], m.vocab)
+    toks = torch.cat([p.to(torch.int32).flatten() for p in prompts])
+    outs = []
+    for lead in (0, 5, 777):
+        g = Hydra(m, HeadCfg(2, 1, True), [-1, 0, 1], w, 3, 960)
+        buf = torch.cat([torch.full((lead,), 1 << 30, dtype=torch.int32), toks]).cuda()       # what lies ahead is no token
+        offs = [lead]
+        for p in prompts:
+            offs.append(offs[-1] + p.numel())
+        g.batch = 3
+        assert lib.hydra_prefill(g._ctx, 3, buf.data_ptr(), (C.c_int32 * 4)(*offs), _stream()) == 0
+        g.poll_status()
+        outs.append([g.get_buffer(n).cpu().clone() for n in ("ROOT_TOK", "LEN", "N_NEW", "H_NEW", "KV_BASE", "KV_PREFIX")])
+        g.close()
+    for other in outs[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(outs[0], other))

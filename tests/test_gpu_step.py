@@ -47,9 +47,8 @@ def test_small_bf16_hydrapp_ragged_batch():
 
 @pytest.mark.parametrize("head_dim,kv_planes", [(128, 2), (128, 1), (64, 2)])
 def test_prompt_lengths_around_the_prefill_chunk(head_dim, kv_planes):
-    """Prompts that end just before, on and just after the 64- and 128-row boundaries of the prompt pass (the bfloat16 path
-    walks 128-row causal chunks: two 64-row attention launches at head_dim 128 with two planes, one 128-row launch otherwise):
-    the lock-step protocol compares the caches of both layers, the last hidden state and the first steps with the oracle."""
+    """Prompts that end just before, on and just after the 64- and 128-row boundaries of the attention's key tiles and query blocks (the
+    bfloat16 path packs them back to back, a block of at most 128 rows of one prompt per CTA column): the lock-step protocol compares the caches of both layers, the last hidden state and the first steps with the oracle."""
     m = ModelCfg(2, 256, 256 // head_dim, head_dim, 512, 1024, dtype="bf16", kv_planes=kv_planes)
     h = HeadCfg(3, 2, True)
     st, _ = run(m, h, load_tree("tree15_d3"), [127, 128, 129, 64, 65, 191, 256, 1], 2, 31, 320, kv_layers=(0, 1))
@@ -234,3 +233,47 @@ def test_step_graph_replay_matches_kernel_by_kernel_launches():
         assert g.launch_count() > 100 * 50
         g.close()
     assert torch.equal(outs[0], outs[1])
+
+
+def test_step_graphs_across_prompt_passes_batches_and_output_buffers():
+    """Step graphs outlive a prompt pass and take new output buffers in place: prompt passes of other batches and length
+    buckets, fresh output tensors on every step and outputs left out give the tokens of kernel-by-kernel launches, and no step writes
+    into an earlier step's tensors."""
+    from paper_2402_05109_b200 import Hydra
+    from paper_2402_05109_b200.binding import lib, _stream
+    m = ModelCfg(2, 256, 2, 128, 512, 1024, dtype="bf16")
+    h = HeadCfg(4, 2, True)
+    w = {k: v.cuda() for k, v in make_weights(m, h, 51).items()}
+    requests = [make_prompts(51, lens, m.vocab) for lens in ([40, 75], [600], [33, 5, 12], [41, 80], [40, 75])]
+    outs = []
+    for graph in (False, True):
+        g = Hydra(m, h, load_tree("tree63_d4"), w, 3, 1100)
+        g.set_step_graph(graph)
+        stream, got, copies = torch.cuda.Stream(), [], []
+        with torch.cuda.stream(stream):
+            for prompts in requests:
+                g.prefill(prompts)
+                kept = torch.empty(len(prompts), dtype=torch.int32, device="cuda"), torch.empty(len(prompts), h.n_heads + 1, dtype=torch.int32, device="cuda")
+                for s in range(9):
+                    if s == 4:                        # neither output
+                        assert lib.hydra_step(g._ctx, None, None, _stream()) == 0
+                        continue
+                    if s == 5:                        # lengths only
+                        n_acc = torch.full((len(prompts),), -7, dtype=torch.int32, device="cuda")
+                        assert lib.hydra_step(g._ctx, n_acc.data_ptr(), None, _stream()) == 0
+                        got.append(n_acc)
+                        copies.append(n_acc.clone())
+                        continue
+                    pair = g.step(*kept) if s in (2, 3) else g.step()
+                    got += [t.clone() for t in pair] if s in (2, 3) else list(pair)
+                    copies += [t.clone() for t in pair]
+                copies.append(g.get_buffer("LEN")[: len(prompts)].clone())
+                got.append(copies[-1])
+                g.poll_status()
+            stream.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, copies))        # later steps left earlier tensors alone
+        outs.append([t.cpu() for t in got])
+        g.close()
+    assert len(outs[0]) == len(outs[1]) and all(torch.equal(a, b) for a, b in zip(*outs))
+    per = len(outs[1]) // len(requests)
+    assert all(torch.equal(a, b) for a, b in zip(outs[1][:per], outs[1][-per:]))      # the first request again: the same tokens

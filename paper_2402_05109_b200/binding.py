@@ -87,8 +87,11 @@ def _check(code: int, what: str):
                                              lib.hydra_last_error().decode()))
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # without the wrapper object; not a public name
+
+
 def _stream() -> int:
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())      # torch.cuda.current_stream().cuda_stream without the wrapper object
+    return _raw_stream(torch.cuda.current_device()) if _raw_stream else torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

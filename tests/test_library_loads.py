@@ -31,3 +31,16 @@ def test_workspace_bytes_and_invalid_configs_without_gpu():
     assert lib.hydra_workspace_bytes(C.byref(mc), C.byref(hc), C.byref(TreeCfgC(5, deep))) == 0
     mc.n_heads = 3                                           # n_heads * head_dim != d_model
     assert lib.hydra_workspace_bytes(C.byref(mc), C.byref(hc), C.byref(TreeCfgC(4, par))) == 0
+
+
+def test_current_stream_without_the_private_torch_function(monkeypatch):
+    """The raw-stream shortcut is not a public name of torch: the binding works where it is absent."""
+    from types import SimpleNamespace
+    import torch
+    from paper_2402_05109_b200 import binding
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=7))
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 100 + device)
+    assert binding._stream() == 103
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    assert binding._stream() == 7

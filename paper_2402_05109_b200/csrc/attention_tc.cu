@@ -34,9 +34,9 @@
 // What bounds a tile of the loop (two planes, head_dim 128): 64 KB from memory (1.1 us with 120 CTAs at 7 TB/s), about 1800
 // cycles of shared memory and 1540 of the tensor pipe (see S_COLS), 512 of exponentials per 32 rows; a softmax step is a chain of
 // about 1600 cycles, of which two run at a time.  With one group of softmax warps (a tile of 64 rows shared by two warps), P in
-// shared memory and the rows of one chunk merged like those of several, a layer took, against now: 64 rows x 8 sequences of 250 to
-// 1100 tokens x 32 heads 49.7 -> 42.7 us, 40 heads x 2000 tokens 30.5 -> 26.8 us, 32 heads x 600 tokens 12.0 -> 10.9 us; 768 prompt
-// rows of two sequences 41.6 -> 27 us, of one sequence at 2000 tokens (40 heads) 85 -> 68 us, of four (52 heads) 84 -> 62 us.
+// shared memory and the rows of one chunk merged like those of several, a stand-alone call of 64 rows took, against now (back to back
+// over caches larger than the L2, graph replay): 8 sequences of 250 to 1100 tokens x 32 heads 56.1 -> 49.2 us, 4 of 1050 x 52 heads
+// 61.4 -> 58.1, 1 of 2000 x 40 heads 23.4 -> 22.7, 1 of 600 x 32 heads 12.6 -> 11.9.
 // Query rows beyond the row count of the call ride along as unused lanes of the M = 128 tile.
 // One chunk: the softmax warps normalise their rows out of tensor memory and write them, through a warp's own piece of the
 // idle ring for whole 128-byte stores; no cluster, no merge.

@@ -9,8 +9,9 @@
 
 namespace {
 
-// Partial sums of the stream-K GEMM: hydra_gemm_partial_floats(m, n, k, 1, 0) floats.  8 MiB per GPU that loads the library, held until
-// the process exits.  Shared by every call (and every thread) on that GPU.
+// Partial sums of the stream-K GEMM: m n floats for every CTA that touches a tile; where those of the usual plan do not fit, fewer CTAs
+// share the work, down to one a tile.  8 MiB per GPU that loads the library, held until the process exits.  Shared by every call (and
+// every thread) on that GPU.
 constexpr size_t NOALLOC_SCRATCH_BYTES = 8u << 20;
 // behind them the counters of one-launch calls (see GemmArrivals)
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + hydra::GEMM_ONE_LAUNCH_TILES * sizeof(unsigned long long)];

@@ -86,7 +86,9 @@ typedef struct {
 } hydra_tree_cfg;
 
 /* Device weight pointers.  Arrays of pointers (attn_norm[l], ...) are HOST arrays of n_layers (or K)
- * DEVICE pointers.  wqkv rows are q, k, v in that order; w_gate_up rows are gate then up. */
+ * DEVICE pointers.  wqkv rows are q, k, v in that order; w_gate_up rows are gate then up.  Matrices lie on 16-byte boundaries (dtype 1)
+ * or on four elements (dtype 0), norm gains and the embedding on four elements (else INVALID, from hydra_create or from the first call that
+ * uses them); biases on an element. */
 typedef struct {
   const void *embed /*[V][d]*/, *lm_head /*[V][d]*/, *final_norm /*[d]*/;
   const void *const *attn_norm /*[d]*/, *const *wqkv /*[3d][d]*/, *const *wo /*[d][d]*/;
@@ -219,7 +221,7 @@ const char* hydra_last_error(void); /* text of the last CUDA error seen by this 
 /* Single-kernel entry points for kernel-level parity tests.  No context; the library makes its own
  * tensor maps.  All pointers are device pointers.
  * hydra_gemm: out[m][n] = sum_k x[m][k] * w[n][k] (float accumulate, float out), dtype as above;
- *   n % 128 == 0 and k % 64 == 0 for mode 0.  x_planes = 1: x is [m][k]; x_planes = 2 (dtype 1, mode 0 only): x is
+ *   n % 128 == 0, k % 64 == 0 and x, w on 16-byte boundaries (else INVALID) for mode 0; k % 4 == 0 and x, w on four elements else.  x_planes = 1: x is [m][k]; x_planes = 2 (dtype 1, mode 0 only): x is
  *   [2][m][k], the hi and lo bfloat16 planes of the activations, and the product uses both.  partial_dev needs
  *   hydra_gemm_partial_floats(m, n, k, dtype, mode) floats: the tensor-core GEMM leaves per-CTA partial sums
  *   there, which a second kernel adds in fixed order.  mode as in hydra_set_gemm_mode; status_dev is an int32
@@ -229,8 +231,8 @@ const char* hydra_last_error(void); /* text of the last CUDA error seen by this 
  *   NULL (= tc), mask [tc] ancestor bitmasks.  Row i of sequence b sees slots < pos0[b] and slot pos0[b]+j when bit j
  *   of mask[i] is set; mask NULL (dtype 1 only) means a causal chunk: slot pos0[b]+j is visible when j <= i.
  *   dtype 0: q, caches and out [rows][n_heads*head_dim] are float, tc <= 64, scratch_dev needs
- *   hydra_attention_scratch_bytes(...) bytes, planes = out_planes = 1, status_dev unused.  dtype 1: q and the caches are
- *   float16 in `planes` planes (2: hi = f16(v), lo = f16(v - hi)), out is bfloat16 [out_planes][rows][n_heads*head_dim]
+ *   hydra_attention_scratch_bytes(...) bytes, planes = out_planes = 1, status_dev unused.  dtype 1: q and the caches (16-byte boundaries, else
+ *   INVALID) are float16 in `planes` planes (2: hi = f16(v), lo = f16(v - hi)), out is bfloat16 [out_planes][rows][n_heads*head_dim]
  *   (2: hi = bf16(v) and lo = bf16(v - hi)); tc <= 64 with a mask, <= 128 causal; scratch_dev unused (may be NULL); status_dev is an int32 status word (bit 2: a bounded wait ran out). */
 size_t hydra_gemm_partial_floats(int m, int n, int k, int dtype, int mode);
 hydra_status hydra_gemm(const void* x_dev, const void* w_dev, float* out_dev, float* partial_dev, int m, int n, int k,

@@ -533,6 +533,11 @@ hydra_status hydra_create(hydra_ctx** out, const hydra_model_cfg* m, const hydra
   if (th.K > 0 && h->n_mlp_layers > 1 && (!w->head_wr || (h->has_bias && !w->head_br))) return HYDRA_ERR_INVALID;
   if (h->prefix_attn && (!w->pfx_attn_norm || !w->pfx_wqkv || !w->pfx_wo || !w->pfx_ffn_norm || !w->pfx_w_gate_up || !w->pfx_w_down))
     return HYDRA_ERR_INVALID;
+  // read four elements at a time
+  auto off4 = [&](const void* p) { return ((uintptr_t)p & (m->dtype == 0 ? 15 : 7)) != 0; };
+  if (off4(w->embed) || off4(w->final_norm)) return HYDRA_ERR_INVALID;
+  for (int l = 0; l < m->n_layers; ++l) if (off4(w->attn_norm[l]) || off4(w->ffn_norm[l])) return HYDRA_ERR_INVALID;
+  if (h->prefix_attn && (off4(w->pfx_attn_norm) || off4(w->pfx_ffn_norm))) return HYDRA_ERR_INVALID;
   if (m->dtype == 1 && !gemm_tc_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
   hydra_ctx* c = new (std::nothrow) hydra_ctx();
   if (!c) return HYDRA_ERR_INVALID;

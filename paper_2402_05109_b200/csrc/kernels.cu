@@ -118,6 +118,7 @@ static void launch_gemm_simt(const void* x, const void* w, float* out, int m, in
 }
 hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, bool w_const, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0 || (k & 3)) return HYDRA_ERR_UNSUPPORTED;
+  if (((uintptr_t)x | (uintptr_t)w) & (dtype == 0 ? 15 : 7)) return HYDRA_ERR_INVALID;      // both are read four elements at a time
   auto rows = [&](auto zero) {
     typedef decltype(zero) T;
     if (m == 1) launch_gemm_simt<T, 1>(x, w, out, m, n, k, w_const, st);

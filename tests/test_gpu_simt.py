@@ -35,3 +35,14 @@ def test_chained_calls_read_the_first_ones_result(m, n, k):
             assert lib.hydra_gemm(a.data_ptr(), b.data_ptr(), c.data_ptr(), part.data_ptr(), mm, nn, kk, 0, 0, 1, None, _stream()) == 0
         # two float products in a row: k^0.5 and n^0.5 ulp on the scale of the largest sum
         assert float((out.double() - ref).abs().max()) <= 2e-5 * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_operands_off_a_boundary_of_four_elements_are_refused(dtype):
+    from paper_2402_05109_b200 import HydraError, gemm
+    buf = torch.zeros(8 * 64 + 4, dtype=dtype, device="cuda")
+    good, off = buf[:8 * 64].view(8, 64), buf[1:1 + 8 * 64].view(8, 64)
+    assert gemm(good, good, mode=1).shape == (8, 8)
+    for x, w in ((off, good), (good, off)):
+        with pytest.raises(HydraError, match="invalid"):
+            gemm(x, w, mode=1)

@@ -44,3 +44,33 @@ def test_current_stream_without_the_private_torch_function(monkeypatch):
     assert binding._stream() == 103
     monkeypatch.setattr(binding, "_raw_stream", None)
     assert binding._stream() == 7
+
+
+def test_weights_off_a_boundary_of_four_elements_are_refused():
+    """The checks come before anything touches the device: made-up addresses do on a machine without a GPU."""
+    import ctypes as C
+    import pytest
+    import torch
+    from paper_2402_05109_b200.binding import lib, HeadCfgC, ModelCfgC, TreeCfgC, WeightsC, _PP
+    if torch.cuda.is_available():
+        pytest.skip("with a GPU the good call would go on to the device")
+    L, K = 2, 1
+    mc, hc = ModelCfgC(L, 256, 4, 64, 688, 1024, 1e-6, 1e4, 0, 1, 128), HeadCfgC(K, 1, 1, 0)
+    tc = TreeCfgC(2, (C.c_int32 * 2)(-1, 0))
+    arrays = ("attn_norm", "wqkv", "wo", "ffn_norm", "w_gate_up", "w_down", "head_w1", "head_b1", "head_wr", "head_br")
+
+    def create(name=None, off=0):
+        w, keep = WeightsC(), []
+        for f, _ in WeightsC._fields_:
+            at = 0x10000 + (off if f == name else 0)
+            if f in arrays:
+                keep.append((C.c_void_p * L)(0x10000, at))
+                setattr(w, f, C.cast(keep[-1], _PP))
+            else:
+                setattr(w, f, at)
+        ctx = C.c_void_p()
+        return lib.hydra_create(C.byref(ctx), C.byref(mc), C.byref(hc), C.byref(tc), C.byref(w), 0x100000, 1 << 40)
+
+    assert create() == 5 and create("head_b1", 4) == 5                    # past the checks, as far as the missing device
+    for name in ("embed", "final_norm", "attn_norm", "ffn_norm", "pfx_attn_norm", "pfx_ffn_norm"):
+        assert create(name, 4) == 1, name

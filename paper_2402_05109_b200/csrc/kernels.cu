@@ -433,20 +433,21 @@ hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cud
 // more SMs.  What the call's earlier kernels cannot change - slot counts, lengths, row table - is read before the wait (the
 // lengths are stable within a forward call, see rope_table_kernel).
 // T: float (float model path) or float16 (bfloat16 model path: q and the caches are float16 in one or two planes).
+// first = 1: the projection has no q columns (a layer of which only the cache rows are wanted).
 template <typename T>
 __global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, SplitDesc sd,
                                                              const float2* table, T* __restrict__ q, size_t q_ps,
                                                              T* __restrict__ kc, T* __restrict__ vc, size_t kv_ps,
-                                                             RowSet rs, int H, int hd, int max_seq,
+                                                             RowSet rs, int H, int hd, int max_seq, int first,
                                                              int* status) {
   pdl_trigger();
-  const int r = blockIdx.x, which = blockIdx.z;
-  const int d = H * hd, half = hd >> 1;
+  const int r = blockIdx.x, which = blockIdx.z + first;
+  const int d = H * hd, half = hd >> 1, cols = (3 - first) * d;
   const int tph = half >> 2;                                       // threads per head
   const int h = blockIdx.y * (blockDim.x / tph) + threadIdx.x / tph;
   const int j = (threadIdx.x % tph) * 4;
-  const int c0 = which * d + h * hd + j;
-  const size_t off[2] = {(size_t)r * 3 * d + c0, (size_t)r * 3 * d + c0 + half};
+  const int c0 = blockIdx.z * d + h * hd + j;
+  const size_t off[2] = {(size_t)r * cols + c0, (size_t)r * cols + c0 + half};
   const int ns[2] = {split_count(sd, r, c0), split_count(sd, r, c0 + half)};
   int b, slot;
   bool live = h < H;
@@ -462,7 +463,7 @@ __global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, 
   const bool in_range = slot >= 0 && slot < max_seq;
   pdl_wait();
   if (!live) return;
-  if (!in_range) { if (threadIdx.x == 0 && blockIdx.y == 0 && which == 0) atomicOr(status, ST_BOUNDS); return; }
+  if (!in_range) { if (threadIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) atomicOr(status, ST_BOUNDS); return; }
   const float4 t01 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j);        // (cos, sin) of j, j+1
   const float4 t23 = *reinterpret_cast<const float4*>(table + (size_t)r * half + j + 2);    // (cos, sin) of j+2, j+3
   float4 v2[2];
@@ -481,16 +482,17 @@ __global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, 
   put4h<T>(dst + j + half, ps, v2[1]);
 }
 hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table, void* q, size_t q_ps, void* kcache, void* vcache,
-                            size_t kv_ps, RowSet rs, int H, int hd, int max_seq, int dtype, int* status, cudaStream_t st) {
+                            size_t kv_ps, RowSet rs, int H, int hd, int max_seq, int dtype, bool kv_only, int* status, cudaStream_t st) {
+  const int first = kv_only ? 1 : 0;
   if (hd % 8 || 128 % (hd / 8)) return HYDRA_ERR_UNSUPPORTED;
   const int heads_per_block = 128 / (hd / 8);
-  dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block, 3);
+  dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block, 3 - first);
   if (dtype == 0)
     launch_pdl(qkv_rope_store_kernel<float>, grid, dim3(128), 0, st, part, sd, table, (float*)q, q_ps, (float*)kcache, (float*)vcache,
-               kv_ps, rs, H, hd, max_seq, status);
+               kv_ps, rs, H, hd, max_seq, first, status);
   else
     launch_pdl(qkv_rope_store_kernel<__half>, grid, dim3(128), 0, st, part, sd, table, (__half*)q, q_ps, (__half*)kcache, (__half*)vcache,
-               kv_ps, rs, H, hd, max_seq, status);
+               kv_ps, rs, H, hd, max_seq, first, status);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

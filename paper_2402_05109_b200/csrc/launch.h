@@ -42,9 +42,10 @@ hydra_status residual_rmsnorm(const float* res, const float* part, SplitDesc sd,
 // table[r][j] = (cos, sin) of (pos0[b]+depth[i]) * theta^(-2j/head_dim), evaluated in double
 hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cudaStream_t st);
 // q ([rows][H][hd], rotated) and the K/V cache rows (rotated K) from the QKV partial sums; float for dtype 0; for dtype 1
-// float16 with a lo plane (f16(v - f16(v))) q_ps / kv_ps elements after the hi plane (0: hi only).
+// float16 with a lo plane (f16(v - f16(v))) q_ps / kv_ps elements after the hi plane (0: hi only).  kv_only: the projection has the
+// 2 d columns of K and V, q is not written.
 hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table, void* q, size_t q_ps, void* kcache, void* vcache,
-                            size_t kv_ps, RowSet rs, int n_heads, int head_dim, int max_seq, int dtype, int* status, cudaStream_t st);
+                            size_t kv_ps, RowSet rs, int n_heads, int head_dim, int max_seq, int dtype, bool kv_only, int* status, cudaStream_t st);
 // Float model path: SIMT kernel + combine kernel, partial rows of ATT_CHUNK_ROWS-row chunks in `scratch`
 // (attention_scratch_bytes).  q, caches and out are float.
 constexpr int ATT_CHUNK_ROWS = 128;

@@ -648,7 +648,7 @@ __global__ void tree_attn_combine_kernel(const float* part_o, const float* part_
 // 16 rows x 4 heads x 48..80 slots: 11.7 us with the kernel above (one row per warp), 2.8 us so (tiny float model, 8 steps: 1013 -> 872 us).
 constexpr int ATT_BATCH = 4;
 constexpr int ATT_FEW_KEYS = 512;
-template <int HD, int R>
+template <int HD, int R, bool VEC>
 __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const float* q, const float* kc, const float* vc, RowSet rs, float* __restrict__ out,
                                                                       int H, int max_seq) {
   pdl_trigger();
@@ -666,7 +666,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const flo
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const bool live = r0 + r < nr;
-    qv[r] = live ? *reinterpret_cast<const float4*>(q + (size_t)(b * rs.tc + r0 + r) * d + h * HD + dim) : make_float4(0.f, 0.f, 0.f, 0.f);
+    qv[r] = live ? load4_at<VEC>(q + (size_t)(b * rs.tc + r0 + r) * d + h * HD + dim) : make_float4(0.f, 0.f, 0.f, 0.f);
     qv[r].x *= scale; qv[r].y *= scale; qv[r].z *= scale; qv[r].w *= scale;
     msk[r] = live ? rs.mask[r0 + r] : 0ull;
     o[r] = make_float4(0.f, 0.f, 0.f, 0.f); m[r] = -INFINITY; l[r] = 0.f;
@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const flo
     for (int u = 0; u < ATT_BATCH; ++u) {
       const int slot = s0 + u * ATT_WARPS * KPW;
       kv[u] = vv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (slot < total) { kv[u] = *reinterpret_cast<const float4*>(kc + base + (size_t)slot * HD); vv[u] = *reinterpret_cast<const float4*>(vc + base + (size_t)slot * HD); }
+      if (slot < total) { kv[u] = load4_at<VEC>(kc + base + (size_t)slot * HD); vv[u] = load4_at<VEC>(vc + base + (size_t)slot * HD); }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -773,17 +773,20 @@ static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSe
   // Short caches: the keys of a row shared out over the warps of a CTA, with the fewest rows a CTA that leave two CTAs per SM.  A CTA reads all keys
   // of its pair and its chain grows with them (one chunk per CTA and the combine kernel do not: 16 rows, 4 heads: 80, 256, 512 keys 3.9, 5.9, 9.4 us
   // against 7.3, 12.2, 11.7).  Four rows a CTA pay from the second chunk on (128 rows, 80 keys: 8.1 against 7.4; 256 keys: 13.7 against 20.0).
-  if (on_vec4(q) && on_vec4(kc) && on_vec4(vc) && len_upper <= ATT_FEW_KEYS) {
+  // (The stand-alone call takes operands on any element boundary; loads of one element then, the same sums.)
+  const bool vec = on_vec4(q) && on_vec4(kc) && on_vec4(vc);
+  if (len_upper <= ATT_FEW_KEYS) {
     const long pairs = (long)H * rs.batch;
-    auto go = [&](auto kernel, int R) { launch_pdl(kernel, dim3(H, rs.batch, (rs.tc + R - 1) / R), dim3(ATT_WARPS * 32), 0, st, q, kc, vc, rs, out, H, max_seq); };
+    auto go = [&](auto kernel, auto scalar, int R) {
+      launch_pdl(vec ? kernel : scalar, dim3(H, rs.batch, (rs.tc + R - 1) / R), dim3(ATT_WARPS * 32), 0, st, q, kc, vc, rs, out, H, max_seq);
+    };
     const int R = pairs * rs.tc <= cap ? 1 : pairs * ((rs.tc + 1) / 2) <= cap ? 2 : len_upper > ATT_CHUNK && pairs * ((rs.tc + 3) / 4) <= 2 * cap ? 4 : 0;
-    if (R == 1) go(tree_attn_few_kernel<HD, 1>, 1);
-    if (R == 2) go(tree_attn_few_kernel<HD, 2>, 2);
-    if (R == 4) go(tree_attn_few_kernel<HD, 4>, 4);
+    if (R == 1) go(tree_attn_few_kernel<HD, 1, true>, tree_attn_few_kernel<HD, 1, false>, 1);
+    if (R == 2) go(tree_attn_few_kernel<HD, 2, true>, tree_attn_few_kernel<HD, 2, false>, 2);
+    if (R == 4) go(tree_attn_few_kernel<HD, 4, true>, tree_attn_few_kernel<HD, 4, false>, 4);
     if (R) { HYDRA_LAUNCH_CHECK(); return HYDRA_OK; }
   }
-  // the stand-alone call takes operands on any element boundary: loads of one element then (the rows of a warp do not change a result)
-  if (!on_vec4(q) || !on_vec4(kc) || !on_vec4(vc)) HYDRA_TRY((launch_tree_attn<T, HD, 8, false>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
+  if (!vec) HYDRA_TRY((launch_tree_attn<T, HD, 8, false>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else if (ctas1 <= cap) HYDRA_TRY((launch_tree_attn<T, HD, 1>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else if (ctas1 <= 2 * cap) HYDRA_TRY((launch_tree_attn<T, HD, 2>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else HYDRA_TRY((launch_tree_attn<T, HD, 8>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));

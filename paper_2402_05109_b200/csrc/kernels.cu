@@ -919,14 +919,14 @@ __global__ void __launch_bounds__(256) topk_stage1_kernel(const float* part, Spl
 // One warp per winner list; dynamic shared memory: nblk * c (value, index) pairs.
 __global__ void __launch_bounds__(32) topk_stage2_kernel(const float* cand_v, const int* cand_i,
                                                          int nblk, int c, LevelDesc lv, const int* __restrict__ first_child,
-                                                         const int* __restrict__ n_child, int* __restrict__ out, int T, int cand_div) {
+                                                         const int* __restrict__ n_child, int* __restrict__ out, int T, int row0, int cand_div) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ float s_cand[];
   float* sv = s_cand;
   int* si = reinterpret_cast<int*>(s_cand + nblk * c);
   const int row = blockIdx.x, lane = threadIdx.x;
-  const int crow = row / cand_div;                         // row of the candidate lists (one per sequence when the parents share them)
+  const int crow = row0 + row / cand_div;                  // row of the candidate lists (one per sequence when the parents share them)
   int* dst = out + row;
   int count = 1;
   if (lv.parents) {
@@ -964,33 +964,44 @@ size_t topk_scratch_bytes(int rows, int vocab) {
   return (size_t)rows * nblk * TOPK_MAX * (sizeof(float) + sizeof(int));
 }
 
-// rows: logits rows (stage 1); out_rows: winner lists (stage 2), out_rows / rows of them per logits row
-static hydra_status topk_rows(const float* part, SplitDesc sd, float* logits_out, void* scratch, int rows_cap, int rows, int out_rows, int vocab,
-                              int c, LevelDesc lv, const int* first_child, const int* n_child, int* out, int T, cudaStream_t st) {
-  if (c < 1 || c > TOPK_MAX || rows > rows_cap || rows < 1 || out_rows % rows) return HYDRA_ERR_UNSUPPORTED;
-  const int nblk = (vocab + TOPK_SPAN - 1) / TOPK_SPAN;
-  const size_t merge_bytes = (size_t)nblk * c * 8;         // stage 2 keeps every candidate of a row in shared memory
-  if (nblk > 32 * TOPK_LISTS_PER_LANE || merge_bytes > 48 * 1024) return HYDRA_ERR_UNSUPPORTED;
-  float* cand_v = (float*)scratch;
-  int* cand_i = (int*)(cand_v + (size_t)rows_cap * nblk * TOPK_MAX);
-  launch_pdl(topk_stage1_kernel, dim3(rows, nblk), dim3(256), 0, st, part, sd, logits_out, cand_v, cand_i, vocab, c);
-  HYDRA_LAUNCH_CHECK();
-  launch_pdl(topk_stage2_kernel, dim3(out_rows), dim3(32), merge_bytes, st, (const float*)cand_v, (const int*)cand_i, nblk, c, lv, first_child, n_child, out, T,
-             out_rows / rows);
-  HYDRA_LAUNCH_CHECK();
-  return HYDRA_OK;
+struct TopkPlan { int nblk; float* cand_v; int* cand_i; };
+static bool topk_plan(void* scratch, int rows_cap, int rows, int vocab, int c, TopkPlan* p) {
+  if (c < 1 || c > TOPK_MAX || rows > rows_cap || rows < 1) return false;
+  p->nblk = (vocab + TOPK_SPAN - 1) / TOPK_SPAN;
+  if (p->nblk > 32 * TOPK_LISTS_PER_LANE || (size_t)p->nblk * c * 8 > 48 * 1024) return false;      // stage 2 keeps every candidate of a row in shared memory
+  p->cand_v = (float*)scratch;
+  p->cand_i = (int*)(p->cand_v + (size_t)rows_cap * p->nblk * TOPK_MAX);
+  return true;
 }
 
 hydra_status argmax_rows(const float* part, SplitDesc sd, float* logits_out, int* amax, void* scratch, int rows_cap, int rows,
                          int vocab, cudaStream_t st) {
-  return topk_rows(part, sd, logits_out, scratch, rows_cap, rows, rows, vocab, 1, LevelDesc{0, 0, nullptr}, nullptr, nullptr, amax, 0, st);
+  TopkPlan p;
+  if (!topk_plan(scratch, rows_cap, rows, vocab, 1, &p)) return HYDRA_ERR_UNSUPPORTED;
+  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits_out, p.cand_v, p.cand_i, vocab, 1);
+  HYDRA_LAUNCH_CHECK();
+  launch_pdl(topk_stage2_kernel, dim3(rows), dim3(32), (size_t)p.nblk * 8, st, (const float*)p.cand_v, (const int*)p.cand_i, p.nblk, 1, LevelDesc{0, 0, nullptr},
+             (const int*)nullptr, (const int*)nullptr, amax, 0, 0, 1);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
 }
 
-hydra_status topk_children(const float* part, SplitDesc sd, float* logits, LevelDesc lv, int max_children, const int* first_child,
-                           const int* n_child, int* tree_tok, void* scratch, int rows_cap, int batch, int T, int vocab, int shared_rows,
-                           cudaStream_t st) {
-  return topk_rows(part, sd, logits, scratch, rows_cap, shared_rows ? batch : batch * lv.n_parents, batch * lv.n_parents, vocab, max_children, lv,
-                   first_child, n_child, tree_tok, T, st);
+hydra_status topk_candidates(const float* part, SplitDesc sd, float* logits, int max_children, void* scratch, int rows_cap, int rows, int vocab, cudaStream_t st) {
+  TopkPlan p;
+  if (!topk_plan(scratch, rows_cap, rows, vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
+  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits, p.cand_v, p.cand_i, vocab, max_children);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
+}
+
+hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int row0,
+                        int batch, int T, int vocab, int shared_rows, cudaStream_t st) {
+  TopkPlan p;
+  if (!topk_plan(scratch, rows_cap, row0 + (shared_rows ? batch : batch * lv.n_parents), vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
+  launch_pdl(topk_stage2_kernel, dim3(batch * lv.n_parents), dim3(32), (size_t)p.nblk * max_children * 8, st, (const float*)p.cand_v, (const int*)p.cand_i, p.nblk,
+             max_children, lv, first_child, n_child, tree_tok, T, row0, shared_rows ? lv.n_parents : 1);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -133,7 +133,10 @@ hydra_status hydra_draft(hydra_ctx*, int32_t* tree_tok_dev, void* stream);
  * row i land in cache slot len+i, its rotary position is len+depth(i).  amax_dev [batch][n_rows] int32 out:
  * argmax of each row's logits (ties: lowest id).  logits_dev [batch][n_rows][vocab] float out, or NULL.
  * tree_tok_dev [batch][n_rows] int32 in; the caller may have edited it since hydra_draft.  A token id outside
- * [0, vocab) raises the BOUNDS bit of the status word (the row is computed for token 0).  Errors: STATE, CAPACITY. */
+ * [0, vocab) raises the BOUNDS bit of the status word (the row is computed for token 0).  From the second call of the context on, the
+ * forward pass is captured into a CUDA graph (again for another batch or attention grid; up to eight are kept) and replayed, on the streams and under
+ * the switch described at hydra_step; the pointers may change freely, and a stream that the caller is capturing gets the launches themselves.
+ * Errors: STATE, CAPACITY. */
 hydra_status hydra_verify(hydra_ctx*, const int32_t* tree_tok_dev, int32_t* amax_dev, float* logits_dev, void* stream);
 
 /* Acceptance and compaction (Background, verification criteria: the greedy criterion keeps a candidate
@@ -153,7 +156,7 @@ hydra_status hydra_accept_compact(hydra_ctx*, const int32_t* tree_tok_dev, const
  * acceptance criterion or the GEMM mode changes; n_acc_dev and out_tok_dev may change freely) and replayed with one launch, unless the stream
  * is a default stream (not capturable) or hydra_set_step_graph switched graphs off.  Errors: STATE, CAPACITY. */
 hydra_status hydra_step(hydra_ctx*, int32_t* n_acc_dev, int32_t* out_tok_dev, void* stream);
-/* on = 0: hydra_step launches kernel by kernel (for profilers that list kernels); on = 1 (default): graph replay. */
+/* on = 0: hydra_step and hydra_verify launch kernel by kernel (for profilers that list kernels); on = 1 (default): graph replay. */
 hydra_status hydra_set_step_graph(hydra_ctx*, int on);
 
 /* Acceptance criterion.  mode 0 (default): greedy, as described at hydra_accept_compact.  mode 1: typical acceptance

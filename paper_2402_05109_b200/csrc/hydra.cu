@@ -111,6 +111,11 @@ struct hydra_ctx {
   };
   struct StepGraph { cudaGraph_t graph; cudaGraphExec_t exec; cudaGraphNode_t accept; AcceptArgs args; long long launches; };
   std::map<GraphKey, StepGraph> graphs;
+  // verifications of the caller's candidates: everything up to the vocabulary projection, from a copy of the tokens (the caller's pointers
+  // are arguments of the launches around it), keyed by batch and attention grid size
+  struct RowsGraph { cudaGraph_t graph; cudaGraphExec_t exec; SplitDesc sd; long long launches; };
+  std::map<std::pair<int, int>, RowsGraph> rows_graphs;
+  long long verifies_done;
   int use_graph; long long steps_done;
   int timing;
   std::vector<Timed> timed;
@@ -484,17 +489,24 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
   return HYDRA_OK;
 }
 
-hydra_status do_verify(hydra_ctx* c, const int* tree_tok, int* amax, float* logits, cudaStream_t st) {
+// Base model over the candidate rows, up to the partial sums of the vocabulary projection (*sd) in c->part.
+hydra_status verify_rows(hydra_ctx* c, const int* tree_tok, SplitDesc* sd, cudaStream_t st) {
+  RowSet rs{c->batch, c->T, nullptr, c->d_len, c->d_depth, c->d_anc};
+  return run_base(c, tree_tok, rs, len_bucket(c, max_len_ub(c) + c->T), c->lm_head, c->m.vocab, sd, true, st);
+}
+hydra_status verify_results(hydra_ctx* c, const SplitDesc& sd, int* amax, float* logits, cudaStream_t st) {
   const hydra_model_cfg& m = c->m;
   const int rows = c->batch * c->T;
-  RowSet rs{c->batch, c->T, nullptr, c->d_len, c->d_depth, c->d_anc};
-  SplitDesc sd;
-  HYDRA_TRY(run_base(c, tree_tok, rs, len_bucket(c, max_len_ub(c) + c->T), c->lm_head, m.vocab, &sd, true, st));
   if (c->acc_mode == 1 && !logits) logits = c->logits;              // the typical criterion reads whole rows of logits
   c->last_logits = logits;
   HYDRA_TRY(argmax_rows(c->part, sd, logits, amax, c->topk_scratch, c->topk_rows_cap, rows, m.vocab, st));
   if (c->acc_mode == 1) HYDRA_TRY(softmax_row_stats(logits, c->d_row_stats, rows, m.vocab, c->acc_tau, st));
   return HYDRA_OK;
+}
+hydra_status do_verify(hydra_ctx* c, const int* tree_tok, int* amax, float* logits, cudaStream_t st) {
+  SplitDesc sd;
+  HYDRA_TRY(verify_rows(c, tree_tok, &sd, st));
+  return verify_results(c, sd, amax, logits, st);
 }
 
 AcceptArgs accept_args(const hydra_ctx* c, const int* tree_tok, const int* amax, int* n_acc, int* path, int* out_tok) {
@@ -533,6 +545,29 @@ hydra_status enqueue_step(hydra_ctx* c, int* n_acc, int* out_tok, cudaStream_t s
 void drop_graphs(hydra_ctx* c) {
   for (auto& g : c->graphs) { cudaGraphExecDestroy(g.second.exec); cudaGraphDestroy(g.second.graph); }
   c->graphs.clear();
+  for (auto& g : c->rows_graphs) { cudaGraphExecDestroy(g.second.exec); cudaGraphDestroy(g.second.graph); }
+  c->rows_graphs.clear();
+}
+
+bool capturable(cudaStream_t st) { return st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread; }      // default streams are not
+bool being_captured(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &s) != cudaSuccess || s != cudaStreamCaptureStatusNone;
+}
+// What `enqueue` puts on the stream, as a graph and not executed; *launches: kernels in it.
+template <typename F>
+hydra_status capture(hydra_ctx* c, cudaStream_t st, F enqueue, cudaGraph_t* out, long long* launches) {
+  const long long before = c->launches;
+  HYDRA_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  const hydra_status es = enqueue();
+  cudaGraph_t graph = nullptr;
+  const cudaError_t ce = cudaStreamEndCapture(st, &graph);
+  *launches = c->launches - before;
+  c->launches = before;
+  if (es != HYDRA_OK) { if (graph) cudaGraphDestroy(graph); return es; }
+  if (ce != cudaSuccess) { set_last_error("cudaStreamEndCapture", ce); return HYDRA_ERR_CUDA; }
+  *out = graph;
+  return HYDRA_OK;
 }
 
 bool capacity_ok(const hydra_ctx* c) {
@@ -597,7 +632,7 @@ hydra_status hydra_create(hydra_ctx** out, const hydra_model_cfg* m, const hydra
   c->embed = w->embed; c->lm_head = w->lm_head; c->final_norm = w->final_norm;
   const size_t need = carve(c, *m, *h, th, (char*)ws);
   if (ws_bytes < need) { delete c; return HYDRA_ERR_CAPACITY; }
-  c->batch = 0; c->state = ST_CREATED; c->gemm_mode = 0; c->plant = nullptr; c->launches = 0; c->timing = 0; c->steps_done = 0;
+  c->batch = 0; c->state = ST_CREATED; c->gemm_mode = 0; c->plant = nullptr; c->launches = 0; c->timing = 0; c->steps_done = 0; c->verifies_done = 0;
   c->use_graph = 1;
   c->acc_mode = 0; c->acc_tau = 1.f; c->acc_eps = 0.f; c->acc_alpha = 0.f; c->acc_u = nullptr; c->last_logits = nullptr;
   c->len_ub.assign(m->max_batch, 0);
@@ -692,7 +727,28 @@ hydra_status hydra_verify(hydra_ctx* c, const int32_t* tree_tok, int32_t* amax, 
   if (c->state != ST_READY && c->state != ST_DRAFTED && c->state != ST_VERIFIED) return HYDRA_ERR_STATE;
   if (!capacity_ok(c)) return HYDRA_ERR_CAPACITY;
   CounterScope cs(c);
-  HYDRA_TRY(do_verify(c, tree_tok, amax, logits, (cudaStream_t)stream));
+  cudaStream_t st = (cudaStream_t)stream;
+  // the first one runs uncaptured (one-time lazy set-up); a stream that its owner is capturing takes the launches themselves
+  if (!c->use_graph || !capturable(st) || c->timing || c->verifies_done == 0 || being_captured(st)) {
+    HYDRA_TRY(do_verify(c, tree_tok, amax, logits, st));
+  } else {
+    // (launched kernel by kernel, 47 rows of the 7B shape behind 700 tokens: 3.542 ms, replayed 3.452)
+    const std::pair<int, int> key(c->batch, len_bucket(c, max_len_ub(c) + c->T));
+    auto it = c->rows_graphs.find(key);
+    if (it == c->rows_graphs.end()) {
+      if (c->rows_graphs.size() >= 8) drop_graphs(c);
+      hydra_ctx::RowsGraph g{};
+      HYDRA_TRY(capture(c, st, [&]() { return verify_rows(c, c->d_tok, &g.sd, st); }, &g.graph, &g.launches));
+      const cudaError_t ce = cudaGraphInstantiate(&g.exec, g.graph, 0);
+      if (ce != cudaSuccess) { cudaGraphDestroy(g.graph); set_last_error("cudaGraphInstantiate", ce); return HYDRA_ERR_CUDA; }
+      it = c->rows_graphs.emplace(key, g).first;
+    }
+    HYDRA_TRY(copy_i32(c->d_tok, tree_tok, c->batch * c->T, st));
+    HYDRA_CUDA(cudaGraphLaunch(it->second.exec, st));
+    c->launches += it->second.launches;
+    HYDRA_TRY(verify_results(c, it->second.sd, amax, logits, st));
+  }
+  ++c->verifies_done;
   c->state = ST_VERIFIED;
   return HYDRA_OK;
 }
@@ -714,8 +770,7 @@ hydra_status hydra_step(hydra_ctx* c, int32_t* n_acc, int32_t* out_tok, void* st
   if (!capacity_ok(c)) return HYDRA_ERR_CAPACITY;
   CounterScope cs(c);
   cudaStream_t st = (cudaStream_t)stream;
-  const bool capturable = st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread;   // default streams cannot be captured
-  if (!c->use_graph || !capturable || c->timing || c->steps_done == 0) {      // the first step runs uncaptured (one-time lazy set-up)
+  if (!c->use_graph || !capturable(st) || c->timing || c->steps_done == 0) {      // the first step runs uncaptured (one-time lazy set-up)
     HYDRA_TRY(enqueue_step(c, n_acc, out_tok, st));
   } else {
     const int lu = max_len_ub(c);
@@ -723,18 +778,12 @@ hydra_status hydra_step(hydra_ctx* c, int32_t* n_acc, int32_t* out_tok, void* st
     auto it = c->graphs.find(key);
     if (it == c->graphs.end()) {
       if (c->graphs.size() >= 8) drop_graphs(c);
-      const long long before = c->launches;
-      HYDRA_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-      hydra_status es = enqueue_step(c, n_acc, out_tok, st);
       cudaGraph_t graph = nullptr;
-      cudaError_t ce = cudaStreamEndCapture(st, &graph);
-      const long long captured = c->launches - before;
-      c->launches = before;
-      if (es != HYDRA_OK) { if (graph) cudaGraphDestroy(graph); return es; }
-      if (ce != cudaSuccess) { set_last_error("cudaStreamEndCapture", ce); return HYDRA_ERR_CUDA; }
+      long long captured = 0;
+      HYDRA_TRY(capture(c, st, [&]() { return enqueue_step(c, n_acc, out_tok, st); }, &graph, &captured));
       cudaGraphExec_t exec = nullptr;
       cudaGraphNode_t accept = nullptr;
-      ce = accept_graph_node(graph, &accept);
+      cudaError_t ce = accept_graph_node(graph, &accept);
       if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
       if (ce != cudaSuccess) { cudaGraphDestroy(graph); set_last_error("cudaGraphInstantiate", ce); return HYDRA_ERR_CUDA; }
       it = c->graphs.emplace(key, hydra_ctx::StepGraph{graph, exec, accept, accept_args(c, c->d_tree_tok, c->d_amax, n_acc, nullptr, out_tok), captured}).first;

@@ -483,8 +483,8 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
                           K + 1, d, m.vocab, dt, c->d_status, st));
     HYDRA_TRY(head_mlp(lvl, rows, lv.n_parents, lvl + 1, 0));
     HYDRA_TRY(run_gemm(c, c->yb, c->RH, c->lm_head, rows, m.vocab, d, &sd, st));
-    HYDRA_TRY(topk_candidates(c->part, sd, c->head_logits, max_children, c->topk_scratch, c->topk_rows_cap, rows, m.vocab, st));
-    HYDRA_TRY(topk_merge(lv, max_children, c->d_first_child, c->d_n_child, tree_tok, c->topk_scratch, c->topk_rows_cap, 0, B, c->T, m.vocab, 0, st));
+    HYDRA_TRY(topk_children(c->part, sd, c->head_logits, lv, max_children, c->d_first_child, c->d_n_child, tree_tok, c->topk_scratch, c->topk_rows_cap,
+                            B, c->T, m.vocab, st));
   }
   return HYDRA_OK;
 }

@@ -854,9 +854,11 @@ constexpr int TOPK_SPAN = 2048;           // columns per stage-1 block (8 per th
 constexpr int TOPK_MAX = 64;              // a tree node has at most 63 children
 constexpr int TOPK_LISTS_PER_LANE = 4;    // stage 2: at most 128 column blocks (262144 tokens)
 
+// out (a vocabulary of one column block): the block's list is the row's, and the winners go where stage 2 would have put them.
 __global__ void __launch_bounds__(256) topk_stage1_kernel(const float* part, SplitDesc sd,
                                                           float* __restrict__ logits_out, float* __restrict__ cand_v,
-                                                          int* __restrict__ cand_i, int vocab, int c) {
+                                                          int* __restrict__ cand_i, int vocab, int c, LevelDesc lv, const int* __restrict__ first_child,
+                                                          const int* __restrict__ n_child, int* __restrict__ out, int T) {
   pdl_trigger();
   __shared__ float wv[8][TOPK_MAX];
   __shared__ int wi[8][TOPK_MAX];
@@ -900,15 +902,21 @@ __global__ void __launch_bounds__(256) topk_stage1_kernel(const float* part, Spl
   }
   __syncthreads();
   if (warp == 0) {                                         // merge: lane w < 8 walks warp w's list
-    int ptr = 0;
-    for (int t = 0; t < c; ++t) {
+    int ptr = 0, count = c;
+    int* dst = out + row;
+    if (out && lv.parents) {
+      const int p = lv.parents[row % lv.n_parents];
+      dst = out + row / lv.n_parents * T + first_child[p];
+      count = n_child[p];
+    }
+    for (int t = 0; t < count; ++t) {
       float hv = -INFINITY; int hi = 0x7fffffff;
       if (lane < 8 && ptr < c) { hv = wv[lane][ptr]; hi = wi[lane][ptr]; }
       float bv = hv; int bi = hi;
       warp_best(bv, bi);
       if (lane == 0) {
-        cand_v[((size_t)row * nblk + blk) * TOPK_MAX + t] = bv;
-        cand_i[((size_t)row * nblk + blk) * TOPK_MAX + t] = bi;
+        if (out) dst[t] = bi;
+        else { cand_v[((size_t)row * nblk + blk) * TOPK_MAX + t] = bv; cand_i[((size_t)row * nblk + blk) * TOPK_MAX + t] = bi; }
       }
       if (hi == bi && bi != 0x7fffffff) ++ptr;
     }
@@ -978,8 +986,11 @@ hydra_status argmax_rows(const float* part, SplitDesc sd, float* logits_out, int
                          int vocab, cudaStream_t st) {
   TopkPlan p;
   if (!topk_plan(scratch, rows_cap, rows, vocab, 1, &p)) return HYDRA_ERR_UNSUPPORTED;
-  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits_out, p.cand_v, p.cand_i, vocab, 1);
+  int* direct = p.nblk == 1 ? amax : nullptr;
+  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits_out, p.cand_v, p.cand_i, vocab, 1, LevelDesc{0, 0, nullptr},
+             (const int*)nullptr, (const int*)nullptr, direct, 0);
   HYDRA_LAUNCH_CHECK();
+  if (direct) return HYDRA_OK;
   launch_pdl(topk_stage2_kernel, dim3(rows), dim3(32), (size_t)p.nblk * 8, st, (const float*)p.cand_v, (const int*)p.cand_i, p.nblk, 1, LevelDesc{0, 0, nullptr},
              (const int*)nullptr, (const int*)nullptr, amax, 0, 0, 1);
   HYDRA_LAUNCH_CHECK();
@@ -989,9 +1000,25 @@ hydra_status argmax_rows(const float* part, SplitDesc sd, float* logits_out, int
 hydra_status topk_candidates(const float* part, SplitDesc sd, float* logits, int max_children, void* scratch, int rows_cap, int rows, int vocab, cudaStream_t st) {
   TopkPlan p;
   if (!topk_plan(scratch, rows_cap, rows, vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
-  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits, p.cand_v, p.cand_i, vocab, max_children);
+  launch_pdl(topk_stage1_kernel, dim3(rows, p.nblk), dim3(256), 0, st, part, sd, logits, p.cand_v, p.cand_i, vocab, max_children, LevelDesc{0, 0, nullptr},
+             (const int*)nullptr, (const int*)nullptr, (int*)nullptr, 0);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
+}
+
+hydra_status topk_children(const float* part, SplitDesc sd, float* logits, LevelDesc lv, int max_children, const int* first_child, const int* n_child,
+                           int* tree_tok, void* scratch, int rows_cap, int batch, int T, int vocab, cudaStream_t st) {
+  TopkPlan p;
+  const int rows = batch * lv.n_parents;
+  if (!topk_plan(scratch, rows_cap, rows, vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
+  // one column block: its list is the row's, and a launch of a chain of short ones goes (tiny float model, 8 steps: 872 -> 813 us)
+  if (p.nblk == 1) {
+    launch_pdl(topk_stage1_kernel, dim3(rows, 1), dim3(256), 0, st, part, sd, logits, p.cand_v, p.cand_i, vocab, max_children, lv, first_child, n_child, tree_tok, T);
+    HYDRA_LAUNCH_CHECK();
+    return HYDRA_OK;
+  }
+  HYDRA_TRY(topk_candidates(part, sd, logits, max_children, scratch, rows_cap, rows, vocab, st));
+  return topk_merge(lv, max_children, first_child, n_child, tree_tok, scratch, rows_cap, 0, batch, T, vocab, 0, st);
 }
 
 hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int row0,

@@ -94,6 +94,10 @@ hydra_status topk_candidates(const float* part, SplitDesc sd, float* logits, int
 hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int row0,
                         int batch, int T, int vocab, int shared_rows, cudaStream_t st);
 
+// Both, for a level whose rows are its own.
+hydra_status topk_children(const float* part, SplitDesc sd, float* logits, LevelDesc lv, int max_children, const int* first_child, const int* n_child,
+                           int* tree_tok, void* scratch, int rows_cap, int batch, int T, int vocab, cudaStream_t st);
+
 // ---- acceptance + compaction (one kernel)
 struct AcceptArgs {
   const int* tree_tok; const int* amax;

@@ -222,7 +222,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int u_begin = blockIdx.x * a.q;
   const int u_end = min(u_begin + a.q, a.total_units);
-  const int n_units = u_end - u_begin, ring = n_units < stages ? n_units : stages, pre = a.w_const ? ring : 0;     // pre: weight tiles requested up front
+  const int n_units = u_end - u_begin, ring = n_units < stages ? n_units : stages, pre = a.w_const ? (ring + 1) / 2 : 0;     // pre: weight tiles requested up front
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -231,11 +231,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     mbar_init_fence();
     prefetch_tensormap(&tmW);
     prefetch_tensormap(&tmX);
-    // weights do not depend on the preceding kernel: request the first ring of weight tiles right away, before the
-    // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait; where they may, bring them nearer
+    // weights do not depend on the preceding kernel: request half a ring of weight tiles right away, before the
+    // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait; where they may, bring them nearer.
+    // (The whole ring, 29 MB over the SMs, is more than the preceding row-wise kernel's time takes in, and its loads then queue behind it: 7B
+    // shape, 32 steps without a tree 94.4 -> 93.7 ms with half, a 64-row tree 147.0 -> 145.6; all but one stage the same, one stage alone no better than the whole ring.)
     const uint64_t pol = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal();
     int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_tiles * BN;
-    for (int i = 0; i < ring; ++i) {
+    for (int i = 0; i < (a.w_const ? pre : ring); ++i) {
       if (!a.w_const) {
         tma_prefetch_2d(&tmW, kb * BLOCK_K, nrow);
       } else if (u_begin + i != a.skip_unit) {

@@ -510,6 +510,14 @@ constexpr int ATT_CHUNK = ATT_CHUNK_ROWS;
 constexpr int ATT_TILE = 64;      // KV rows staged per iteration: two keys per lane
 constexpr int ATT_WARPS = 8;
 
+// Rows and keys of sequence b: no more rows than the call has and no key past the cache, whatever the device-side lengths say.  (A row past the
+// cache is not in it: qkv_rope_store skips it and raises the status bit; the row then attends to what there is.)
+struct AttSpan { int nr, p0, total; };
+__device__ __forceinline__ AttSpan att_span(const RowSet& rs, int b, int max_seq) {
+  const int nr = min(rs.n_rows ? rs.n_rows[b] : rs.tc, rs.tc), p0 = rs.pos0[b];
+  return AttSpan{nr, p0, min(min(p0, max_seq) + nr, max_seq)};
+}
+
 template <typename T, int HD, int RPW, bool VEC>
 __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* q, const T* kc,
                                                                    const T* vc, RowSet rs,
@@ -525,9 +533,7 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* q, c
   float* vs = ks + ATT_TILE * (HD + 1);                   // [ATT_TILE][HD]
   const int h = blockIdx.x, b = blockIdx.y, c = blockIdx.z % nchunks, r0 = blockIdx.z / nchunks * ROWS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nr = rs.n_rows ? rs.n_rows[b] : rs.tc;
-  const int p0 = rs.pos0[b];
-  const int total = p0 + nr;
+  const auto [nr, p0, total] = att_span(rs, b, max_seq);
   const int s0 = c * ATT_CHUNK;
   const int s1 = min(s0 + ATT_CHUNK, total);
   const int d = H * HD;
@@ -620,15 +626,15 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_kernel(const T* q, c
 
 template <typename T, int HD>
 __global__ void tree_attn_combine_kernel(const float* part_o, const float* part_ml, RowSet rs,
-                                         T* __restrict__ out, int H, int nchunks) {
+                                         T* __restrict__ out, int H, int max_seq, int nchunks) {
   pdl_trigger();
   pdl_wait();
   const int r = blockIdx.x, h = blockIdx.y, b = r / rs.tc, i = r % rs.tc;
-  const int nr = rs.n_rows ? rs.n_rows[b] : rs.tc;
+  const auto [nr, p0, total] = att_span(rs, b, max_seq);
   const int k = threadIdx.x;
   T* dst = out + (size_t)r * H * HD + h * HD;
   if (i >= nr) { dst[k] = from_f<T>(0.f); return; }
-  const int used = min(nchunks, (rs.pos0[b] + nr + ATT_CHUNK - 1) / ATT_CHUNK);
+  const int used = min(nchunks, (total + ATT_CHUNK - 1) / ATT_CHUNK);
   size_t idx = ((size_t)r * H + h) * nchunks;
   float M = -INFINITY;
   for (int c = 0; c < used; ++c) M = fmaxf(M, part_ml[(idx + c) * 2]);
@@ -659,7 +665,8 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const flo
   __shared__ float s_m[R][ATT_WARPS], s_l[R][ATT_WARPS];
   __shared__ __align__(16) float s_o[R][ATT_WARPS][HD];
   pdl_wait();
-  const int nr = rs.n_rows ? rs.n_rows[b] : rs.tc, p0 = rs.pos0[b], total = r0 < nr ? p0 + nr : 0;
+  const auto [nr, p0, end] = att_span(rs, b, max_seq);
+  const int total = r0 < nr ? end : 0;
   const float scale = rsqrtf((float)HD);
   float4 qv[R], o[R];
   float m[R], l[R];
@@ -792,7 +799,7 @@ static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSe
   else if (ctas1 <= 2 * cap) HYDRA_TRY((launch_tree_attn<T, HD, 2>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else HYDRA_TRY((launch_tree_attn<T, HD, 8>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   if (nchunks == 1) return HYDRA_OK;
-  launch_pdl(tree_attn_combine_kernel<T, HD>, dim3(dim3((unsigned)rows, H)), dim3(HD), 0, st, part_o, part_ml, rs, out, H, nchunks);
+  launch_pdl(tree_attn_combine_kernel<T, HD>, dim3(dim3((unsigned)rows, H)), dim3(HD), 0, st, part_o, part_ml, rs, out, H, max_seq, nchunks);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

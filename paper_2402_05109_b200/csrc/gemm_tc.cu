@@ -444,13 +444,14 @@ SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t pa
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
                      SplitDesc* sd_out, bool w_const, int* status, int* diag, const GemmDebug* dbg, cudaStream_t st, size_t part_cap, float* out,
-                     const GemmArrivals* arrivals) {
+                     const GemmArrivals* arrivals, int x_row0) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
   int grid = 1;
   const SplitDesc sd = gemm_tc_plan(m, n, k, &grid, nullptr, part_cap);
   const GemmShape sh = gemm_shape(m, n, k);
-  if (x_rows_alloc < m) x_rows_alloc = m;
+  if (x_rows_alloc < x_row0 + m) x_rows_alloc = x_row0 + m;
+  x += (size_t)x_row0 * k;
   GemmArgs a{};
   a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.m_tiles = sd.m_tiles; a.mt = sd.mt;
   a.total_units = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles * sd.kb; a.q = sd.q; a.status = status;
@@ -469,7 +470,7 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   a.stages = RING_BYTES / stage_bytes < MAX_STAGES ? RING_BYTES / stage_bytes : MAX_STAGES;
   CUtensorMap tw, tx;
   if (!get_tensor_map(w, (uint64_t)n, (uint64_t)k, (uint32_t)(sh.nh * BLOCK_N), false, &tw) ||
-      !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes, (uint64_t)k, (uint32_t)sd.mt, false, &tx)) {
+      !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes - x_row0, (uint64_t)k, (uint32_t)sd.mt, false, &tx)) {      // what the buffer holds from x on; rows past it read as zeros
     set_last_error("cuTensorMapEncodeTiled", cudaErrorUnknown);
     return HYDRA_ERR_CUDA;
   }

@@ -273,19 +273,21 @@ struct TimeScope {                // brackets the launches issued during its lif
   ~TimeScope() { if (a) { cudaEventRecord(b, st); c->timed.push_back({a, b, cls, bytes}); } }
 };
 
-// Partial sums of x @ w^T into c->part; *sd says where the slots of each output tile are.
+// Partial sums of x @ w^T into c->part; *sd says where the slots of each output tile are.  The rows begin at row x_row0 of x, which is an
+// operand buffer of x_rows_alloc rows a plane.
 hydra_status run_gemm(hydra_ctx* c, const void* x, int x_rows_alloc, const void* w, int m, int n, int k, SplitDesc* sd,
-                      cudaStream_t st) {
+                      cudaStream_t st, int x_row0 = 0) {
   // algorithmic bytes of the launch: the weight matrix and the activation slab read once, the output written once
   TimeScope ts(c, HYDRA_TIME_GEMM, (double)c->esize * ((double)n * k + (double)c->planes * m * k) + 4.0 * m * n, st);
   if (c->m.dtype == 1 && c->gemm_mode != 1) {
     int slots = 1;
     gemm_tc_plan(m, n, k, nullptr, &slots);
     if ((size_t)slots * m * n > c->part_floats) return HYDRA_ERR_CAPACITY;
-    return gemm_tc((const bf16*)x, x_rows_alloc, c->planes, (const bf16*)w, c->part, m, n, k, sd, true, c->d_status, c->d_status + 8, nullptr, st);
+    return gemm_tc((const bf16*)x, x_rows_alloc, c->planes, (const bf16*)w, c->part, m, n, k, sd, true, c->d_status, c->d_status + 8, nullptr, st, 0,
+                   nullptr, nullptr, x_row0);
   }
   *sd = single_slot((size_t)m * n);
-  return gemm_simt(x, w, c->part, m, n, k, c->m.dtype, true, st);      // bfloat16: the hi plane only (debug mode)
+  return gemm_simt((const char*)x + (size_t)x_row0 * k * c->esize, w, c->part, m, n, k, c->m.dtype, true, st);      // bfloat16: the hi plane only (debug mode)
 }
 
 // element distance between the hi and lo planes of an operand buffer of `rows_alloc` rows of `cols` (0 for float)
@@ -448,7 +450,7 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     for (int l = 0; l + 1 < c->h.n_mlp_layers; ++l) {
       const char* wr = (const char*)c->head_wr[lvl - 1] + (size_t)l * d * d * c->esize;
       const char* br = c->h.has_bias ? (const char*)c->head_br[lvl - 1] + (size_t)l * d * c->esize : nullptr;
-      HYDRA_TRY(run_gemm(c, yb, c->RH, wr, rows, d, d, &sd, st));
+      HYDRA_TRY(run_gemm(c, c->yb, c->RH, wr, rows, d, d, &sd, st, y0));
       HYDRA_TRY(head_act(y, 0, rows_per_b, c->part, sd, br, y, yb, ps(c, c->RH, d), rows, d, dt, st));
     }
     return HYDRA_OK;

@@ -7,7 +7,8 @@ namespace hydra {
 // ---- GEMM: partial sums of x[m][k] * w[n][k] (see SplitDesc for where they land)
 // tcgen05 path (bfloat16 operands).  x_rows_alloc = rows the x buffer really holds (>= m); rows of the last
 // tile beyond m are computed and dropped.  part needs gemm_tc_plan(...)'s max_slots * m * n floats.
-// x holds x_planes (1 or 2) planes of x_rows_alloc rows each: plane 0 = bf16(v), plane 1 = bf16(v - plane 0).
+// x holds x_planes (1 or 2) planes of x_rows_alloc rows each: plane 0 = bf16(v), plane 1 = bf16(v - plane 0).  The m rows begin at row x_row0
+// of a plane; x itself is the buffer's beginning, so that no row behind its end is ever described to the hardware.
 // w_const: no kernel in flight writes w (the weights of a context); its first tiles are then read ahead of the preceding kernel's completion.
 // dbg (tests of the bounded waits only): a shorter poll limit and one weight-tile request that CTA 0 leaves out.
 struct GemmDebug { uint32_t wait_limit; int skip_unit; };
@@ -15,7 +16,7 @@ struct GemmArrivals { unsigned long long* count; unsigned long long ticket; };
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
                      SplitDesc* sd_out, bool w_const, int* status, int* diag /*int[8] or null*/, const GemmDebug* dbg /*null: defaults*/, cudaStream_t st,
                      size_t part_cap = 0 /*floats in part; 0: as many as the plan asks for*/,
-                     float* out = nullptr /*[m][n]: the sums themselves*/, const GemmArrivals* arrivals = nullptr /*with out: for one-launch calls*/);
+                     float* out = nullptr /*[m][n]: the sums themselves*/, const GemmArrivals* arrivals = nullptr /*with out: for one-launch calls*/, int x_row0 = 0);
 // Stand-alone calls of up to GEMM_ONE_LAUNCH_WEIGHTS weights and 16 rows add their partial sums in the GEMM's own launch (gemm_tc.cu has the
 // figures).  A counter per tile (128 columns, at least 64 k) says how many CTAs have stored it: the call's ticket in the upper 48 bits,
 // the count below.  Tickets rise from call to call, so whatever an earlier call left in a counter - one that timed out, or that another call

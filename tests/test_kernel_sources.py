@@ -27,3 +27,15 @@ def test_only_weights_and_tables_are_declared_constant():
     for body in kernel_bodies("kernels.cu"):
         constant |= set(re.findall(r"const \w+\s*\*\s*__restrict__\s+(\w+)", body[:body.index("{")]))
     assert constant <= {"embed", "gain", "bias", "first_child", "n_child", "path_tab"}
+
+
+def test_gemm_operands_are_whole_buffers():
+    """The tensor-core GEMM reads row tiles of up to 15 rows more than it is asked for, as far as the buffer that it is told of goes: operand and row
+    count of a call are those of one buffer of the workspace, and rows inside it are named by their number."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "hydra.cu")).read())
+    carved = dict(re.findall(r"auto\* (\w+) = b\.take<char>\(\(size_t\)np \* (\w+) \*", text))
+    assert {"xn", "attn_out", "act", "z", "yb"} <= set(carved)
+    calls = re.findall(r"run_gemm\(c, ([^,]+), ([^,]+),", text)
+    assert len(calls) >= 10
+    for x, rows in calls:
+        assert x.startswith("c->") and rows == "c->" + carved[x[3:]], (x, rows)

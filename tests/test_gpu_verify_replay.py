@@ -1,4 +1,4 @@
-"""hydra_verify replays a captured graph from its second call on a stream of the caller's own: other candidates, other result buffers, other
+"""hydra_verify replays a captured graph from the eighth call of a batch on a stream of the caller's own: other candidates, other result buffers, other
 prompt lengths and batches give bit for bit what launching kernel by kernel gives."""
 import pytest
 import torch
@@ -28,7 +28,7 @@ def test_replay_matches_launches(dtype, typical):
             gen = torch.Generator().manual_seed(5)
             for lens in ([70, 33], [70, 33, 1], [20, 9], [600, 1]):        # the last one needs another attention grid
                 g.prefill([p.cuda() for p in make_prompts(91, lens, m.vocab)])
-                for want in (True, True, False):
+                for want in (True, True, False) * 3:
                     cand = torch.randint(0, m.vocab, (len(lens), len(parent)), dtype=torch.int32, generator=gen).cuda()
                     res = g.verify(cand, want_logits=want)
                     amax = res[0] if want else res

@@ -134,7 +134,7 @@ hydra_status hydra_draft(hydra_ctx*, int32_t* tree_tok_dev, void* stream);
  * argmax of each row's logits (ties: lowest id).  logits_dev [batch][n_rows][vocab] float out, or NULL.
  * tree_tok_dev [batch][n_rows] int32 in; the caller may have edited it since hydra_draft.  A token id outside
  * [0, vocab) raises the BOUNDS bit of the status word (the row is computed for token 0).  At the eighth call
- * of a batch and attention grid (earlier a capture costs more than it saves) the forward pass is captured into a CUDA graph (up to eight are kept) and from then on replayed, on the streams and under
+ * of a batch and attention grid (earlier a capture costs more than it saves) the forward pass is captured into a CUDA graph (eight are kept, the one used longest ago goes) and from then on replayed, on the streams and under
  * the switch described at hydra_step; the pointers may change freely, and a stream that the caller is capturing gets the launches themselves.
  * Errors: STATE, CAPACITY. */
 hydra_status hydra_verify(hydra_ctx*, const int32_t* tree_tok_dev, int32_t* amax_dev, float* logits_dev, void* stream);
@@ -152,7 +152,7 @@ hydra_status hydra_accept_compact(hydra_ctx*, const int32_t* tree_tok_dev, const
 /* One whole decoding step (the three passages above): draft + (optional planting) + verify + accept_compact
  * on the library's own buffers.  n_acc_dev [batch], out_tok_dev [batch][K+1] as in hydra_accept_compact (either
  * may be NULL).  From the second step of the context on, the step is captured into a CUDA graph (again
- * when the batch or the planting buffer changes or an attention grid must grow; up to eight graphs are kept, across prompt passes too, until the
+ * when the batch or the planting buffer changes or an attention grid must grow; eight graphs are kept (the one used longest ago goes), across prompt passes too, until the
  * acceptance criterion or the GEMM mode changes; n_acc_dev and out_tok_dev may change freely) and replayed with one launch, unless the stream
  * is a default stream (not capturable) or hydra_set_step_graph switched graphs off.  Errors: STATE, CAPACITY. */
 hydra_status hydra_step(hydra_ctx*, int32_t* n_acc_dev, int32_t* out_tok_dev, void* stream);

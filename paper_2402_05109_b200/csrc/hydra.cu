@@ -58,6 +58,31 @@ int pad_rows(int m) { return (m + 15) / 16 * 16; }
 // 81 waited-for calls over nine batches in random order, launched 4.45 ms: 4.60 with a capture at the second call, 4.74 at the fourth, 4.46 at the eighth.
 constexpr int VERIFY_CAPTURE_CALL = 8;
 
+// Captured graphs by what they freeze (G: graph, exec - null while there is none yet).  At most GRAPHS_KEPT; a new key takes the place of the one
+// that was asked for longest ago.
+constexpr size_t GRAPHS_KEPT = 8;
+template <typename Key, typename G>
+struct GraphStore {
+  struct Entry { G g; long long used; };
+  std::map<Key, Entry> entries;
+  long long clock = 0;
+  static void release(G& g) { if (g.exec) cudaGraphExecDestroy(g.exec); if (g.graph) cudaGraphDestroy(g.graph); }
+  G& at(const Key& key) {                          // the key's entry, a new one all zero
+    auto it = entries.find(key);
+    if (it == entries.end()) {
+      if (entries.size() >= GRAPHS_KEPT) {
+        auto oldest = std::min_element(entries.begin(), entries.end(), [](const auto& a, const auto& b) { return a.second.used < b.second.used; });
+        release(oldest->second.g);
+        entries.erase(oldest);
+      }
+      it = entries.emplace(key, Entry{}).first;
+    }
+    it->second.used = ++clock;
+    return it->second.g;
+  }
+  void clear() { for (auto& e : entries) release(e.second.g); entries.clear(); }
+};
+
 enum State { ST_CREATED = 0, ST_READY = 1, ST_DRAFTED = 2, ST_VERIFIED = 3 };
 
 }  // namespace
@@ -115,11 +140,11 @@ struct hydra_ctx {
     }
   };
   struct StepGraph { cudaGraph_t graph; cudaGraphExec_t exec; cudaGraphNode_t accept; AcceptArgs args; long long launches; };
-  std::map<GraphKey, StepGraph> graphs;
+  GraphStore<GraphKey, StepGraph> graphs;
   // verifications of the caller's candidates: everything up to the vocabulary projection, from a copy of the tokens (the caller's pointers
   // are arguments of the launches around it), keyed by batch and attention grid size
   struct RowsGraph { cudaGraph_t graph; cudaGraphExec_t exec; SplitDesc sd; long long launches; int calls; };      // exec null: launched `calls` times so far
-  std::map<std::pair<int, int>, RowsGraph> rows_graphs;
+  GraphStore<std::pair<int, int>, RowsGraph> rows_graphs;
   int use_graph; long long steps_done;
   int timing;
   std::vector<Timed> timed;
@@ -548,12 +573,7 @@ hydra_status enqueue_step(hydra_ctx* c, int* n_acc, int* out_tok, cudaStream_t s
   return do_accept(c, c->d_tree_tok, c->d_amax, n_acc, nullptr, out_tok, st);
 }
 
-void drop_graphs(hydra_ctx* c) {
-  for (auto& g : c->graphs) { cudaGraphExecDestroy(g.second.exec); cudaGraphDestroy(g.second.graph); }
-  c->graphs.clear();
-  for (auto& g : c->rows_graphs) if (g.second.exec) { cudaGraphExecDestroy(g.second.exec); cudaGraphDestroy(g.second.graph); }
-  c->rows_graphs.clear();
-}
+void drop_graphs(hydra_ctx* c) { c->graphs.clear(); c->rows_graphs.clear(); }
 
 bool capturable(cudaStream_t st) { return st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread; }      // default streams are not
 bool being_captured(cudaStream_t st) {
@@ -738,8 +758,7 @@ hydra_status hydra_verify(hydra_ctx* c, const int32_t* tree_tok, int32_t* amax, 
   // a stream that its owner is capturing takes the launches themselves
   if (c->use_graph && capturable(st) && !c->timing && !being_captured(st)) {
     const std::pair<int, int> key(c->batch, len_bucket(c, max_len_ub(c) + c->T));
-    if (!c->rows_graphs.count(key) && c->rows_graphs.size() >= 8) drop_graphs(c);
-    g = &c->rows_graphs[key];
+    g = &c->rows_graphs.at(key);
     if (!g->exec && ++g->calls >= VERIFY_CAPTURE_CALL) {
       cudaGraph_t graph = nullptr;
       cudaGraphExec_t exec = nullptr;
@@ -784,28 +803,24 @@ hydra_status hydra_step(hydra_ctx* c, int32_t* n_acc, int32_t* out_tok, void* st
   } else {
     const int lu = max_len_ub(c);
     hydra_ctx::GraphKey key{c->batch, len_bucket(c, lu + c->T), len_bucket(c, lu), c->plant};
-    auto it = c->graphs.find(key);
-    if (it == c->graphs.end()) {
-      if (c->graphs.size() >= 8) drop_graphs(c);
+    hydra_ctx::StepGraph& g = c->graphs.at(key);
+    if (!g.exec) {
       cudaGraph_t graph = nullptr;
-      long long captured = 0;
-      HYDRA_TRY(capture(c, st, [&]() { return enqueue_step(c, n_acc, out_tok, st); }, &graph, &captured));
+      HYDRA_TRY(capture(c, st, [&]() { return enqueue_step(c, n_acc, out_tok, st); }, &graph, &g.launches));
       cudaGraphExec_t exec = nullptr;
-      cudaGraphNode_t accept = nullptr;
-      cudaError_t ce = accept_graph_node(graph, &accept);
+      cudaError_t ce = accept_graph_node(graph, &g.accept);
       if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
       if (ce != cudaSuccess) { cudaGraphDestroy(graph); set_last_error("cudaGraphInstantiate", ce); return HYDRA_ERR_CUDA; }
-      it = c->graphs.emplace(key, hydra_ctx::StepGraph{graph, exec, accept, accept_args(c, c->d_tree_tok, c->d_amax, n_acc, nullptr, out_tok), captured}).first;
+      g.graph = graph; g.exec = exec; g.args = accept_args(c, c->d_tree_tok, c->d_amax, n_acc, nullptr, out_tok);
     }
-    AcceptArgs& aa = it->second.args;
-    if (aa.n_acc != n_acc || aa.out_tok != out_tok) {        // other output buffers: two arguments of one node
-      AcceptArgs na = aa;
+    if (g.args.n_acc != n_acc || g.args.out_tok != out_tok) {        // other output buffers: two arguments of one node
+      AcceptArgs na = g.args;
       na.n_acc = n_acc; na.out_tok = out_tok;
-      HYDRA_CUDA(accept_graph_update(it->second.exec, it->second.accept, na));
-      aa = na;
+      HYDRA_CUDA(accept_graph_update(g.exec, g.accept, na));
+      g.args = na;
     }
-    HYDRA_CUDA(cudaGraphLaunch(it->second.exec, st));
-    c->launches += it->second.launches;
+    HYDRA_CUDA(cudaGraphLaunch(g.exec, st));
+    c->launches += g.launches;
   }
   bump_len_ub(c);
   ++c->steps_done;

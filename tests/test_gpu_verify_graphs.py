@@ -53,3 +53,28 @@ def test_capture_at_the_eighth_call_of_a_batch():
     assert d.verify(3, CAPTURED_AT) == [False] * (CAPTURED_AT - 1) + [True]      # a batch of its own, counted from its own first call
     assert d.verify(1, 2) == [True] * 2
     d.g.close()
+
+
+def test_the_batch_that_was_asked_for_longest_ago_goes():
+    d = Driver()
+    assert d.verify(1, CAPTURED_AT)[-1]
+    for b in range(2, 11):                         # nine others pass by while batch 1 is in use
+        assert d.verify(b) == [False] and d.verify(1) == [True]
+    for b in range(2, 10):                         # eight others while it is not
+        d.verify(b)
+    assert d.verify(1) == [False]
+    d.g.close()
+
+
+def test_steps_leave_the_verifications_graphs():
+    d = Driver(1)
+    assert d.verify(1, CAPTURED_AT)[-1]
+    plants = [torch.full((1, 16), -1, dtype=torch.int32, device="cuda") for _ in range(11)]
+    with torch.cuda.stream(d.stream):
+        d.g.prefill(d.prompts[:1])
+        for p in plants:                           # a step graph for each but the first
+            d.g.set_plant(p)
+            d.g.step()
+        d.g.set_plant(None)
+    assert d.verify(1) == [True]
+    d.g.close()

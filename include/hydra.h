@@ -134,7 +134,7 @@ hydra_status hydra_draft(hydra_ctx*, int32_t* tree_tok_dev, void* stream);
  * argmax of each row's logits (ties: lowest id).  logits_dev [batch][n_rows][vocab] float out, or NULL.
  * tree_tok_dev [batch][n_rows] int32 in; the caller may have edited it since hydra_draft.  A token id outside
  * [0, vocab) raises the BOUNDS bit of the status word (the row is computed for token 0).  At the eighth call
- * of a batch and attention grid (earlier a capture costs more than it saves) the forward pass is captured into a CUDA graph (eight are kept, the one used longest ago goes) and from then on replayed, on the streams and under
+ * of a batch and attention grid (earlier a capture costs more than it saves) the forward pass is captured into a CUDA graph (eight are kept until the GEMM mode changes, the one used longest ago goes) and from then on replayed, on the streams and under
  * the switch described at hydra_step; the pointers may change freely, and a stream that the caller is capturing gets the launches themselves.
  * Errors: STATE, CAPACITY. */
 hydra_status hydra_verify(hydra_ctx*, const int32_t* tree_tok_dev, int32_t* amax_dev, float* logits_dev, void* stream);

@@ -838,7 +838,7 @@ hydra_status hydra_set_acceptance(hydra_ctx* c, int mode, float tau, float eps, 
   if (mode == 1 && !(tau > 0.f && eps >= 0.f && alpha >= 0.f)) return HYDRA_ERR_INVALID;
   if (c->state == ST_VERIFIED && mode != c->acc_mode) return HYDRA_ERR_STATE;      // the last verification prepared for the other criterion
   c->acc_mode = mode; c->acc_tau = tau; c->acc_eps = eps; c->acc_alpha = alpha; c->acc_u = mode == 1 ? u_dev : nullptr;
-  drop_graphs(c);
+  c->graphs.clear();                               // (a verification's graph ends before the criterion comes in)
   return HYDRA_OK;
 }
 

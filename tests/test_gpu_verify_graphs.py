@@ -78,3 +78,21 @@ def test_steps_leave_the_verifications_graphs():
         d.g.set_plant(None)
     assert d.verify(1) == [True]
     d.g.close()
+
+
+def test_the_criterion_leaves_the_verifications_graphs():
+    """A sampling loop sets the criterion before every verification; the graph ends before the criterion comes in."""
+    d = Driver(2)
+    assert d.verify(2, CAPTURED_AT)[-1]
+    u = torch.tensor([0.25, 0.75], device="cuda")
+    for mode, tau in ((1, 0.7), (1, 1.3), (0, 1.0)):
+        d.batch = 0                                # a prompt pass: the criterion may then change
+        with torch.cuda.stream(d.stream):
+            d.g.prefill(d.prompts[:2])
+            d.batch = 2
+            d.g.set_acceptance(mode, tau, 0.1, 0.3, u if mode else None)
+        assert d.verify(2, 2) == [True] * 2
+    d.g.set_gemm_mode(1)                           # another kernel: nothing captured survives
+    d.g.set_gemm_mode(0)
+    assert d.verify(2) == [False]
+    d.g.close()

@@ -235,7 +235,8 @@ const char* hydra_last_error(void); /* text of the last CUDA error seen by this 
  *   of mask[i] is set; mask NULL (dtype 1 only) means a causal chunk: slot pos0[b]+j is visible when j <= i.
  *   dtype 0: q, caches and out [rows][n_heads*head_dim] are float, tc <= 64, scratch_dev needs
  *   hydra_attention_scratch_bytes(...) bytes, planes = out_planes = 1, status_dev unused; n_rows[b] past tc counts as tc, and slots from
- *   max_seq on are not read.  dtype 1: q and the caches (16-byte boundaries, else
+ *   max_seq on are not read.  The order of a row's sums follows from batch, tc, n_heads and max_seq (inside a context: the bound of its lengths), so a
+ *   row may differ in its last bits from the same row in another batch.  dtype 1: q and the caches (16-byte boundaries, else
  *   INVALID) are float16 in `planes` planes (2: hi = f16(v), lo = f16(v - hi)), out is bfloat16 [out_planes][rows][n_heads*head_dim]
  *   (2: hi = bf16(v) and lo = bf16(v - hi)); tc <= 64 with a mask, <= 128 causal; scratch_dev unused (may be NULL); status_dev is an int32 status word (bit 2: a bounded wait ran out). */
 size_t hydra_gemm_partial_floats(int m, int n, int k, int dtype, int mode);

@@ -233,8 +233,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     prefetch_tensormap(&tmX);
     // weights do not depend on the preceding kernel: request half a ring of weight tiles right away, before the
     // CTA-wide set-up (TMEM allocation, barrier hand-over) and before griddepcontrol.wait; where they may, bring them nearer.
-    // (The whole ring, 29 MB over the SMs, is more than the preceding row-wise kernel's time takes in, and its loads then queue behind it: 7B
-    // shape, 32 steps without a tree 94.4 -> 93.7 ms with half, a 64-row tree 147.0 -> 145.6; all but one stage the same, one stage alone no better than the whole ring.)
+    // (The weight tiles of a whole ring are 128 KB an SM at 64 rows and 160 KB at one, 19 and 24 MB over the SMs; the preceding row-wise kernel's
+    // loads queue behind them.  7B shape, 32 steps with a 64-row tree 145.2 -> 144.0 ms with half a ring, runs of one side 0.3 % apart; without a
+    // tree, and 47 supplied rows, the same either way.  All stages but one gained as much as half, one stage alone nothing.)
     const uint64_t pol = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal();
     int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_tiles * BN;
     for (int i = 0; i < (a.w_const ? pre : ring); ++i) {

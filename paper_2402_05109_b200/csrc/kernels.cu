@@ -656,10 +656,13 @@ __global__ void tree_attn_combine_kernel(const float* part_o, const float* part_
 // The same for short caches and few rows: R query rows per CTA, its warps share the keys out (HD / 4 lanes a key, 16 bytes of it
 // each, ATT_BATCH keys of a lane group in flight), every lane group keeps an online softmax of its keys, and they meet once, in shared memory.  A row's chain
 // is then a handful of keys instead of all of them; each CTA reads the K, V of its pair again, out of L2.
-// 16 rows x 4 heads x 48..80 slots: 11.7 us with the kernel above (one row per warp), 2.8 us so (tiny float model, 8 steps: 1013 -> 872 us).
+// AHEAD: the next keys are fetched while these are worked on, which is most of the time of a round where many CTAs share the L2.  (A cache of a round or
+// two has nothing to fetch ahead, and the longer code shows: tiny float model 814 -> 821 us; four rows leave no registers for it.)
+// Full caches, back to back in a graph, head_dim 64, 4 heads; the kernel above / this one without / with AHEAD: 16 rows, 80 keys 6.6 / 3.3 us; 256 keys
+// 9.0 / 5.6 / 5.1; 512 keys 9.4 / 9.2 / 8.2; 4 x 16 rows, 512 keys 13.0 / 15.4 / 9.2.  Tiny float model, 8 steps: 1013 -> 872 us.
 constexpr int ATT_BATCH = 4;
 constexpr int ATT_FEW_KEYS = 512;
-template <int HD, int R, bool VEC>
+template <int HD, int R, bool VEC, bool AHEAD>
 __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const float* q, const float* kc, const float* vc, RowSet rs, float* __restrict__ out,
                                                                       int H, int max_seq) {
   pdl_trigger();
@@ -684,14 +687,21 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const flo
     o[r] = make_float4(0.f, 0.f, 0.f, 0.f); m[r] = -INFINITY; l[r] = 0.f;
   }
   const size_t base = ((size_t)b * H + h) * max_seq * HD + dim;
-  for (int s0 = warp * KPW + sub; s0 - sub < total; s0 += ATT_WARPS * KPW * ATT_BATCH) {
-    float4 kv[ATT_BATCH], vv[ATT_BATCH];
+  float4 kv[ATT_BATCH], vv[ATT_BATCH];
+  auto fetch = [&](int at, float4 (&k)[ATT_BATCH], float4 (&v)[ATT_BATCH]) {
 #pragma unroll
     for (int u = 0; u < ATT_BATCH; ++u) {
-      const int slot = s0 + u * ATT_WARPS * KPW;
-      kv[u] = vv[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (slot < total) { kv[u] = load4_at<VEC>(kc + base + (size_t)slot * HD); vv[u] = load4_at<VEC>(vc + base + (size_t)slot * HD); }
+      const int slot = at + u * ATT_WARPS * KPW;
+      k[u] = v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (slot < total) { k[u] = load4_at<VEC>(kc + base + (size_t)slot * HD); v[u] = load4_at<VEC>(vc + base + (size_t)slot * HD); }
     }
+  };
+  constexpr int STEP = ATT_WARPS * KPW * ATT_BATCH;
+  if (AHEAD) fetch(warp * KPW + sub, kv, vv);
+  for (int s0 = warp * KPW + sub; s0 - sub < total; s0 += STEP) {
+    float4 kn[ATT_BATCH], vn[ATT_BATCH];
+    if (AHEAD) fetch(s0 + STEP, kn, vn);
+    else fetch(s0, kv, vv);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       float s[ATT_BATCH], mn = m[r];
@@ -717,6 +727,10 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) tree_attn_few_kernel(const flo
         const float w = expf(s[u] - mn);
         l[r] += w; o[r].x += w * vv[u].x; o[r].y += w * vv[u].y; o[r].z += w * vv[u].z; o[r].w += w * vv[u].w;
       }
+    }
+    if (AHEAD) {
+#pragma unroll
+      for (int u = 0; u < ATT_BATCH; ++u) { kv[u] = kn[u]; vv[u] = vn[u]; }
     }
   }
 #pragma unroll
@@ -782,21 +796,29 @@ static hydra_status tree_attention_t(const T* q, const T* kc, const T* vc, RowSe
   float* part_ml = scratch + rows * H * nchunks_max * HD;
   // one row per warp while that leaves at most two CTAs per SM; more rows per warp share the staged K,V tile instead
   const long ctas1 = (long)H * rs.batch * nchunks * ((rs.tc + ATT_WARPS - 1) / ATT_WARPS), cap = 2L * sm_count();
-  // Short caches: the keys of a row shared out over the warps of a CTA, with the fewest rows a CTA that leave two CTAs per SM.  A CTA reads all keys
-  // of its pair and its chain grows with them (one chunk per CTA and the combine kernel do not: 16 rows, 4 heads: 80, 256, 512 keys 3.9, 5.9, 9.4 us
-  // against 7.3, 12.2, 11.7).  Four rows a CTA pay from the second chunk on (128 rows, 80 keys: 8.1 against 7.4; 256 keys: 13.7 against 20.0).
+  // Short caches: the keys of a row shared out over the warps of a CTA, with the fewest rows a CTA that leave two CTAs per SM, or four rows and up to four
+  // CTAs, which pay from the second chunk on (head_dim 64, 2 x 64 rows x 4 heads: two rows a CTA, 80 keys 7.3 us with a chunk per CTA and the combine
+  // kernel, 5.6 so, 256 keys 10.5 and 8.4; 4 x 64 rows, four a CTA, 256 keys 15.3 and 12.7).  len_upper bounds lengths that only the device knows, and a
+  // CTA's chain follows the length.  Timed from 1 to 8 sequences, 2 to 8 heads, 1 to 64 rows and 66 to 512 keys, nothing at head_dim 64 is slower than with
+  // chunks, at any length.  At head_dim 128 nothing is up to 384 keys; the full 512 take 1.04 to 1.31 as long (4 x 16 rows x 4 heads 13.3 -> 16.9 us), 256 and
+  // 80 keys under the same bound a half and a third, so the line stays at 512 there too.
   // (The stand-alone call takes operands on any element boundary; loads of one element then, the same sums.)
   const bool vec = on_vec4(q) && on_vec4(kc) && on_vec4(vc);
-  if (len_upper <= ATT_FEW_KEYS) {
-    const long pairs = (long)H * rs.batch;
-    auto go = [&](auto kernel, auto scalar, int R) {
+  const long pairs = (long)H * rs.batch;
+  const int R = pairs * rs.tc <= cap ? 1 : pairs * ((rs.tc + 1) / 2) <= cap ? 2 : len_upper > ATT_CHUNK && pairs * ((rs.tc + 3) / 4) <= 2 * cap ? 4 : 0;
+  if (R && len_upper <= ATT_FEW_KEYS) {
+    // (head_dim 128 and few CTAs: the L2 answers as fast as they ask; 16 rows x 4 heads, 256 keys 8.4 us without, 8.9 with)
+    const bool ahead = len_upper > ATT_CHUNK && (HD == 64 || pairs * ((rs.tc + R - 1) / R) > sm_count() / 2);
+    auto go = [&](auto kernel, auto scalar) {
       launch_pdl(vec ? kernel : scalar, dim3(H, rs.batch, (rs.tc + R - 1) / R), dim3(ATT_WARPS * 32), 0, st, q, kc, vc, rs, out, H, max_seq);
     };
-    const int R = pairs * rs.tc <= cap ? 1 : pairs * ((rs.tc + 1) / 2) <= cap ? 2 : len_upper > ATT_CHUNK && pairs * ((rs.tc + 3) / 4) <= 2 * cap ? 4 : 0;
-    if (R == 1) go(tree_attn_few_kernel<HD, 1, true>, tree_attn_few_kernel<HD, 1, false>, 1);
-    if (R == 2) go(tree_attn_few_kernel<HD, 2, true>, tree_attn_few_kernel<HD, 2, false>, 2);
-    if (R == 4) go(tree_attn_few_kernel<HD, 4, true>, tree_attn_few_kernel<HD, 4, false>, 4);
-    if (R) { HYDRA_LAUNCH_CHECK(); return HYDRA_OK; }
+    if (R == 1 && ahead) go(tree_attn_few_kernel<HD, 1, true, true>, tree_attn_few_kernel<HD, 1, false, true>);
+    else if (R == 1) go(tree_attn_few_kernel<HD, 1, true, false>, tree_attn_few_kernel<HD, 1, false, false>);
+    else if (R == 2 && ahead) go(tree_attn_few_kernel<HD, 2, true, true>, tree_attn_few_kernel<HD, 2, false, true>);
+    else if (R == 2) go(tree_attn_few_kernel<HD, 2, true, false>, tree_attn_few_kernel<HD, 2, false, false>);
+    else go(tree_attn_few_kernel<HD, 4, true, false>, tree_attn_few_kernel<HD, 4, false, false>);
+    HYDRA_LAUNCH_CHECK();
+    return HYDRA_OK;
   }
   if (!vec) HYDRA_TRY((launch_tree_attn<T, HD, 8, false>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));
   else if (ctas1 <= cap) HYDRA_TRY((launch_tree_attn<T, HD, 1>(q, kc, vc, rs, part_o, part_ml, out, H, max_seq, nchunks, st)));

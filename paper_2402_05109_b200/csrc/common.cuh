@@ -65,6 +65,33 @@ __device__ __forceinline__ float warp_max(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
+// Sum of v[r] over the warp, for R values at once: lanes first trade halves of the values (R-1 shuffles for R values), then the
+// remaining lane bits are folded.  Value warp_sum_owner(lane) ends up in lanes 0..R-1.
+template <int R>
+__device__ __forceinline__ float warp_sum_multi(float (&v)[R], int lane) {
+#pragma unroll
+  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int r = 0; r < n; ++r) {
+      const float give = up ? v[r] : v[r + n], keep = up ? v[r + n] : v[r];
+      v[r] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
+  }
+  float s = v[0];
+#pragma unroll
+  for (int bit = R; bit < 32; bit *= 2) s += __shfl_xor_sync(0xffffffffu, s, bit);
+  return s;
+}
+// which of the R values: the lowest lane bit chose the upper half, the next bit the upper quarter, ...
+template <int R>
+__device__ __forceinline__ int warp_sum_owner(int lane) {
+  int r = 0;
+#pragma unroll
+  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) r += (lane & bit) ? n : 0;
+  return r;
+}
+
 // Programmatic dependent launch: every kernel of the library starts with pdl_trigger() (lets the next kernel
 // in the stream get resident early) and pdl_wait() (blocks until the preceding kernel has completed and its
 // writes are visible) before it touches what other kernels write, so dependencies stay transitive along the stream.  What an earlier

@@ -322,20 +322,17 @@ hydra_status run_gemm(hydra_ctx* c, const void* x, int x_rows_alloc, const void*
 // element distance between the hi and lo planes of an operand buffer of `rows_alloc` rows of `cols` (0 for float)
 size_t ps(const hydra_ctx* c, int rows_alloc, size_t cols) { return c->planes == 2 ? (size_t)rows_alloc * cols : 0; }
 
-// RoPE + KV append + tree attention of one layer from the QKV partial sums (*sd) in c->part; result in c->attn_out.
-// stable_lengths: every forward call of the library starts with rope_table, which lets nothing of the call start before all
+// bfloat16 path: RoPE + KV append + tree attention of one layer from the QKV partial sums (*sd) in c->part; result in c->attn_out.
+// stable_lengths: every forward call of the library starts with forward_start, which lets nothing of the call start before all
 // earlier kernels have completed; the row set's lengths and the committed cache rows are written before that kernel, so
 // the attention kernels of the call may fetch committed tiles ahead of their predecessor.
 hydra_status attention_block(hydra_ctx* c, char* kc, char* vc, const RowSet& rs, int len_upper, const SplitDesc& sd, bool stable_lengths,
                              cudaStream_t st) {
   const hydra_model_cfg& m = c->m;
-  const int d = m.d_model, dt = m.dtype;
+  const int d = m.d_model;
   const size_t q_ps = c->kv_planes == 2 ? (size_t)c->R * d : 0, kv_ps = c->kv_planes == 2 ? kv_layer_elems(m) : 0;
-  HYDRA_TRY(qkv_rope_store(c->part, sd, c->rope, c->q, q_ps, kc, vc, kv_ps, rs, m.n_heads, m.head_dim, m.max_seq, dt, false, c->d_status, st));
+  HYDRA_TRY(qkv_rope_store(c->part, sd, c->rope, c->q, q_ps, kc, vc, kv_ps, rs, m.n_heads, m.head_dim, m.max_seq, false, c->d_status, st));
   TimeScope ts(c, HYDRA_TIME_ATTENTION, 0.0, st);
-  if (dt == 0)
-    return tree_attention_f32((const float*)c->q, (const float*)kc, (const float*)vc, rs, (float*)c->attn_out, c->att_scratch, m.n_heads,
-                              m.head_dim, m.max_seq, len_upper, st);
   return tree_attention_tc((const __half*)c->q, c->R, (const __half*)kc, (const __half*)vc, m.max_batch, c->kv_planes, rs, (bf16*)c->attn_out,
                            ps(c, c->R, d), m.n_heads, m.head_dim, m.max_seq, len_upper, c->d_status, stable_lengths, st);
 }
@@ -344,7 +341,7 @@ double gemm_bytes(const hydra_ctx* c, int m, int n, int k) {        // weights +
   return (double)c->esize * ((double)n * k + (double)c->planes * m * k) + 4.0 * m * n;
 }
 
-// The rest of a layer after its attention: O projection, + residual, RMSNorm, gate/up, SiLU * up, down, + residual and,
+// bfloat16 path: the rest of a layer after its attention: O projection, + residual, RMSNorm, gate/up, SiLU * up, down, + residual and,
 // when next_gain is given, xn = rmsnorm(x) * next_gain (hn: the same in float); when next_w is given, also the
 // GEMM xn @ next_w^T (the next layer's QKV projection, or the LM head), whose partial sums stay in c->part (*sd).
 hydra_status mlp_block(hydra_ctx* c, const LayerW& w, int rows, const void* next_gain, float* hn, const void* next_w, int next_n,
@@ -355,11 +352,31 @@ hydra_status mlp_block(hydra_ctx* c, const LayerW& w, int rows, const void* next
   HYDRA_TRY(run_gemm(c, c->attn_out, c->R, w.wo, rows, d, d, &s1, st));
   HYDRA_TRY(residual_rmsnorm(c->x, c->part, s1, c->x, w.ffn_norm, c->xn, ps(c, c->R, d), nullptr, rows, d, m.rms_eps, dt, st));
   HYDRA_TRY(run_gemm(c, c->xn, c->R, w.w_gate_up, rows, 2 * f, d, &s1, st));
-  HYDRA_TRY(silu_mul(c->part, s1, c->act, ps(c, c->R, f), rows, f, dt, st));
+  HYDRA_TRY(silu_mul(c->part, s1, c->act, ps(c, c->R, f), rows, f, st));
   HYDRA_TRY(run_gemm(c, c->act, c->R, w.w_down, rows, d, f, &s1, st));
   HYDRA_TRY(residual_rmsnorm(c->x, c->part, s1, c->x, next_gain, next_gain ? c->xn : nullptr, ps(c, c->R, d), hn, rows, d, m.rms_eps, dt, st));
   if (next_w) HYDRA_TRY(run_gemm(c, c->xn, c->R, next_w, rows, next_n, d, sd, st));
   return HYDRA_OK;
+}
+
+// A layer of the float path: the rows `src` go in, the residual stream comes out in c->x (src may be c->x).
+hydra_status f32_layer(hydra_ctx* c, const LayerW& w, const float* src, char* kc, char* vc, const RowSet& rs, int len_upper, cudaStream_t st) {
+  const hydra_model_cfg& m = c->m;
+  const int rows = rs.rows(), d = m.d_model, f = m.d_ffn;
+  auto product = [&](int n, int k, auto launch) -> hydra_status {
+    TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, n, k), st);
+    return launch();
+  };
+  HYDRA_TRY(product(3 * d, d, [&]() {
+    return f32_qkv(src, (const float*)w.attn_norm, (const float*)w.wqkv, c->rope, (float*)c->q, (float*)kc, (float*)vc, rs, m.n_heads, m.head_dim, m.max_seq, false, m.rms_eps, c->d_status, st);
+  }));
+  {
+    TimeScope ts(c, HYDRA_TIME_ATTENTION, 0.0, st);
+    HYDRA_TRY(tree_attention_f32((const float*)c->q, (const float*)kc, (const float*)vc, rs, (float*)c->attn_out, c->att_scratch, m.n_heads, m.head_dim, m.max_seq, len_upper, st));
+  }
+  HYDRA_TRY(product(d, d, [&]() { return f32_add((const float*)c->attn_out, (const float*)w.wo, src, c->x, rows, d, d, st); }));
+  HYDRA_TRY(product(2 * f, d, [&]() { return f32_glu(c->x, (const float*)w.ffn_norm, (const float*)w.w_gate_up, (float*)c->act, rows, f, d, m.rms_eps, st); }));
+  return product(d, f, [&]() { return f32_add((const float*)c->act, (const float*)w.w_down, c->x, c->x, rows, d, f, st); });
 }
 
 // Base model over the rows of `rs` whose tokens are tok[rows]: leaves post-final-norm hidden rows in c->h_tree
@@ -369,8 +386,13 @@ hydra_status run_base(hydra_ctx* c, const int* tok, const RowSet& rs, int len_up
   const hydra_model_cfg& m = c->m;
   const int rows = rs.rows(), d = m.d_model;
   const size_t kvl = kv_layer_elems(m) * c->kv_esize * c->kv_planes;      // bytes of one layer's K (or V) cache, all planes
-  HYDRA_TRY(rope_table(rs, c->rope, m.head_dim, m.rope_theta, st));
-  HYDRA_TRY(embed_rows(c->embed, tok, c->x, rows, d, m.vocab, m.dtype, c->d_status, st));
+  HYDRA_TRY(forward_start(rs, c->rope, m.head_dim, m.rope_theta, c->embed, tok, c->x, d, m.vocab, m.dtype, c->d_status, st));
+  if (m.dtype == 0) {
+    for (int l = 0; l < m.n_layers; ++l)
+      HYDRA_TRY(f32_layer(c, c->layers[l], c->x, c->kv_base + (size_t)(2 * l) * kvl, c->kv_base + (size_t)(2 * l + 1) * kvl, rs, len_upper, st));
+    HYDRA_TRY(residual_rmsnorm(c->x, nullptr, single_slot(0), c->x, c->final_norm, c->xn, 0, c->h_tree, rows, d, m.rms_eps, 0, st));
+    return tail_w ? run_gemm(c, c->xn, c->R, tail_w, rows, tail_n, d, tail_sd, st) : HYDRA_OK;
+  }
   HYDRA_TRY(residual_rmsnorm(c->x, nullptr, single_slot(0), c->x, c->layers[0].attn_norm, c->xn, ps(c, c->R, d), nullptr, rows, d, m.rms_eps, m.dtype, st));
   SplitDesc sd;
   HYDRA_TRY(run_gemm(c, c->xn, c->R, c->layers[0].wqkv, rows, 3 * d, d, &sd, st));
@@ -388,7 +410,8 @@ hydra_status run_prefix(hydra_ctx* c, const float* src, const RowSet& rs, int le
   const hydra_model_cfg& m = c->m;
   const int rows = rs.rows(), d = m.d_model;
   const size_t kvl = kv_layer_elems(m) * c->kv_esize * c->kv_planes;      // bytes of one layer's K (or V) cache, all planes
-  HYDRA_TRY(rope_table(rs, c->rope, m.head_dim, m.rope_theta, st));
+  HYDRA_TRY(forward_start(rs, c->rope, m.head_dim, m.rope_theta, nullptr, nullptr, nullptr, 0, 0, m.dtype, c->d_status, st));
+  if (m.dtype == 0) return f32_layer(c, c->pfx, src, c->kv_pfx, c->kv_pfx + kvl, rs, len_upper, st);
   HYDRA_TRY(residual_rmsnorm(src, nullptr, single_slot(0), c->x, c->pfx.attn_norm, c->xn, ps(c, c->R, d), nullptr, rows, d, m.rms_eps, m.dtype, st));
   SplitDesc sd;
   HYDRA_TRY(run_gemm(c, c->xn, c->R, c->pfx.wqkv, rows, 3 * d, d, &sd, st));
@@ -405,11 +428,16 @@ hydra_status prefix_cache_rows(hydra_ctx* c, const float* src, const RowSet& rs,
   const hydra_model_cfg& m = c->m;
   const int rows = rs.rows(), d = m.d_model;
   const size_t kvl = kv_layer_elems(m) * c->kv_esize * c->kv_planes;
+  if (m.dtype == 0) {
+    TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, 2 * d, d), st);
+    return f32_qkv(src, (const float*)c->pfx.attn_norm, (const float*)c->pfx.wqkv + (size_t)d * d, c->rope, nullptr, (float*)c->kv_pfx, (float*)(c->kv_pfx + kvl), rs, m.n_heads,
+                   m.head_dim, m.max_seq, true, m.rms_eps, c->d_status, st);
+  }
   HYDRA_TRY(residual_rmsnorm(src, nullptr, single_slot(0), c->x, c->pfx.attn_norm, c->xn, ps(c, c->R, d), nullptr, rows, d, m.rms_eps, m.dtype, st));
   SplitDesc sd;
   HYDRA_TRY(run_gemm(c, c->xn, c->R, (const char*)c->pfx.wqkv + (size_t)d * d * c->esize, rows, 2 * d, d, &sd, st));
   return qkv_rope_store(c->part, sd, c->rope, nullptr, 0, c->kv_pfx, c->kv_pfx + kvl, c->kv_planes == 2 ? kv_layer_elems(m) : 0, rs, m.n_heads,
-                        m.head_dim, m.max_seq, m.dtype, true, c->d_status, st);
+                        m.head_dim, m.max_seq, true, c->d_status, st);
 }
 
 // Prompt pass of the bfloat16 path: the concatenated prompts (c->d_offsets) go through the base model (and the prefix layer)
@@ -475,12 +503,28 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     float* y = c->y + (size_t)y0 * d;
     char* yb = (char*)c->yb + (size_t)y0 * d * c->esize;
     HYDRA_TRY(run_gemm(c, c->z, c->RH, c->head_w1[lvl - 1], rows, d, in_blocks * d, &sd, st));
-    HYDRA_TRY(head_act(c->hprime, 1, rows_per_b, c->part, sd, c->h.has_bias ? c->head_b1[lvl - 1] : nullptr, y, yb, ps(c, c->RH, d), rows, d, dt, st));
+    HYDRA_TRY(head_act(c->hprime, 1, rows_per_b, c->part, sd, c->h.has_bias ? c->head_b1[lvl - 1] : nullptr, y, yb, ps(c, c->RH, d), rows, d, st));
     for (int l = 0; l + 1 < c->h.n_mlp_layers; ++l) {
       const char* wr = (const char*)c->head_wr[lvl - 1] + (size_t)l * d * d * c->esize;
       const char* br = c->h.has_bias ? (const char*)c->head_br[lvl - 1] + (size_t)l * d * c->esize : nullptr;
       HYDRA_TRY(run_gemm(c, c->yb, c->RH, wr, rows, d, d, &sd, st, y0));
-      HYDRA_TRY(head_act(y, 0, rows_per_b, c->part, sd, br, y, yb, ps(c, c->RH, d), rows, d, dt, st));
+      HYDRA_TRY(head_act(y, 0, rows_per_b, c->part, sd, br, y, yb, ps(c, c->RH, d), rows, d, st));
+    }
+    return HYDRA_OK;
+  };
+  // Float path: the layers of a head over the level's rows (sequence, parent), input rows read where they are; the result ends up in rows y0.. of c->yb
+  auto f32_mlp = [&](int lvl, const LevelDesc& lv, bool write_root, int y0) -> hydra_status {
+    const int rows = B * lv.n_parents, layers = c->h.n_mlp_layers;
+    float *out = (layers & 1 ? (float*)c->yb : c->y) + (size_t)y0 * d, *other = (layers & 1 ? c->y : (float*)c->yb) + (size_t)y0 * d;
+    {
+      TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, d, (lv.d + 1) * d), st);
+      HYDRA_TRY(f32_head_first(c->hprime, (const float*)c->embed, c->d_root_tok, tree_tok, c->d_path_tab, lv, write_root, (const float*)c->head_w1[lvl - 1],
+                               c->h.has_bias ? (const float*)c->head_b1[lvl - 1] : nullptr, out, B, c->T, K + 1, d, m.vocab, c->d_status, st));
+    }
+    for (int l = 0; l + 1 < layers; ++l, std::swap(out, other)) {
+      TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, d, d), st);
+      HYDRA_TRY(f32_head_next(out, (const float*)c->head_wr[lvl - 1] + (size_t)l * d * d, c->h.has_bias ? (const float*)c->head_br[lvl - 1] + (size_t)l * d : nullptr, other,
+                              rows, d, st));
     }
     return HYDRA_OK;
   };
@@ -492,11 +536,12 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     // one-parent level for the gather).  No head waits for another's tokens, so the vocabulary projection takes the rows of all heads at once.
     // The last head's rows come first: its logits are the ones that stay readable.
     // (One projection a head: 7B shape, 4 heads, a step of one sequence 3.30 -> 3.17 ms.)
-    HYDRA_TRY(head_gather(c->hprime, c->embed, c->d_root_tok, tree_tok, c->d_path_tab, LevelDesc{0, 1, c->d_level_parents[0]}, 1, c->z, ps(c, c->RH, d), B, c->T,
-                          K + 1, d, m.vocab, dt, c->d_status, st));
+    const LevelDesc alone{0, 1, c->d_level_parents[0]};
+    if (dt == 1)
+      HYDRA_TRY(head_gather(c->hprime, c->embed, c->d_root_tok, tree_tok, c->d_path_tab, alone, 1, c->z, ps(c, c->RH, d), B, c->T, K + 1, d, m.vocab, c->d_status, st));
     int max_children = 1;
     for (int lvl = 1; lvl <= c->Ktree; ++lvl) {
-      HYDRA_TRY(head_mlp(lvl, B, 1, 1, (c->Ktree - lvl) * B));
+      HYDRA_TRY(dt == 0 ? f32_mlp(lvl, alone, lvl == 1, (c->Ktree - lvl) * B) : head_mlp(lvl, B, 1, 1, (c->Ktree - lvl) * B));
       max_children = std::max(max_children, children_of(lvl));
     }
     HYDRA_TRY(run_gemm(c, c->yb, c->RH, c->lm_head, c->Ktree * B, m.vocab, d, &sd, st));
@@ -510,9 +555,13 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     // one row per (sequence, parent), input [h' ; E of the path tokens]
     const LevelDesc lv = level(lvl);
     const int rows = B * lv.n_parents, max_children = children_of(lvl);
-    HYDRA_TRY(head_gather(c->hprime, c->embed, c->d_root_tok, tree_tok, c->d_path_tab, lv, lvl == 1, c->z, ps(c, c->RH, (size_t)(lvl + 1) * d), B, c->T,
-                          K + 1, d, m.vocab, dt, c->d_status, st));
-    HYDRA_TRY(head_mlp(lvl, rows, lv.n_parents, lvl + 1, 0));
+    if (dt == 0) {
+      HYDRA_TRY(f32_mlp(lvl, lv, lvl == 1, 0));
+    } else {
+      HYDRA_TRY(head_gather(c->hprime, c->embed, c->d_root_tok, tree_tok, c->d_path_tab, lv, lvl == 1, c->z, ps(c, c->RH, (size_t)(lvl + 1) * d), B, c->T,
+                            K + 1, d, m.vocab, c->d_status, st));
+      HYDRA_TRY(head_mlp(lvl, rows, lv.n_parents, lvl + 1, 0));
+    }
     HYDRA_TRY(run_gemm(c, c->yb, c->RH, c->lm_head, rows, m.vocab, d, &sd, st));
     HYDRA_TRY(topk_children(c->part, sd, c->head_logits, lv, max_children, c->d_first_child, c->d_n_child, tree_tok, c->topk_scratch, c->topk_rows_cap,
                             B, c->T, m.vocab, st));

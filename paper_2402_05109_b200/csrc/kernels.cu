@@ -8,7 +8,8 @@
 namespace hydra {
 
 // ------------------------------------------------------------------------------------------------
-// SIMT GEMM: out[m][n] = sum_k x[m][k] w[n][k].  One warp per output feature, MR rows per pass.
+// SIMT GEMM of bfloat16 operands (the debug mode): out[m][n] = sum_k x[m][k] w[n][k].  One warp per output feature, MR rows per pass.
+// (Float operands: float_path.cu.)
 // ------------------------------------------------------------------------------------------------
 template <typename T> struct Vec4 { };
 template <> struct Vec4<float> {
@@ -21,33 +22,6 @@ template <> struct Vec4<bf16> {
     __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&t.x), b = *reinterpret_cast<__nv_bfloat162*>(&t.y);
     v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b); }
 };
-
-// Sum of v[r] over the warp, for R values at once: lanes first trade halves of the values (R-1 shuffles for R values), then the
-// remaining lane bits are folded.  Value warp_sum_owner(lane) ends up in lanes 0..R-1.
-template <int R>
-__device__ __forceinline__ float warp_sum_multi(float (&v)[R], int lane) {
-#pragma unroll
-  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) {
-    const bool up = lane & bit;
-#pragma unroll
-    for (int r = 0; r < n; ++r) {
-      const float give = up ? v[r] : v[r + n], keep = up ? v[r + n] : v[r];
-      v[r] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
-    }
-  }
-  float s = v[0];
-#pragma unroll
-  for (int bit = R; bit < 32; bit *= 2) s += __shfl_xor_sync(0xffffffffu, s, bit);
-  return s;
-}
-// which of the R values: the lowest lane bit chose the upper half, the next bit the upper quarter, ...
-template <int R>
-__device__ __forceinline__ int warp_sum_owner(int lane) {
-  int r = 0;
-#pragma unroll
-  for (int n = R / 2, bit = 1; n >= 1; n /= 2, bit *= 2) r += (lane & bit) ? n : 0;
-  return r;
-}
 
 // MR activation rows; KS warps share an output column (each every KS-th 512-byte piece of its weight row), 8 / KS columns per
 // block.  The small models of the float path spend their time in the chain launch -> loads -> reduction: the first WPRE weight
@@ -120,14 +94,11 @@ static void launch_gemm_simt(const void* x, const void* w, float* out, int m, in
 hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, bool w_const, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0 || (k & 3)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & (dtype == 0 ? 15 : 7)) return HYDRA_ERR_INVALID;      // both are read four elements at a time
-  auto rows = [&](auto zero) {
-    typedef decltype(zero) T;
-    if (m == 1) launch_gemm_simt<T, 1>(x, w, out, m, n, k, w_const, st);
-    else if (m <= 4) launch_gemm_simt<T, 4>(x, w, out, m, n, k, w_const, st);
-    else if (m <= 8) launch_gemm_simt<T, 8>(x, w, out, m, n, k, w_const, st);
-    else launch_gemm_simt<T, 16>(x, w, out, m, n, k, w_const, st);
-  };
-  if (dtype == 0) rows(float{}); else rows(bf16{});
+  if (dtype == 0) return f32_gemm((const float*)x, (const float*)w, out, m, n, k, w_const, st);
+  if (m == 1) launch_gemm_simt<bf16, 1>(x, w, out, m, n, k, w_const, st);
+  else if (m <= 4) launch_gemm_simt<bf16, 4>(x, w, out, m, n, k, w_const, st);
+  else if (m <= 8) launch_gemm_simt<bf16, 8>(x, w, out, m, n, k, w_const, st);
+  else launch_gemm_simt<bf16, 16>(x, w, out, m, n, k, w_const, st);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -148,9 +119,6 @@ hydra_status reduce_splits(const float* part, SplitDesc sd, float* out, int m, i
   return HYDRA_OK;
 }
 
-// ------------------------------------------------------------------------------------------------
-// Embedding gather
-// ------------------------------------------------------------------------------------------------
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
 template <> __device__ __forceinline__ float4 load4<bf16>(const bf16* p) {
@@ -161,25 +129,6 @@ template <typename T> inline bool on_vec4(const T* p) { return ((uintptr_t)p & (
 template <bool VEC, typename T> __device__ __forceinline__ float4 load4_at(const T* p) {
   if constexpr (VEC) return load4<T>(p);
   else return make_float4(to_f<T>(p[0]), to_f<T>(p[1]), to_f<T>(p[2]), to_f<T>(p[3]));
-}
-
-template <typename T>
-__global__ void embed_rows_kernel(const T* __restrict__ embed, const int* tok, float* __restrict__ x, int d,
-                                  int vocab, int* status) {
-  pdl_trigger();
-  pdl_wait();
-  int r = blockIdx.x;
-  int t = tok[r];
-  if (t < 0 || t >= vocab) { if (threadIdx.x == 0) atomicOr(status, ST_BOUNDS); t = 0; }
-  const T* e = embed + (size_t)t * d;
-  for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) *reinterpret_cast<float4*>(x + (size_t)r * d + i) = load4<T>(e + i);   // d % 4 == 0
-}
-hydra_status embed_rows(const void* embed, const int* tok, float* x, int rows, int d, int vocab, int dtype, int* status,
-                        cudaStream_t st) {
-  if (dtype == 0) launch_pdl(embed_rows_kernel<float>, dim3(rows), dim3(256), 0, st, (const float*)embed, tok, x, d, vocab, status);
-  else launch_pdl(embed_rows_kernel<bf16>, dim3(rows), dim3(256), 0, st, (const bf16*)embed, tok, x, d, vocab, status);
-  HYDRA_LAUNCH_CHECK();
-  return HYDRA_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -210,10 +159,8 @@ template <> __device__ __forceinline__ void store4<__half>(__half* p, float4 v) 
   uint2 u; u.x = *reinterpret_cast<uint32_t*>(&a); u.y = *reinterpret_cast<uint32_t*>(&b);
   *reinterpret_cast<uint2*>(p) = u;
 }
-// float: one plane.  float16: hi = f16(v) and, ps elements further on, lo = f16(v - hi) (ps = 0: hi only).
-template <typename T> __device__ __forceinline__ void put4h(T* p, size_t ps, float4 v);
-template <> __device__ __forceinline__ void put4h<float>(float* p, size_t, float4 v) { *reinterpret_cast<float4*>(p) = v; }
-template <> __device__ __forceinline__ void put4h<__half>(__half* p, size_t ps, float4 v) {
+// hi = f16(v) and, ps elements further on, lo = f16(v - hi) (ps = 0: hi only).
+__device__ __forceinline__ void put4h(__half* p, size_t ps, float4 v) {
   const float4 h = make_float4(__half2float(__float2half_rn(v.x)), __half2float(__float2half_rn(v.y)),
                                __half2float(__float2half_rn(v.z)), __half2float(__float2half_rn(v.w)));
   store4<__half>(p, h);
@@ -405,14 +352,23 @@ hydra_status residual_rmsnorm(const float* res, const float* part, SplitDesc sd,
 // ------------------------------------------------------------------------------------------------
 // Rotary table + QKV post-processing (sum partials, rotate q and k, append K,V to the cache)
 // ------------------------------------------------------------------------------------------------
-// The first kernel of every forward call.  It lets its successors start only AFTER it has waited for everything before
-// it (trigger after wait): no kernel of this call can be resident, however early the following launches are, while a
+// The first kernel of every forward call: the rotary table of its rows and, where they come as tokens, their embeddings.  It lets its successors start only
+// AFTER it has waited for everything before it (trigger after wait): no kernel of this call can be resident, however early the following launches are, while a
 // kernel of an earlier call (the acceptance kernel that wrote the lengths, the kernels that filled the committed cache
 // rows) is still running.  The early cache fetches of the attention kernel rely on that.
-__global__ void rope_table_kernel(RowSet rs, float2* __restrict__ table, int half, float theta) {
+template <typename T>
+__global__ void forward_start_kernel(RowSet rs, float2* __restrict__ table, int half, float theta, const T* __restrict__ embed, const int* tok, float* __restrict__ x, int d,
+                                     int vocab, int* status) {
   pdl_wait();
   pdl_trigger();
-  int r = blockIdx.x, pos;
+  const int r = blockIdx.x;
+  if (tok) {
+    int t = tok[r];
+    if (t < 0 || t >= vocab) { if (threadIdx.x == 0) atomicOr(status, ST_BOUNDS); t = 0; }
+    const T* e = embed + (size_t)t * d;
+    for (int i = threadIdx.x * 4; i < d; i += blockDim.x * 4) *reinterpret_cast<float4*>(x + (size_t)r * d + i) = load4<T>(e + i);   // d % 4 == 0
+  }
+  int pos;
   if (rs.row_at) pos = rs.row_at[r].y;
   else pos = rs.pos0[r / rs.tc] + rs.depth[r % rs.tc];
   for (int j = threadIdx.x; j < half; j += blockDim.x) {
@@ -422,8 +378,11 @@ __global__ void rope_table_kernel(RowSet rs, float2* __restrict__ table, int hal
     table[(size_t)r * half + j] = make_float2((float)c, (float)s);
   }
 }
-hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cudaStream_t st) {
-  launch_pdl(rope_table_kernel, dim3(rs.rows()), dim3(64), 0, st, rs, table, head_dim / 2, theta);
+hydra_status forward_start(RowSet rs, float2* table, int head_dim, float theta, const void* embed, const int* tok, float* x, int d, int vocab, int dtype, int* status,
+                           cudaStream_t st) {
+  const dim3 threads(tok ? 256 : 64);
+  if (dtype == 0) launch_pdl(forward_start_kernel<float>, dim3(rs.rows()), threads, 0, st, rs, table, head_dim / 2, theta, (const float*)embed, tok, x, d, vocab, status);
+  else launch_pdl(forward_start_kernel<bf16>, dim3(rs.rows()), threads, 0, st, rs, table, head_dim / 2, theta, (const bf16*)embed, tok, x, d, vocab, status);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -432,13 +391,12 @@ hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cud
 // k and v appended to the cache; all loads and stores are 16 bytes wide.  Three short threads instead of one long one: the sums
 // of two pieces leave registers for twice the warps (512 rows of 32 heads: 23 us with one thread for q, k and v, 17 so), and 64 rows spread over
 // more SMs.  What the call's earlier kernels cannot change - slot counts, lengths, row table - is read before the wait (the
-// lengths are stable within a forward call, see rope_table_kernel).
-// T: float (float model path) or float16 (bfloat16 model path: q and the caches are float16 in one or two planes).
+// lengths are stable within a forward call, see forward_start_kernel).
+// (The float path does this in its product: float_path.cu.)
 // first = 1: the projection has no q columns (a layer of which only the cache rows are wanted).
-template <typename T>
 __global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, SplitDesc sd,
-                                                             const float2* table, T* __restrict__ q, size_t q_ps,
-                                                             T* __restrict__ kc, T* __restrict__ vc, size_t kv_ps,
+                                                             const float2* table, __half* __restrict__ q, size_t q_ps,
+                                                             __half* __restrict__ kc, __half* __restrict__ vc, size_t kv_ps,
                                                              RowSet rs, int H, int hd, int max_seq, int first,
                                                              int* status) {
   pdl_trigger();
@@ -477,23 +435,18 @@ __global__ void __launch_bounds__(128) qkv_rope_store_kernel(const float* part, 
     for (int e = 0; e < 4; ++e) { l[e] = av[e] * cs[e] - bv[e] * sn[e]; hh[e] = bv[e] * cs[e] + av[e] * sn[e]; }
     v2[0] = make_float4(l[0], l[1], l[2], l[3]); v2[1] = make_float4(hh[0], hh[1], hh[2], hh[3]);
   }
-  T* dst = which == 0 ? q + (size_t)r * d + h * hd : (which == 1 ? kc : vc) + (((size_t)b * H + h) * max_seq + slot) * hd;
+  __half* dst = which == 0 ? q + (size_t)r * d + h * hd : (which == 1 ? kc : vc) + (((size_t)b * H + h) * max_seq + slot) * hd;
   const size_t ps = which == 0 ? q_ps : kv_ps;
-  put4h<T>(dst + j, ps, v2[0]);
-  put4h<T>(dst + j + half, ps, v2[1]);
+  put4h(dst + j, ps, v2[0]);
+  put4h(dst + j + half, ps, v2[1]);
 }
 hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table, void* q, size_t q_ps, void* kcache, void* vcache,
-                            size_t kv_ps, RowSet rs, int H, int hd, int max_seq, int dtype, bool kv_only, int* status, cudaStream_t st) {
+                            size_t kv_ps, RowSet rs, int H, int hd, int max_seq, bool kv_only, int* status, cudaStream_t st) {
   const int first = kv_only ? 1 : 0;
   if (hd % 8 || 128 % (hd / 8)) return HYDRA_ERR_UNSUPPORTED;
   const int heads_per_block = 128 / (hd / 8);
   dim3 grid(rs.rows(), (H + heads_per_block - 1) / heads_per_block, 3 - first);
-  if (dtype == 0)
-    launch_pdl(qkv_rope_store_kernel<float>, grid, dim3(128), 0, st, part, sd, table, (float*)q, q_ps, (float*)kcache, (float*)vcache,
-               kv_ps, rs, H, hd, max_seq, first, status);
-  else
-    launch_pdl(qkv_rope_store_kernel<__half>, grid, dim3(128), 0, st, part, sd, table, (__half*)q, q_ps, (__half*)kcache, (__half*)vcache,
-               kv_ps, rs, H, hd, max_seq, first, status);
+  launch_pdl(qkv_rope_store_kernel, grid, dim3(128), 0, st, part, sd, table, (__half*)q, q_ps, (__half*)kcache, (__half*)vcache, kv_ps, rs, H, hd, max_seq, first, status);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -842,8 +795,7 @@ hydra_status tree_attention_f32(const float* q, const float* kc, const float* vc
 // SiLU(gate) * up from the gate/up partial sums: four columns a thread, rows on the grid's y, so that nothing but the slot counts is
 // worked out and that before the wait (512 x 11008: 28 us with a flat index divided by the row length, 21 so; 64 rows: 6.0 and 3.5)
 // ------------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) silu_mul_kernel(const float* part, SplitDesc sd, T* __restrict__ act, size_t act_ps, int f) {
+__global__ void __launch_bounds__(256) silu_mul_kernel(const float* part, SplitDesc sd, bf16* __restrict__ act, size_t act_ps, int f) {
   pdl_trigger();
   const int r = blockIdx.y, c = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   const size_t off[2] = {(size_t)r * 2 * f + c, (size_t)r * 2 * f + f + c};
@@ -853,13 +805,12 @@ __global__ void __launch_bounds__(256) silu_mul_kernel(const float* part, SplitD
   float4 gu[2];
   sum_slots_multi<2, 4>(part, sd.stride, off, ns, gu);     // the widest output: few CTAs, hence few slots, per tile
   const float4 g = gu[0], u = gu[1];
-  put4<T>(act + (size_t)r * f + c, act_ps, make_float4(silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w));
+  put4<bf16>(act + (size_t)r * f + c, act_ps, make_float4(silu_f(g.x) * u.x, silu_f(g.y) * u.y, silu_f(g.z) * u.z, silu_f(g.w) * u.w));
 }
-hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, int dtype, cudaStream_t st) {
+hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, cudaStream_t st) {
   if (f & 3) return HYDRA_ERR_UNSUPPORTED;
   const dim3 grid((f / 4 + 255) / 256, rows);
-  if (dtype == 0) launch_pdl(silu_mul_kernel<float>, grid, dim3(256), 0, st, part, sd, (float*)act, act_ps, f);
-  else launch_pdl(silu_mul_kernel<bf16>, grid, dim3(256), 0, st, part, sd, (bf16*)act, act_ps, f);
+  launch_pdl(silu_mul_kernel, grid, dim3(256), 0, st, part, sd, (bf16*)act, act_ps, f);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -1115,40 +1066,35 @@ hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, 
 }
 
 // ------------------------------------------------------------------------------------------------
-// Hydra heads: input gather and the residual SiLU layer epilogue
+// Draft heads (bfloat16 path): input gather and the residual SiLU layer epilogue
 // ------------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) head_gather_kernel(const float* hprime, const T* __restrict__ embed,
+__global__ void __launch_bounds__(256) head_gather_kernel(const float* hprime, const bf16* __restrict__ embed,
                                                           const int* root_tok, int* tree_tok,
-                                                          const int* __restrict__ path_tab, LevelDesc lv, int write_root, T* __restrict__ z,
+                                                          const int* __restrict__ path_tab, LevelDesc lv, int write_root, bf16* __restrict__ z,
                                                           size_t z_ps, int T_rows, int kp1, int d_model, int vocab, int* status) {
   pdl_trigger();
   pdl_wait();
   const int row = blockIdx.x, b = row / lv.n_parents, j = row % lv.n_parents;
   const int blk = blockIdx.y;                               // 0: hidden, 1..d: path tokens root..parent
   const int p = lv.parents[j];
-  T* dst = z + ((size_t)row * (lv.d + 1) + blk) * d_model;
+  bf16* dst = z + ((size_t)row * (lv.d + 1) + blk) * d_model;
   if (blk == 0) {                                          // 16-byte pieces (d_model is a multiple of 4)
     for (int i = threadIdx.x * 4; i < d_model; i += blockDim.x * 4)
-      put4<T>(dst + i, z_ps, *reinterpret_cast<const float4*>(hprime + (size_t)b * d_model + i));
+      put4<bf16>(dst + i, z_ps, *reinterpret_cast<const float4*>(hprime + (size_t)b * d_model + i));
     if (write_root && j == 0 && threadIdx.x == 0) tree_tok[b * T_rows] = root_tok[b];
     return;
   }
   int node = path_tab[p * kp1 + (blk - 1)];
   int t = node == 0 ? root_tok[b] : tree_tok[b * T_rows + node];
   if (t < 0 || t >= vocab) { if (threadIdx.x == 0) atomicOr(status, ST_BOUNDS); t = 0; }
-  const T* e = embed + (size_t)t * d_model;
-  for (int i = threadIdx.x * 4; i < d_model; i += blockDim.x * 4) put4<T>(dst + i, z_ps, load4<T>(e + i));      // embeddings are exact: lo = 0
+  const bf16* e = embed + (size_t)t * d_model;
+  for (int i = threadIdx.x * 4; i < d_model; i += blockDim.x * 4) put4<bf16>(dst + i, z_ps, load4<bf16>(e + i));      // embeddings are exact: lo = 0
 }
 hydra_status head_gather(const float* hprime, const void* embed, const int* root_tok, int* tree_tok, const int* path_tab,
-                         LevelDesc lv, int write_root, void* z, size_t z_ps, int batch, int T, int kp1, int d_model, int vocab, int dtype,
+                         LevelDesc lv, int write_root, void* z, size_t z_ps, int batch, int T, int kp1, int d_model, int vocab,
                          int* status, cudaStream_t st) {
   dim3 grid(batch * lv.n_parents, lv.d + 1);
-  if (dtype == 0)
-    launch_pdl(head_gather_kernel<float>, dim3(grid), dim3(256), 0, st, hprime, (const float*)embed, root_tok, tree_tok, path_tab, lv, write_root,
-               (float*)z, z_ps, T, kp1, d_model, vocab, status);
-  else
-    launch_pdl(head_gather_kernel<bf16>, dim3(grid), dim3(256), 0, st, hprime, (const bf16*)embed, root_tok, tree_tok, path_tab, lv, write_root,
+  launch_pdl(head_gather_kernel, grid, dim3(256), 0, st, hprime, (const bf16*)embed, root_tok, tree_tok, path_tab, lv, write_root,
                (bf16*)z, z_ps, T, kp1, d_model, vocab, status);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
@@ -1157,9 +1103,9 @@ hydra_status head_gather(const float* hprime, const void* embed, const int* root
 // Four columns per thread in small CTAs (a level has 1 to a few dozen rows); the bias and the slot counts before the wait.
 // VEC: the bias, a caller's vector, lies on a boundary of four elements.
 constexpr int HEAD_ACT_THREADS = 64;
-template <typename T, bool VEC>
+template <bool VEC>
 __global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float* res, int res_is_hprime, int rows_per_b, const float* part,
-                                SplitDesc sd, const T* __restrict__ bias, float* y_out, T* __restrict__ yb, size_t yb_ps,
+                                SplitDesc sd, const bf16* __restrict__ bias, float* y_out, bf16* __restrict__ yb, size_t yb_ps,
                                 int rows, int d) {
   pdl_trigger();
   const int d4 = d / 4, p = blockIdx.x * blockDim.x + threadIdx.x, r = p / d4, c = (p - r * d4) * 4;
@@ -1174,18 +1120,14 @@ __global__ void __launch_bounds__(HEAD_ACT_THREADS) head_act_kernel(const float*
   sum_slots_multi<1, 12>(part, sd.stride, off, ns, acc);
   const float4 y = make_float4(base.x + silu_f(v.x + acc[0].x), base.y + silu_f(v.y + acc[0].y), base.z + silu_f(v.z + acc[0].z), base.w + silu_f(v.w + acc[0].w));
   *reinterpret_cast<float4*>(y_out + off[0]) = y;
-  put4<T>(yb + off[0], yb_ps, y);
+  put4<bf16>(yb + off[0], yb_ps, y);
 }
 hydra_status head_act(const float* res, int res_is_hprime, int rows_per_b, const float* part, SplitDesc sd,
-                      const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, int dtype, cudaStream_t st) {
+                      const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, cudaStream_t st) {
   if (d & 3) return HYDRA_ERR_UNSUPPORTED;
   const unsigned grid = (unsigned)(((size_t)rows * d / 4 + HEAD_ACT_THREADS - 1) / HEAD_ACT_THREADS);
-  auto go = [&](auto zero, auto kernel) {
-    typedef decltype(zero) T;
-    launch_pdl(kernel, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd, (const T*)bias, y_out, (T*)yb, yb_ps, rows, d);
-  };
-  if (dtype == 0) on_vec4((const float*)bias) ? go(float{}, head_act_kernel<float, true>) : go(float{}, head_act_kernel<float, false>);
-  else on_vec4((const bf16*)bias) ? go(bf16{}, head_act_kernel<bf16, true>) : go(bf16{}, head_act_kernel<bf16, false>);
+  launch_pdl(on_vec4((const bf16*)bias) ? head_act_kernel<true> : head_act_kernel<false>, dim3(grid), dim3(HEAD_ACT_THREADS), 0, st, res, res_is_hprime, rows_per_b, part, sd,
+             (const bf16*)bias, y_out, (bf16*)yb, yb_ps, rows, d);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

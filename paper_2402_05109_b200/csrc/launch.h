@@ -33,20 +33,19 @@ hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, i
 hydra_status reduce_splits(const float* part, SplitDesc sd, float* out, int m, int n, cudaStream_t st);
 
 // ---- element-wise / row-wise stages of a decoder layer (dtype: 0 float, 1 bfloat16 for the "act" outputs)
-hydra_status embed_rows(const void* embed, const int* tok, float* x, int rows, int d, int vocab, int dtype, int* status,
-                        cudaStream_t st);
 // x_out = (res ? res : 0) + sum_s part[s]; if gain: xn = rmsnorm(x_out)*gain (act dtype, optional) and hn = the same in
 // float (optional).  part may be null.  x_out may alias res.
 hydra_status residual_rmsnorm(const float* res, const float* part, SplitDesc sd, float* x_out,
                               const void* gain, void* xn, size_t xn_ps, float* hn, int rows, int d, float eps, int dtype,
                               cudaStream_t st);
-// table[r][j] = (cos, sin) of (pos0[b]+depth[i]) * theta^(-2j/head_dim), evaluated in double
-hydra_status rope_table(RowSet rs, float2* table, int head_dim, float theta, cudaStream_t st);
-// q ([rows][H][hd], rotated) and the K/V cache rows (rotated K) from the QKV partial sums; float for dtype 0; for dtype 1
+// The first kernel of a forward call: table[r][j] = (cos, sin) of (pos0[b]+depth[i]) * theta^(-2j/head_dim), evaluated in double, and with tok x[r] = embed[tok[r]]
+hydra_status forward_start(RowSet rs, float2* table, int head_dim, float theta, const void* embed, const int* tok, float* x, int d, int vocab, int dtype, int* status,
+                           cudaStream_t st);
+// bfloat16 path: q ([rows][H][hd], rotated) and the K/V cache rows (rotated K) from the QKV partial sums;
 // float16 with a lo plane (f16(v - f16(v))) q_ps / kv_ps elements after the hi plane (0: hi only).  kv_only: the projection has the
 // 2 d columns of K and V, q is not written.
 hydra_status qkv_rope_store(const float* part, SplitDesc sd, const float2* table, void* q, size_t q_ps, void* kcache, void* vcache,
-                            size_t kv_ps, RowSet rs, int n_heads, int head_dim, int max_seq, int dtype, bool kv_only, int* status, cudaStream_t st);
+                            size_t kv_ps, RowSet rs, int n_heads, int head_dim, int max_seq, bool kv_only, int* status, cudaStream_t st);
 // Float model path: SIMT kernel + combine kernel, partial rows of ATT_CHUNK_ROWS-row chunks in `scratch`
 // (attention_scratch_bytes).  q, caches and out are float.
 constexpr int ATT_CHUNK_ROWS = 128;
@@ -66,15 +65,14 @@ hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, co
                                bf16* out, size_t out_ps, int n_heads, int head_dim, int max_seq, int len_upper, int* status,
                                bool stable_lengths, cudaStream_t st);
 constexpr int ATT_BLOCK_ROWS = 128;
-hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, int dtype,
-                      cudaStream_t st);
+hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, cudaStream_t st);
 // amax[r] = argmax_v of the summed partial logits (lowest id among equal maxima); the sums go to logits_out if given
 // scratch: topk_scratch_bytes(rows_cap, vocab) bytes of candidate storage
 size_t topk_scratch_bytes(int rows, int vocab);
 hydra_status argmax_rows(const float* part, SplitDesc sd, float* logits_out, int* amax, void* scratch, int rows_cap, int rows,
                          int vocab, cudaStream_t st);
 
-// ---- Hydra heads
+// ---- draft heads
 struct LevelDesc {           // one tree level d (1-based): the parents that have children
   int d, n_parents;
   const int* parents;        // device [n_parents] row ids
@@ -82,11 +80,11 @@ struct LevelDesc {           // one tree level d (1-based): the parents that hav
 // z[b*P+j] = [hprime[b] ; E[tok[b][path(parent j)]]] in act dtype (lv.d path tokens; lv.d = 0: the hidden state alone);
 // with write_root also tree_tok[b][0] = root_tok[b].
 hydra_status head_gather(const float* hprime, const void* embed, const int* root_tok, int* tree_tok, const int* path_tab,
-                         LevelDesc lv, int write_root, void* z, size_t z_ps, int batch, int T, int kp1, int d_model, int vocab, int dtype,
+                         LevelDesc lv, int write_root, void* z, size_t z_ps, int batch, int T, int kp1, int d_model, int vocab,
                          int* status, cudaStream_t st);
 // y_out = res + silu(sum_s part[s] + bias); res row = hprime[b] when res_is_hprime else y row.  yb = act-dtype copy.
 hydra_status head_act(const float* res, int res_is_hprime, int rows_per_b, const float* part, SplitDesc sd,
-                      const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, int dtype, cudaStream_t st);
+                      const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, cudaStream_t st);
 // Children of a level in two steps.  The max_children best tokens of every logits row, descending (ties: lower id first); the logits are the
 // summed partials, also written to `logits` [rows][vocab].  Then the children of parent j of sequence b = the first n_child of row row0 + b*P+j's;
 // shared_rows: the level has ONE row per sequence (sequentially independent heads), row0 + b, and every parent takes its children from that.
@@ -98,6 +96,22 @@ hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, 
 // Both, for a level whose rows are its own.
 hydra_status topk_children(const float* part, SplitDesc sd, float* logits, LevelDesc lv, int max_children, const int* first_child, const int* n_child,
                            int* tree_tok, void* scratch, int rows_cap, int batch, int T, int vocab, cudaStream_t st);
+
+// ---- float path: products with what follows them (float_path.cu).  w rows, x and gain on four elements; sums in one slot
+// out[m][n] = x[m][k] w[n][k]^T.  w_const as in gemm_simt
+hydra_status f32_gemm(const float* x, const float* w, float* out, int m, int n, int k, bool w_const, cudaStream_t st);
+// out[m][n] = res[m][n] + x[m][k] w[n][k]^T; out may be res
+hydra_status f32_add(const float* x, const float* w, const float* res, float* out, int m, int n, int k, cudaStream_t st);
+// act[m][f] = SiLU(gate) * up of rmsnorm(x)*gain, w [2 f][d]: gate rows, then up rows
+hydra_status f32_glu(const float* x, const float* gain, const float* w, float* act, int m, int f, int d, float eps, cudaStream_t st);
+// qkv_rope_store of the projection of rmsnorm(x)*gain; w [3 d][d], or the [2 d][d] of K and V (kv_only)
+hydra_status f32_qkv(const float* x, const float* gain, const float* w, const float2* table, float* q, float* kc, float* vc, RowSet rs, int n_heads, int head_dim, int max_seq,
+                     bool kv_only, float eps, int* status, cudaStream_t st);
+// first layer of a head: y = h' + SiLU(W [h' ; E of lv.d path tokens] + bias), rows (sequence, parent); write_root as in head_gather
+hydra_status f32_head_first(const float* hprime, const float* embed, const int* root_tok, int* tree_tok, const int* path_tab, LevelDesc lv, int write_root,
+                            const float* w, const float* bias, float* y, int batch, int T, int kp1, int d_model, int vocab, int* status, cudaStream_t st);
+// a further layer: y = y_in + SiLU(W y_in + bias); y is another buffer than y_in
+hydra_status f32_head_next(const float* y_in, const float* w, const float* bias, float* y, int m, int d, cudaStream_t st);
 
 // ---- acceptance + compaction (one kernel)
 struct AcceptArgs {

@@ -102,11 +102,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + __expf(-x)); }
 
-// Where the partial sums of a GEMM output element live.  The tensor-core GEMM cuts the (tile, k-block) line
-// into ranges of q units per CTA; tile t = (n >> bn_shift) * m_tiles + m / mt (weight tiles of
-// 128 or 256 rows; the row tiles that read the same weights are neighbours) owns units [t*kb, (t+1)*kb), so its
-// partial sums sit in slots 0 .. split_count-1 (slot s at part + s*stride + m*N + n), one per CTA that
-// touched the tile, in CTA order.  A single-slot output is described by q = kb = 1.
+// Where the partial sums of a GEMM output element live.  The tensor-core GEMM lays its (tile, k-block) pairs out in one line and cuts it
+// into ranges of q units; tile t = (n >> bn_shift) * m_tiles + m / mt (weight tiles of 128 or 256 rows; mt: the rows of a group of row tiles that walk
+// the line together) owns units [t*kb, (t+1)*kb), so its
+// partial sums sit in slots 0 .. split_count-1 (slot s at part + s*stride + m*N + n), one per range that
+// touches the tile, in their order.  A single-slot output is described by q = kb = 1.
 struct SplitDesc {
   int q, kb, m_tiles, mt, bn_shift;
   unsigned long long q_inv, mt_inv;      // ceil(2^63 / q), ceil(2^32 / mt)
@@ -119,7 +119,7 @@ struct SplitDesc {
   __host__ __device__ unsigned div_q(unsigned u) const {
     return (unsigned)(((unsigned long long)u * (unsigned)(q_inv >> 32) + ((unsigned long long)u * (unsigned)q_inv >> 32)) >> 31);
   }
-  // m / mt, exact while m mt < 2^32; row tiles of 256 (every m above 4096 has tiles of more than 240, that is 256 rows) are exact for all m
+  // m / mt, exact while m mt < 2^32; other mt than 256 and 4096, which are exact for all m, come with at most 65536 rows
   __host__ __device__ int div_mt(int m) const { return (int)(((unsigned)m * mt_inv) >> 32); }
 };
 __host__ __device__ __forceinline__ int split_count(const SplitDesc& sd, int m, int n) {

@@ -13,6 +13,13 @@
 // possibly whole tiles, and the head of another; each such run is a "segment" whose partial sum goes to
 // slot (CTA - first CTA of the tile) of the partial buffer.  The consumer kernel adds the slots of a tile in
 // fixed order (SplitDesc), so results are deterministic.
+// Several row tiles: the line is that of the weight tiles alone, and a group of neighbouring CTAs, one for each row tile, walks a range of it together, so
+// that they read the same weights at the same time and those come from memory once.  (One line of all tiles, row tiles next to each other, had them read the same
+// weights a third of the kernel's time apart: 768 x 22016 x 4096 read 505 MB, 203 so, for 180 MB of weights; 768 x 4096 x 11008 147 and 124.  The tensor cores
+// run at the clock that power leaves them, so it shows in time: layers of a 7B prompt pass of 768 / 675 / 512 / 300 rows 544 / 523 / 382 / 274 -> 522 / 488 / 371 / 250 us,
+// of the 13B shape 768 rows 901 -> 876, of the 33B shape 512 rows 884 -> 849.  Weights marked to go first: 6 us less a 7B layer than left to the L2.)
+// (Ranges that end with the tiles where that makes them at most 5 % longer - 144 whole tiles of 768 x 12288 on 147 CTAs - leave fewer partial sums, 522 -> 500 us,
+// but longer ones, and with those the error below: 6.6e-6 -> 9.3e-6.  Not done.)
 //
 // A unit is 64 k of NH = 1 or 2 weight tiles of 128 rows (one TMA box, one accumulator each) that share the activation tile.
 //
@@ -161,7 +168,7 @@ __device__ __forceinline__ void sum_tile(const float* part, size_t stride, int s
 struct GemmArgs {
   float* part; size_t slot_stride;
   float* out; GemmArrivals arr;            // REDUCE only: the output, and per tile how many of its CTAs have stored
-  int m, n, kb, m_tiles, total_units, q;
+  int m, n, kb, group, m_blocks, total_units, q;      // group: CTAs (row tiles) that walk a range together; m_blocks: groups of row tiles
   int x_lo_rows;                 // row offset of the lo plane inside the activation tensor map (0: single plane)
   // activation rows per tile, boxes (planes) of a stage, MMA passes over a weight tile and columns of one, ring stages,
   // accumulator columns and buffers, tensor-memory columns
@@ -220,7 +227,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __shared__ int s_abort, s_last;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int u_begin = blockIdx.x * a.q;
+  // this CTA's range of the line, and which of its group's row tiles is its own
+  const int range = blockIdx.x / a.group, member = blockIdx.x - range * a.group, u_begin = range * a.q;
   const int u_end = min(u_begin + a.q, a.total_units);
   const int n_units = u_end - u_begin, ring = n_units < stages ? n_units : stages, pre = a.w_const ? (ring + 1) / 2 : 0;     // pre: weight tiles requested up front
 
@@ -236,8 +244,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // (The weight tiles of a whole ring are 128 KB an SM at 64 rows and 160 KB at one, 19 and 24 MB over the SMs; the preceding row-wise kernel's
     // loads queue behind them.  7B shape, 32 steps with a 64-row tree 145.2 -> 144.0 ms with half a ring, runs of one side 0.3 % apart; without a
     // tree, and 47 supplied rows, the same either way.  All stages but one gained as much as half, one stage alone nothing.)
-    const uint64_t pol = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal();
-    int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_tiles * BN;
+    const uint64_t pol = policy_evict_first();
+    int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_blocks * BN;
     for (int i = 0; i < (a.w_const ? pre : ring); ++i) {
       if (!a.w_const) {
         tma_prefetch_2d(&tmW, kb * BLOCK_K, nrow);
@@ -245,7 +253,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         mbar_arrive_expect_tx(full_bar(i), W_BYTES);
         tma_load_2d(tiles + i * stage_bytes, &tmW, kb * BLOCK_K, nrow, full_bar(i), pol);
       }
-      if (++kb == a.kb) { kb = 0; nrow = ++tile / a.m_tiles * BN; }
+      if (++kb == a.kb) { kb = 0; nrow = ++tile / a.m_blocks * BN; }
     }
   }
   if (warp == 1) tmem_alloc(tmem_slot, a.tmem_cols);
@@ -258,13 +266,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint64_t pol_w = a.m_tiles == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
+      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
       int kcol = 0, nrow = 0, mrow = 0;                  // (k column, weight row, activation row) of the unit being issued, advanced without divisions
       if (n_units > 0) {
         const int tile = u_begin / a.kb;
-        kcol = (u_begin - tile * a.kb) * BLOCK_K; nrow = tile / a.m_tiles * BN; mrow = tile % a.m_tiles * a.mt;
+        kcol = (u_begin - tile * a.kb) * BLOCK_K; nrow = tile / a.m_blocks * BN; mrow = (tile % a.m_blocks * a.group + member) * a.mt;
       }
-      const int kend = a.kb * BLOCK_K, mend = a.m_tiles * a.mt;
+      const int kend = a.kb * BLOCK_K, mstep = a.group * a.mt, mend = a.m_blocks * mstep;
       int s = 0; uint32_t eph = 1;                       // ring stage, parity of its empty barrier
       grid_dep_wait();                                   // activations are the preceding kernel's output
       for (int i = 0; i < n_units; ++i) {
@@ -280,7 +288,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         tma_load_2d(dst + W_BYTES, &tmX, kcol, mrow, full_bar(s), pol_x);
         if (a.x_boxes == 2) tma_load_2d(dst + W_BYTES + x_box_bytes, &tmX, kcol, mrow + a.x_lo_rows, full_bar(s), pol_x);
         if (++s == stages) { s = 0; eph ^= 1u; }
-        if ((kcol += BLOCK_K) == kend) { kcol = 0; if ((mrow += a.mt) == mend) { mrow = 0; nrow += BN; } }
+        if ((kcol += BLOCK_K) == kend) { kcol = 0; if ((mrow += mstep) >= mend) { mrow -= mend; nrow += BN; } }
       }
     }
   } else if (warp == 1) {
@@ -329,8 +337,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     uint32_t acc_ph = 0;
     for (int i = 0, tile = u_begin / a.kb; i < n_units; ++tile) {
       // where the segment goes, worked out while its accumulator fills
-      const int seg_len = min((tile + 1) * a.kb, u_end) - (u_begin + i), slot = (int)blockIdx.x - tile * a.kb / a.q;
-      const int n_tile = tile / a.m_tiles, n0 = n_tile * BN, m0 = (tile - n_tile * a.m_tiles) * a.mt, rows = min(a.mt, a.m - m0);
+      const int seg_len = min((tile + 1) * a.kb, u_end) - (u_begin + i), slot = range - tile * a.kb / a.q;
+      const int n_tile = tile / a.m_blocks, n0 = n_tile * BN, m0 = ((tile - n_tile * a.m_blocks) * a.group + member) * a.mt, rows = min(a.mt, a.m - m0);
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * NH * a.acc_cols);
       float* dst = a.part + (size_t)slot * a.slot_stride + (size_t)m0 * a.n + n0 + quarter * 32 + lane;
       if (REDUCE && threadIdx.x == 64) atomicMax(a.arr.count + tile, a.arr.ticket << 16);      // an older call's count, if one is left, is gone
@@ -415,32 +423,46 @@ static GemmShape gemm_shape(int m, int n, int k) {
   return GemmShape{wide ? 2 : 1, mt, (m + mt - 1) / mt};
 }
 
-// Stream-K plan: equal contiguous unit ranges, one per CTA, at most one CTA per SM and at least 4 k-blocks each.
-SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap) {
-  SplitDesc sd{};
-  const GemmShape sh = gemm_shape(m, n, k);
-  sd.mt = sh.mt; sd.m_tiles = sh.m_tiles; sd.kb = k / BLOCK_K; sd.stride = (size_t)m * n;
-  sd.bn_shift = sh.nh == 2 ? 8 : 7;
-  const int tiles = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles;
-  const long long total = (long long)tiles * sd.kb;
-  long long g = sm_count();
-  if (g > total / 4) g = total / 4 > 0 ? total / 4 : 1;
-  sd.q = (int)((total + g - 1) / g);
-  if (max_slots || part_cap) {
-    auto slots = [&]() {                                   // CTAs that touch a tile, at most: tile t begins rem units into a CTA's range
-      const unsigned q = (unsigned)sd.q, kb = (unsigned)sd.kb, top = (q + kb - 2) / q + 1;
+// Stream-K plan: equal contiguous ranges of the line, at most one CTA per SM and at least 4 k-blocks each.
+constexpr int GROUP_MAX = 16;            // (a prompt pass has at most 3 row tiles, 64 sequences of a 64-row tree 16)
+struct GemmPlan { GemmShape sh; int group, ranges, max_slots; SplitDesc sd; };
+static GemmPlan gemm_plan(int m, int n, int k, bool want_slots, size_t part_cap) {
+  GemmPlan p{};
+  p.sh = gemm_shape(m, n, k);
+  SplitDesc& sd = p.sd;
+  const int kb = k / BLOCK_K, sms = sm_count(), n_tiles = p.sh.nh == 2 ? (n + 255) / 256 : n / BLOCK_N;
+  const long long total = (long long)n_tiles * p.sh.m_tiles * kb;
+  const int blocks = total / 4 >= sms ? (p.sh.m_tiles + GROUP_MAX - 1) / GROUP_MAX : p.sh.m_tiles;
+  p.group = (p.sh.m_tiles + blocks - 1) / blocks;
+  sd.kb = kb; sd.stride = (size_t)m * n; sd.bn_shift = p.sh.nh == 2 ? 8 : 7; sd.m_tiles = blocks; sd.mt = p.group * p.sh.mt;
+  const int tiles = n_tiles * blocks;
+  const long long line = (long long)tiles * kb;
+  long long g = sms / p.group;
+  if (g > line / 4) g = line / 4 > 0 ? line / 4 : 1;
+  sd.q = (int)((line + g - 1) / g);
+  if (want_slots || part_cap) {
+    auto slots = [&]() {                                   // ranges that touch a tile, at most: tile t begins rem units into a range
+      const unsigned q = (unsigned)sd.q, kbu = (unsigned)sd.kb, top = (q + kbu - 2) / q + 1;
       unsigned mx = 1, rem = 0;
-      for (int t = 0; t < tiles && mx < top; ++t, rem = (rem + kb) % q) mx = std::max(mx, (rem + kb - 1) / q + 1);
+      for (int t = 0; t < tiles && mx < top; ++t, rem = (rem + kbu) % q) mx = std::max(mx, (rem + kbu - 1) / q + 1);
       return (int)mx;
     };
-    int mx = slots();
-    // whole tiles per CTA need one slot
-    while (part_cap && mx > 1 && (size_t)mx * sd.stride > part_cap) { sd.q = sd.q < sd.kb ? sd.q + 1 : (sd.q + sd.kb) / sd.kb * sd.kb; mx = slots(); }
-    if (max_slots) *max_slots = mx;
+    p.max_slots = slots();
+    // whole tiles per range need one slot
+    while (part_cap && p.max_slots > 1 && (size_t)p.max_slots * sd.stride > part_cap) {
+      sd.q = sd.q < kb ? sd.q + 1 : (sd.q + kb) / kb * kb;
+      p.max_slots = slots();
+    }
   }
-  if (grid) *grid = (int)((total + sd.q - 1) / sd.q);
+  p.ranges = (int)((line + sd.q - 1) / sd.q);
   sd.set_inverses();
-  return sd;
+  return p;
+}
+SplitDesc gemm_tc_plan(int m, int n, int k, int* grid, int* max_slots, size_t part_cap) {
+  const GemmPlan p = gemm_plan(m, n, k, max_slots != nullptr, part_cap);
+  if (grid) *grid = p.ranges * p.group;
+  if (max_slots) *max_slots = p.max_slots;
+  return p.sd;
 }
 
 hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* w, float* part, int m, int n, int k,
@@ -448,30 +470,31 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
                      const GemmArrivals* arrivals, int x_row0) {
   if (m <= 0 || n <= 0 || k <= 0 || n % BLOCK_N || k % BLOCK_K || (x_planes != 1 && x_planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & 15) return HYDRA_ERR_INVALID;
-  int grid = 1;
-  const SplitDesc sd = gemm_tc_plan(m, n, k, &grid, nullptr, part_cap);
-  const GemmShape sh = gemm_shape(m, n, k);
+  const GemmPlan plan = gemm_plan(m, n, k, false, part_cap);
+  const SplitDesc& sd = plan.sd;
+  const GemmShape& sh = plan.sh;
+  const int grid = plan.ranges * plan.group;
   if (x_rows_alloc < x_row0 + m) x_rows_alloc = x_row0 + m;
   x += (size_t)x_row0 * k;
   GemmArgs a{};
-  a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.m_tiles = sd.m_tiles; a.mt = sd.mt;
-  a.total_units = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles * sd.kb; a.q = sd.q; a.status = status;
+  a.part = part; a.slot_stride = sd.stride; a.m = m; a.n = n; a.kb = sd.kb; a.mt = sh.mt;
+  a.group = plan.group; a.m_blocks = sd.m_tiles; a.total_units = ((n + (1 << sd.bn_shift) - 1) >> sd.bn_shift) * sd.m_tiles * sd.kb; a.q = sd.q; a.status = status;
   a.x_lo_rows = x_planes == 2 ? x_rows_alloc : 0; a.diag = diag;
   a.wait_limit = dbg && dbg->wait_limit ? dbg->wait_limit : WAIT_LIMIT; a.skip_unit = dbg ? dbg->skip_unit : -1; a.w_const = w_const;
   // Two planes, up to 128 rows: the hi and lo activation tiles sit back to back and form ONE MMA operand of 2 mt rows, so each
   // weight tile is read from shared memory once; taller tiles take a pass per plane.
-  a.cat = x_planes == 2 && sd.mt <= 128;
+  a.cat = x_planes == 2 && sh.mt <= 128;
   a.passes = x_planes == 2 && !a.cat ? 2 : 1;
-  a.x_boxes = x_planes; a.mma_n = a.cat ? 2 * sd.mt : sd.mt;
-  const int read_cols = (sd.mt + 31) / 32 * 32;          // the epilogue reads whole batches of 32 columns
-  a.acc_cols = a.cat ? sd.mt + read_cols : read_cols;
+  a.x_boxes = x_planes; a.mma_n = a.cat ? 2 * sh.mt : sh.mt;
+  const int read_cols = (sh.mt + 31) / 32 * 32;          // the epilogue reads whole batches of 32 columns
+  a.acc_cols = a.cat ? sh.mt + read_cols : read_cols;
   a.acc_bufs = 2 * sh.nh * a.acc_cols <= 512 ? 2 : 1;
   for (a.tmem_cols = 32; a.tmem_cols < a.acc_bufs * sh.nh * a.acc_cols;) a.tmem_cols *= 2;
-  const int stage_bytes = sh.nh * A_BYTES + a.x_boxes * sd.mt * BLOCK_K * 2;
+  const int stage_bytes = sh.nh * A_BYTES + a.x_boxes * sh.mt * BLOCK_K * 2;
   a.stages = RING_BYTES / stage_bytes < MAX_STAGES ? RING_BYTES / stage_bytes : MAX_STAGES;
   CUtensorMap tw, tx;
   if (!get_tensor_map(w, (uint64_t)n, (uint64_t)k, (uint32_t)(sh.nh * BLOCK_N), false, &tw) ||
-      !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes - x_row0, (uint64_t)k, (uint32_t)sd.mt, false, &tx)) {      // what the buffer holds from x on; rows past it read as zeros
+      !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes - x_row0, (uint64_t)k, (uint32_t)sh.mt, false, &tx)) {      // what the buffer holds from x on; rows past it read as zeros
     set_last_error("cuTensorMapEncodeTiled", cudaErrorUnknown);
     return HYDRA_ERR_CUDA;
   }

@@ -22,6 +22,19 @@ def test_gemm_tile_edges(m, n, k):
         assert float((out - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
 
 
+@pytest.mark.parametrize("m", [4097, 4360])
+@pytest.mark.parametrize("n,k", [(1152, 1024), (4224, 2048)])
+def test_gemm_groups_of_row_tiles(m, n, k):
+    """More row tiles than walk the weights together: two groups of 9, with 4097 rows one of the 18 places empty."""
+    from paper_2402_05109_b200 import gemm
+    x = normal_(torch.empty(m, k, device="cuda"), 77, m, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 78, n, 0.02)
+    planes = split_hi_lo(x)
+    ref = planes.double().sum(0) @ w.double().T
+    # as above
+    assert float((gemm(planes, w, mode=0).double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 128, 64), (1, 256, 256), (11, 2048, 2048), (16, 640, 5632), (16, 1408, 4288), (17, 1408, 4288), (3, 4096, 4096)])
 def test_gemm_noalloc_one_and_two_launches(m, n, k):
     """Both sides of the choice between adding the partial sums in the GEMM's own launch and in a second one; several calls in a

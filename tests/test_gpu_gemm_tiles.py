@@ -22,6 +22,20 @@ def test_gemm_tile_edges(m, n, k):
         assert float((out - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
 
 
+@pytest.mark.parametrize("m", [96, 97, 112, 128])
+@pytest.mark.parametrize("n", [18816, 18944, 19072])
+def test_gemm_wide_units_at_97_to_128_rows(m, n):
+    """Both sides of the lines in rows and in width, and an output that ends inside its last unit."""
+    from paper_2402_05109_b200 import gemm
+    k = 320
+    x = normal_(torch.empty(m, k, device="cuda"), 79, m, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 80, n, 0.02)
+    planes = split_hi_lo(x)
+    ref = planes.double().sum(0) @ w.double().T
+    # as above
+    assert float((gemm(planes, w, mode=0).double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
+
+
 @pytest.mark.parametrize("m", [4097, 4360])
 @pytest.mark.parametrize("n,k", [(1152, 1024), (4224, 2048)])
 def test_gemm_groups_of_row_tiles(m, n, k):

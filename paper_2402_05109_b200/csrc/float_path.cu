@@ -23,6 +23,9 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 __device__ __forceinline__ float dot4(float4 a, float4 b, float s) { return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s)))); }
 __device__ __forceinline__ float4 mul4(float4 a, float4 b) { return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w); }
 
+// Row n[b] - 1 of sequence b's tc rows (n null: its only one).
+__device__ __forceinline__ const float* last_row(const LastRows& h, int b, int d) { return h.rows + ((size_t)b * h.tc + (h.n ? max(h.n[b] - 1, 0) : 0)) * d; }
+
 // ---- where the rows of x come from.  prepare() waits for the preceding kernel and readies rows m0 .. m0 + R - 1; at(r, k): four elements of row m0 + r.
 // tab: smem(R) bytes of shared memory.
 struct Rows {
@@ -33,7 +36,7 @@ struct Rows {
 };
 // [h' ; E of the lv.d path tokens] of row (sequence, parent), read where they are; with write_root also tree_tok[b][0] = root_tok[b]
 struct HeadRows {
-  const float *hprime, *embed;
+  LastRows h; const float* embed;
   const int *root_tok, *path_tab; int* tree_tok;
   LevelDesc lv;
   int write_root, T, kp1, vocab, m, d;
@@ -45,7 +48,7 @@ struct HeadRows {
       const int r = min(m0 + e / blocks, m - 1), blk = e % blocks, b = r / lv.n_parents, j = r - b * lv.n_parents;
       const int node = blk ? path_tab[lv.parents[j] * kp1 + blk - 1] : 0;       // (tables, older than any call)
       pdl_wait();
-      const float* src = hprime + (size_t)b * d;
+      const float* src = last_row(h, b, d);
       if (blk) {
         int t = node == 0 ? root_tok[b] : tree_tok[b * T + node];
         if (t < 0 || t >= vocab) { atomicOr(status, ST_BOUNDS); t = 0; }
@@ -57,6 +60,11 @@ struct HeadRows {
     }
     pdl_wait();
     __syncthreads();
+    if (h.copy && blockIdx.x == 0)                         // (one parent a sequence then: row r is sequence r)
+      for (int e = threadIdx.x * 4; e < R * d; e += THREADS * 4) {
+        const int r = e / d;
+        if (m0 + r < m) *reinterpret_cast<float4*>(h.copy + (size_t)m0 * d + e) = ld4(static_cast<const float* const*>(tab)[r * blocks] + (e - r * d));
+      }
   }
   __device__ __forceinline__ const float* at(int, int r, int kk, const void* tab) const {      // (d % 4 == 0: four elements lie in one block)
     const int blk = kk / d;
@@ -69,6 +77,16 @@ struct HeadRows {
 struct Plain {
   static constexpr int NC = 1; static constexpr bool NORM = false;
   float* out; int n;
+  struct Pre {};
+  int units() const { return n; }
+  __device__ __forceinline__ int w_row(int u, int) const { return u; }
+  __device__ __forceinline__ Pre load(int, int) const { return Pre{}; }
+  __device__ __forceinline__ void store(int row, int u, const Pre&, const float (&s)[1]) const { out[(size_t)row * n + u] = s[0]; }
+};
+// the product of rmsnorm(x) * gain, and those rows themselves
+struct NormedOut {
+  static constexpr int NC = 1; static constexpr bool NORM = true;
+  float *out, *hn; int n;
   struct Pre {};
   int units() const { return n; }
   __device__ __forceinline__ int w_row(int u, int) const { return u; }
@@ -100,7 +118,6 @@ struct Qkv {
   int H, hd, max_seq, first; int* status;
   struct Pre { float2 cs; int b, slot; };                  // slot -2: a row that the call does not have
   int units() const { return (3 - first) * H * (hd >> 1); }
-  __device__ __forceinline__ int head_of(int u) const { return u / (hd >> 1); }       // heads of q, k and v in a row
   __device__ __forceinline__ int w_row(int u, int c) const { const int half = hd >> 1, head = u / half; return head * hd + (u - head * half) + c * half; }
   __device__ __forceinline__ Pre load(int row, int u) const {
     const int half = hd >> 1, b = row / rs.tc, i = row - b * rs.tc;
@@ -120,16 +137,30 @@ struct Qkv {
     dst[j + half] = which < 2 ? s[1] * p.cs.x + s[0] * p.cs.y : s[1];
   }
 };
-// y = res + SiLU(s + bias), res row = row / rows_per_res
+// y = res + SiLU(s + bias), res: the last row of sequence row / rows_per_res
 struct HeadAct {
   static constexpr int NC = 1; static constexpr bool NORM = false;
-  const float *res, *bias; float* y; int d, rows_per_res;
+  LastRows res; const float* bias; float* y; int d, rows_per_res;
   struct Pre { float base, add; };
   int units() const { return d; }
   __device__ __forceinline__ int w_row(int u, int) const { return u; }
-  __device__ __forceinline__ Pre load(int row, int u) const { return Pre{res[(size_t)(row / rows_per_res) * d + u], bias ? bias[u] : 0.f}; }
+  __device__ __forceinline__ Pre load(int row, int u) const { return Pre{last_row(res, row / rows_per_res, d)[u], bias ? bias[u] : 0.f}; }
   __device__ __forceinline__ void store(int row, int u, const Pre& p, const float (&s)[1]) const { y[(size_t)row * d + u] = p.base + silu_f(s[0] + p.add); }
 };
+
+// The normed rows of a block's row group, dealt out over the blocks that share it: inv[r] of rows m0 .. m0 + R - 1 in shared memory.
+template <int R, typename Src, typename Op>
+__device__ __forceinline__ void normed_rows(const Src& src, const Op& op, const float* gain, const float* inv, int m0, int m, int k) {
+  if constexpr (std::is_same<Op, NormedOut>::value) {
+    __syncthreads();
+    for (int e = (blockIdx.x * THREADS + threadIdx.x) * 4; e < R * k; e += gridDim.x * THREADS * 4) {
+      const int r = e / k, c = e - r * k;
+      if (m0 + r >= m) break;
+      const float4 x = ld4(src.at(m0, r, c, nullptr)), g = ld4(gain + c);
+      *reinterpret_cast<float4*>(op.hn + (size_t)(m0 + r) * k + c) = make_float4(x.x * (inv[r] * g.x), x.y * (inv[r] * g.y), x.z * (inv[r] * g.z), x.w * (inv[r] * g.w));
+    }
+  }
+}
 
 // ---- few rows: one warp per output column and MR rows
 // What a warp makes of its share of the contraction: s[c] = sum_k w_c[k] x[r][k] for C weight rows, with NORM also s[C] = sum_k x[r][k]^2, of row
@@ -222,13 +253,17 @@ __global__ void __launch_bounds__(THREADS, 2) f32_rows_kernel(const Src src, con
     __syncthreads();
     if (mine) s[1] = s_mate[warp + KS][lane];
   }
-  if (!mine) return;
   if constexpr (Op::NORM) {
+    __shared__ float s_inv[MR];
     const float inv = rsqrtf(t[C] / (float)k + eps);
 #pragma unroll
     for (int c = 0; c < NC; ++c) s[c] *= inv;
+    if (std::is_same<Op, NormedOut>::value && warp == 0 && lane < MR) s_inv[warp_sum_owner<MR>(lane)] = inv;
+    if (mine) op.store(row, unit, pre, s);
+    normed_rows<MR>(src, op, gain, s_inv, m0, m, k);
+  } else {
+    if (mine) op.store(row, unit, pre, s);
   }
-  op.store(row, unit, pre, s);
 }
 
 // ---- many rows: tiles of 32 rows x 32 weight rows (32 units, or 16 of two columns).  64 k a stage come by asynchronous copies, four stages, so that d = 256 is
@@ -247,7 +282,7 @@ __global__ void __launch_bounds__(THREADS, 2) f32_tile_kernel(const Src src, con
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float* stage0 = reinterpret_cast<float*>(s_dyn);
   void* tab = s_dyn + TILE_SMEM;
-  __shared__ float s_ss[WARPS][TM];
+  __shared__ float s_ss[WARPS][TM], s_inv[TM];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, m0 = blockIdx.y * TM, u0 = blockIdx.x * UNITS, n_stages = (k + TK - 1) / TK;
   // a thread copies 16 bytes of rows cr and cr + 16 of x and of w
   const int cr = tid >> 4, ck = (tid & 15) * 4;
@@ -323,6 +358,12 @@ __global__ void __launch_bounds__(THREADS, 2) f32_tile_kernel(const Src src, con
 #pragma unroll
   for (int o = 0; o < OUT; ++o) {
     const int r = tid / UNITS + o * (THREADS / UNITS), c0 = tid % UNITS, row = m0 + r, unit = u0 + c0;
+    if (std::is_same<Op, NormedOut>::value && c0 == 0) {
+      float t = 0.f;
+#pragma unroll
+      for (int v = 0; v < WARPS; ++v) t += s_ss[v][r];
+      s_inv[r] = rsqrtf(t / (float)k + eps);
+    }
     if (row >= m || unit >= n_units) continue;
     float s[NC] = {}, t = 0.f;
 #pragma unroll
@@ -338,6 +379,7 @@ __global__ void __launch_bounds__(THREADS, 2) f32_tile_kernel(const Src src, con
     }
     op.store(row, unit, pre[o], s);
   }
+  normed_rows<TM>(src, op, gain, s_inv, m0, m, k);
 }
 static_assert(WARPS * TM * (TN + 1) <= STAGES * STAGE_FLOATS, "the warps' sums take the place of the stages");
 
@@ -398,6 +440,10 @@ hydra_status f32_gemm(const float* x, const float* w, float* out, int m, int n, 
   if (off16(x)) return HYDRA_ERR_INVALID;
   return product(Rows{x, m, k}, w, nullptr, Plain{out, n}, m, k, 0.f, w_const, st);
 }
+hydra_status f32_normed_gemm(const float* x, const float* gain, const float* w, float* out, float* hn, int m, int n, int k, float eps, cudaStream_t st) {
+  if (off16(x) || off16(hn)) return HYDRA_ERR_INVALID;
+  return product(Rows{x, m, k}, w, gain, NormedOut{out, hn, n}, m, k, eps, true, st);
+}
 hydra_status f32_add(const float* x, const float* w, const float* res, float* out, int m, int n, int k, cudaStream_t st) {
   if (off16(x)) return HYDRA_ERR_INVALID;
   return product(Rows{x, m, k}, w, nullptr, Add{res, out, n}, m, k, 0.f, true, st);
@@ -413,17 +459,18 @@ hydra_status f32_qkv(const float* x, const float* gain, const float* w, const fl
   const int m = rs.rows(), d = H * hd;
   return product(Rows{x, m, d}, w, gain, Qkv{rs, table, q, kc, vc, H, hd, max_seq, kv_only ? 1 : 0, status}, m, d, eps, true, st);
 }
-hydra_status f32_head_first(const float* hprime, const float* embed, const int* root_tok, int* tree_tok, const int* path_tab, LevelDesc lv, int write_root,
+hydra_status f32_head_first(const LastRows& h, const float* embed, const int* root_tok, int* tree_tok, const int* path_tab, LevelDesc lv, int write_root,
                             const float* w, const float* bias, float* y, int batch, int T, int kp1, int d, int vocab, int* status, cudaStream_t st) {
   if (d & 3) return HYDRA_ERR_UNSUPPORTED;
-  if (off16(hprime) || off16(embed)) return HYDRA_ERR_INVALID;
+  if (off16(h.rows) || off16(embed)) return HYDRA_ERR_INVALID;
+  if (h.copy && lv.n_parents != 1) return HYDRA_ERR_INVALID;
   const int m = batch * lv.n_parents;
-  return product(HeadRows{hprime, embed, root_tok, path_tab, tree_tok, lv, write_root, T, kp1, vocab, m, d, status}, w, nullptr, HeadAct{hprime, bias, y, d, lv.n_parents}, m,
+  return product(HeadRows{h, embed, root_tok, path_tab, tree_tok, lv, write_root, T, kp1, vocab, m, d, status}, w, nullptr, HeadAct{h, bias, y, d, lv.n_parents}, m,
                  (lv.d + 1) * d, 0.f, true, st);
 }
 hydra_status f32_head_next(const float* y_in, const float* w, const float* bias, float* y, int m, int d, cudaStream_t st) {
   if (off16(y_in)) return HYDRA_ERR_INVALID;
-  return product(Rows{y_in, m, d}, w, nullptr, HeadAct{y_in, bias, y, d, 1}, m, d, 0.f, true, st);
+  return product(Rows{y_in, m, d}, w, nullptr, HeadAct{LastRows{y_in, nullptr, 1, nullptr}, bias, y, d, 1}, m, d, 0.f, true, st);
 }
 
 }  // namespace hydra

@@ -390,8 +390,10 @@ hydra_status run_base(hydra_ctx* c, const int* tok, const RowSet& rs, int len_up
   if (m.dtype == 0) {
     for (int l = 0; l < m.n_layers; ++l)
       HYDRA_TRY(f32_layer(c, c->layers[l], c->x, c->kv_base + (size_t)(2 * l) * kvl, c->kv_base + (size_t)(2 * l + 1) * kvl, rs, len_upper, st));
-    HYDRA_TRY(residual_rmsnorm(c->x, nullptr, single_slot(0), c->x, c->final_norm, c->xn, 0, c->h_tree, rows, d, m.rms_eps, 0, st));
-    return tail_w ? run_gemm(c, c->xn, c->R, tail_w, rows, tail_n, d, tail_sd, st) : HYDRA_OK;
+    if (!tail_w) return residual_rmsnorm(c->x, nullptr, single_slot(0), c->x, c->final_norm, nullptr, 0, c->h_tree, rows, d, m.rms_eps, 0, st);
+    TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, tail_n, d), st);
+    *tail_sd = single_slot((size_t)rows * tail_n);
+    return f32_normed_gemm(c->x, (const float*)c->final_norm, (const float*)tail_w, c->part, c->h_tree, rows, tail_n, d, m.rms_eps, st);
   }
   HYDRA_TRY(residual_rmsnorm(c->x, nullptr, single_slot(0), c->x, c->layers[0].attn_norm, c->xn, ps(c, c->R, d), nullptr, rows, d, m.rms_eps, m.dtype, st));
   SplitDesc sd;
@@ -492,10 +494,10 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     HYDRA_TRY(prefix_rowset(c->d_len, c->d_n_new, c->d_pos0, c->d_nrows, B, st));
     RowSet rs{B, K + 1, c->d_nrows, c->d_pos0, c->d_chain_depth, c->d_chain_mask};
     HYDRA_TRY(run_prefix(c, c->h_new, rs, len_bucket(c, max_len_ub(c)), st));
-    HYDRA_TRY(pick_last_row(c->x, c->d_nrows, K + 1, c->hprime, B, d, st));
-  } else {
-    HYDRA_TRY(pick_last_row(c->h_new, c->d_n_new, K + 1, c->hprime, B, d, st));
   }
+  // h': the last of the rows that the prefix layer, or else the base model, took this step (float path: the first head picks them itself)
+  const LastRows last{c->h.prefix_attn ? c->x : c->h_new, c->h.prefix_attn ? c->d_nrows : c->d_n_new, K + 1, c->hprime}, hprime{c->hprime, nullptr, 1, nullptr};
+  if (dt == 1 || c->Ktree == 0) HYDRA_TRY(pick_last_row(last.rows, last.n, K + 1, c->hprime, B, d, st));
   if (c->Ktree == 0) return copy_i32(tree_tok, c->d_root_tok, B, st);      // root-only tree (T == 1)
   // W x + b of one head's layers over `rows` rows of c->z; the head's last hidden rows go to rows y0.. of c->y and c->yb
   auto head_mlp = [&](int lvl, int rows, int rows_per_b, int in_blocks, int y0) -> hydra_status {
@@ -518,7 +520,7 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     float *out = (layers & 1 ? (float*)c->yb : c->y) + (size_t)y0 * d, *other = (layers & 1 ? c->y : (float*)c->yb) + (size_t)y0 * d;
     {
       TimeScope ts(c, HYDRA_TIME_GEMM, gemm_bytes(c, rows, d, (lv.d + 1) * d), st);
-      HYDRA_TRY(f32_head_first(c->hprime, (const float*)c->embed, c->d_root_tok, tree_tok, c->d_path_tab, lv, write_root, (const float*)c->head_w1[lvl - 1],
+      HYDRA_TRY(f32_head_first(lvl == 1 ? last : hprime, (const float*)c->embed, c->d_root_tok, tree_tok, c->d_path_tab, lv, write_root, (const float*)c->head_w1[lvl - 1],
                                c->h.has_bias ? (const float*)c->head_b1[lvl - 1] : nullptr, out, B, c->T, K + 1, d, m.vocab, c->d_status, st));
     }
     for (int l = 0; l + 1 < layers; ++l, std::swap(out, other)) {

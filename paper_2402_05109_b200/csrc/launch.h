@@ -100,6 +100,8 @@ hydra_status topk_children(const float* part, SplitDesc sd, float* logits, Level
 // ---- float path: products with what follows them (float_path.cu).  w rows, x and gain on four elements; sums in one slot
 // out[m][n] = x[m][k] w[n][k]^T.  w_const as in gemm_simt
 hydra_status f32_gemm(const float* x, const float* w, float* out, int m, int n, int k, bool w_const, cudaStream_t st);
+// the same of rmsnorm(x)*gain, whose rows also go to hn
+hydra_status f32_normed_gemm(const float* x, const float* gain, const float* w, float* out, float* hn, int m, int n, int k, float eps, cudaStream_t st);
 // out[m][n] = res[m][n] + x[m][k] w[n][k]^T; out may be res
 hydra_status f32_add(const float* x, const float* w, const float* res, float* out, int m, int n, int k, cudaStream_t st);
 // act[m][f] = SiLU(gate) * up of rmsnorm(x)*gain, w [2 f][d]: gate rows, then up rows
@@ -107,8 +109,10 @@ hydra_status f32_glu(const float* x, const float* gain, const float* w, float* a
 // qkv_rope_store of the projection of rmsnorm(x)*gain; w [3 d][d], or the [2 d][d] of K and V (kv_only)
 hydra_status f32_qkv(const float* x, const float* gain, const float* w, const float2* table, float* q, float* kc, float* vc, RowSet rs, int n_heads, int head_dim, int max_seq,
                      bool kv_only, float eps, int* status, cudaStream_t st);
-// first layer of a head: y = h' + SiLU(W [h' ; E of lv.d path tokens] + bias), rows (sequence, parent); write_root as in head_gather
-hydra_status f32_head_first(const float* hprime, const float* embed, const int* root_tok, int* tree_tok, const int* path_tab, LevelDesc lv, int write_root,
+// first layer of a head: y = h' + SiLU(W [h' ; E of lv.d path tokens] + bias), rows (sequence, parent); write_root as in head_gather.  h' of sequence b is row
+// n[b] - 1 of its tc rows (n null: the only one) and goes to copy[b] as well if that is given (one parent then)
+struct LastRows { const float* rows; const int* n; int tc; float* copy; };
+hydra_status f32_head_first(const LastRows& h, const float* embed, const int* root_tok, int* tree_tok, const int* path_tab, LevelDesc lv, int write_root,
                             const float* w, const float* bias, float* y, int batch, int T, int kp1, int d_model, int vocab, int* status, cudaStream_t st);
 // a further layer: y = y_in + SiLU(W y_in + bias); y is another buffer than y_in
 hydra_status f32_head_next(const float* y_in, const float* w, const float* bias, float* y, int m, int d, cudaStream_t st);

@@ -19,8 +19,8 @@
  *    hydra_destroy.  The library owns only the opaque context; KV caches, tables and scratch are
  *    carved out of the caller's workspace (hydra_workspace_bytes, 256-byte aligned base).
  *  - Calls enqueue work on `stream` (a cudaStream_t passed as void*) and do not synchronise, except
- *    hydra_create (uploads tables; synchronises the device), hydra_prefill (synchronises the stream once,
- *    after uploading the prompt offsets, before its first kernel), hydra_poll_status, hydra_get_timing and
+ *    hydra_create (uploads tables; synchronises the device), hydra_prefill of a bfloat16 model (synchronises the stream once,
+ *    after uploading the blocks of its attention; not under stream capture), hydra_poll_status, hydra_get_timing and
  *    hydra_destroy.
  *  - Order: create -> prefill -> (draft -> verify -> accept_compact | step)*.  A call out of order
  *    returns HYDRA_ERR_STATE.  The host keeps an upper bound of every sequence length (it grows by

@@ -206,7 +206,7 @@ bool valid_cfg(const hydra_model_cfg* m, const hydra_head_cfg* h) {
 hydra_status supported_cfg(const hydra_model_cfg* m) {
   if (m->head_dim != 64 && m->head_dim != 128) return HYDRA_ERR_UNSUPPORTED;
   if (m->d_model % 4 || m->d_ffn % 4) return HYDRA_ERR_UNSUPPORTED;
-  if (m->max_batch > 64) return HYDRA_ERR_UNSUPPORTED;
+  if (m->max_batch > MAX_BATCH) return HYDRA_ERR_UNSUPPORTED;
   if (m->dtype == 1 && (m->d_model % 128 || m->d_ffn % 64 || m->vocab % 128)) return HYDRA_ERR_UNSUPPORTED;
   return HYDRA_OK;
 }
@@ -629,7 +629,9 @@ void drop_graphs(hydra_ctx* c) { c->graphs.clear(); c->rows_graphs.clear(); }
 bool capturable(cudaStream_t st) { return st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread; }      // default streams are not
 bool being_captured(cudaStream_t st) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &s) != cudaSuccess || s != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  cudaGetLastError();                              // (the default stream while another one captures)
+  return true;
 }
 // What `enqueue` puts on the stream, as a graph and not executed; *launches: kernels in it.
 template <typename F>
@@ -753,20 +755,23 @@ hydra_status hydra_prefill(hydra_ctx* c, int batch, const int32_t* tokens, const
   cudaStream_t st = (cudaStream_t)stream;
   const hydra_model_cfg& m = c->m;
   std::vector<int> plen(batch);
+  PromptOffsets po{};
   int maxlen = 0;
   for (int b = 0; b < batch; ++b) {
     plen[b] = offs[b + 1] - offs[b];
     if (plen[b] < 1) return HYDRA_ERR_INVALID;
     if (plen[b] + c->T > m.max_seq) return HYDRA_ERR_CAPACITY;
     maxlen = std::max(maxlen, plen[b]);
+    po.off[b] = offs[b];
   }
+  po.off[batch] = offs[batch];
+  // a prompt pass belongs to one request and its host-side bounds to one call: nothing to replay
+  if (being_captured(st)) { set_last_error("hydra_prefill on a stream under capture", cudaErrorStreamCaptureUnsupported); return HYDRA_ERR_CUDA; }
   c->batch = batch;
-  HYDRA_CUDA(cudaMemcpyAsync(c->d_prompt_len, plen.data(), batch * sizeof(int), cudaMemcpyHostToDevice, st));
-  HYDRA_CUDA(cudaMemcpyAsync(c->d_offsets, offs, (batch + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
+  HYDRA_TRY(set_prompts(po, batch, c->d_prompt_len, c->d_offsets, st));
   if (m.dtype == 1) {
     HYDRA_TRY(prompt_packed(c, tokens, offs, st));
   } else {
-    HYDRA_CUDA(cudaStreamSynchronize(st));         // the host vectors above go out of scope
     const int nchunks = (maxlen + CHUNK - 1) / CHUNK;
     // a chunk is a chain: row i sees the rows before it
     RowSet rs{batch, CHUNK, c->d_nrows, c->d_pos0, c->d_chain_depth, c->d_chain_mask};

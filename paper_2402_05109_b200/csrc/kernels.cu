@@ -1392,6 +1392,20 @@ cudaError_t accept_graph_update(cudaGraphExec_t exec, cudaGraphNode_t node, cons
 // ------------------------------------------------------------------------------------------------
 // Small state kernels
 // ------------------------------------------------------------------------------------------------
+__global__ void set_prompts_kernel(const PromptOffsets p, int batch, int* prompt_len, int* offsets) {
+  pdl_trigger();
+  pdl_wait();
+  for (int i = threadIdx.x; i <= batch; i += blockDim.x) {
+    offsets[i] = p.off[i];
+    if (i < batch) prompt_len[i] = p.off[i + 1] - p.off[i];
+  }
+}
+hydra_status set_prompts(const PromptOffsets& p, int batch, int* prompt_len, int* offsets, cudaStream_t st) {
+  launch_pdl(set_prompts_kernel, dim3(1), dim3(MAX_BATCH + 1), 0, st, p, batch, prompt_len, offsets);
+  HYDRA_LAUNCH_CHECK();
+  return HYDRA_OK;
+}
+
 __global__ void set_chunk_kernel(const int* prompt_len, int chunk, int tc, int* pos0, int* n_rows, int batch) {
   pdl_trigger();
   pdl_wait();

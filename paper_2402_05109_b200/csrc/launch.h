@@ -143,6 +143,10 @@ cudaError_t accept_graph_node(cudaGraph_t graph, cudaGraphNode_t* node);
 cudaError_t accept_graph_update(cudaGraphExec_t exec, cudaGraphNode_t node, const AcceptArgs& a);
 
 // ---- small state kernels
+// prompt lengths and offsets of a batch, as kernel arguments: no copy from host memory, which would have to outlive the call
+constexpr int MAX_BATCH = 64;
+struct PromptOffsets { int off[MAX_BATCH + 1]; };
+hydra_status set_prompts(const PromptOffsets& p, int batch, int* prompt_len, int* offsets, cudaStream_t st);
 hydra_status set_chunk(const int* prompt_len, int chunk, int tc, int* pos0, int* n_rows, int batch, cudaStream_t st);
 hydra_status gather_chunk_tokens(const int* tokens, const int* offsets, int chunk, int tc, int* tok_out, int batch,
                                  cudaStream_t st);

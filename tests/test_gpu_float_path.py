@@ -1,5 +1,6 @@
 """Float path: products with what follows them, in both forms (a warp per column, 32 x 32 tiles) and at their edges, over whole steps against the oracle."""
 import pytest
+import torch
 
 from synth import load_tree
 from synth.configs import ModelCfg, HeadCfg
@@ -23,3 +24,25 @@ def test_steps_against_the_oracle(model, head, tree, lens):
     assert st.steps == 3
     # rounded at 24 bits: each product and norm adds about 1e-7, and a layer amplifies what comes in by a small factor (heads: several times a layer)
     assert st.max_hidden_err < 2e-5 and st.max_logit_err < 1e-3 and st.max_hprime_err < 1e-4
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_prompt_pass_is_refused_under_stream_capture(dtype):
+    """The float path copies nothing from host memory and waits for nothing, but a prompt pass still belongs to one call."""
+    import ctypes as C
+    from paper_2402_05109_b200 import Hydra
+    from paper_2402_05109_b200.binding import lib, _stream
+    from synth import make_prompts, make_weights
+    m, h = ModelCfg(2, 256, 2, 128, 512, 1024, dtype=dtype), HeadCfg(3, 1, False)
+    g = Hydra(m, h, load_tree("tree15_d3"), {k: v.cuda() for k, v in make_weights(m, h, 7).items()}, 1, 128)
+    toks, offs = make_prompts(7, [40], m.vocab)[0].to(torch.int32).cuda(), (C.c_int32 * 2)(0, 40)
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        x += 1
+        assert lib.hydra_prefill(g._ctx, 1, toks.data_ptr(), offs, _stream()) != 0
+    graph.replay()
+    g.prefill([toks])
+    assert g.get_buffer("LEN")[0].item() == 40 and x[0].item() == 1
+    g.close()

@@ -92,7 +92,7 @@ using namespace hydra;
 
 struct hydra_ctx {
   hydra_model_cfg m; hydra_head_cfg h;
-  int T, Ktree;                                  // tree rows, tree depth
+  int T, Ktree, n_parents;                       // tree rows, tree depth, rows with children
   std::vector<int> parent, depth, first_child, n_child, path_tab;
   std::vector<uint64_t> anc;
   std::vector<std::vector<int>> level_parents;   // [Ktree]
@@ -248,8 +248,12 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
   auto* parent = b.take<int>(T); auto* depth = b.take<int>(T); auto* fc = b.take<int>(T); auto* nc = b.take<int>(T);
   auto* path_tab = b.take<int>((size_t)T * (K + 1)); auto* chain_depth = b.take<int>(2 * CHUNK);
   auto* anc = b.take<uint64_t>(T); auto* chain_mask = b.take<uint64_t>(CHUNK);
+  // the parents level by level, back to back (the list of all of them is wanted too)
   std::vector<int*> lvl;
-  for (auto& lv : t.level_parents) lvl.push_back(b.take<int>(lv.size()));
+  size_t parents = 0;
+  for (auto& lv : t.level_parents) parents += lv.size();
+  auto* all_parents = b.take<int>(parents);
+  for (auto& lv : t.level_parents) { lvl.push_back(all_parents); if (all_parents) all_parents += lv.size(); }
   auto* len = b.take<int>(m.max_batch); auto* n_new = b.take<int>(m.max_batch); auto* root = b.take<int>(m.max_batch);
   auto* status = b.take<int>(64);          // [0] status word, [8..15] where a bounded wait gave up
   auto* pos0 = b.take<int>(m.max_batch); auto* nrows = b.take<int>(m.max_batch);
@@ -279,7 +283,7 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
   if (c) {
     c->R = R; c->RH = RH; c->part_floats = part_floats; c->esize = es; c->planes = np; c->kv_esize = ces; c->kv_planes = kvp;
     c->d_parent = parent; c->d_depth = depth; c->d_first_child = fc; c->d_n_child = nc; c->d_path_tab = path_tab;
-    c->d_chain_depth = chain_depth; c->d_anc = anc; c->d_chain_mask = chain_mask; c->d_level_parents = lvl;
+    c->d_chain_depth = chain_depth; c->d_anc = anc; c->d_chain_mask = chain_mask; c->d_level_parents = lvl; c->n_parents = (int)parents;
     c->d_len = len; c->d_n_new = n_new; c->d_root_tok = root; c->d_status = status; c->d_pos0 = pos0; c->d_nrows = nrows;
     c->d_prompt_len = plen; c->d_offsets = offs; c->d_tok = tok; c->d_tree_tok = tree_tok; c->d_amax = amax; c->d_done = done;
     c->d_row_at = row_at; c->d_blocks = blocks;
@@ -548,10 +552,9 @@ hydra_status do_draft(hydra_ctx* c, int* tree_tok, cudaStream_t st) {
     }
     HYDRA_TRY(run_gemm(c, c->yb, c->RH, c->lm_head, c->Ktree * B, m.vocab, d, &sd, st));
     HYDRA_TRY(topk_candidates(c->part, sd, c->head_logits, max_children, c->topk_scratch, c->topk_rows_cap, c->Ktree * B, m.vocab, st));
-    for (int lvl = 1; lvl <= c->Ktree; ++lvl)
-      HYDRA_TRY(topk_merge(level(lvl), max_children, c->d_first_child, c->d_n_child, tree_tok, c->topk_scratch, c->topk_rows_cap, (c->Ktree - lvl) * B,
-                           B, c->T, m.vocab, 1, st));
-    return HYDRA_OK;
+    // the children of all levels in one launch (one a level: four heads at the 7B shape, 4.6 us each)
+    return topk_merge(LevelDesc{0, c->n_parents, c->d_level_parents[0]}, max_children, c->d_first_child, c->d_n_child, tree_tok, c->topk_scratch, c->topk_rows_cap, c->Ktree * B,
+                      B, c->T, m.vocab, c->d_depth, c->Ktree - 1, st);
   }
   for (int lvl = 1; lvl <= c->Ktree; ++lvl) {
     // one row per (sequence, parent), input [h' ; E of the path tokens]

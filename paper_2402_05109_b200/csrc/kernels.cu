@@ -951,23 +951,24 @@ __global__ void __launch_bounds__(256) argmax_stage1_kernel(const float* part, S
 }
 
 // out_of(row) and count_of(row): where the winners go.  lv.parents == null: argmax (one winner per row to amax[row]).
-// One warp per winner list; dynamic shared memory: nblk * c (value, index) pairs.
+// One warp per winner list; dynamic shared memory: nblk * c (value, index) pairs.  depth (sequentially independent heads): the parents of all levels at once; those at
+// depth t of sequence b share candidate row (top - t) * batch + b.
 __global__ void __launch_bounds__(32) topk_stage2_kernel(const float* cand_v, const int* cand_i,
                                                          int nblk, int c, LevelDesc lv, const int* __restrict__ first_child,
-                                                         const int* __restrict__ n_child, int* __restrict__ out, int T, int row0, int cand_div) {
+                                                         const int* __restrict__ n_child, int* __restrict__ out, int T, const int* depth, int top, int batch) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ float s_cand[];
   float* sv = s_cand;
   int* si = reinterpret_cast<int*>(s_cand + nblk * c);
   const int row = blockIdx.x, lane = threadIdx.x;
-  const int crow = row0 + row / cand_div;                  // row of the candidate lists (one per sequence when the parents share them)
   int* dst = out + row;
-  int count = 1;
+  int count = 1, crow = row;                               // crow: row of the candidate lists
   if (lv.parents) {
     const int b = row / lv.n_parents, p = lv.parents[row % lv.n_parents];
     dst = out + b * T + first_child[p];
     count = n_child[p];
+    if (depth) crow = (top - depth[p]) * batch + b;
   }
   for (int e = lane; e < nblk * c; e += 32) {
     const size_t at = ((size_t)crow * nblk + e / c) * TOPK_MAX + e % c;
@@ -1026,7 +1027,7 @@ hydra_status argmax_rows(const float* part, SplitDesc sd, float* logits_out, int
   HYDRA_LAUNCH_CHECK();
   if (direct) return HYDRA_OK;
   launch_pdl(topk_stage2_kernel, dim3(rows), dim3(32), (size_t)p.nblk * 8, st, (const float*)p.cand_v, (const int*)p.cand_i, p.nblk, 1, LevelDesc{0, 0, nullptr},
-             (const int*)nullptr, (const int*)nullptr, amax, 0, 0, 1);
+             (const int*)nullptr, (const int*)nullptr, amax, 0, (const int*)nullptr, 0, 0);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -1052,15 +1053,15 @@ hydra_status topk_children(const float* part, SplitDesc sd, float* logits, Level
     return HYDRA_OK;
   }
   HYDRA_TRY(topk_candidates(part, sd, logits, max_children, scratch, rows_cap, rows, vocab, st));
-  return topk_merge(lv, max_children, first_child, n_child, tree_tok, scratch, rows_cap, 0, batch, T, vocab, 0, st);
+  return topk_merge(lv, max_children, first_child, n_child, tree_tok, scratch, rows_cap, rows, batch, T, vocab, nullptr, 0, st);
 }
 
-hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int row0,
-                        int batch, int T, int vocab, int shared_rows, cudaStream_t st) {
+hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int cand_rows,
+                        int batch, int T, int vocab, const int* depth, int top, cudaStream_t st) {
   TopkPlan p;
-  if (!topk_plan(scratch, rows_cap, row0 + (shared_rows ? batch : batch * lv.n_parents), vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
+  if (!topk_plan(scratch, rows_cap, cand_rows, vocab, max_children, &p)) return HYDRA_ERR_UNSUPPORTED;
   launch_pdl(topk_stage2_kernel, dim3(batch * lv.n_parents), dim3(32), (size_t)p.nblk * max_children * 8, st, (const float*)p.cand_v, (const int*)p.cand_i, p.nblk,
-             max_children, lv, first_child, n_child, tree_tok, T, row0, shared_rows ? lv.n_parents : 1);
+             max_children, lv, first_child, n_child, tree_tok, T, depth, top, batch);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }

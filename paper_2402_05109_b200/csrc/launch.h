@@ -86,12 +86,12 @@ hydra_status head_gather(const float* hprime, const void* embed, const int* root
 hydra_status head_act(const float* res, int res_is_hprime, int rows_per_b, const float* part, SplitDesc sd,
                       const void* bias, float* y_out, void* yb, size_t yb_ps, int rows, int d, cudaStream_t st);
 // Children of a level in two steps.  The max_children best tokens of every logits row, descending (ties: lower id first); the logits are the
-// summed partials, also written to `logits` [rows][vocab].  Then the children of parent j of sequence b = the first n_child of row row0 + b*P+j's;
-// shared_rows: the level has ONE row per sequence (sequentially independent heads), row0 + b, and every parent takes its children from that.
+// summed partials, also written to `logits` [rows][vocab].  Then the children of parent j of sequence b = the first n_child of row b*P+j's; with depth, lv has
+// the parents of all levels (sequentially independent heads, one row per sequence and head), and those at depth t take theirs from row (top - t)*batch + b.
 hydra_status topk_candidates(const float* part, SplitDesc sd, float* logits, int max_children, void* scratch, int rows_cap, int rows, int vocab,
                              cudaStream_t st);
-hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int row0,
-                        int batch, int T, int vocab, int shared_rows, cudaStream_t st);
+hydra_status topk_merge(LevelDesc lv, int max_children, const int* first_child, const int* n_child, int* tree_tok, void* scratch, int rows_cap, int cand_rows,
+                        int batch, int T, int vocab, const int* depth, int top, cudaStream_t st);
 
 // Both, for a level whose rows are its own.
 hydra_status topk_children(const float* part, SplitDesc sd, float* logits, LevelDesc lv, int max_children, const int* first_child, const int* n_child,

@@ -65,6 +65,9 @@ hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, co
                                bf16* out, size_t out_ps, int n_heads, int head_dim, int max_seq, int len_upper, int* status,
                                bool stable_lengths, cudaStream_t st);
 constexpr int ATT_BLOCK_ROWS = 128;
+// The same for one or two rows a sequence, without tensor cores (attention_rows.cu).
+hydra_status tree_attention_rows(const __half* q, int q_rows, const __half* kc, const __half* vc, int cache_batch, int planes, RowSet rs, bf16* out, size_t out_ps, int n_heads,
+                                 int head_dim, int max_seq, int len_upper, bool stable_lengths, cudaStream_t st);
 hydra_status silu_mul(const float* part, SplitDesc sd, void* act, size_t act_ps, int rows, int f, cudaStream_t st);
 // amax[r] = argmax_v of the summed partial logits (lowest id among equal maxima); the sums go to logits_out if given
 // scratch: topk_scratch_bytes(rows_cap, vocab) bytes of candidate storage

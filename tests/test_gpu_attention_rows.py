@@ -1,0 +1,43 @@
+"""Float16 attention of one and two rows a sequence: lengths around the lane groups' rounds (32 or 64 keys a round of a CTA, four rounds in flight) and the chunks' cuts, empty
+sequences and rows, with and without a mask.  What lies behind a sequence's keys in its cache is not a number and would show in every result that read it."""
+import pytest
+import torch
+
+from oracle.hydra_oracle import masked_attention
+from tests.test_gpu_kernels import rnd, _dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("hd,planes", [(128, 2), (128, 1), (64, 2), (64, 1)])
+@pytest.mark.parametrize("tc,masked", [(1, True), (1, False), (2, True), (2, False)])
+@pytest.mark.parametrize("H,S,pos0", [(1, 96, [0, 1, 31, 33, 63]), (5, 300, [64, 127, 128, 129, 297]), (60, 700, [255, 257, 511, 0, 690])])
+def test_few_rows(H, S, pos0, tc, masked, hd, planes):
+    from paper_2402_05109_b200 import tree_attention
+    B, n_rows = len(pos0), [tc, tc, tc - 1, tc, tc]
+    src = torch.float32 if planes == 2 else torch.float16
+    (q_d, q), (k_d, kc), (v_d, vc) = (_dev(rnd(shape, 91, i, src), planes) for i, shape in ((3, (B * tc, H, hd)), (1, (B, H, S, hd)), (2, (B, H, S, hd))))
+    for b in range(B):
+        for cache in (k_d, v_d):
+            cache[..., b, :, pos0[b] + n_rows[b]:, :] = float("nan")
+    bits = [1, 2]                                         # two siblings: the second does not see the first
+    dev = lambda x, t=torch.int32: torch.tensor(x, dtype=t).cuda()
+    out = tree_attention(q_d, k_d, v_d, dev(pos0), dev(n_rows), dev(bits[:tc], torch.int64) if masked else None, tc, out_planes=2).float().cpu().sum(0).view(B, tc, H, hd)
+    for b in range(B):
+        n, L = n_rows[b], pos0[b] + n_rows[b]
+        assert n == tc or float(out[b, n:].abs().max()) == 0.0
+        if n == 0:
+            continue
+        new = torch.eye(n, dtype=torch.bool) if masked else torch.tril(torch.ones(n, n, dtype=torch.bool))
+        allowed = torch.cat([torch.ones(n, pos0[b], dtype=torch.bool), new], dim=1)
+        ref = masked_attention(q.view(B, tc, H, hd)[b, :n].double(), kc[b, :, :L].permute(1, 0, 2).double(), vc[b, :, :L].permute(1, 0, 2).double(), allowed)
+        # weights and sums are float; the result is rounded to two bfloat16 planes (2^-17 of at most 4)
+        assert float((out[b, :n].double() - ref).abs().max()) <= 1e-4
+
+
+def test_lengths_past_the_cache_give_zeros():
+    from paper_2402_05109_b200 import tree_attention
+    H, S, hd = 3, 80, 128
+    q, k, v = (rnd(s, 92, i, torch.float16).cuda() for i, s in ((3, (5, H, hd)), (1, (5, H, S, hd)), (2, (5, H, S, hd))))
+    out = tree_attention(q, k, v, torch.tensor([S, -1, 1 << 30, 2147483647, S - 1], dtype=torch.int32).cuda(), None, None, 1, out_planes=2).float().sum(0).view(5, H, hd)
+    assert float(out[:4].abs().max()) == 0.0 and float(out[4].abs().min(-1).values.max()) > 0.0

@@ -508,7 +508,10 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   // 1024 10.2 / 8.3: the sums of a tile are one CTA's work).
   // sum_tile stores 16 bytes at a time; a result buffer off that boundary takes the second launch, which stores single floats.  (Units
   // of two weight tiles begin at 9 million weights on 148 SMs.)
-  if (out && arrivals && sh.nh == 1 && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && !((uintptr_t)out & 15)) {
+  // And only while a tile has few slots, which one CTA adds eight rows at a time: a call from Python takes 9.2 us with two launches whatever these sizes, and with one 11 x 256 x
+  // 4096 (17 slots at most) 8.5, 11 x 1024 x 5632 (19) 10.7, 8 x 640 x 5632 (23) 8.5, 8 x 768 x 7744 (25) 10.0, 11 x 256 x 11008 (44) 18.7.
+  const int most_slots = (sd.kb + sd.q - 2) / sd.q + 1;
+  if (out && arrivals && sh.nh == 1 && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && most_slots <= (m > 8 ? 17 : 23) && !((uintptr_t)out & 15)) {
     a.out = out; a.arr = *arrivals;
     return launch<1, true>(tw, tx, a, grid, st);
   }

@@ -65,6 +65,12 @@ def test_gemm_noalloc_one_and_two_launches(m, n, k):
     assert int(status.item()) == 0
 
 
+@pytest.mark.parametrize("m,n,k", [(8, 640, 5632), (9, 640, 5632), (9, 256, 4096), (8, 768, 7744), (16, 256, 11008), (64, 8192, 2048), (40, 3072, 1920)])
+def test_gemm_noalloc_slots_of_a_tile(m, n, k):
+    """Up to 17 or 23 slots a tile in one launch, more in two; in the second one up to twelve in flight together, more in turn."""
+    test_gemm_noalloc_one_and_two_launches(m, n, k)
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 128, 64), (11, 2048, 2048), (3, 4096, 4096)])
 @pytest.mark.parametrize("offset", [1, 2, 3])
 def test_gemm_noalloc_result_off_a_16_byte_boundary(m, n, k, offset):

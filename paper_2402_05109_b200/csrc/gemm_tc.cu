@@ -203,8 +203,11 @@ __device__ __forceinline__ bool epilogue_all(bool v) {       // v of all 128 epi
 constexpr int MAX_STAGES = 10;
 constexpr int EPI_WARPS = 4;                             // one per quadrant of tensor memory (two measured no faster: the L2 takes the stores no sooner)
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr int RING_BYTES = 200 * 1024;
-constexpr int SMEM_BYTES = RING_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
+// Shared memory of the ring: 200 KB, above 64 rows up to 220 KB where that is another stage.  There a stage is 36 to 96 KB and two or three of them do
+// not hide a load: 22016 x 4096, two planes, 144 rows 44.5 us with three stages / 40.1 with four, 288 rows 88 / 76, 320 rows 92 / 84 (two / three); 4096 x
+// 4096, 400 and 432 rows 31.3 / 25.8, 33.3 / 27.6 (two / three).  Up to 64 rows the kernels around a GEMM want the rest: with 216 KB 1 and 16 rows took
+// 27.7 and 28.2 instead of 26.8 and 27.2, and with 160 KB as long.
+constexpr int RING_BYTES = 200 * 1024, RING_BYTES_MAX = 220 * 1024, RING_EXTRA_BYTES = 1024 /*alignment slack*/ + 512 /*barriers*/;
 
 // Shapes are run-time arguments (one copy of the code for all row counts); NH: 128-row weight tiles per CTA and unit.
 // REDUCE (stand-alone calls): the last CTA to store a tile's partial sums adds them, so the call is one launch.  (Inside a
@@ -218,7 +221,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int stages = a.stages;
   const uint32_t x_box_bytes = (uint32_t)a.mt * (BLOCK_K * 2), x_bytes = a.x_boxes * x_box_bytes, stage_bytes = W_BYTES + x_bytes;
-  const uint32_t bars = tiles + RING_BYTES;
+  const uint32_t bars = tiles + stages * stage_bytes;
   auto full_bar = [&](int s) { return bars + 8u * s; };
   auto empty_bar = [&](int s) { return bars + 8u * (MAX_STAGES + s); };
   auto accfull_bar = [&](int i) { return bars + 8u * (2 * MAX_STAGES + i); };
@@ -385,14 +388,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 }
 
 template <int NH, bool REDUCE>
-hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, cudaStream_t st) {
+hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs& a, int grid, int smem, cudaStream_t st) {
   static PerDeviceFlag attr_done;
   if (!attr_done.get()) {
-    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<NH, REDUCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
+    HYDRA_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<NH, REDUCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, RING_BYTES_MAX + RING_EXTRA_BYTES));
     attr_done.set();
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -494,7 +497,8 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   a.acc_bufs = 2 * sh.nh * a.acc_cols <= 512 ? 2 : 1;
   for (a.tmem_cols = 32; a.tmem_cols < a.acc_bufs * sh.nh * a.acc_cols;) a.tmem_cols *= 2;
   const int stage_bytes = sh.nh * A_BYTES + a.x_boxes * sh.mt * BLOCK_K * 2;
-  a.stages = RING_BYTES / stage_bytes < MAX_STAGES ? RING_BYTES / stage_bytes : MAX_STAGES;
+  a.stages = std::min((sh.mt > 64 ? RING_BYTES_MAX : RING_BYTES) / stage_bytes, MAX_STAGES);
+  const int smem = std::max(a.stages * stage_bytes, RING_BYTES) + RING_EXTRA_BYTES;
   CUtensorMap tw, tx;
   if (!get_tensor_map(w, (uint64_t)n, (uint64_t)k, (uint32_t)(sh.nh * BLOCK_N), false, &tw) ||
       !get_tensor_map(x, (uint64_t)x_rows_alloc * x_planes - x_row0, (uint64_t)k, (uint32_t)sh.mt, false, &tx)) {      // what the buffer holds from x on; rows past it read as zeros
@@ -513,9 +517,9 @@ hydra_status gemm_tc(const bf16* x, int x_rows_alloc, int x_planes, const bf16* 
   const int most_slots = (sd.kb + sd.q - 2) / sd.q + 1;
   if (out && arrivals && sh.nh == 1 && m <= 16 && (long long)n * k <= GEMM_ONE_LAUNCH_WEIGHTS && most_slots <= (m > 8 ? 17 : 23) && !((uintptr_t)out & 15)) {
     a.out = out; a.arr = *arrivals;
-    return launch<1, true>(tw, tx, a, grid, st);
+    return launch<1, true>(tw, tx, a, grid, smem, st);
   }
-  const hydra_status s = sh.nh == 2 ? launch<2, false>(tw, tx, a, grid, st) : launch<1, false>(tw, tx, a, grid, st);
+  const hydra_status s = sh.nh == 2 ? launch<2, false>(tw, tx, a, grid, smem, st) : launch<1, false>(tw, tx, a, grid, smem, st);
   return s == HYDRA_OK && out ? reduce_splits(part, sd, out, m, n, st) : s;
 }
 

@@ -171,3 +171,17 @@ def test_gemm_noalloc_takes_fewer_ctas_where_the_sums_would_not_fit(m, n, k):
     ref = x.double() @ w.double().T
     assert float((out.double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("m", [64, 65, 80, 112, 144, 160, 208, 224, 240, 288, 320])
+@pytest.mark.parametrize("n", [512, 22016])
+def test_gemm_ring_above_64_rows(m, n):
+    """Row tiles whose stages fill more than 200 KB, and their neighbours; more blocks of k than stages, units of one and of two weight tiles."""
+    from paper_2402_05109_b200 import gemm
+    k = 1088
+    x = normal_(torch.empty(m, k, device="cuda"), 81, m, 1.0)
+    w = normal_(torch.empty(n, k, dtype=torch.bfloat16, device="cuda"), 82, n, 0.02)
+    # as above
+    for planes in (split_hi_lo(x), x.to(torch.bfloat16)):
+        ref = (planes.double().sum(0) if planes.dim() == 3 else planes.double()) @ w.double().T
+        assert float((gemm(planes, w, mode=0).double() - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5

@@ -415,9 +415,11 @@ bool gemm_tc_available() { return tensor_map_encoder_available(); }
 //    30.2, 64 rows: 42.2 / 42.4; 4096 x 11008, 1 row: 19.0 / 17.5, 64 rows: 20.9 / 20.3
 //  * above, 128 (tensor memory then holds two accumulators, and fewer partial sums are left): 12288 x 4096, 96 rows: 29.4 / 30.9;
 //    4096 x 4096, 128 rows: 16.0 / 19.0; 22016 x 4096, 192 rows: 77 / 82; except for
-//  * 97 to 128 rows of an output wide enough that a tile meets one or two ranges all the same (half as many tiles as SMs): the activation tile is twice the weight
+//  * 97 to 160 rows of an output wide enough that a tile meets one or two ranges all the same (half as many tiles as SMs): the activation tile is twice the weight
 //    tile there, and an SM takes in a third less.  In a forward pass, 128 rows: 22016 x 4096 37.9 / 36.6, 32000 x 4096 54.0 / 51.1, 27648 x 5120 58.2 / 54.5,
-//    35840 x 6656 97.8 / 90.5, 19968 x 6656 56.8 / 54.1; 12288 x 4096 23.0 / 23.7, 6656 x 17920 with its norm 59.4 / 61.2; 80 rows 22016 x 4096 32.0 / 32.7; and for
+//    35840 x 6656 97.8 / 90.5, 19968 x 6656 56.8 / 54.1; 12288 x 4096 23.0 / 23.7, 6656 x 17920 with its norm 59.4 / 61.2; 80 rows 22016 x 4096 32.0 / 32.7.
+//    160 rows: 22016 x 4096 47.3 / 41.8, 32000 x 4096 66.8 / 56.5, 27648 x 5120 74.8 / 63.0, 35840 x 6656 127 / 105, 19968 x 6656 73.3 / 64.5; 129 rows 39.4 / 38.8,
+//    56.3 / 52.9, 63.0 / 58.8, 103 / 95, 60.8 / 57.9; 12288 x 4096 144 rows 25.0 / 25.6 (176 rows would have two stages: 192 rows 22016 x 4096 54.2 / 56.2); and for
 //  * tall row tiles with 16 and more units per SM, where the activation tile is most of what an SM takes in: 22016 x 4096, 256
 //    rows: 111 / 103, 512 rows: 222 / 192; 4096 x 11008, 512 rows: 96 / 91; but 4096 x 4096, 512 rows: 49 / 54
 struct GemmShape { int nh, mt, m_tiles; };
@@ -425,7 +427,7 @@ static GemmShape gemm_shape(int m, int n, int k) {
   // equal row tiles of a multiple of 16 rows, so that the MMA work and the activation traffic follow m
   const int row_tiles = (m + 255) / 256, mt = ((m + row_tiles - 1) / row_tiles + 15) / 16 * 16;
   const long long units = (long long)row_tiles * (n / 256) * (k / BLOCK_K), sms = sm_count();
-  const bool wide = m <= 64 ? 4 * units >= 15 * sms : m <= 128 ? m > 96 && n / 256 * 2 >= sms : (mt > 192 || row_tiles > 1) && units >= 16 * sms;
+  const bool wide = m <= 64 ? 4 * units >= 15 * sms : m <= 160 ? m > 96 && n / 256 * 2 >= sms : (mt > 192 || row_tiles > 1) && units >= 16 * sms;
   return GemmShape{wide ? 2 : 1, mt, (m + mt - 1) / mt};
 }
 

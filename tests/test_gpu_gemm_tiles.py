@@ -22,9 +22,9 @@ def test_gemm_tile_edges(m, n, k):
         assert float((out - ref).abs().max()) <= 1e-5 * float(ref.abs().max()) + 1e-6 * k ** 0.5
 
 
-@pytest.mark.parametrize("m", [96, 97, 112, 128])
+@pytest.mark.parametrize("m", [96, 97, 112, 128, 129, 160, 161])
 @pytest.mark.parametrize("n", [18816, 18944, 19072])
-def test_gemm_wide_units_at_97_to_128_rows(m, n):
+def test_gemm_wide_units_at_97_to_160_rows(m, n):
     """Both sides of the lines in rows and in width, and an output that ends inside its last unit."""
     from paper_2402_05109_b200 import gemm
     k = 320

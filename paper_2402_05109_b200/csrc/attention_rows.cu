@@ -110,22 +110,24 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_rows_kernel(const RowsAr
 #pragma unroll
         for (int u = 0; u < BATCH; ++u) s[r][u] += __shfl_xor_sync(0xffffffffu, s[r][u], bit);
     float w[R][BATCH];
+    bool seen[R][BATCH];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       float mn = m[r];
 #pragma unroll
       for (int u = 0; u < BATCH; ++u) {
         const int slot = s0 + u * GROUPS;
-        if (!(r < nr && slot < k1 && (slot < p0 || ((mask[r] >> (slot - p0)) & 1ull)))) s[r][u] = -INFINITY;
+        seen[r][u] = r < nr && slot < k1 && (slot < p0 || ((mask[r] >> (slot - p0)) & 1ull));
+        if (!seen[r][u]) s[r][u] = -INFINITY;
         mn = fmaxf(mn, s[r][u]);
       }
-      const float f = mn == -INFINITY ? 1.f : ex2(m[r] - mn);
+      const float f = mn == -INFINITY ? 1.f : ex2(m[r] - mn), ref = mn == -INFINITY ? 0.f : mn;
       m[r] = mn;
       l[r] *= f;
 #pragma unroll
       for (int d = 0; d < 8; ++d) o[r][d] *= f;
 #pragma unroll
-      for (int u = 0; u < BATCH; ++u) { w[r][u] = s[r][u] == -INFINITY ? 0.f : ex2(s[r][u] - mn); l[r] += w[r][u]; }
+      for (int u = 0; u < BATCH; ++u) { w[r][u] = ex2(s[r][u] - ref); l[r] += w[r][u]; }
     }
 #pragma unroll
     for (int u = 0; u < BATCH; ++u) {
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_rows_kernel(const RowsAr
       unpack8<NP>(vv[u], v);
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        if (w[r][u] != 0.f) {                              // (a key that a row does not see adds nothing, whatever it holds)
+        if (seen[r][u]) {                                  // (a key that a row does not see adds nothing, whatever it holds)
 #pragma unroll
           for (int d = 0; d < 8; ++d) o[r][d] = fmaf(w[r][u], v[d], o[r][d]);
         }
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(THREADS, 1) tree_attn_rows_kernel(const RowsAr
     const float mi = s_part[i][r][HD], f = mi == -INFINITY ? 0.f : ex2(mi - M);
     L += s_part[i][r][HD + 1] * f; acc += s_part[i][r][k] * f;
   }
-  const float y = L > 0.f ? acc / L : 0.f;                 // rows past nr get zeros
+  const float y = L == 0.f ? 0.f : acc / L;                // rows without keys get zeros; a sum that is no number stays none
   bf16* dst = a.out + (size_t)(b * rs.tc + r) * H * HD + h * HD + k;
   const bf16 hi = __float2bfloat16_rn(y);
   *dst = hi;

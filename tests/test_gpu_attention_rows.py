@@ -1,5 +1,6 @@
 """Float16 attention of one and two rows a sequence: lengths around the lane groups' rounds (32 or 64 keys a round of a CTA, four rounds in flight) and the chunks' cuts, empty
-sequences and rows, with and without a mask.  What lies behind a sequence's keys in its cache is not a number and would show in every result that read it."""
+sequences and rows, with and without a mask.  What lies behind a sequence's keys in its cache is not a number and would show in every result that read it
+(in the zeros of rows past the call's, too: a sum that is no number stays none)."""
 import pytest
 import torch
 
@@ -41,3 +42,46 @@ def test_lengths_past_the_cache_give_zeros():
     q, k, v = (rnd(s, 92, i, torch.float16).cuda() for i, s in ((3, (5, H, hd)), (1, (5, H, S, hd)), (2, (5, H, S, hd))))
     out = tree_attention(q, k, v, torch.tensor([S, -1, 1 << 30, 2147483647, S - 1], dtype=torch.int32).cuda(), None, None, 1, out_planes=2).float().sum(0).view(5, H, hd)
     assert float(out[:4].abs().max()) == 0.0 and float(out[4].abs().min(-1).values.max()) > 0.0
+
+
+@pytest.mark.parametrize("planes", [1, 2])
+@pytest.mark.parametrize("tc", [1, 2])
+@pytest.mark.parametrize("H,B,length", [(4, 2, 20), (4, 2, 700), (50, 3, 70)])      # one round, several chunks, one chunk
+def test_what_is_not_a_number_shows(H, B, length, tc, planes):
+    """A key, a value or a score that is not finite reaches every row that sees it, as on the tensor cores (three rows), and no other sequence, head or row."""
+    from paper_2402_05109_b200 import tree_attention
+    hd, S, b0, h0, bad = 128, length + 8, B - 1, H - 2, float("nan")
+    base = [rnd(shape, 93, i, torch.float16) for i, shape in ((3, (B, 3, H, hd)), (1, (B, H, S, hd)), (2, (B, H, S, hd)))]
+    pos0, bits = torch.full((B,), length, dtype=torch.int32).cuda(), [1, 2, 4]
+
+    def call(rows, poison):
+        q, k, v = (torch.stack([t, torch.zeros_like(t)]) if planes == 2 else t[None].clone() for t in base)
+        poison(q, k, v)
+        q = q[:, :, :rows].reshape(planes, B * rows, H, hd)
+        q, k, v = (t.contiguous().cuda() if planes == 2 else t[0].contiguous().cuda() for t in (q, k, v))
+        out = tree_attention(q, k, v, pos0, None, torch.tensor(bits[:rows], dtype=torch.int64).cuda(), rows, out_planes=2)
+        return out.float().sum(0).view(B, rows, H, hd)[:, :tc].cpu()
+
+    def key_nan(q, k, v): k[:, b0, h0, length // 2, 5] = bad
+
+    def key_inf(q, k, v):                                  # a value past float16: hi is inf, lo what is left of it
+        k[0, b0, h0, length // 3, :] = float("inf")
+        if planes == 2: k[1, b0, h0, length // 3, :] = -float("inf")
+    def score_inf(q, k, v): q[0, b0, :, h0, 7] = 1.0; k[0, b0, h0, 3, 7] = float("inf")
+    def value_nan(q, k, v): v[:, b0, h0, length - 1, :] = bad
+    def faint_value_nan(q, k, v): q[0, b0, :, h0, :] = 8.0; k[0, b0, h0, :length] = 8.0; k[0, b0, h0, 0] = -8.0; v[:, b0, h0, 0, :] = bad      # a weight of zero
+    where = torch.zeros(B, tc, H, hd, dtype=torch.bool)
+    where[b0, :, h0] = True
+    for poison in (key_nan, key_inf, score_inf, value_nan, faint_value_nan):
+        got = call(tc, poison)
+        assert torch.equal(got.isnan(), where), poison.__name__
+        assert torch.equal(call(3, poison).isnan(), where), poison.__name__
+    # the query of the last row, and the key of the last row, which only that one sees
+    def query_nan(q, k, v): q[:, b0, tc - 1, h0, 9] = bad
+    def own_nan(q, k, v): k[:, b0, h0, length + tc - 1] = bad; v[:, b0, h0, length + tc - 1] = bad
+    where[b0, :tc - 1, h0] = False
+    for poison in (query_nan, own_nan):
+        assert torch.equal(call(tc, poison).isnan(), where), poison.__name__
+    if planes == 1:                                        # every visible score -inf: no weight at all, and zeros as on the tensor cores
+        def no_weight(q, k, v): q[0, b0, :, h0] = 1.0; k[0, b0, h0, :length + tc] = -float("inf")
+        assert float(call(tc, no_weight)[b0, :, h0].abs().max()) == 0.0

@@ -50,3 +50,50 @@ def test_slot_counts_against_divisions(tmp_path):
                     "-L", PKG, "-lhydra", "-Xlinker", "-rpath=" + PKG], check=True, capture_output=True, text=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stdout
+
+
+ERRORS = r"""
+#include "launch.h"
+#include <cstdio>
+#include <cmath>
+using namespace hydra;
+// Error of a product by its plan, up to a factor: sums are drained where a range or a tile ends, and an error grows with a sum's length to the power 1.5.
+static double error(long long line, int kb, int q) {
+  double s = 0;
+  for (long long u = 0; u < line;) {
+    const long long end = std::min({(u / kb + 1) * kb, (u / q + 1) * q, line});
+    s += std::pow((double)(end - u), 3);
+    u = end;
+  }
+  return std::sqrt(s / (double)line);
+}
+int main() {
+  const int shapes[][2] = {{4096, 4096}, {12288, 4096}, {22016, 4096}, {4096, 11008}, {32000, 4096}, {5120, 5120}, {5120, 13824}, {6656, 6656}, {35840, 6656}, {6656, 17920},
+                           {2048, 2048}, {1024, 1024}, {3072, 1024}, {4224, 2048}};
+  int bad = 0;
+  for (auto& s : shapes)
+    for (int tiles = 2; tiles <= 64; ++tiles) {
+      const int n = s[0], k = s[1], m = 256 * tiles - 16, kb = k / 64;      // row tiles of 256
+      int grid = 0;
+      const SplitDesc sd = gemm_tc_plan(m, n, k, &grid, nullptr);
+      const long long n_tiles = (n + (1 << sd.bn_shift) - 1) >> sd.bn_shift, all = n_tiles * tiles * kb, sms = sm_count();
+      if (all / 4 < sms) continue;
+      const int q1 = (int)((all + sms - 1) / sms);
+      const double one = error(all, kb, q1), now = error(n_tiles * sd.m_tiles * kb, kb, sd.q);
+      if (now > 1.051 * one || 8ll * sd.q > 9ll * q1 || grid > sms) ++bad, printf("%d row tiles of %d x %d: error %.3f, ranges %d / %d, grid %d\n", tiles, n, k, now / one, sd.q, q1, grid);
+    }
+  return bad != 0;
+}
+"""
+
+
+def test_row_tiles_that_walk_together_have_sums_as_short_as_alone(tmp_path):
+    from paper_2402_05109_b200.build import build
+    build()
+    src, exe = tmp_path / "errors.cu", tmp_path / "errors"
+    src.write_text("#include <algorithm>\n#include <initializer_list>\n" + ERRORS)
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O2", "-I", os.path.join(PKG, "csrc"), str(src), "-o", str(exe),
+                    "-L", PKG, "-lhydra", "-Xlinker", "-rpath=" + PKG], check=True, capture_output=True, text=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout

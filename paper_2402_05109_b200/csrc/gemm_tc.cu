@@ -247,7 +247,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // (The weight tiles of a whole ring are 128 KB an SM at 64 rows and 160 KB at one, 19 and 24 MB over the SMs; the preceding row-wise kernel's
     // loads queue behind them.  7B shape, 32 steps with a 64-row tree 145.2 -> 144.0 ms with half a ring, runs of one side 0.3 % apart; without a
     // tree, and 47 supplied rows, the same either way.  All stages but one gained as much as half, one stage alone nothing.)
-    const uint64_t pol = policy_evict_first();
+    const uint64_t pol = a.m_blocks == 1 ? policy_evict_first() : policy_evict_normal();
     int tile = u_begin / a.kb, kb = u_begin - tile * a.kb, nrow = tile / a.m_blocks * BN;
     for (int i = 0; i < (a.w_const ? pre : ring); ++i) {
       if (!a.w_const) {
@@ -269,7 +269,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == 0) {
     if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
+      // (several groups of row tiles: the next one reads the weights again)
+      const uint64_t pol_w = a.m_blocks == 1 ? policy_evict_first() : policy_evict_normal(), pol_x = policy_evict_last();
       int kcol = 0, nrow = 0, mrow = 0;                  // (k column, weight row, activation row) of the unit being issued, advanced without divisions
       if (n_units > 0) {
         const int tile = u_begin / a.kb;
@@ -452,25 +453,26 @@ static int range_units(long long line, long long most) {
 }
 // Row tiles that walk the line together: all of them up to 16, else groups as equal as they come, unless fewer at a time are as exact as one line of all
 // tiles and more are not.  Ranges that end with the tiles leave whole tiles in one sum, and a group whose size does not divide the SMs makes ranges longer: a group is taken when its
-// plan's error is at most 5 % above that of the one line and its ranges at most an eighth longer.  4096 x 4096, 9 row tiles: one line 6.58e-6, nine
-// together (whole tiles) 9.25e-6 against float64; 17 row tiles of 2048 x 2048: 3.12e-6, two nines 4.56e-6.
+// plan's error is at most 5 % above that of the one line and its ranges at most a sixteenth longer, or an eighth if no group has such.  4096 x 4096, 9 row tiles: one line 6.58e-6, nine
+// together (whole tiles) 9.25e-6 against float64, three 6.04e-6; 17 row tiles of 2048 x 2048: 3.12e-6, two nines 4.56e-6.
 constexpr int GROUP_MAX = 16;            // (a prompt pass has at most 3 row tiles, 64 sequences of a 64-row tree 16)
 static int row_tile_group(int m, int m_tiles, int n_tiles, int kb, int sms) {
   const long long all = (long long)n_tiles * m_tiles * kb;
   if (m_tiles == 1 || all / 4 < sms) return 1;
   const int most = (m_tiles + GROUP_MAX - 1) / GROUP_MAX;
-  int group = (m_tiles + most - 1) / most;
+  const int group = (m_tiles + most - 1) / most;
   if (m > 65536) return group;           // (SplitDesc::div_mt: groups of 16 whole tiles)
   const int q1 = range_units(all, sms);
   const double cubes1 = segment_cubes(all, kb, q1) / (double)all;
-  for (; group > 1; --group) {
-    const int blocks = (m_tiles + group - 1) / group;
-    group = (m_tiles + blocks - 1) / blocks;
-    const long long line = (long long)n_tiles * blocks * kb;
-    const int q = range_units(line, sms / group);
-    if (8ll * q <= 9ll * q1 && segment_cubes(line, kb, q) <= 1.1 * cubes1 * (double)line) break;
-  }
-  return group;
+  for (const int part : {16, 8})
+    for (int g = group; g > 1; --g) {
+      const int blocks = (m_tiles + g - 1) / g;
+      g = (m_tiles + blocks - 1) / blocks;
+      const long long line = (long long)n_tiles * blocks * kb;
+      const int q = range_units(line, sms / g);
+      if ((long long)part * q <= (part + 1ll) * q1 && segment_cubes(line, kb, q) <= 1.1 * cubes1 * (double)line) return g;
+    }
+  return 1;
 }
 
 // Stream-K plan: equal contiguous ranges of the line, at most one CTA per SM and at least 4 k-blocks each.

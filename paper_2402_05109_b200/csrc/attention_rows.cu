@@ -199,8 +199,12 @@ hydra_status tree_attention_rows(const __half* q, int q_rows, const __half* kc, 
                                  int max_seq, int len_upper, bool stable_lengths, cudaStream_t st) {
   if (rs.blocks || rs.tc < 1 || rs.tc > 2 || (hd != 64 && hd != 128) || (planes != 1 && planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   const RowsArgs a{q, kc, vc, (size_t)q_rows * H * hd, (size_t)cache_batch * H * max_seq * hd, rs, out, out_ps, H, max_seq, stable_lengths ? 1 : 0};
-  // a chunk per 64 keys while the pairs leave SMs idle
-  const int pairs = H * rs.batch, n = std::max(1, std::min({MAX_CHUNKS, sm_count() / pairs, (len_upper + 63) / 64}));
+  // A chunk per 64 keys while the pairs leave SMs idle.  With more pairs, two where the last wave would fill at most half of the SMs with long CTAs, which
+  // alone do not keep memory busy.  One chunk / two, us, two planes: 160 pairs of 500 keys 24.5 / 23.7, 1000 41.6 / 37.8, 4000 141 / 120; 208 of 1000 43.6 / 41.4, 8000 282 / 250; 352 of
+  // 1000 68.1 / 69.4, 2000 123 / 118; 512 of 1000 91 / 94, 4000 321 / 311; but 256 (a last wave of 108) of 1000 47 / 53, 8000 307 / 322.
+  const long long pairs = (long long)H * rs.batch, sms = sm_count(), last = pairs % sms;
+  int n = (int)std::max(1ll, std::min({(long long)MAX_CHUNKS, sms / pairs, (len_upper + 63ll) / 64}));
+  if (pairs > sms && last && 2 * last <= sms && len_upper >= 768 * (pairs / sms)) n = 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(H, rs.batch, n); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = 0; cfg.stream = st;
   cudaLaunchAttribute attr[2];

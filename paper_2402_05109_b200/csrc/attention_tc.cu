@@ -704,8 +704,9 @@ hydra_status tree_attention_tc(const __half* q, int q_rows, const __half* kc, co
   if ((!rs.blocks && (rs.tc > 128 || (rs.mask && rs.tc > 64))) || (planes != 1 && planes != 2)) return HYDRA_ERR_UNSUPPORTED;
   if (!tensor_map_encoder_available()) { set_last_error("cuTensorMapEncodeTiled entry point", cudaErrorUnknown); return HYDRA_ERR_CUDA; }
   if (((uintptr_t)q | (uintptr_t)kc | (uintptr_t)vc) & 15) return HYDRA_ERR_INVALID;
-  // One row always (5 to 40 % faster from 40 to 2400 keys, 1 to 8 sequences); two rows up to 1024 keys (1 sequence of 160 keys 7.7 / 5.8 us, 1000 12.7 / 11.6; 4 of 1000
-  // 27.2 / 27.4, 2 of 2400 31.1 / 32.2); four rows took as long at 160 keys and 10 to 40 % longer above
+  // One row always: 3 to 48 % faster, 40 to 32000 keys, 1 to 64 sequences of 8 to 52 heads; two sequences of 32 heads with one plane from 8000 keys on 1 to 2 % slower.
+  // Two rows up to 1024 keys: 0.53 to 0.95 of the time at 40 to 160 keys; at 1000 1 sequence of 32 heads 12.8 / 11.8 us, 8 52.7 / 51.4, 16 107 / 99, but 2 17.2 / 17.4, 4 26.2 / 27.5, 5 45.4 /
+  // 48.1 (kept: with one plane the weights of these rows are float, not float16), 2 of 2400 31.1 / 32.2.  Four rows took as long at 160 keys and 10 to 40 % longer above.
   if (!rs.blocks && (rs.tc == 1 || (rs.tc == 2 && len_upper <= 1024)))
     return tree_attention_rows(q, q_rows, kc, vc, cache_batch, planes, rs, out, out_ps, H, hd, max_seq, len_upper, stable_lengths, st);
   return planes == 2 ? dispatch<2>(q, q_rows, kc, vc, cache_batch, rs, out, out_ps, H, hd, max_seq, len_upper, status, stable_lengths, st)

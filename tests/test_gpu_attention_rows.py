@@ -85,3 +85,18 @@ def test_what_is_not_a_number_shows(H, B, length, tc, planes):
     if planes == 1:                                        # every visible score -inf: no weight at all, and zeros as on the tensor cores
         def no_weight(q, k, v): q[0, b0, :, h0] = 1.0; k[0, b0, h0, :length + tc] = -float("inf")
         assert float(call(tc, no_weight)[b0, :, h0].abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("hd,planes", [(128, 2), (64, 1)])
+@pytest.mark.parametrize("tc", [1, 2])
+@pytest.mark.parametrize("H,S,pos0", [(1, 440, [0, 1, 200, 300, 437]), (2, 700, [0, 63, 100, 640, 697]),      # six to eight chunks
+                                      (32, 800, [0, 127, 400, 766, 798]), (32, 767, [0, 63, 384, 700, 765]), (41, 768, [1, 63, 384, 700, 766]),      # two for a short last wave
+                                      (7, 1024, [0, 64, 600, 1000, 1022])])
+def test_chunks(H, S, pos0, tc, hd, planes):
+    test_few_rows(H, S, pos0, tc, True, hd, planes)
+
+
+@pytest.mark.parametrize("hd", [64, 128])
+def test_two_rows_past_the_line(hd):
+    """The tensor cores' side of 1024 keys; two planes leave the same error."""
+    test_few_rows(7, 1025, [0, 64, 600, 1000, 1023], 2, True, hd, 2)

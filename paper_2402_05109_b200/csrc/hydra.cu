@@ -630,11 +630,10 @@ hydra_status enqueue_step(hydra_ctx* c, int* n_acc, int* out_tok, cudaStream_t s
 void drop_graphs(hydra_ctx* c) { c->graphs.clear(); c->rows_graphs.clear(); }
 
 bool capturable(cudaStream_t st) { return st != nullptr && st != cudaStreamLegacy && st != cudaStreamPerThread; }      // default streams are not
-bool being_captured(cudaStream_t st) {
+hydra_status being_captured(cudaStream_t st, bool* captured) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
-  cudaGetLastError();                              // (the default stream while another one captures)
-  return true;
+  const cudaError_t asked = cudaStreamIsCapturing(st, &s);
+  return capture_answer(asked, s, captured);
 }
 // What `enqueue` puts on the stream, as a graph and not executed; *launches: kernels in it.
 template <typename F>
@@ -769,7 +768,9 @@ hydra_status hydra_prefill(hydra_ctx* c, int batch, const int32_t* tokens, const
   }
   po.off[batch] = offs[batch];
   // a prompt pass belongs to one request and its host-side bounds to one call: nothing to replay
-  if (being_captured(st)) { set_last_error("hydra_prefill on a stream under capture", cudaErrorStreamCaptureUnsupported); return HYDRA_ERR_CUDA; }
+  bool captured = false;
+  HYDRA_TRY(being_captured(st, &captured));
+  if (captured) { set_last_error("hydra_prefill on a stream under capture", cudaErrorStreamCaptureUnsupported); return HYDRA_ERR_CUDA; }
   c->batch = batch;
   HYDRA_TRY(set_prompts(po, batch, c->d_prompt_len, c->d_offsets, st));
   if (m.dtype == 1) {
@@ -815,7 +816,9 @@ hydra_status hydra_verify(hydra_ctx* c, const int32_t* tree_tok, int32_t* amax, 
   cudaStream_t st = (cudaStream_t)stream;
   hydra_ctx::RowsGraph* g = nullptr;
   // a stream that its owner is capturing takes the launches themselves
-  if (c->use_graph && capturable(st) && !c->timing && !being_captured(st)) {
+  bool captured = true;
+  if (c->use_graph && capturable(st) && !c->timing) HYDRA_TRY(being_captured(st, &captured));
+  if (!captured) {
     const std::pair<int, int> key(c->batch, len_bucket(c, max_len_ub(c) + c->T));
     g = &c->rows_graphs.at(key);
     if (!g->exec && ++g->calls >= VERIFY_CAPTURE_CALL) {

@@ -145,6 +145,17 @@ hydra_status accept_compact(const AcceptArgs& a, cudaStream_t st);
 cudaError_t accept_graph_node(cudaGraph_t graph, cudaGraphNode_t* node);
 cudaError_t accept_graph_update(cudaGraphExec_t exec, cudaGraphNode_t node, const AcceptArgs& a);
 
+// Whether a stream is being captured, from what cudaStreamIsCapturing answered.  The default stream cannot be used while another one captures: that counts as
+// captured.  Any other error is reported as it is.  Either way the runtime does not hand it to the next launch's check.
+inline hydra_status capture_answer(cudaError_t asked, cudaStreamCaptureStatus s, bool* captured) {
+  *captured = s != cudaStreamCaptureStatusNone;
+  if (asked == cudaSuccess) return HYDRA_OK;
+  cudaGetLastError();
+  if (asked == cudaErrorStreamCaptureImplicit) { *captured = true; return HYDRA_OK; }
+  set_last_error("cudaStreamIsCapturing", asked);
+  return HYDRA_ERR_CUDA;
+}
+
 // ---- small state kernels
 // prompt lengths and offsets of a batch, as kernel arguments: no copy from host memory, which would have to outlive the call
 constexpr int MAX_BATCH = 64;

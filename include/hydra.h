@@ -20,7 +20,7 @@
  *    carved out of the caller's workspace (hydra_workspace_bytes, 256-byte aligned base).
  *  - Calls enqueue work on `stream` (a cudaStream_t passed as void*) and do not synchronise, except
  *    hydra_create (uploads tables; synchronises the device), hydra_prefill of a bfloat16 model (synchronises the stream once,
- *    after uploading the blocks of its attention; not under stream capture), hydra_poll_status, hydra_get_timing and
+ *    after uploading the blocks of its attention), hydra_poll_status, hydra_get_timing and
  *    hydra_destroy.
  *  - Order: create -> prefill -> (draft -> verify -> accept_compact | step)*.  A call out of order
  *    returns HYDRA_ERR_STATE.  The host keeps an upper bound of every sequence length (it grows by
@@ -115,9 +115,11 @@ hydra_status hydra_destroy(hydra_ctx*);
  * prompt token) and the last hidden state.  tokens_dev holds the prompts back to back; seq_offsets_host
  * has batch+1 entries (read before the call returns).  The prompts are processed in passes, every pass
  * streaming the weights once: of up to 768 tokens of the prompts packed back to back (dtype 1), or of 64 rows per sequence
- * (dtype 0).  Synchronises the stream once (see Conventions).
+ * (dtype 0).  A bfloat16 model synchronises the stream once (see Conventions).  A prompt pass of either model cannot be
+ * captured: it depends on the prompt lengths, which the host reads.
  * Errors: INVALID (null pointer, batch outside 1..max_batch, empty prompt), CAPACITY (prompt + tree rows
- * exceed max_seq). */
+ * exceed max_seq), CUDA with nothing enqueued (the stream is under capture, or is the default stream while another one
+ * captures). */
 hydra_status hydra_prefill(hydra_ctx*, int batch, const int32_t* tokens_dev, const int32_t* seq_offsets_host,
                            void* stream);
 

@@ -221,25 +221,27 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
   const int d = m.d_model, f = m.d_ffn, V = m.vocab, K = h.n_heads, T = t.T;
   const int R = pad_rows(call_rows(m, T, K));
   const int RH = pad_rows(m.max_batch * std::max(t.maxP, h.medusa ? t.K : 1));      // (a Medusa draft projects the rows of all its heads together)
-  // largest partial-sum buffer over every GEMM shape and row count the library issues
+  // largest partial-sum buffer over every GEMM shape and row count the library issues; float: the logits of a verification, of a draft level or of the prompts
+  // (every other product of that path leaves its sums where they are wanted)
   size_t part_floats = 0;
-  {
+  if (m.dtype == 0) {
+    part_floats = (size_t)std::max(m.max_batch * T, RH) * V;
+  } else {
     auto need = [&](int mm, int n, int k) {
       int slots = 1;
-      if (m.dtype == 1) gemm_tc_plan(mm, n, k, nullptr, &slots);
+      gemm_tc_plan(mm, n, k, nullptr, &slots);
       part_floats = std::max(part_floats, (size_t)slots * mm * n);
     };
     const int shapes[][2] = {{3 * d, d}, {2 * d, d}, {d, d}, {2 * f, d}, {d, f}, {V, d}};
-    const int per_seq[] = {T, K + 1, 1, m.dtype == 1 ? 1 : CHUNK};
+    const int per_seq[] = {T, K + 1, 1};
     for (auto& sh : shapes) {
       // packed prompt passes have any row count; the plan depends on the count rounded up to 16 rows
-      if (m.dtype == 1) for (int rows = 16; rows <= PROMPT_ROWS; rows += 16) need(rows, sh[0], sh[1]);
+      for (int rows = 16; rows <= PROMPT_ROWS; rows += 16) need(rows, sh[0], sh[1]);
       for (int rows : per_seq)
         for (int bb = 1; bb <= m.max_batch; ++bb)
-          if (m.dtype != 1 || rows * bb > PROMPT_ROWS) need(rows * bb, sh[0], sh[1]);
+          if (rows * bb > PROMPT_ROWS) need(rows * bb, sh[0], sh[1]);
     }
-    const int g = m.dtype == 1 ? 16 : 1;
-    for (int mm = g; mm < RH + g; mm += g) {
+    for (int mm = 16; mm < RH + 16; mm += 16) {
       for (int i = 1; i <= K; ++i) need(mm, d, (i + 1) * d);
       need(mm, d, d);
       need(mm, V, d);
@@ -274,9 +276,9 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
   auto* hprime = b.take<float>((size_t)m.max_batch * d);
   auto* y = b.take<float>((size_t)RH * d); auto* head_logits = b.take<float>((size_t)RH * V);
   auto* rope = b.take<float2>((size_t)R * (m.head_dim / 2));
-  auto* xn = b.take<char>((size_t)np * R * d * es); auto* attn_out = b.take<char>((size_t)np * R * d * es);
+  auto* xn = b.take<char>(m.dtype == 1 ? (size_t)np * R * d * es : 0); auto* attn_out = b.take<char>((size_t)np * R * d * es);
   auto* act = b.take<char>((size_t)np * R * f * es);
-  auto* z = b.take<char>((size_t)np * RH * (K + 1) * d * es); auto* yb = b.take<char>((size_t)np * RH * d * es);
+  auto* z = b.take<char>(m.dtype == 1 ? (size_t)np * RH * (K + 1) * d * es : 0); auto* yb = b.take<char>((size_t)np * RH * d * es);
   const int topk_cap = std::max(R, RH);
   auto* topk_s = b.take<char>(topk_scratch_bytes(topk_cap, V));
   auto* att = b.take<char>(m.dtype == 0 ? attention_scratch_bytes(m.max_batch, CHUNK, m.n_heads, m.head_dim, m.max_seq) : 0);
@@ -384,7 +386,7 @@ hydra_status f32_layer(hydra_ctx* c, const LayerW& w, const float* src, char* kc
 }
 
 // Base model over the rows of `rs` whose tokens are tok[rows]: leaves post-final-norm hidden rows in c->h_tree
-// (float) and c->xn (operand type); with tail_w also the partial sums of xn @ tail_w^T (the LM head) in c->part (*tail_sd).
+// (float) and, on the bfloat16 path, c->xn (operand planes); with tail_w also the partial sums of their product with tail_w (the LM head) in c->part (*tail_sd).
 hydra_status run_base(hydra_ctx* c, const int* tok, const RowSet& rs, int len_upper, const void* tail_w, int tail_n, SplitDesc* tail_sd,
                       bool stable_lengths, cudaStream_t st) {
   const hydra_model_cfg& m = c->m;

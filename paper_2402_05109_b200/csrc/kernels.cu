@@ -11,26 +11,18 @@ namespace hydra {
 // SIMT GEMM of bfloat16 operands (the debug mode): out[m][n] = sum_k x[m][k] w[n][k].  One warp per output feature, MR rows per pass.
 // (Float operands: float_path.cu.)
 // ------------------------------------------------------------------------------------------------
-template <typename T> struct Vec4 { };
-template <> struct Vec4<float> {
-  static __device__ __forceinline__ void load(const float* p, float (&v)[4]) {
-    float4 t = *reinterpret_cast<const float4*>(p); v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w; }
-};
-template <> struct Vec4<bf16> {
-  static __device__ __forceinline__ void load(const bf16* p, float (&v)[4]) {
-    uint2 t = *reinterpret_cast<const uint2*>(p);
-    __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&t.x), b = *reinterpret_cast<__nv_bfloat162*>(&t.y);
-    v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b); }
-};
+__device__ __forceinline__ void load_bf16x4(const bf16* p, float (&v)[4]) {
+  uint2 t = *reinterpret_cast<const uint2*>(p);
+  __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162*>(&t.x), b = *reinterpret_cast<__nv_bfloat162*>(&t.y);
+  v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b);
+}
 
-// MR activation rows; KS warps share an output column (each every KS-th 512-byte piece of its weight row), 8 / KS columns per
-// block.  The small models of the float path spend their time in the chain launch -> loads -> reduction: the first WPRE weight
-// pieces of a lane are loaded before the wait for the preceding kernel (w_const: the weights of a context, which no kernel writes; a
-// stand-alone call's w may be the preceding kernel's result), the MR sums share one transposing reduction, and the
-// split keeps the activation loads of a lane to one or two rounds and fills the SMs (16 x 256 x 688: 10.5 us with one warp per
-// column, 32 blocks).
-template <typename T, int MR, int KS>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w,      // not __restrict__: such loads may be moved over the wait
+// MR activation rows; KS warps share an output column (each every KS-th piece of 128 weights of its row), 8 / KS columns per
+// block.  The first WPRE weight pieces of a lane are loaded before the wait for the preceding kernel (w_const: the weights of a context, which no
+// kernel writes; a stand-alone call's w may be the preceding kernel's result), the MR sums share one transposing reduction, and the
+// split keeps the activation loads of a lane to one or two rounds and fills the SMs.
+template <int MR, int KS>
+__global__ void __launch_bounds__(256) gemm_simt_kernel(const bf16* x, const bf16* w,      // not __restrict__: such loads may be moved over the wait
                                                         float* __restrict__ out, int m, int n, int k, int w_const) {
   constexpr int WPRE = 2;
   pdl_trigger();
@@ -38,12 +30,12 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w, 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int col = blockIdx.x * (8 / KS) + warp / KS, k0 = (warp % KS) * 128 + lane * 4;
   const int m0 = blockIdx.y * MR;
-  const T* wr = w + (size_t)min(col, n - 1) * k;
+  const bf16* wr = w + (size_t)min(col, n - 1) * k;
   float wv[WPRE][4];
   if (!w_const) pdl_wait();
 #pragma unroll
   for (int i = 0; i < WPRE; ++i)
-    if (k0 + i * KS * 128 < k) Vec4<T>::load(wr + k0 + i * KS * 128, wv[i]);
+    if (k0 + i * KS * 128 < k) load_bf16x4(wr + k0 + i * KS * 128, wv[i]);
   if (w_const) pdl_wait();
   float acc[MR];
 #pragma unroll
@@ -53,7 +45,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w, 
     for (int r = 0; r < MR; ++r) {
       const int row = m0 + r < m ? m0 + r : m - 1;
       float xv[4];
-      Vec4<T>::load(x + (size_t)row * k + kk, xv);
+      load_bf16x4(x + (size_t)row * k + kk, xv);
       acc[r] += wk[0] * xv[0] + wk[1] * xv[1] + wk[2] * xv[2] + wk[3] * xv[3];
     }
   };
@@ -62,7 +54,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w, 
     if (k0 + i * KS * 128 < k) step(k0 + i * KS * 128, wv[i]);
   for (int kk = k0 + WPRE * KS * 128; kk < k; kk += KS * 128) {
     float wk[4];
-    Vec4<T>::load(wr + kk, wk);
+    load_bf16x4(wr + kk, wk);
     step(kk, wk);
   }
   float s = warp_sum_multi<MR>(acc, lane);
@@ -79,26 +71,26 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* x, const T* w, 
   if (lane < MR && m0 + r < m && col < n) out[(size_t)(m0 + r) * n + col] = s;
 }
 
-template <typename T, int MR>
+template <int MR>
 static void launch_gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, bool w_const, cudaStream_t st) {
   const int groups = (m + MR - 1) / MR;
   auto go = [&](auto kernel, int ks) {
-    launch_pdl(kernel, dim3((n * ks + 7) / 8, groups), dim3(256), 0, st, (const T*)x, (const T*)w, out, m, n, k, (int)w_const);
+    launch_pdl(kernel, dim3((n * ks + 7) / 8, groups), dim3(256), 0, st, (const bf16*)x, (const bf16*)w, out, m, n, k, (int)w_const);
   };
   // warps per column: until there are two blocks per SM or a lane has one piece
   const int pieces = (k + 127) / 128, want = 2 * sm_count();
-  if (pieces >= 4 && (long)n * groups / 4 <= want) go(gemm_simt_kernel<T, MR, 4>, 4);
-  else if (pieces >= 2 && (long)n * groups / 8 <= want) go(gemm_simt_kernel<T, MR, 2>, 2);
-  else go(gemm_simt_kernel<T, MR, 1>, 1);
+  if (pieces >= 4 && (long)n * groups / 4 <= want) go(gemm_simt_kernel<MR, 4>, 4);
+  else if (pieces >= 2 && (long)n * groups / 8 <= want) go(gemm_simt_kernel<MR, 2>, 2);
+  else go(gemm_simt_kernel<MR, 1>, 1);
 }
 hydra_status gemm_simt(const void* x, const void* w, float* out, int m, int n, int k, int dtype, bool w_const, cudaStream_t st) {
   if (m <= 0 || n <= 0 || k <= 0 || (k & 3)) return HYDRA_ERR_UNSUPPORTED;
   if (((uintptr_t)x | (uintptr_t)w) & (dtype == 0 ? 15 : 7)) return HYDRA_ERR_INVALID;      // both are read four elements at a time
   if (dtype == 0) return f32_gemm((const float*)x, (const float*)w, out, m, n, k, w_const, st);
-  if (m == 1) launch_gemm_simt<bf16, 1>(x, w, out, m, n, k, w_const, st);
-  else if (m <= 4) launch_gemm_simt<bf16, 4>(x, w, out, m, n, k, w_const, st);
-  else if (m <= 8) launch_gemm_simt<bf16, 8>(x, w, out, m, n, k, w_const, st);
-  else launch_gemm_simt<bf16, 16>(x, w, out, m, n, k, w_const, st);
+  if (m == 1) launch_gemm_simt<1>(x, w, out, m, n, k, w_const, st);
+  else if (m <= 4) launch_gemm_simt<4>(x, w, out, m, n, k, w_const, st);
+  else if (m <= 8) launch_gemm_simt<8>(x, w, out, m, n, k, w_const, st);
+  else launch_gemm_simt<16>(x, w, out, m, n, k, w_const, st);
   HYDRA_LAUNCH_CHECK();
   return HYDRA_OK;
 }
@@ -148,7 +140,7 @@ hydra_status reduce_splits(const float* part, SplitDesc sd, float* out, int m, i
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
 template <> __device__ __forceinline__ float4 load4<bf16>(const bf16* p) {
-  float v[4]; Vec4<bf16>::load(p, v); return make_float4(v[0], v[1], v[2], v[3]);
+  float v[4]; load_bf16x4(p, v); return make_float4(v[0], v[1], v[2], v[3]);
 }
 // Four elements at an element boundary (VEC: at a boundary of four).
 template <bool VEC, typename T> __device__ __forceinline__ float4 load4_at(const T* p) {

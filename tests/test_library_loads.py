@@ -74,3 +74,25 @@ def test_weights_off_a_boundary_of_four_elements_are_refused():
     assert create() == 5 and create("head_b1", 4) == 5                    # past the checks, as far as the missing device
     for name in ("embed", "final_norm", "attn_norm", "ffn_norm", "pfx_attn_norm", "pfx_ffn_norm"):
         assert create(name, 4) == 1, name
+
+
+def test_workspace_of_a_float_model_holds_what_its_kernels_use():
+    """The float model's products leave their sums where they are wanted: no normed rows, no gathered head inputs, and partial sums for vocabulary projections only.
+    Sizes grow accordingly (256-byte steps aside; 64 sequences, so no row count is rounded up)."""
+    import ctypes as C
+    from paper_2402_05109_b200.binding import lib, HeadCfgC, ModelCfgC, TreeCfgC
+    B, S, V, T = 64, 64, 128, 2
+
+    def size(d=256, ffn=512, K=3):
+        n = lib.hydra_workspace_bytes(C.byref(ModelCfgC(1, d, d // 64, 64, ffn, V, 1e-6, 1e4, 0, B, S)), C.byref(HeadCfgC(K, 1, 0, 1)),
+                                      C.byref(TreeCfgC(T, (C.c_int32 * T)(-1, 0))))
+        assert n > 0
+        return n
+    R, RH, slack, base = 64 * B, B, 64 * 256, size()       # rows of a prompt pass and of a draft level
+    # activations after SiLU
+    assert size(ffn=4096) - base <= 4 * R * (4096 - 512) + slack
+    # hidden rows of the last step (and the tree's path table)
+    assert size(K=60) - base <= 4 * 57 * (B * 256 + T) + slack
+    # K and V; residual rows, q, hidden rows and attention output; last step's rows, h' and the heads' two row buffers; attention's partial rows
+    att = lib.hydra_attention_scratch_bytes(B, 64, 8, 64, S) - lib.hydra_attention_scratch_bytes(B, 64, 4, 64, S)
+    assert size(d=512) - base <= 4 * 256 * (2 * B * S + 4 * R + B * 4 + B + 2 * RH) + att + slack

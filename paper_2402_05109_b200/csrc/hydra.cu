@@ -276,9 +276,10 @@ size_t carve(hydra_ctx* c, const hydra_model_cfg& m, const hydra_head_cfg& h, co
   auto* hprime = b.take<float>((size_t)m.max_batch * d);
   auto* y = b.take<float>((size_t)RH * d); auto* head_logits = b.take<float>((size_t)RH * V);
   auto* rope = b.take<float2>((size_t)R * (m.head_dim / 2));
-  auto* xn = b.take<char>(m.dtype == 1 ? (size_t)np * R * d * es : 0); auto* attn_out = b.take<char>((size_t)np * R * d * es);
+  const int gathered = m.dtype == 1 ? 1 : 0;     // the float path's products read normed rows and head inputs where they are
+  auto* xn = b.take<char>((size_t)np * R * d * es * gathered); auto* attn_out = b.take<char>((size_t)np * R * d * es);
   auto* act = b.take<char>((size_t)np * R * f * es);
-  auto* z = b.take<char>(m.dtype == 1 ? (size_t)np * RH * (K + 1) * d * es : 0); auto* yb = b.take<char>((size_t)np * RH * d * es);
+  auto* z = b.take<char>((size_t)np * RH * (K + 1) * d * es * gathered); auto* yb = b.take<char>((size_t)np * RH * d * es);
   const int topk_cap = std::max(R, RH);
   auto* topk_s = b.take<char>(topk_scratch_bytes(topk_cap, V));
   auto* att = b.take<char>(m.dtype == 0 ? attention_scratch_bytes(m.max_batch, CHUNK, m.n_heads, m.head_dim, m.max_seq) : 0);

@@ -4,8 +4,8 @@
 // stores to the next one's loads, so what counts is how many there are.  Sums are whole here (no partial-sum slots), so the residual, SiLU and the
 // rotary embedding with the cache rows happen where they are formed; and a norm needs the rows that are read for the product anyway: their squares
 // are summed along, the gain goes to an operand and the row's factor to the sums.  A decoder layer is five launches (QKV with norm, rotation and cache rows; attention;
-// O with the residual; gate and up with norm and SiLU; down with the residual) where it was nine, a draft head's layer one where it was two or
-// three (gather, product, SiLU and residual).  Tiny float model (2 layers, d 256), a request of 32 tokens and 8 steps: 855 -> 655 us.
+// O with the residual; gate and up with norm and SiLU; down with the residual; a sixth where the attention adds its chunks up) where it was nine, a draft head's layer one where it was two or
+// three (gather, product, SiLU and residual).  Tiny float model (2 layers, d 256), a request of 32 tokens and 8 steps: 810 -> 577 us.
 //
 // Two forms.  Few rows or columns: a warp per output column (row_sums), so that a few hundred columns fill the SMs and the chain in a
 // warp is short.  Many: 32 x 32 tiles out of shared memory, since a warp per column reads every row again for every column: 512 rows, d 256, f 688: QKV 21 -> 14 us, gate

@@ -410,19 +410,31 @@ hydra_status launch(const CUtensorMap& tw, const CUtensorMap& tx, const GemmArgs
 
 bool gemm_tc_available() { return tensor_map_encoder_available(); }
 
-// Tile shape.  128 or 256 weight rows per unit, measured with the reduction of the partial sums (us; n x k):
-//  * units of 256 rows take enough of them for ~4 per SM: 2048 x 2048, 1 row: 4.8 (128) against 5.6 (256); 3072 x 3072: 8.4 / 7.6
-//  * up to 64 activation rows 256 (fewer activation bytes per weight byte, more weight bytes in flight): 22016 x 4096, 1 row: 32.1 /
-//    30.2, 64 rows: 42.2 / 42.4; 4096 x 11008, 1 row: 19.0 / 17.5, 64 rows: 20.9 / 20.3
-//  * above, 128 (tensor memory then holds two accumulators, and fewer partial sums are left): 12288 x 4096, 96 rows: 29.4 / 30.9;
-//    4096 x 4096, 128 rows: 16.0 / 19.0; 22016 x 4096, 192 rows: 77 / 82; except for
-//  * 97 to 160 rows of an output wide enough that a tile meets one or two ranges all the same (half as many tiles as SMs): the activation tile is twice the weight
-//    tile there, and an SM takes in a third less.  In a forward pass, 128 rows: 22016 x 4096 37.9 / 36.6, 32000 x 4096 54.0 / 51.1, 27648 x 5120 58.2 / 54.5,
-//    35840 x 6656 97.8 / 90.5, 19968 x 6656 56.8 / 54.1; 12288 x 4096 23.0 / 23.7, 6656 x 17920 with its norm 59.4 / 61.2; 80 rows 22016 x 4096 32.0 / 32.7.
-//    160 rows: 22016 x 4096 47.3 / 41.8, 32000 x 4096 66.8 / 56.5, 27648 x 5120 74.8 / 63.0, 35840 x 6656 127 / 105, 19968 x 6656 73.3 / 64.5; 129 rows 39.4 / 38.8,
-//    56.3 / 52.9, 63.0 / 58.8, 103 / 95, 60.8 / 57.9; 12288 x 4096 144 rows 25.0 / 25.6 (176 rows would have two stages: 192 rows 22016 x 4096 54.2 / 56.2); and for
-//  * tall row tiles with 16 and more units per SM, where the activation tile is most of what an SM takes in: 22016 x 4096, 256
-//    rows: 111 / 103, 512 rows: 222 / 192; 4096 x 11008, 512 rows: 96 / 91; but 4096 x 4096, 512 rows: 49 / 54
+// Tile shape: 128 or 256 weight rows per unit.
+//  * Units of 256 rows take enough of them for ~4 per SM.
+//  * Up to 64 activation rows 256: fewer activation bytes per weight byte, more weight bytes in flight.
+//  * Above, 128: tensor memory then holds two accumulators, and fewer partial sums are left.  Except for
+//  * 97 to 160 rows of an output wide enough that a tile meets one or two ranges all the same (half as many tiles as SMs): the activation tile is twice the
+//    weight tile there, and an SM takes in a third less (176 rows would have two stages); and for
+//  * tall row tiles with 16 and more units per SM, where the activation tile is most of what an SM takes in.
+// Measured, us with 128 / 256 weight rows.  With the reduction of the partial sums:
+//    rows  n x k                                      rows  n x k
+//       1  2048 x 2048     4.8 / 5.6                     1  3072 x 3072    8.4 / 7.6
+//       1  22016 x 4096   32.1 / 30.2                   64  22016 x 4096  42.2 / 42.4
+//       1  4096 x 11008   19.0 / 17.5                   64  4096 x 11008  20.9 / 20.3
+//      96  12288 x 4096   29.4 / 30.9                  128  4096 x 4096   16.0 / 19.0
+//     192  22016 x 4096     77 / 82                    256  22016 x 4096   111 / 103
+//     512  22016 x 4096    222 / 192                   512  4096 x 11008    96 / 91
+//     512  4096 x 4096      49 / 54
+// In a forward pass:
+//    rows  22016 x 4096  32000 x 4096  27648 x 5120  35840 x 6656  19968 x 6656  12288 x 4096
+//      80  32.0 / 32.7
+//     128  37.9 / 36.6   54.0 / 51.1   58.2 / 54.5   97.8 / 90.5   56.8 / 54.1   23.0 / 23.7
+//     129  39.4 / 38.8   56.3 / 52.9   63.0 / 58.8    103 / 95     60.8 / 57.9
+//     144                                                                        25.0 / 25.6
+//     160  47.3 / 41.8   66.8 / 56.5   74.8 / 63.0    127 / 105    73.3 / 64.5
+//     192  54.2 / 56.2
+//    6656 x 17920 with its norm, 128 rows: 59.4 / 61.2
 struct GemmShape { int nh, mt, m_tiles; };
 static GemmShape gemm_shape(int m, int n, int k) {
   // equal row tiles of a multiple of 16 rows, so that the MMA work and the activation traffic follow m
